@@ -51,8 +51,20 @@ constexpr int kPLight = 128;
 constexpr int kPHeavySlots = 4096;  // per-block shared table (degree <= 2048); larger: global
 constexpr int kPSortSmem = 2048;    // overflow sets sorted in shared memory up to this size
 constexpr int kPBuckets = 4096;     // few-label overflow: priority buckets (top 12 bits)
+constexpr int kPScan = 8;           // few-label overflow: keys of the set in flight per thread
 constexpr int kPCross = 1024;       // few-label overflow: crossing-bucket entries kept in shared memory
-constexpr int kPFewLabels = 256;    // labels up to this count: per-target overflow resolution
+// overflow sets above kPSortOne entries with at most kPFewLabels labels are resolved one target per block
+// (every block reads the whole set, so more labels than a few per block would not pay); smaller sets are
+// sorted by one block in shared memory
+constexpr int kPFewLabels = 1024;
+constexpr int kPSortOne = 1024;
+// 2.5x cap: digits of the radix select (11 bits from the top), and the keys left at which the
+// remaining ones are listed and ranked directly
+constexpr int kPCapBits = 11;
+constexpr int kPCapBins = 1 << kPCapBits;
+constexpr int kPCapPasses = 6;
+constexpr int kPCapList = 256;
+constexpr int kPPropBuf = 32;       // proposals a warp collects before it takes list slots for them
 constexpr int kPAggLabels = 4096;   // labels up to this count: weight updates aggregated per block
 constexpr int kPWeightSmem = 1024;  // refinement with labels up to this count: weights in shared memory
 constexpr int kPKeys = 64 * 4;      // (sub-round, degree class) lists of a round
@@ -69,8 +81,8 @@ constexpr int kPKeys = 64 * 4;      // (sub-round, degree class) lists of a roun
 struct PCount {
   int nprop, nheavy, nov, ecount;
   long long delta, moved;
-  int touched;  // few-label overflow: at least one entry seen (unused otherwise)
-  int pad;
+  int over;     // some target's incoming weight exceeds its room
+  int nleft;    // cap: keys listed for the direct ranking
 };
 
 struct PResult {
@@ -105,7 +117,8 @@ struct PArgs {
   int32_t *depw;         // [nlabels] clustering: weight leaving a cluster, zero between sub-rounds
   unsigned long long *dkey;  // [nlabels] clustering: latest departure key, zero between sub-rounds
   uint64_t *ekeys;       // [n] emptying keys
-  unsigned *chist;       // [8][256] cap select histograms
+  unsigned *chist;       // [kPCapPasses][kPCapBins] cap select histograms
+  uint64_t *cleft;       // [kPCapList] cap select: the keys of the last digit's bin
   int32_t *gtk, *gtv;    // per-block global tables for heavy nodes beyond kPHeavySlots
   int64_t gstride;
   int hblocks;           // the first hblocks blocks rate the heavy nodes (one table each)
@@ -176,11 +189,38 @@ __device__ __forceinline__ uint64_t pkey(uint64_t kprio, int v) {
   return ((uint64_t)h32(kprio, (uint32_t)v, 0) << 32) | (uint32_t)v;
 }
 
-// Appends one proposal (lane 0 of the rating warp / thread 0 of the rating block).
+// Adds a proposal's weight to its target.  The additions to a target see every partial total, the last
+// one the full one, so the sub-round's overflow flag is raised iff some target's total does not fit.
+__device__ __forceinline__ void add_incoming(const PArgs &a, PCount *c, int K, int cv, int wK) {
+  const int before = atomicAdd(&a.incoming[K], cv);
+  if ((int64_t)wK + before + cv > a.bound) *(volatile int *)&c->over = 1;
+}
+
+// Appends one proposal (thread 0 of the rating block).
 __device__ __forceinline__ void propose(const PArgs &a, PCount *c, int v, int K, int own, int cv) {
   const int i = atomicAdd(&c->nprop, 1);
   a.prop[i] = make_int4(v, K, own, cv);
-  atomicAdd(&a.incoming[K], cv);
+  add_incoming(a, c, K, cv, a.weight[K]);
+}
+
+// A warp's proposals are collected in shared memory and take their places in the list 32 at a time:
+// one add to the list length per 32 proposals instead of one each (all warps add to the same word,
+// and such adds are served one after another).
+struct PropBuf {
+  int4 *buf;
+  int cnt;
+};
+
+__device__ __forceinline__ void flush_props(const PArgs &a, PCount *c, PropBuf &b) {
+  if (b.cnt == 0) return;
+  const int lane = (int)lane_id();
+  int base = 0;
+  if (lane == 0) base = atomicAdd(&c->nprop, b.cnt);
+  base = __shfl_sync(FULL, base, 0);
+  __syncwarp();
+  if (lane < b.cnt) a.prop[base + lane] = b.buf[lane];
+  __syncwarp();
+  b.cnt = 0;
 }
 
 // Best candidate over a rating table (keys tk, sums tv, `size` slots) walked by
@@ -292,7 +332,7 @@ __device__ void bitonic(uint64_t *k, uint32_t *v, int32_t *ix, int P) {
 template <int G, int E>
 __device__ __forceinline__ void rate_list(const PArgs &a, PCount *c, const int32_t *list, int count, int gw,
                                           int nw, int *tk, int *tv, uint64_t ktie, const int *s_wl,
-                                          unsigned long long &ue, unsigned long long &uv) {
+                                          PropBuf &pb, unsigned long long &ue, unsigned long long &uv) {
   constexpr int NV = 32 / G;
   constexpr int TS = GroupTable<G, E>::TS;
   static_assert(NV * TS <= kPSlots, "table size");
@@ -314,10 +354,20 @@ __device__ __forceinline__ void rate_list(const PArgs &a, PCount *c, const int32
     const unsigned best = rate_group<G, E, false>(a.adjncy, a.adjwgt, a.label, a.label8, a.weight, s_wl, a.bound,
                                                   ktie, v, st, deg, own, cv, tk + grp * TS, tv + grp * TS, gmask,
                                                   gl, false, nc, stable);
-    if (gl == 0 && v >= 0) {
+    const bool mine = gl == 0 && v >= 0;
+    const bool prop = mine && best != 0xFFFFFFFFu;
+    const unsigned pm = __ballot_sync(FULL, prop);
+    if (pm) {
+      if (pb.cnt + __popc(pm) > kPPropBuf) flush_props(a, c, pb);
+      if (prop) {
+        pb.buf[pb.cnt + __popc(pm & lanemask_lt())] = make_int4(v, (int)best, own, cv);
+        add_incoming(a, c, (int)best, cv, s_wl ? s_wl[best] : a.weight[best]);
+      }
+      pb.cnt += __popc(pm);
+    }
+    if (mine) {
       ue += deg;
       uv += 1;
-      if (best != 0xFFFFFFFFu) propose(a, c, v, (int)best, own, cv);
       if (a.dirty && stable) a.dirty[v] = 0;
     }
   }
@@ -339,7 +389,8 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
   __shared__ int s_ri[kPWarps];
   __shared__ uint64_t s_ru[kPWarps];
   __shared__ long long s_ll[kPWarps];
-  __shared__ unsigned s_h[256];
+  __shared__ int s_dig, s_binc;
+  __shared__ long long s_rank;
   __shared__ int s_bc[kPKeys], s_bb[kPKeys], s_bo[kPKeys + 1];
   __shared__ int s_wl[kPWeightSmem];
 
@@ -439,7 +490,7 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
       if (blockIdx.x == 0 && threadIdx.x == 0) {
         PCount *nx = a.cnt + ((subs + 1) % 3);
         nx->nprop = 0; nx->nheavy = 0; nx->nov = 0; nx->ecount = 0;
-        nx->delta = 0; nx->moved = 0; nx->touched = 0;
+        nx->delta = 0; nx->moved = 0; nx->over = 0; nx->nleft = 0;
       }
       // ---------------------------------------------------------- rate
       const int32_t *lo = a.boffs + (r & 1) * (kPKeys + 1) + s * 4;  // this sub-round's four lists
@@ -497,13 +548,23 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
       }
       {
         const int *wl = few_w ? s_wl : nullptr;
-        rate_list<32, 4>(a, c, a.blist + lo[2], lo[3] - lo[2], gw, nw, tk, tv, ktie, wl, ue, uv);
-        rate_list<32, 1>(a, c, a.blist + lo[1], lo[2] - lo[1], gw, nw, tk, tv, ktie, wl, ue, uv);
-        rate_list<8, 1>(a, c, a.blist + lo[0], lo[1] - lo[0], gw, nw, tk, tv, ktie, wl, ue, uv);
+        // the proposal buffers lie behind the heavy nodes' tables in the shared area
+        PropBuf pb{reinterpret_cast<int4 *>(area + sizeof(int) * 2 * kPHeavySlots) + wib * kPPropBuf, 0};
+        rate_list<32, 4>(a, c, a.blist + lo[2], lo[3] - lo[2], gw, nw, tk, tv, ktie, wl, pb, ue, uv);
+        rate_list<32, 1>(a, c, a.blist + lo[1], lo[2] - lo[1], gw, nw, tk, tv, ktie, wl, pb, ue, uv);
+        rate_list<8, 1>(a, c, a.blist + lo[0], lo[1] - lo[0], gw, nw, tk, tv, ktie, wl, pb, ue, uv);
+        flush_props(a, c, pb);
       }
       if (!grid_sync(a)) return;
-      // -------------------------------------------------------- decide
       const int nprop = *(volatile int *)&c->nprop;
+      if (nprop == 0) {  // nothing to decide or apply: on to the next sub-round
+        subs++;
+        continue;
+      }
+      // -------------------------------------------------------- decide
+      // when no target overflows every proposal is accepted, and there is nothing to decide
+      const bool over_any = *(volatile int *)&c->over != 0;
+      if (over_any) {
       for (int b0 = blockIdx.x * blockDim.x; b0 < nprop; b0 += gthreads) {
         const int i = b0 + (int)threadIdx.x;
         bool over = false;
@@ -522,10 +583,11 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
         }
       }
       if (!grid_sync(a)) return;
+      }
       // ------------------------------------------------------ overflow
-      const int nov = *(volatile int *)&c->nov;
+      const int nov = over_any ? *(volatile int *)&c->nov : 0;
       if (nov > 0) {
-        if (few) {
+        if (few && nov > kPSortOne) {
           // per target: weighted histogram over the top 12 priority bits finds the
           // bucket where the running weight passes the room; only that bucket's
           // entries are ranked exactly
@@ -539,11 +601,20 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
             for (int q = threadIdx.x; q < kPBuckets; q += blockDim.x) hist[q] = 0;
             if (threadIdx.x == 0) { s_any = 0; s_nx = 0; }
             __syncthreads();
-            for (int j = threadIdx.x; j < nov; j += blockDim.x) {
-              const uint64_t k = a.ovk[j];
-              if ((int)(k >> 32) != t) continue;
-              atomicAdd((unsigned long long *)&hist[(uint32_t)k >> 20], (unsigned long long)a.vwgt[a.ovv[j]]);
-              s_any = 1;
+            for (int j0 = threadIdx.x; j0 < nov; j0 += blockDim.x * kPScan) {  // kPScan keys in flight
+              uint64_t k[kPScan];
+#pragma unroll
+              for (int q = 0; q < kPScan; q++) {
+                const int j = j0 + q * kPThreads;
+                k[q] = j < nov ? a.ovk[j] : ~0ull;
+              }
+#pragma unroll
+              for (int q = 0; q < kPScan; q++) {
+                if ((int)(k[q] >> 32) != t) continue;
+                atomicAdd((unsigned long long *)&hist[(uint32_t)k[q] >> 20],
+                          (unsigned long long)a.vwgt[a.ovv[j0 + q * kPThreads]]);
+                s_any = 1;
+              }
             }
             __syncthreads();
             if (!s_any) continue;
@@ -577,19 +648,29 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
             }
             __syncthreads();
             const int cross = s_cross;
-            for (int j = threadIdx.x; j < nov; j += blockDim.x) {
-              const uint64_t k = a.ovk[j];
-              if ((int)(k >> 32) != t) continue;
-              const int bk = (int)((uint32_t)k >> 20);
-              if (bk != cross) {
-                a.acc[a.ovi[j]] = bk < cross ? 1 : 0;
-                continue;
+            for (int j0 = threadIdx.x; j0 < nov; j0 += blockDim.x * kPScan) {
+              uint64_t k8[kPScan];
+#pragma unroll
+              for (int q = 0; q < kPScan; q++) {
+                const int j = j0 + q * kPThreads;
+                k8[q] = j < nov ? a.ovk[j] : ~0ull;
               }
-              const int x = atomicAdd(&s_nx, 1);
-              if (x < kPCross) {
-                xk[x] = ((uint64_t)(uint32_t)k << 32) | a.ovv[j];
-                xc[x] = a.vwgt[a.ovv[j]];
-                xi[x] = a.ovi[j];
+#pragma unroll
+              for (int q = 0; q < kPScan; q++) {
+                const uint64_t k = k8[q];
+                const int j = j0 + q * kPThreads;
+                if ((int)(k >> 32) != t) continue;
+                const int bk = (int)((uint32_t)k >> 20);
+                if (bk != cross) {
+                  a.acc[a.ovi[j]] = bk < cross ? 1 : 0;
+                  continue;
+                }
+                const int x = atomicAdd(&s_nx, 1);
+                if (x < kPCross) {
+                  xk[x] = ((uint64_t)(uint32_t)k << 32) | a.ovv[j];
+                  xc[x] = a.vwgt[a.ovv[j]];
+                  xi[x] = a.ovi[j];
+                }
               }
             }
             __syncthreads();
@@ -673,19 +754,18 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
       if (a.count_clusters && (long long)nprop > ncl - a.n_min) {
         const long long D = ncl - a.n_min;
         for (int i = gt; i < nprop; i += gthreads) {
-          if (!a.acc[i]) continue;
+          if (over_any && !a.acc[i]) continue;
           const int4 p = a.prop[i];
           atomicAdd(&a.depw[p.z], p.w);
           atomicMax(&a.dkey[p.z], (unsigned long long)pkey(kprio, p.x));
         }
-        if (blockIdx.x == 0)
-          for (int q = threadIdx.x; q < 8 * 256; q += blockDim.x) a.chist[q] = 0;
+        for (int q = gt; q < kPCapPasses * kPCapBins; q += gthreads) a.chist[q] = 0;
         if (!grid_sync(a)) return;
         for (int b0 = blockIdx.x * blockDim.x; b0 < nprop; b0 += gthreads) {
           const int i = b0 + (int)threadIdx.x;
           bool emit_key = false;
           uint64_t key = 0;
-          if (i < nprop && a.acc[i]) {
+          if (i < nprop && (!over_any || a.acc[i])) {
             const int4 p = a.prop[i];
             key = pkey(kprio, p.x);
             emit_key = a.depw[p.z] == a.weight[p.z] && key == a.dkey[p.z];
@@ -697,36 +777,79 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
         const int E = *(volatile int *)&c->ecount;
         // the per-cluster departure state is cleared for the next sub-round
         for (int i = gt; i < nprop; i += gthreads) {
-          if (!a.acc[i]) continue;
+          if (over_any && !a.acc[i]) continue;
           const int own = a.prop[i].z;
           a.depw[own] = 0;
           a.dkey[own] = 0;
         }
         if (E > D) {
-          // MSD radix select of the (D+1)-th smallest emptying key, 8 bits per pass
+          // MSD radix select of the (D+1)-th smallest emptying key, 11 bits per pass; once few keys
+          // share the prefix (after two passes, as a rule: the upper half of a key is a hash) they
+          // are listed and every block ranks them
+          unsigned *s_h = reinterpret_cast<unsigned *>(area);  // [kPCapBins]
+          constexpr int PER = kPCapBins / kPThreads;
           uint64_t prefix = 0, mask = 0;
-          long long rank = D;
-          for (int pass = 0; pass < 8; pass++) {
-            const int shift = 56 - 8 * pass;
-            for (int q = threadIdx.x; q < 256; q += blockDim.x) s_h[q] = 0;
+          long long rank = D, left = E;
+          for (int pass = 0; pass < kPCapPasses && left > kPCapList; pass++) {
+            const int shift = max(0, 64 - kPCapBits * (pass + 1));
+            const unsigned dmask = pass == kPCapPasses - 1 ? (1u << (64 - kPCapBits * pass)) - 1u : kPCapBins - 1u;
+            for (int q = threadIdx.x; q < kPCapBins; q += blockDim.x) s_h[q] = 0;
             __syncthreads();
             for (int i = gt; i < E; i += gthreads) {
               const uint64_t key = a.ekeys[i];
-              if ((key & mask) == prefix) atomicAdd(&s_h[(key >> shift) & 255u], 1u);
+              if ((key & mask) == prefix) atomicAdd(&s_h[(unsigned)(key >> shift) & dmask], 1u);
             }
             __syncthreads();
-            for (int q = threadIdx.x; q < 256; q += blockDim.x)
-              if (s_h[q]) atomicAdd(&a.chist[pass * 256 + q], s_h[q]);
+            for (int q = threadIdx.x; q < kPCapBins; q += blockDim.x)
+              if (s_h[q]) atomicAdd(&a.chist[pass * kPCapBins + q], s_h[q]);
             if (!grid_sync(a)) return;
-            const volatile unsigned *hh = a.chist + pass * 256;
-            int d = 0;
-            for (; d < 255; d++) {
-              const long long x = hh[d];
-              if (rank < x) break;
-              rank -= x;
+            // the digit whose bin holds the rank: a block scan over the bins, PER per thread
+            const volatile unsigned *hh = a.chist + pass * kPCapBins + threadIdx.x * PER;
+            unsigned bin[PER];
+            long long loc = 0;
+#pragma unroll
+            for (int q = 0; q < PER; q++) { bin[q] = hh[q]; loc += bin[q]; }
+            long long tot;
+            long long run = block_incl_scan(loc, s_ll, tot) - loc;
+            if (rank >= run && rank < run + loc) {  // exactly one thread: the bins hold more than `rank` keys
+#pragma unroll
+              for (int q = 0; q < PER; q++) {
+                if (rank >= run && rank < run + bin[q]) {
+                  s_dig = (int)threadIdx.x * PER + q;
+                  s_rank = run;
+                  s_binc = (int)bin[q];
+                }
+                run += bin[q];
+              }
             }
-            prefix |= (uint64_t)d << shift;
-            mask |= (uint64_t)255 << shift;
+            __syncthreads();
+            rank -= s_rank;
+            left = s_binc;
+            prefix |= (uint64_t)(unsigned)s_dig << shift;
+            mask |= (uint64_t)dmask << shift;
+            __syncthreads();
+          }
+          if (left > 1 || mask != ~0ull) {
+            for (int b0 = blockIdx.x * blockDim.x; b0 < E; b0 += gthreads) {
+              const int i = b0 + (int)threadIdx.x;
+              const uint64_t key = i < E ? a.ekeys[i] : 0;
+              const bool in = i < E && (key & mask) == prefix;
+              const int pos = warp_append(&c->nleft, in);
+              if (in) a.cleft[pos] = key;
+            }
+            if (!grid_sync(a)) return;
+            uint64_t *s_left = reinterpret_cast<uint64_t *>(area);
+            const int nl = (int)left;
+            for (int q = threadIdx.x; q < nl; q += blockDim.x) s_left[q] = *(volatile uint64_t *)&a.cleft[q];
+            __syncthreads();
+            for (int q = threadIdx.x; q < nl; q += blockDim.x) {
+              int below = 0;  // keys are distinct
+              for (int y = 0; y < nl; y++) below += s_left[y] < s_left[q] ? 1 : 0;
+              if (below == (int)rank) s_ru[0] = s_left[q];
+            }
+            __syncthreads();
+            prefix = s_ru[0];
+            __syncthreads();
           }
           cutoff = prefix;
           capped++;
@@ -742,7 +865,7 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
       for (int i = gt; i < nprop; i += gthreads) {
         const int4 p = a.prop[i];
         a.incoming[p.y] = 0;
-        if (!a.acc[i]) continue;
+        if (over_any && !a.acc[i]) continue;
         if (cutoff != ~0ull && pkey(kprio, p.x) >= cutoff) continue;
         a.label[p.x] = p.y;
         if (a.label8) a.label8[p.x] = (uint8_t)p.y;
@@ -763,7 +886,7 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
       }
       if (a.dirty) {  // every applied move marks its node and the node's neighbours, a warp per move
         for (int i = gw; i < nprop; i += nw) {
-          if (!a.acc[i]) continue;
+          if (over_any && !a.acc[i]) continue;
           const int v = a.prop[i].x;
           if (cutoff != ~0ull && pkey(kprio, v) >= cutoff) continue;
           const int e0 = a.xadj[v], e1 = a.xadj[v + 1];
@@ -811,7 +934,8 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
 
 constexpr size_t kAreaBytes() {
   // the largest phase use of the shared area
-  size_t heavy = sizeof(int) * 2 * kPHeavySlots;
+  size_t heavy = sizeof(int) * 2 * kPHeavySlots + sizeof(int4) * kPWarps * kPPropBuf;
+  size_t cap = sizeof(unsigned) * kPCapBins;
   size_t sort = (sizeof(uint64_t) + sizeof(uint32_t) + sizeof(int32_t) + sizeof(long long)) * kPSortSmem;
   size_t fewb = sizeof(long long) * kPBuckets + (sizeof(uint64_t) + 2 * sizeof(int)) * kPCross;
   size_t aggb = sizeof(int) * kPAggLabels;
@@ -819,6 +943,7 @@ constexpr size_t kAreaBytes() {
   m = sort > m ? sort : m;
   m = fewb > m ? fewb : m;
   m = aggb > m ? aggb : m;
+  m = cap > m ? cap : m;
   return m;
 }
 
@@ -875,11 +1000,14 @@ LpResult lp_run_small(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *w
   DBuf<int32_t> depw;
   DBuf<unsigned long long> dkey;
   DBuf<uint64_t> ekeys;
-  DBuf<unsigned> chist(ctx, 8 * 256);
+  DBuf<unsigned> chist;
+  DBuf<uint64_t> cleft;
   if (p.count_clusters) {
     depw.reset(ctx, (size_t)nlabels);
     dkey.reset(ctx, (size_t)nlabels);
     ekeys.reset(ctx, (size_t)n);
+    chist.reset(ctx, kPCapPasses * kPCapBins);
+    cleft.reset(ctx, kPCapList);
     depw.zero();
     dkey.zero();
   }
@@ -931,6 +1059,7 @@ LpResult lp_run_small(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *w
   a.bcnt = bcnt.get(); a.bfill = bfill.get(); a.boffs = boffs.get();
   a.ovk = ovk.get(); a.ovv = ovv.get(); a.ovi = ovi.get(); a.ovps = ovps.get(); a.cap2 = cap2;
   a.depw = depw.get(); a.dkey = dkey.get(); a.ekeys = ekeys.get(); a.chist = chist.get();
+  a.cleft = cleft.get();
   a.gtk = gtk.get(); a.gtv = gtv.get(); a.gstride = gstride; a.hblocks = hblocks;
   a.cnt = dc->cnt; a.bar = dc->bar; a.status = &dc->status;
   a.spin_cap = ctx->wait_spins > 0 ? ctx->wait_spins : (ctx->wait_spins == 0 ? kDefaultWaitSpins : -1);
