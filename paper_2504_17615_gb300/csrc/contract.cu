@@ -6,9 +6,9 @@
 //  reserve: every fine node reserves room for its row inside its coarse
 //           node's segment (an atomic add on the segment length returns the
 //           node's offset) and adds its weight to the coarse node;
-//  map    : warps walk 32 consecutive fine rows at a time (one contiguous
-//           range of entries) and write (coarse id of the neighbour, weight)
-//           into the owner's segment; entries inside the cluster are marked;
+//  map    : the fine entries are split evenly over the warps (EntryWalk),
+//           which write (coarse id of the neighbour, weight) into the owner's
+//           segment; entries inside the cluster are marked;
 //  merge  : each segment is summed by coarse neighbour in a hash table (a
 //           warp with a shared-memory table up to 256 entries, a block with
 //           a 4096-slot shared or a global table above) and written back in
@@ -70,19 +70,14 @@ __global__ void __launch_bounds__(kThreads) k_map(const int32_t *xadj, const int
   const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int nw = (int)((gridDim.x * blockDim.x) >> 5);
   unsigned long long ue = 0;
-  for (int64_t u0 = (int64_t)wid * 32; u0 < n; u0 += (int64_t)nw * 32) {
-    const int64_t u = u0 + lane;
-    const bool valid = u < n;
-    int xs = 0, xe = 0x7FFFFFFF, A = -2, base = 0;
-    if (valid) {
-      xs = xadj[u];
-      xe = xadj[u + 1];
+  for (EntryWalk wk(xadj, n, wid, nw); wk.next();) {
+    const int64_t u = wk.u0 + lane;
+    int A = -2, base = 0;
+    if (u < n) {
       A = cmap[u];
-      base = tstart[A] + moff[u] - xs;
+      base = tstart[A] + moff[u] - xadj[u];
     }
-    const int e0 = __shfl_sync(FULL, xs, 0);
-    const int last = (int)((n - u0) < 32 ? (n - u0) : 32) - 1;
-    const int e1 = __shfl_sync(FULL, xe, last);
+    const int e0 = wk.e0, e1 = wk.e1;
     if (lane == 0) ue += (unsigned long long)(e1 - e0);
     // kMapUnroll entries per lane in flight: ids, then coarse ids, then the writes
     for (int f0 = e0; f0 < e1; f0 += 32 * kMapUnroll) {
@@ -90,12 +85,7 @@ __global__ void __launch_bounds__(kThreads) k_map(const int32_t *xadj, const int
 #pragma unroll
       for (int r = 0; r < kMapUnroll; r++) {
         e[r] = f0 + r * 32 + lane;
-        int j = 0;  // owner: lanes whose row ends at or before e
-#pragma unroll
-        for (int step = 16; step > 0; step >>= 1) {
-          const int val = __shfl_sync(FULL, xe, j + step - 1);
-          if (val <= e[r]) j += step;
-        }
+        const int j = wk.owner(e[r]);
         bj[r] = __shfl_sync(FULL, base, j);
         Aj[r] = __shfl_sync(FULL, A, j);
       }
@@ -281,8 +271,8 @@ void contract_graph(gp_ctx *ctx, const DevGraph &g, const int32_t *cmap, int32_t
   }
   {
     ProfScope ps(ctx, PROF_CONTRACT);
-    if (n > 0) {
-      k_map<<<grid_for((int64_t)n, kThreads, ctx->num_sms * 16), kThreads, 0, ctx->stream>>>(
+    if (g.m2 > 0) {
+      k_map<<<walk_grid(g.m2, ctx->num_sms), kThreads, 0, ctx->stream>>>(
           g.xadj, g.adjncy, g.unit_w ? nullptr : g.adjwgt, cmap, moff.get(), tstart.get(), n, temp.get(), units);
       GP_LAUNCH_CHECK();
     }

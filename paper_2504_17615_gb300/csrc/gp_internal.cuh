@@ -360,6 +360,74 @@ __device__ __forceinline__ int row_of(const int32_t *xadj, int n, int64_t e) {
   return lo;
 }
 
+// A walk of one warp over its share of a graph's CSR entries, 32 consecutive rows (a window) at a
+// time.  The entries are split evenly over the warps, not the rows: with 32 rows per warp step one warp
+// walked a hub's whole row (4e5 entries of the scale-24 R-MAT graph) while the rest of the device
+// waited.  One search per warp (32 probes a step) finds the first row; a window without entries (a long
+// run of empty rows) is left by another search.
+//
+//   for (EntryWalk w(xadj, n, wid, nw); w.next(); )
+//     entries [w.e0, w.e1) lie in rows [w.u0, w.u0 + 32); lane i's row ends at w.xe (INT_MAX past n)
+struct EntryWalk {
+  const int32_t *xadj;
+  int n;
+  int64_t pos, end;  // entries still to walk
+  int64_t u0, row;   // this window's first row, the next one's
+  int e0, e1, xe;
+  __device__ __forceinline__ EntryWalk(const int32_t *x, int nn, int wid, int nw) : xadj(x), n(nn) {
+    const int64_t lo = nn > 0 ? x[0] : 0, hi = nn > 0 ? x[nn] : 0;
+    const int64_t per = (((hi - lo + nw - 1) / nw) + 31) & ~(int64_t)31;
+    pos = lo + per * wid;
+    end = pos + per < hi ? pos + per : hi;
+    row = pos < end ? find(pos) : 0;
+    u0 = 0; e0 = e1 = xe = 0;
+  }
+  __device__ __forceinline__ bool next() {
+    while (pos < end) {
+      u0 = row;
+      const int64_t u = u0 + lane_id();
+      xe = u < n ? xadj[u + 1] : 0x7FFFFFFF;
+      const int last = (int)((n - u0) < 32 ? (n - u0) : 32) - 1;
+      const int64_t wend = __shfl_sync(0xFFFFFFFFu, xe, last);
+      if (wend <= pos) {  // nothing here: jump
+        row = find(pos);
+        continue;
+      }
+      e0 = (int)pos;
+      e1 = (int)(wend < end ? wend : end);
+      pos = e1;
+      row = u0 + 32;
+      return true;
+    }
+    return false;
+  }
+  // Row of entry e (xadj[0] <= e < xadj[n]); the whole warp asks for the same e.
+  __device__ __forceinline__ int64_t find(int64_t e) const {
+    int64_t a = 0, b = n;  // xadj[a] <= e < xadj[b]
+    while (b - a > 1) {
+      const int64_t step = (b - a + 32) / 33, p = a + (int64_t)(lane_id() + 1) * step;
+      const unsigned m = __ballot_sync(0xFFFFFFFFu, p < b && (int64_t)xadj[p] <= e);
+      a += step * __popc(m);
+      b = a + step < b ? a + step : b;
+    }
+    return a;
+  }
+  // Lane index of the row that holds entry e: the lanes whose row ends at or before e.
+  __device__ __forceinline__ int owner(int e) const {
+    int q = 0;
+#pragma unroll
+    for (int step = 16; step > 0; step >>= 1) {
+      const int val = __shfl_sync(0xFFFFFFFFu, xe, q + step - 1);
+      if (val <= e) q += step;
+    }
+    return q;
+  }
+};
+
+// Blocks of 256 threads for an EntryWalk over m2 entries: at least 2048 entries a warp, so that the
+// search for its first row stays a small part, and at most 16 blocks an SM.
+inline int walk_grid(int64_t m2, int num_sms) { return grid_for(m2, 8 * 2048, num_sms * 16); }
+
 // ---------------------------------------------------------- primitives
 
 // Exclusive prefix sum of n values; total (device pointer, may be null)

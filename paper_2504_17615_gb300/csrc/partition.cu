@@ -49,8 +49,8 @@ __device__ __forceinline__ unsigned long long pair_hash(uint32_t lo, uint32_t hi
 // increasing rows, and symmetry by comparing, over the entries below and
 // above the diagonal, their counts and the sums of a 64-bit hash of
 // (min, max, weight) (equal sums unless the graph is asymmetric, up to a
-// 2^-64 collision).  Runs after the row offsets were checked; a warp walks 32
-// consecutive rows (one contiguous range of entries) at a time.
+// 2^-64 collision).  Runs after the row offsets were checked.  The entries are
+// split evenly over the warps (EntryWalk).
 constexpr int kValUnroll = 4;
 
 __global__ void __launch_bounds__(256) k_validate_entries(const int32_t *xadj, const int32_t *adjncy,
@@ -61,25 +61,18 @@ __global__ void __launch_bounds__(256) k_validate_entries(const int32_t *xadj, c
   const int nw = (int)((gridDim.x * blockDim.x) >> 5);
   int err = 0;
   unsigned long long ws = 0, hlo = 0, hhi = 0, nlo = 0, nhi = 0;
-  for (int64_t u0 = (int64_t)wid * 32; u0 < n; u0 += (int64_t)nw * 32) {
-    const int64_t u = u0 + lane;
-    const bool valid = u < n;
-    const int xs = valid ? xadj[u] : 0x7FFFFFFF;
-    const int xe = valid ? xadj[u + 1] : 0x7FFFFFFF;
-    const int e0 = __shfl_sync(FULL, xs, 0);
-    const int last = (int)((n - u0) < 32 ? (n - u0) : 32) - 1;
-    const int e1 = __shfl_sync(FULL, xe, last);
+  for (EntryWalk wk(xadj, n, wid, nw); wk.next();) {
+    const int64_t u0 = wk.u0;
+    const int e0 = wk.e0, e1 = wk.e1;
+    // lane i's row start: the previous row's end
+    const int up = __shfl_up_sync(FULL, wk.xe, 1);
+    const int xs = lane == 0 ? xadj[u0] : up;
     for (int f0 = e0; f0 < e1; f0 += 32 * kValUnroll) {
       int e[kValUnroll], row[kValUnroll], rs[kValUnroll], v[kValUnroll], w[kValUnroll], pv[kValUnroll];
 #pragma unroll
       for (int r = 0; r < kValUnroll; r++) {
         e[r] = f0 + r * 32 + lane;
-        int q = 0;  // owner: lanes whose row ends at or before e
-#pragma unroll
-        for (int step = 16; step > 0; step >>= 1) {
-          const int val = __shfl_sync(FULL, xe, q + step - 1);
-          if (val <= e[r]) q += step;
-        }
+        const int q = wk.owner(e[r]);
         row[r] = (int)(u0 + q);
         rs[r] = __shfl_sync(FULL, xs, q);
       }
@@ -121,8 +114,8 @@ __global__ void k_project(int n, const int32_t *cmap, const int32_t *coarse, int
     fine[v] = coarse[cmap[v]];
 }
 
-// cut = 1/2 sum over CSR entries whose endpoints lie in different blocks: a
-// warp walks 32 consecutive rows (one contiguous range of entries), finds each
+// cut = 1/2 sum over CSR entries whose endpoints lie in different blocks: the
+// entries are split evenly over the warps (EntryWalk); a warp finds each
 // entry's row among its lanes by a shuffle search, and keeps four entries per
 // lane in flight.
 template <typename B>
@@ -134,26 +127,16 @@ __global__ void __launch_bounds__(256) k_cut(const int32_t *xadj, const int32_t 
   const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int nw = (int)((gridDim.x * blockDim.x) >> 5);
   unsigned long long s = 0;
-  for (int64_t u0 = (int64_t)wid * 32; u0 < n; u0 += (int64_t)nw * 32) {
-    const int64_t u = u0 + lane;
-    const bool valid = u < n;
-    const int xe = valid ? xadj[u + 1] : 0x7FFFFFFF;
-    const int bu = valid ? (int)blk[u] : -1;
-    const int e0 = __shfl_sync(FULL, valid ? xadj[u] : 0, 0);
-    const int last = (int)((n - u0) < 32 ? (n - u0) : 32) - 1;
-    const int e1 = __shfl_sync(FULL, xe, last);
+  for (EntryWalk wk(xadj, n, wid, nw); wk.next();) {
+    const int64_t u = wk.u0 + lane;
+    const int bu = u < n ? (int)blk[u] : -1;
+    const int e0 = wk.e0, e1 = wk.e1;
     for (int f0 = e0; f0 < e1; f0 += 32 * R) {
       int e[R], bo[R], v[R], w[R];
 #pragma unroll
       for (int r = 0; r < R; r++) {
         e[r] = f0 + r * 32 + lane;
-        int q = 0;  // owner: lanes whose row ends at or before e
-#pragma unroll
-        for (int step = 16; step > 0; step >>= 1) {
-          const int val = __shfl_sync(FULL, xe, q + step - 1);
-          if (val <= e[r]) q += step;
-        }
-        bo[r] = __shfl_sync(FULL, bu, q);
+        bo[r] = __shfl_sync(FULL, bu, wk.owner(e[r]));
       }
 #pragma unroll
       for (int r = 0; r < R; r++) {
@@ -239,7 +222,7 @@ GraphTotals validate_graph(gp_ctx *ctx, const DevGraph &g, bool full) {
   GP_REQUIRE(h.csum <= 0x7FFFFFFFull, GP_ERR_OVERFLOW, "total node weight exceeds 2^31 - 1");
   prof_bytes(ctx, PROF_VALIDATE, 8.0 * g.n + 8.0 * g.m2);  // offsets, node weights, ids, edge weights
   if (g.m2 > 0) {
-    k_validate_entries<<<grid_for(g.n, 256, ctx->num_sms * 16), 256, 0, ctx->stream>>>(
+    k_validate_entries<<<walk_grid(g.m2, ctx->num_sms), 256, 0, ctx->stream>>>(
         g.xadj, g.adjncy, g.adjwgt, g.n, g.m2, o.get());
     GP_LAUNCH_CHECK();
     read_back(ctx, o.get(), sizeof(ValOut), &h);
@@ -269,7 +252,7 @@ void cut_and_weights(gp_ctx *ctx, const DevGraph &g, const int32_t *blocks, int3
   DBuf<unsigned long long> c(ctx, 1);
   c.zero();
   if (g.m2 > 0) {
-    const int grid = grid_for(g.n, 256, ctx->num_sms * 16);
+    const int grid = walk_grid(g.m2, ctx->num_sms);
     if (k <= 255) {
       DBuf<uint8_t> b8(ctx, (size_t)g.n);
       k_narrow<<<grid_for(g.n, 256, ctx->num_sms * 8), 256, 0, ctx->stream>>>(blocks, g.n, b8.get());

@@ -12,11 +12,11 @@
 // its hash is below floor(m_hat 2^32 / m).  Both CSR directions of an edge
 // see the same hash, so the result stays symmetric.
 //
-// Two passes over the entries, each warp walking 32 consecutive rows (one
-// contiguous range of entries): the first counts the kept entries of every
-// row, a prefix sum turns the counts into the new row offsets, and the second
-// takes the same keep decisions again and writes the kept entries of the 32
-// rows contiguously from the first row's new offset.
+// Two passes over the entries, split evenly over the warps (EntryWalk): the
+// first counts the kept entries of every row and of every warp's share, prefix
+// sums turn the counts into the new row offsets and into each share's place in
+// the output (kept entries stay in order), and the second takes the same keep
+// decisions again and writes each share's kept entries contiguously.
 #include "gp_internal.cuh"
 
 #include <algorithm>
@@ -60,8 +60,8 @@ struct KeepArgs {
   uint64_t T;   // modes 1, 2: 32-bit hash threshold; mode 4: the last kept 64-bit hash
   uint64_t key;
   uint32_t blo, bhi;  // mode 4: the last kept edge among those whose hash equals T
-  int32_t *cnt;         // count pass: kept entries per row
-  const int32_t *nxadj; // write pass: new row offsets
+  int32_t *cnt;         // count pass: kept entries per row (zeroed before: a row may lie in two shares)
+  int32_t *share;       // per warp: kept entries of its share (count pass), their place (write pass)
   int32_t *oadj, *ow;
 };
 
@@ -88,28 +88,18 @@ __global__ void __launch_bounds__(256) k_keep(KeepArgs a) {
   const int lane = (int)lane_id(), wib = threadIdx.x >> 5;
   const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-  for (int64_t u0 = (int64_t)wid * 32; u0 < a.n; u0 += (int64_t)nw * 32) {
-    const int64_t u = u0 + lane;
-    const bool valid = u < a.n;
-    const int xe = valid ? a.xadj[u + 1] : 0x7FFFFFFF;
-    const int e0 = a.xadj[u0];
-    const int last = (int)((a.n - u0) < 32 ? (a.n - u0) : 32) - 1;
-    const int e1 = __shfl_sync(FULL, xe, last);
+  int out = WRITE ? a.share[wid] : 0;
+  for (EntryWalk wk(a.xadj, a.n, wid, nw); wk.next();) {
+    const int64_t u0 = wk.u0, u = u0 + lane;
+    const int e0 = wk.e0, e1 = wk.e1;
     if (!WRITE) s_cnt[wib][lane] = 0;
-    int out = WRITE ? a.nxadj[u0] : 0;
     __syncwarp();
     for (int f0 = e0; f0 < e1; f0 += 32 * kKeepUnroll) {
       int e[kKeepUnroll], j[kKeepUnroll], v[kKeepUnroll], x[kKeepUnroll];
 #pragma unroll
       for (int r = 0; r < kKeepUnroll; r++) {
         e[r] = f0 + r * 32 + lane;
-        int q = 0;  // owner: lanes whose row ends at or before e
-#pragma unroll
-        for (int step = 16; step > 0; step >>= 1) {
-          const int val = __shfl_sync(FULL, xe, q + step - 1);
-          if (val <= e[r]) q += step;
-        }
-        j[r] = q;
+        j[r] = wk.owner(e[r]);
       }
 #pragma unroll
       for (int r = 0; r < kKeepUnroll; r++) {
@@ -134,16 +124,22 @@ __global__ void __launch_bounds__(256) k_keep(KeepArgs a) {
     }
     if (!WRITE) {
       __syncwarp();
-      if (valid) a.cnt[u] = s_cnt[wib][lane];
+      const int c = s_cnt[wib][lane];
+      if (c) atomicAdd(&a.cnt[u], c);
+      out += c;
       __syncwarp();
     }
+  }
+  if (!WRITE) {
+    out = warp_sum(out);
+    if (lane == 0) a.share[wid] = out;
   }
 }
 
 // Exact-count mode: histogram of one digit of the 64-bit hash of the edges of
 // weight wt (entries with row < neighbour, so every edge once), restricted to
-// the hashes whose bits above the digit equal `prefix`; the same 32-row walk
-// as k_keep.
+// the hashes whose bits above the digit equal `prefix`; the same walk as
+// k_keep.
 struct HashHistArgs {
   const int32_t *xadj, *adjncy, *adjwgt;
   int n;
@@ -168,20 +164,12 @@ __global__ void __launch_bounds__(256) k_hash_digit(HashHistArgs a) {
   const int lane = (int)lane_id();
   const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-  for (int64_t u0 = (int64_t)wid * 32; u0 < a.n; u0 += (int64_t)nw * 32) {
-    const int64_t u = u0 + lane;
-    const int xe = u < a.n ? a.xadj[u + 1] : 0x7FFFFFFF;
-    const int e0 = a.xadj[u0];
-    const int last = (int)((a.n - u0) < 32 ? (a.n - u0) : 32) - 1;
-    const int e1 = __shfl_sync(FULL, xe, last);
-    for (int f0 = e0; f0 < e1; f0 += 32) {
+  for (EntryWalk wk(a.xadj, a.n, wid, nw); wk.next();) {
+    const int64_t u0 = wk.u0;
+    const int e1 = wk.e1;
+    for (int f0 = wk.e0; f0 < e1; f0 += 32) {
       const int e = f0 + lane;
-      int q = 0;  // owner: lanes whose row ends at or before e
-#pragma unroll
-      for (int step = 16; step > 0; step >>= 1) {
-        const int val = __shfl_sync(FULL, xe, q + step - 1);
-        if (val <= e) q += step;
-      }
+      const int q = wk.owner(e);
       if (e >= e1) continue;
       const int row = (int)(u0 + q), v = __ldcs(a.adjncy + e);
       if (row >= v || __ldcs(a.adjwgt + e) != a.wt) continue;
@@ -212,7 +200,7 @@ void exact_boundary(gp_ctx *ctx, const DevGraph &g, int32_t wt, uint64_t key, in
   DBuf<unsigned long long> hist(ctx, 2048);
   std::vector<unsigned long long> h(2048);
   HashHistArgs a{g.xadj, g.adjncy, g.adjwgt, g.n, wt, key, 0, 0, 0, 0, hist.get(), nullptr, nullptr, 0};
-  const int grid = grid_for(g.n, 256, ctx->num_sms * 16);
+  const int grid = walk_grid(g.m2, ctx->num_sms);
   uint64_t prefix = 0;
   int64_t below = 0, equal = 0;
   for (int d = 0; d < 6; d++) {
@@ -342,11 +330,12 @@ void sparsify_graph(gp_ctx *ctx, const DevGraph &g, int64_t m_hat, int32_t level
     exact_boundary(ctx, g, wt, key, m_hat - ng, &T, &blo, &bhi);
   }
   KeepArgs a{g.xadj, g.adjncy, g.adjwgt, n, kmode, wt, T, key, blo, bhi, nullptr, nullptr, nullptr, nullptr};
-  DBuf<int32_t> cnt(ctx, (size_t)n + 1), total(ctx, 1);
-  const int kgrid = grid_for(n, 256, ctx->num_sms * 16);
-  GP_CUDA(cudaMemsetAsync(cnt.get() + n, 0, sizeof(int32_t), ctx->stream));
-  if (n > 0) {
+  const int kgrid = walk_grid(m2, ctx->num_sms);
+  DBuf<int32_t> cnt(ctx, (size_t)n + 1), total(ctx, 1), share(ctx, (size_t)kgrid * 8);
+  cnt.zero();
+  if (m2 > 0) {
     a.cnt = cnt.get();
+    a.share = share.get();
     k_keep<false><<<kgrid, 256, 0, ctx->stream>>>(a);
     GP_LAUNCH_CHECK();
   }
@@ -354,6 +343,7 @@ void sparsify_graph(gp_ctx *ctx, const DevGraph &g, int64_t m_hat, int32_t level
   out.bx.reset(ctx, (size_t)n + 1);
   out.xadj = out.bx.get();
   scan_exclusive_i32(ctx, cnt.get(), out.xadj, n + 1, total.get());
+  if (m2 > 0) scan_exclusive_i32(ctx, share.get(), share.get(), (int64_t)kgrid * 8, nullptr);
   const int32_t m2_out = read_scalar(ctx, total.get());
   out.m2 = m2_out;
   out.ba.reset(ctx, (size_t)m2_out);
@@ -363,7 +353,7 @@ void sparsify_graph(gp_ctx *ctx, const DevGraph &g, int64_t m_hat, int32_t level
   out.bv.reset(ctx, (size_t)n);
   out.vwgt = out.bv.get();
   if (n > 0 && m2_out > 0) {
-    a.nxadj = out.xadj; a.oadj = out.adjncy; a.ow = out.adjwgt;
+    a.oadj = out.adjncy; a.ow = out.adjwgt;
     k_keep<true><<<kgrid, 256, 0, ctx->stream>>>(a);
     GP_LAUNCH_CHECK();
   }
