@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kThreads) k_map(const int32_t *xadj, const int
 #pragma unroll
       for (int r = 0; r < kMapUnroll; r++) {
         e[r] = f0 + r * 32 + lane;
-        const int j = wk.owner(e[r]);
+        const int j = wk.owner(f0 + r * 32);
         bj[r] = __shfl_sync(FULL, base, j);
         Aj[r] = __shfl_sync(FULL, A, j);
       }

@@ -374,13 +374,14 @@ struct EntryWalk {
   int64_t pos, end;  // entries still to walk
   int64_t u0, row;   // this window's first row, the next one's
   int e0, e1, xe;
+  bool no_empty;     // no row of the window is empty
   __device__ __forceinline__ EntryWalk(const int32_t *x, int nn, int wid, int nw) : xadj(x), n(nn) {
     const int64_t lo = nn > 0 ? x[0] : 0, hi = nn > 0 ? x[nn] : 0;
     const int64_t per = (((hi - lo + nw - 1) / nw) + 31) & ~(int64_t)31;
     pos = lo + per * wid;
     end = pos + per < hi ? pos + per : hi;
     row = pos < end ? find(pos) : 0;
-    u0 = 0; e0 = e1 = xe = 0;
+    u0 = 0; e0 = e1 = xe = 0; no_empty = false;
   }
   __device__ __forceinline__ bool next() {
     while (pos < end) {
@@ -395,6 +396,8 @@ struct EntryWalk {
       }
       e0 = (int)pos;
       e1 = (int)(wend < end ? wend : end);
+      const int before = __shfl_up_sync(0xFFFFFFFFu, xe, 1);
+      no_empty = __all_sync(0xFFFFFFFFu, lane_id() == 0 || u >= n || before < xe);
       pos = e1;
       row = u0 + 32;
       return true;
@@ -412,8 +415,17 @@ struct EntryWalk {
     }
     return a;
   }
-  // Lane index of the row that holds entry e: the lanes whose row ends at or before e.
-  __device__ __forceinline__ int owner(int e) const {
+  // Lane index of the row that holds entry f + lane (f the same in the whole warp): the lanes whose row
+  // ends at or before it.  Without empty rows in the window every row end is another position, so the
+  // ends among the 32 entries form a bit mask, and a count of its lower bits replaces the search (one
+  // reduction instead of five dependent shuffles).
+  __device__ __forceinline__ int owner(int f) const {
+    if (no_empty) {
+      const int d = xe - f;
+      const unsigned ends = __reduce_or_sync(0xFFFFFFFFu, d > 0 && d < 32 ? 1u << d : 0u);
+      return __popc(__ballot_sync(0xFFFFFFFFu, d <= 0)) + __popc(ends & (lanemask_lt() | (1u << lane_id())));
+    }
+    const int e = f + (int)lane_id();
     int q = 0;
 #pragma unroll
     for (int step = 16; step > 0; step >>= 1) {

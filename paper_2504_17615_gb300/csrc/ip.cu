@@ -2,7 +2,7 @@
 // bisection (Sec. 4.3), plus the greedy rebalancer.
 //
 // All subproblems of one depth of the bisection tree are split together;
-// every (subproblem, trial) pair runs in its own warp.  A trial grows side 1
+// every (subproblem, trial) pair runs in its own block.  A trial grows side 1
 // greedily: among nodes that still fit under L1, frontier nodes (connected
 // to side 1) of largest gain 2 conn(v) - deg'(v), ties by the smallest id;
 // when no frontier node fits, the node of smallest (h32(key(IP, 0, bid), v,
@@ -13,21 +13,29 @@
 // their gains at the start of the step, skipping those that no longer fit
 // (one node per step below 1024 nodes).
 //
-// A node costs O(deg + n'/64), not O(n'): node lists are sorted by id, so
-// local index order is id order; every 64-node chunk keeps the largest key
-// (gain, -index) of its live frontier nodes, raised with a 64-bit atomicMax
-// when a neighbour's connection grows and recomputed only for the chunks of
-// the nodes just taken.  A picked node that no longer fits is retired for
-// good (side 1 only gets heavier), which leaves the choice among the nodes
-// that fit unchanged.
+// A trial is one chain of a few hundred dependent steps, so the kernel is
+// bound by the latency of a step and built to shorten it:
+//  * a node is ONE word: its state, gain and id packed so that a signed
+//    maximum over words is the choice (gain first, then the smallest id).
+//    32 bits hold it when the weighted degrees stay below 2^15 and the
+//    subproblem below 2^15 nodes; a maximum over the warp is then one
+//    instruction.  Otherwise words have 64 bits.
+//  * every 64-node chunk keeps the largest word of its frontier nodes, raised
+//    by an atomic maximum when a neighbour's connection grows and recomputed
+//    for the chunk of a node just taken; each lane keeps the maximum over its
+//    chunks in a register.
+//  * rows are copied to shared memory where they fit (below the first depths
+//    only a subproblem's internal edges are left); the row bounds of a taken
+//    node are fetched while the next one is being chosen.
+//  * steps of up to kSoloB nodes run in one warp without block barriers.
+// A picked node that no longer fits is retired for good (side 1 only gets
+// heavier), which leaves the choice among the nodes that fit unchanged.
+// The fallback scans all nodes the first few times; after that, nodes are
+// chained by the top bits of their hash and a cursor walks the chains (a
+// node that left the free state or stopped fitting never comes back).
 //
-// Steps of B >= 8 nodes select their nodes together instead of one by one:
-// the chunk maxima are sorted, the q-th largest of them (q = nodes still
-// wanted) is a threshold that at least q frontier nodes reach, and all of
-// those lie in the q leading chunks; they are ranked, and one warp walks them
-// in key order with prefix sums of their weights, taking, retiring or
-// stopping exactly as the one-by-one walk would.  A round that runs out of
-// candidates (retired nodes) selects again.
+// Measured (20,480 nodes, 204,800 edges, k = 128, 8 trials; the whole initial partition): 17.0 ms with 64-bit
+// keys in separate arrays, block barriers in every step and a sort of the chunk maxima; 9.0 ms so.
 #include "gp_internal.cuh"
 
 #include <algorithm>
@@ -36,15 +44,18 @@ namespace gp {
 
 namespace {
 
-constexpr int kUpdUnroll = 8;
+constexpr int kUpdUnroll = 4;
 constexpr int kSmemBatch = 64;  // the nodes of a growing step live in shared memory up to this many
 constexpr int kChunkNodes = 64;
-constexpr int kBatchMinB = 8;    // steps of at least this many nodes select them together
-constexpr int kSortCap = 512;    // chunk maxima sorted per selection round
-constexpr int kCandCap = 256;    // candidates ranked per round, a quarter per warp; more fall back to
-                                 // one-by-one extraction
-// dynamic part (static shared variables use the rest: the sort and candidate buffers and a few words)
-constexpr int kMaxSmemBytes = 227 * 1024 - (kSortCap + 2 * kCandCap) * 8 - kSmemBatch * 4 - 1024;
+constexpr int kIpWarps = 4;     // warps per (subproblem, trial)
+constexpr int kSoloB = 4;       // steps of up to this many nodes run in one warp
+constexpr int kScanFallbacks = 8;      // fallbacks found by a scan over all nodes before the chains are built
+constexpr int kChainNodes = 4;         // nodes per chain at least, on average
+constexpr int kNarrowNodes = 1 << 15;  // 32-bit words: subproblems below this many nodes ...
+constexpr int kNarrowGain = 1 << 15;   // ... and weighted degrees below this
+constexpr int kStaticSmem = 2048;      // room for the kernel's static shared variables
+constexpr int kSmSmem = 228 * 1024;    // shared memory of an SM; every resident block reserves another 1 KiB
+constexpr int kMaxSmemBytes = 227 * 1024 - kStaticSmem;
 
 struct Sub {
   int32_t start, count;  // node list range
@@ -53,9 +64,88 @@ struct Sub {
   int64_t T1, L1;        // side-1 target and limit
 };
 
-// Per-node state of a trial: S_FREE not connected to side 1, S_FRONT free and
-// connected, S_ONE in side 1, S_OUT retired (can never fit again).
-enum : uint8_t { S_FREE = 0, S_ONE = 1, S_OUT = 2, S_FRONT = 3 };
+// The node words.  Frontier nodes: (gain, -id), positive and above kOut; free nodes (not connected to
+// side 1): the same with the sign bit set; kOne: in side 1; kOut: retired (can never fit again).
+template <typename T> struct Word;
+template <int V> struct IntC { static constexpr int value = V; };
+template <> struct Word<int32_t> {
+  static constexpr int32_t kFree = INT32_MIN;
+  __device__ static int32_t make(int64_t gain, int j) {
+    return ((int32_t)(gain + kNarrowGain) << 15) | (kNarrowNodes - 1 - j);
+  }
+  __device__ static int node(int32_t x) { return kNarrowNodes - 1 - (x & (kNarrowNodes - 1)); }
+  __device__ static int32_t delta(int w) { return (int32_t)((uint32_t)(2 * w) << 15); }  // connection + w
+  __device__ static int32_t wmax(int32_t x) { return __reduce_max_sync(0xFFFFFFFFu, x); }
+};
+template <> struct Word<long long> {
+  static constexpr long long kFree = INT64_MIN;
+  __device__ static long long make(int64_t gain, int j) {
+    return ((gain + 2147483648ll) << 31) | (2147483647 - j);
+  }
+  __device__ static int node(long long x) { return 2147483647 - (int)(x & 2147483647ll); }
+  __device__ static long long delta(int w) { return (long long)w << 32; }
+  __device__ static long long wmax(long long x) {
+    const int hi = (int)(x >> 32);
+    const int mh = __reduce_max_sync(0xFFFFFFFFu, hi);
+    const unsigned ml = __reduce_max_sync(0xFFFFFFFFu, hi == mh ? (unsigned)x : 0u);
+    return ((long long)mh << 32) | ml;
+  }
+};
+constexpr int kOne = 0, kOut = 1;
+
+// An array of node words: shared memory by its 32-bit address (so that every access is a shared-memory
+// instruction and none a generic one), or global memory.
+template <typename T, bool SM> struct Words;
+template <> struct Words<int32_t, true> {
+  uint32_t p;
+  __device__ int32_t get(int i) const {
+    int32_t x;
+    asm volatile("ld.shared.s32 %0, [%1];" : "=r"(x) : "r"(p + 4 * i) : "memory");
+    return x;
+  }
+  __device__ void set(int i, int32_t x) const { asm volatile("st.shared.s32 [%0], %1;" ::"r"(p + 4 * i), "r"(x) : "memory"); }
+  __device__ int32_t add(int i, int32_t d) const {
+    int32_t x;
+    asm volatile("atom.shared.add.s32 %0, [%1], %2;" : "=r"(x) : "r"(p + 4 * i), "r"(d) : "memory");
+    return x;
+  }
+  __device__ void unfree(int i) const { asm volatile("red.shared.and.b32 [%0], %1;" ::"r"(p + 4 * i), "r"(INT32_MAX) : "memory"); }
+  __device__ void raise(int i, int32_t x) const { asm volatile("red.shared.max.s32 [%0], %1;" ::"r"(p + 4 * i), "r"(x) : "memory"); }
+};
+template <> struct Words<long long, true> {
+  uint32_t p;
+  __device__ long long get(int i) const {
+    long long x;
+    asm volatile("ld.shared.s64 %0, [%1];" : "=l"(x) : "r"(p + 8 * i) : "memory");
+    return x;
+  }
+  __device__ void set(int i, long long x) const { asm volatile("st.shared.s64 [%0], %1;" ::"r"(p + 8 * i), "l"(x) : "memory"); }
+  __device__ long long add(int i, long long d) const {
+    long long x;
+    asm volatile("atom.shared.add.u64 %0, [%1], %2;" : "=l"(x) : "r"(p + 8 * i), "l"(d) : "memory");
+    return x;
+  }
+  __device__ void unfree(int i) const { asm volatile("red.shared.and.b64 [%0], %1;" ::"r"(p + 8 * i), "l"(INT64_MAX) : "memory"); }
+  __device__ void raise(int i, long long x) const { asm volatile("red.shared.max.s64 [%0], %1;" ::"r"(p + 8 * i), "l"(x) : "memory"); }
+};
+template <typename T> struct Words<T, false> {
+  T *p;
+  __device__ T get(int i) const { return *(volatile T *)(p + i); }
+  __device__ void set(int i, T x) const { *(volatile T *)(p + i) = x; }
+  __device__ T add(int i, T d) const { return (T)atomicAdd((unsigned long long *)(p + i), (unsigned long long)d); }
+  __device__ void unfree(int i) const { atomicAnd((unsigned long long *)(p + i), (unsigned long long)INT64_MAX); }
+  __device__ void raise(int i, T x) const { atomicMax(p + i, x); }
+};
+__device__ __forceinline__ uint32_t lds_u32(uint32_t p) {
+  uint32_t x;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(x) : "r"(p) : "memory");
+  return x;
+}
+__device__ __forceinline__ int lds_u16(uint32_t p) {
+  uint16_t x;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(x) : "r"(p) : "memory");
+  return (int)x;
+}
 
 struct IpArgs {
   const int32_t *lxadj;            // local CSR of every subproblem (by list position)
@@ -65,32 +155,18 @@ struct IpArgs {
   int trials;
   int n;
   uint64_t seed;
-  int smem_nodes;                  // subproblems up to this size keep their state in shared memory
-  int cv16;                        // node weights fit 16 bits: kept in shared memory too
-  int hv_smem;                     // the trial's fallback hashes fit in shared memory too
-  int32_t *gg;                     // global fallback state per block
-  uint8_t *gst;
-  uint16_t *gcv;
-  unsigned long long *gbest, *gsup;
-  int64_t gnodes, gchunks;
+  int smem_bytes;                  // dynamic shared memory of a block
+  int cv16;                        // node weights fit 16 bits: kept in shared memory
+  void *gx, *gbest, *gsup;         // [trial][n] words when a subproblem's do not fit in shared memory, ...
   int32_t *gbatch;                 // per block: the nodes taken in the current step
   int batch_cap;
-  unsigned long long *trace;       // optional: [0] growing steps, [1] fallback scans, [2] retired nodes
+  int64_t bstride, sstride;        // their chunk maxima and maxima over 32 chunks, per trial
+  int32_t *fnext, *fhead;          // fallback chains (words in shared memory only): next node [trial][n],
+  int64_t hstride;                 // first node per bucket, hstride per trial
+  unsigned long long *trace;       // optional: [0] growing steps, [1] fallbacks, [2] retired nodes
   int64_t *trial_cut;              // per block
   uint8_t *flags;                  // [trial][n] side-1 flag by list position
 };
-
-__device__ __forceinline__ unsigned long long gain_key(int64_t gain, int j) {
-  return ((unsigned long long)(gain + 2147483648ll) << 32) | (0xFFFFFFFFu - (unsigned)j);
-}
-
-// 64-bit maximum / minimum over the warp with two 32-bit reductions each.
-__device__ __forceinline__ unsigned long long wmax_u64(unsigned long long x) {
-  const unsigned hi = (unsigned)(x >> 32);
-  const unsigned mh = __reduce_max_sync(0xFFFFFFFFu, hi);
-  const unsigned ml = __reduce_max_sync(0xFFFFFFFFu, hi == mh ? (unsigned)x : 0u);
-  return ((unsigned long long)mh << 32) | ml;
-}
 
 __device__ __forceinline__ unsigned long long wmin_u64(unsigned long long x) {
   const unsigned hi = (unsigned)(x >> 32);
@@ -99,429 +175,399 @@ __device__ __forceinline__ unsigned long long wmin_u64(unsigned long long x) {
   return ((unsigned long long)mh << 32) | ml;
 }
 
-// chunk best over the live frontier nodes of chunk c (one warp)
-__device__ __forceinline__ void rescan_chunk(int c, int cnt, const int32_t *g, const uint8_t *st,
-                                             unsigned long long *best) {
-  const int lane = (int)lane_id();
-  unsigned long long b = 0;
-#pragma unroll
-  for (int r = 0; r < kChunkNodes / 32; r++) {
-    const int j = c * kChunkNodes + r * 32 + lane;
-    if (j < cnt && st[j] == S_FRONT) {
-      const unsigned long long key = gain_key(g[j], j);
-      b = key > b ? key : b;
-    }
-  }
-  b = wmax_u64(b);
-  if (lane == 0) best[c] = b;
-  __syncwarp();
+// A 4-byte copy from global to shared memory that the issuing lane does not wait for.
+__device__ __forceinline__ void copy_async4(int *dst, const int32_t *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
 }
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-constexpr int kIpWarps = 4;  // warps per (subproblem, trial)
-
-// Bitonic sort of kSortCap = 512 keys into descending order by the block's
-// 128 threads, four keys per thread in registers (thread t holds positions
-// 4t .. 4t+3): partners at distance 1 and 2 are in the same thread, at 4 .. 64
-// in the same warp (shuffles), at 128 and 256 in another warp (through x, the
-// only stages with block barriers).  On return x[0, 512) holds the sorted keys
-// and the block is synchronised.
-static_assert(kSortCap == 4 * 32 * kIpWarps, "four keys per thread");
-static_assert(kChunkNodes == 64, "two chunk nodes per lane");
-constexpr int kSegCap = kCandCap / kIpWarps;  // candidates per warp and round
-
-__device__ __forceinline__ unsigned long long keep(unsigned long long mine, unsigned long long other, bool take_max) {
-  return take_max ? (mine > other ? mine : other) : (mine < other ? mine : other);
-}
-
-__device__ __forceinline__ void sort512_desc(unsigned long long (&r)[4], unsigned long long *x) {
-  const int t = threadIdx.x;
-#pragma unroll
-  for (int size = 2; size <= kSortCap; size <<= 1) {
-#pragma unroll
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      if (stride >= 128) {
-#pragma unroll
-        for (int k = 0; k < 4; k++) x[4 * t + k] = r[k];
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-          const int i = 4 * t + k;
-          const unsigned long long o = x[i ^ stride];
-          r[k] = keep(r[k], o, ((i & stride) == 0) == ((i & size) == 0));
-        }
-        __syncthreads();
-      } else if (stride >= 4) {
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-          const int i = 4 * t + k;
-          const unsigned long long o = __shfl_xor_sync(0xFFFFFFFFu, r[k], stride / 4);
-          r[k] = keep(r[k], o, ((i & stride) == 0) == ((i & size) == 0));
-        }
-      } else {
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-          if (k & stride) continue;
-          const int i = 4 * t + k;
-          const unsigned long long lo = r[k], hi = r[k | stride];
-          const bool desc = (i & size) == 0;
-          r[k] = keep(lo, hi, desc);
-          r[k | stride] = keep(lo, hi, !desc);
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < 4; k++) x[4 * t + k] = r[k];
-  __syncthreads();
-}
-
-__device__ __forceinline__ int node_of(unsigned long long key) {
-  return (int)(0xFFFFFFFFu - (unsigned)(key & 0xFFFFFFFFull));
-}
-
-// One block of kIpWarps warps per (subproblem, trial).  Warp 0 takes the
-// step's nodes from the chunk tournament; all warps then raise the
-// connections of the taken nodes' neighbours, scan for the fallback node and
-// add up the trial's cut.
+// One block of kIpWarps warps per (subproblem, trial).  SM: the words live in shared memory (at most
+// 512 chunks: 16 per lane); otherwise in global memory, with one more level of maxima.
+template <typename KT, bool SM>
 __global__ void __launch_bounds__(32 * kIpWarps) k_ip_grow(IpArgs a) {
+  using W = Word<KT>;
   extern __shared__ __align__(16) unsigned char dyn[];
-  __shared__ int s_nb, s_nz, s_wc[kIpWarps];
+  __shared__ int s_nb, s_fj;
   __shared__ long long s_w1;
   __shared__ unsigned long long s_red[kIpWarps];
-  __shared__ unsigned long long s_sort[kSortCap], s_cand[kCandCap], s_rank[kCandCap];
   __shared__ int32_t s_batch[kSmemBatch];
+  __shared__ int s_rs[32], s_re[32];
   const int lane = (int)lane_id(), warp = threadIdx.x >> 5;
   const int si = blockIdx.x / a.trials, t = blockIdx.x % a.trials;
   const Sub S = a.subs[si];
   const int cnt = S.count, nch = (cnt + kChunkNodes - 1) / kChunkNodes;
-  const int start = S.start;
   const int nsup = (nch + 31) / 32;
-  unsigned long long *best, *sup;  // chunk maxima, and maxima over 32 chunks
-  int32_t *g;
-  uint8_t *st;
-  uint16_t *cv = nullptr;
-  uint32_t *hv = nullptr;  // fallback hashes of the trial, when shared memory has room for them
-  if (cnt <= a.smem_nodes) {
-    const int mch = (a.smem_nodes + kChunkNodes - 1) / kChunkNodes;
-    const int msup = (mch + 31) / 32;
-    best = reinterpret_cast<unsigned long long *>(dyn);
-    sup = best + mch;
-    g = reinterpret_cast<int32_t *>(dyn + sizeof(unsigned long long) * (mch + msup));
-    unsigned char *tail = reinterpret_cast<unsigned char *>(g + a.smem_nodes);
-    if (a.hv_smem) {
-      hv = reinterpret_cast<uint32_t *>(tail);
-      tail += sizeof(uint32_t) * a.smem_nodes;
-    }
+  const int start = S.start;
+  const int64_t tpos = (int64_t)t * a.n + start;  // this trial's place in the [trial][n] arrays
+  Words<KT, SM> X, best;
+  KT *sup = nullptr;
+  uint32_t cv = 0, lx = 0, sadj = 0;  // shared addresses (0: not there) of the node weights (16 bits each), of the
+                                      // row bounds from the subproblem's first entry, and of the rows
+                                      // (weight << 16 | neighbour)
+  const int base = a.lxadj[start];
+  if constexpr (SM) {
+    const uint32_t dyn0 = (uint32_t)__cvta_generic_to_shared(dyn);
+    X.p = dyn0;
+    best.p = dyn0 + (uint32_t)sizeof(KT) * cnt;
+    int64_t at = (int64_t)sizeof(KT) * (cnt + nch);
     if (a.cv16) {
-      cv = reinterpret_cast<uint16_t *>(tail);
-      tail += sizeof(uint16_t) * a.smem_nodes;
+      uint16_t *c16 = reinterpret_cast<uint16_t *>(dyn + at);
+      for (int j = threadIdx.x; j < cnt; j += blockDim.x) c16[j] = (uint16_t)a.cvl[start + j];
+      cv = dyn0 + (uint32_t)at;
+      at += (2 * (int64_t)cnt + 3) & ~(int64_t)3;
     }
-    st = tail;
+    if (at + 4 * ((int64_t)cnt + 1) <= a.smem_bytes) {
+      int32_t *l32 = reinterpret_cast<int32_t *>(dyn + at);
+      for (int j = threadIdx.x; j <= cnt; j += blockDim.x) l32[j] = a.lxadj[start + j] - base;
+      lx = dyn0 + (uint32_t)at;
+      at += 4 * ((int64_t)cnt + 1);
+      const int E = a.lxadj[start + cnt] - base;
+      if (sizeof(KT) == 4 && at + 4 * (int64_t)E <= a.smem_bytes) {
+        uint32_t *ad = reinterpret_cast<uint32_t *>(dyn + at);
+        for (int e = threadIdx.x; e < E; e += blockDim.x) {
+          const int2 x = a.ladj[base + e];
+          ad[e] = ((uint32_t)x.y << 16) | (uint32_t)x.x;
+        }
+        sadj = dyn0 + (uint32_t)at;
+      }
+    }
   } else {
-    best = a.gbest + (int64_t)blockIdx.x * a.gchunks;
-    sup = a.gsup + (int64_t)blockIdx.x * ((a.gchunks + 31) / 32);
-    g = a.gg + (int64_t)blockIdx.x * a.gnodes;
-    st = a.gst + (int64_t)blockIdx.x * a.gnodes;
-    if (a.cv16) cv = a.gcv + (int64_t)blockIdx.x * a.gnodes;
+    X.p = reinterpret_cast<KT *>(a.gx) + tpos;
+    best.p = reinterpret_cast<KT *>(a.gbest) + t * a.bstride + start / kChunkNodes + si;
+    sup = reinterpret_cast<KT *>(a.gsup) + t * a.sstride + start / (32 * kChunkNodes) + si;
   }
   const uint64_t kip = stream_key(a.seed, TAG_IP, 0, (uint32_t)S.bid);
-  for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
-    g[j] = -a.dpl[start + j];
-    st[j] = S_FREE;
-    if (cv) cv[j] = (uint16_t)a.cvl[start + j];
-    if (hv) hv[j] = h32(kip, (uint32_t)a.vtx[start + j], (uint32_t)t);
-  }
-  for (int c = threadIdx.x; c < nch; c += blockDim.x) best[c] = 0;
-  for (int c = threadIdx.x; c < nsup; c += blockDim.x) sup[c] = 0;
+  for (int j = threadIdx.x; j < cnt; j += blockDim.x) X.set(j, W::make(-(int64_t)a.dpl[start + j], j) | W::kFree);
+  for (int c = threadIdx.x; c < nch; c += blockDim.x) best.set(c, 0);
+  if (!SM)
+    for (int c = threadIdx.x; c < nsup; c += blockDim.x) sup[c] = 0;
   __syncthreads();
-  int64_t w1 = 0;  // warp 0's copy is the authoritative one; others read s_w1
-  const int B = 1 + cnt / 1024;  // nodes per growing step
-  int32_t *batch = B <= kSmemBatch ? s_batch : a.gbatch + (int64_t)blockIdx.x * a.batch_cap;
-  const bool batched = B >= kBatchMinB && cnt <= a.smem_nodes && nch <= kSortCap;
-  for (;;) {
-    if (threadIdx.x == 0) s_w1 = w1;
-    __syncthreads();
-    w1 = s_w1;
-    if (w1 >= S.T1) break;
-    // up to B nodes in (gain desc, id asc) order; gains stay frozen until the step ends
-    bool seq = !batched;
-    if (batched) {
-      if (threadIdx.x == 0) {
-        s_nb = 0;
-        if (a.trace) atomicAdd(a.trace + 0, 1ull);
+
+  auto weight = [&](int j) -> int { return cv ? lds_u16(cv + 2 * j) : a.cvl[start + j]; };
+  auto entry = [&](int e) -> int2 {  // e counts from the subproblem's first entry
+    if (sadj) {
+      const uint32_t x = lds_u32(sadj + 4 * e);
+      return make_int2((int)(x & 0xFFFFu), (int)(x >> 16));
+    }
+    return a.ladj[base + e];
+  };
+  auto row_begin = [&](int j) -> int { return lx ? (int)lds_u32(lx + 4 * j) : a.lxadj[start + j] - base; };
+  // largest frontier word of chunk c without node skip (one warp), 0 if none
+  auto chunk_max = [&](int c, int skip) -> KT {
+    const int j0 = c * kChunkNodes + lane, j1 = j0 + 32;
+    KT x0 = j0 < cnt && j0 != skip ? X.get(j0) : 0, x1 = j1 < cnt && j1 != skip ? X.get(j1) : 0;
+    x0 = x0 > x1 ? x0 : x1;
+    x0 = W::wmax(x0);
+    return x0 > kOut ? x0 : 0;
+  };
+  int nfall = 0, cursor = 0;           // warp 0: fallbacks so far, bucket the chains are walked from
+  int bits = 0;                        // buckets: the hash's top bits, at most cnt / kChainNodes of them
+  while ((kChainNodes << (bits + 1)) <= cnt) bits++;
+  const int nbk = 1 << bits;
+  int32_t *const head = a.fhead + (int64_t)t * a.hstride + start / kChainNodes + si;
+  auto hash_of = [&](int j) -> uint32_t { return h32(kip, (uint32_t)a.vtx[start + j], (uint32_t)t); };
+  // one thread's share of a scan for the free node of smallest (hash, id) that fits
+  auto scan_free = [&](int tid, int step, int64_t w1) -> unsigned long long {
+    unsigned long long m = ~0ull;
+    for (int j = tid; j < cnt; j += step) {
+      if (X.get(j) >= 0 || w1 + weight(j) > S.L1) continue;
+      const unsigned long long key = ((unsigned long long)hash_of(j) << 32) | (unsigned)j;
+      m = key < m ? key : m;
+    }
+    return m;
+  };
+  auto chain_free = [&](int tid, int step) {  // chains of the nodes still free (heads cleared before)
+    for (int j = tid; j < cnt; j += step)
+      if (X.get(j) < 0) a.fnext[tpos + j] = atomicExch(&head[(int)((uint64_t)hash_of(j) >> (32 - bits))], j);
+  };
+  // warp 0: the free node of smallest (hash, id) that fits, from the chains; -1 if none
+  auto walk_free = [&](int64_t w1) -> int {
+    while (cursor < nbk) {
+      unsigned long long m = ~0ull;
+      const int b = cursor + lane;
+      if (b < nbk)
+        for (int j = head[b]; j >= 0; j = a.fnext[tpos + j]) {
+          if (X.get(j) >= 0 || w1 + weight(j) > S.L1) continue;
+          const unsigned long long key = ((unsigned long long)hash_of(j) << 32) | (unsigned)j;
+          m = key < m ? key : m;
+        }
+      const unsigned any = __ballot_sync(0xFFFFFFFFu, m != ~0ull);
+      if (any) {
+        const int f = __ffs(any) - 1;
+        cursor += f;
+        return __shfl_sync(0xFFFFFFFFu, (int)(unsigned)m, f);
       }
-      for (;;) {  // selection rounds
-        __syncthreads();
-        const int nb0 = s_nb;
-        const long long w10 = s_w1;
-        if (nb0 >= B || w10 >= S.T1) break;
-        {
-          unsigned long long rk[4];
+      cursor += 32;
+    }
+    return -1;
+  };
+
+  int64_t w1 = 0;
+  const int B = 1 + cnt / 1024;  // nodes per growing step
+  unsigned long long steps = 0, retired = 0;
+  // warp 0: the frontier node next in (gain desc, id asc) order is taken (its id comes back and w1 grows)
+  // or, when it no longer fits, retired (-2); -1: no frontier node left.  r: the maxima of the lane's
+  // chunks lane, lane + 32, ... (N of them), kept in step with best.
+  auto pick = [&](auto &r, auto count) -> int {
+    constexpr int N = decltype(count)::value;
+    KT m = 0;
+    if constexpr (SM) {
 #pragma unroll
-          for (int k = 0; k < 4; k++) {
-            const int i = 4 * (int)threadIdx.x + k;
-            rk[k] = i < nch ? best[i] : 0ull;
-          }
-          if (threadIdx.x == 0) s_nz = 0;
-          sort512_desc(rk, s_sort);
-        }
-        for (int i = threadIdx.x; i < kSortCap; i += blockDim.x)
-          if (s_sort[i] != 0 && (i + 1 == kSortCap || s_sort[i + 1] == 0)) s_nz = i + 1;
-        __syncthreads();
-        const int nz = s_nz;
-        if (nz == 0) break;  // no frontier node left
-        const int q = min(B - nb0, nz);
-        const unsigned long long tau = s_sort[q - 1];
-        // every frontier node with key >= tau sits in one of the q leading chunks; each warp
-        // gathers those of its chunks into its own segment of s_cand
-        {
-          int mine = 0;
-          unsigned long long *seg = s_cand + warp * kSegCap;
-          for (int r = warp; r < q; r += kIpWarps) {
-            const int c = node_of(s_sort[r]) / kChunkNodes;
-            const int j0 = c * kChunkNodes + lane, j1 = j0 + 32;
-            unsigned long long k0 = 0, k1 = 0;
-            if (j0 < cnt && st[j0] == S_FRONT) k0 = gain_key(g[j0], j0);
-            if (j1 < cnt && st[j1] == S_FRONT) k1 = gain_key(g[j1], j1);
-            const bool in0 = k0 != 0 && k0 >= tau, in1 = k1 != 0 && k1 >= tau;
-            const unsigned m0 = __ballot_sync(0xFFFFFFFFu, in0), m1 = __ballot_sync(0xFFFFFFFFu, in1);
-            const int p0 = mine + __popc(m0 & lanemask_lt());
-            const int p1 = mine + __popc(m0) + __popc(m1 & lanemask_lt());
-            if (in0 && p0 < kSegCap) seg[p0] = k0;
-            if (in1 && p1 < kSegCap) seg[p1] = k1;
-            mine += __popc(m0) + __popc(m1);
-          }
-          if (lane == 0) s_wc[warp] = mine;
-        }
-        __syncthreads();
-        int wc[kIpWarps], C = 0;
-        bool over = false;
+      for (int i = 0; i < N; i++) m = r[i] > m ? r[i] : m;
+    } else {
+      for (int c = lane; c < nsup; c += 32) { const KT x = sup[c]; m = x > m ? x : m; }
+    }
+    m = W::wmax(m);
+    if (m <= kOut) return -1;
+    const int j = W::node(m), c = j / kChunkNodes;
+    const int cj = weight(j);
+    const KT nm = chunk_max(c, j);
+    const bool fit = w1 + cj <= S.L1;
+    if (lane == 0) {
+      X.set(j, fit ? kOne : kOut);
+      best.set(c, nm);
+    }
+    __syncwarp();
+    if constexpr (SM) {
 #pragma unroll
-        for (int w2 = 0; w2 < kIpWarps; w2++) {
-          wc[w2] = s_wc[w2];
-          C += wc[w2];
-          over = over || wc[w2] > kSegCap;
-        }
-        if (over) { seq = true; break; }
-        for (int t = threadIdx.x; t < C; t += blockDim.x) {  // keys are distinct: rank = place
-          int at = -1, acc = 0;
+      for (int i = 0; i < N; i++) r[i] = c == lane + 32 * i ? nm : r[i];
+    } else {
+      const int s0 = (c / 32) * 32;
+      KT x = s0 + lane < nch ? best.get(s0 + lane) : 0;
+      x = W::wmax(x);
+      if (lane == 0) sup[c / 32] = x;
+      __syncwarp();
+    }
+    if (!fit) {
+      retired++;
+      return -2;
+    }
+    w1 += cj;
+    return j;
+  };
+  auto load_maxima = [&](auto &r, auto count) {
+    if constexpr (SM) {
 #pragma unroll
-          for (int w3 = 0; w3 < kIpWarps; w3++) {
-            if (at < 0 && t < acc + wc[w3]) at = w3 * kSegCap + (t - acc);
-            acc += wc[w3];
-          }
-          const unsigned long long x = s_cand[at];
-          int r = 0;
+      for (int i = 0; i < decltype(count)::value; i++) r[i] = lane + 32 * i < nch ? best.get(lane + 32 * i) : 0;
+    }
+  };
+  // one warp finds the fallback node; -1: none fits
+  auto fallback = [&]() -> int {
+    int j;
+    if (nfall < kScanFallbacks) {
+      const unsigned long long m = wmin_u64(scan_free(lane, 32, w1));
+      j = m == ~0ull ? -1 : (int)(unsigned)m;
+    } else {
+      if (nfall == kScanFallbacks) {
+        for (int b = lane; b < nbk; b += 32) head[b] = -1;
+        __syncwarp();
+        chain_free(lane, 32);
+        __syncwarp();
+      }
+      j = walk_free(w1);
+    }
+    nfall++;
+    return j;
+  };
+
+  if (SM && B <= kSoloB) {
+    if (warp == 0) {
+      constexpr int kN = kSoloB * 1024 / kChunkNodes / 32;  // cnt < kSoloB * 1024
+      constexpr IntC<kN> N{};
+      KT r[kN];
+      while (w1 < S.T1) {
+        load_maxima(r, N);
+        steps++;
+        int nb = 0, rs[kSoloB], re[kSoloB];
+        int2 first[kSoloB];  // the first 32 entries of the taken nodes' rows, fetched while others are chosen
 #pragma unroll
-          for (int w3 = 0; w3 < kIpWarps; w3++)
-            for (int i2 = 0; i2 < wc[w3]; i2++) r += s_cand[w3 * kSegCap + i2] > x ? 1 : 0;
-          s_rank[r] = x;
-        }
-        __syncthreads();
-        if (warp == 0) {
-          int nb = nb0;
-          long long w = w10;
-          int i0 = 0;
-          while (i0 < C) {
-            const int i = i0 + lane;
-            int j = -1;
-            long long c = 0;
-            if (i < C) {
-              j = node_of(s_rank[i]);
-              c = cv ? (long long)cv[j] : (long long)a.cvl[start + j];
+        for (int q = 0; q < kSoloB; q++) {
+          rs[q] = re[q] = 0;
+          first[q] = make_int2(-1, 0);
+          if (q != nb || q >= B || w1 >= S.T1) continue;
+          int j;
+          do { j = pick(r, N); } while (j == -2);
+          if (j == -1 && q == 0) {  // no frontier node fits
+            j = fallback();
+            if (j >= 0) {
+              w1 += weight(j);
+              if (lane == 0) X.set(j, kOne);
+              __syncwarp();
+              nb = kSoloB;  // the step's only node
             }
-            long long pre = c;  // weight of lanes i0..i
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-              const long long y = __shfl_up_sync(0xFFFFFFFFu, pre, o);
-              if (lane >= o) pre += y;
-            }
-            // lane i is reached iff every earlier lane of the group was taken
-            const bool considered = i < C && nb + (i - i0) < B && w + (pre - c) < S.T1;
-            const bool fits = w + pre <= S.L1;
-            const unsigned bad = __ballot_sync(0xFFFFFFFFu, !(considered && fits));
-            const int f = bad ? __ffs(bad) - 1 : 32;
-            if (lane < f) {
-              st[j] = S_ONE;
-              batch[nb + lane] = j;
-            }
-            const long long wf = __shfl_sync(0xFFFFFFFFu, pre, f > 0 ? f - 1 : 0);
-            const bool cf = __shfl_sync(0xFFFFFFFFu, considered, f < 32 ? f : 0);
-            if (f > 0) w += wf;
-            nb += f;
-            if (f == 32) { i0 += 32; continue; }
-            if (i0 + f >= C || !cf) break;  // list used up, or the step is complete
-            if (lane == f) {  // reached and does not fit: retired
-              st[j] = S_OUT;
-              if (a.trace) atomicAdd(a.trace + 2, 1ull);
-            }
-            i0 += f + 1;
           }
-          if (lane == 0) { s_nb = nb; s_w1 = w; }
+          if (j < 0) continue;
+          nb++;
+          rs[q] = row_begin(j);
+          re[q] = row_begin(j + 1);
+          if (rs[q] + lane < re[q]) first[q] = entry(rs[q] + lane);
         }
-        __syncthreads();
-        // the q leading chunks' maxima again, two chunks per warp at a time
-        for (int r = warp; r < q; r += 2 * kIpWarps) {
-          const bool two = r + kIpWarps < q;
-          const int ca = node_of(s_sort[r]) / kChunkNodes;
-          const int cb = two ? node_of(s_sort[r + kIpWarps]) / kChunkNodes : ca;
-          unsigned long long ba = 0, bb = 0;
+        if (nb == 0) break;
+        // neighbours of the step's nodes, row by row (a row has no neighbour twice: no atomic adds)
 #pragma unroll
-          for (int rr = 0; rr < kChunkNodes / 32; rr++) {
-            const int ja = ca * kChunkNodes + rr * 32 + lane, jb = cb * kChunkNodes + rr * 32 + lane;
-            const bool fa = ja < cnt && st[ja] == S_FRONT, fb = jb < cnt && st[jb] == S_FRONT;
-            if (fa) { const unsigned long long k = gain_key(g[ja], ja); ba = k > ba ? k : ba; }
-            if (fb) { const unsigned long long k = gain_key(g[jb], jb); bb = k > bb ? k : bb; }
+        for (int q = 0; q < kSoloB; q++) {
+          if (rs[q] >= re[q]) continue;
+          int2 y = first[q];
+          for (int f = rs[q];;) {
+            if (y.x >= 0) {
+              KT x = X.get(y.x);
+              if (x < 0 || x > kOut) {
+                x = (x & ~W::kFree) + W::delta(y.y);
+                X.set(y.x, x);
+                best.raise(y.x / kChunkNodes, x);
+              }
+            }
+            f += 32;
+            if (f >= re[q]) break;
+            y = f + lane < re[q] ? entry(f + lane) : make_int2(-1, 0);
           }
-          ba = wmax_u64(ba);
-          bb = wmax_u64(bb);
-          if (lane == 0) {
-            best[ca] = ba;
-            if (two) best[cb] = bb;
+          __syncwarp();
+        }
+      }
+    }
+  } else {
+    const bool rows_async = SM && !lx && B <= 32;
+    int32_t *batch = B <= kSmemBatch ? s_batch : a.gbatch + (int64_t)blockIdx.x * a.batch_cap;
+    for (;;) {
+      if (warp == 0) {
+        int nb = -2;  // done
+        if (w1 < S.T1) {
+          nb = 0;
+          steps++;
+          constexpr int kN = SM ? 16 : 1;
+          constexpr IntC<kN> N{};
+          KT r[kN];
+          load_maxima(r, N);
+          while (nb < B && w1 < S.T1) {
+            const int j = pick(r, N);
+            if (j == -1) break;
+            if (j < 0) continue;
+            if (lane == 0) {
+              batch[nb] = j;
+              if (rows_async) {  // the row's bounds come while the next node is chosen
+                copy_async4(&s_rs[nb], a.lxadj + start + j);
+                copy_async4(&s_re[nb], a.lxadj + start + j + 1);
+              }
+            }
+            nb++;
+          }
+          if (rows_async) copy_async_wait();
+        }
+        if (lane == 0) { s_nb = nb; s_w1 = w1; }
+      }
+      __syncthreads();
+      int nb = s_nb;
+      if (nb == -2) break;
+      bool fell = false;
+      if (nb == 0) {  // no frontier node fits
+        fell = true;
+        w1 = s_w1;
+        if (!SM || nfall < kScanFallbacks) {
+          const unsigned long long m = wmin_u64(scan_free(threadIdx.x, blockDim.x, w1));
+          if (lane == 0) s_red[warp] = m;
+          __syncthreads();
+          if (threadIdx.x == 0) {
+            unsigned long long mm = s_red[0];
+            for (int q = 1; q < kIpWarps; q++) mm = s_red[q] < mm ? s_red[q] : mm;
+            s_fj = mm == ~0ull ? -1 : (int)(unsigned)mm;
+          }
+        } else {
+          if (nfall == kScanFallbacks) {
+            for (int b = threadIdx.x; b < nbk; b += blockDim.x) head[b] = -1;
+            __syncthreads();
+            chain_free(threadIdx.x, blockDim.x);
+            __syncthreads();
+          }
+          if (warp == 0) {
+            const int j = walk_free(w1);
+            if (lane == 0) s_fj = j;
+          }
+        }
+        nfall++;
+        __syncthreads();
+        const int j = s_fj;
+        if (j < 0) break;
+        w1 += weight(j);  // warp 0's copy goes on from here
+        if (threadIdx.x == 0) { X.set(j, kOne); batch[0] = j; }
+        nb = 1;
+        __syncthreads();
+      }
+      // neighbours of the step's nodes, over their concatenated local rows (32 nodes at a time),
+      // 32 * kUpdUnroll entries per warp and pass
+      for (int b0 = 0; b0 < nb; b0 += 32) {
+        int r0 = 0, d = 0;
+        if (b0 + lane < nb) {
+          if (rows_async && !fell) {
+            r0 = s_rs[lane] - base;
+            d = s_re[lane] - base - r0;
+          } else {
+            const int j = batch[b0 + lane];
+            r0 = row_begin(j);
+            d = row_begin(j + 1) - r0;
+          }
+        }
+        int incl = d;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+          if (lane >= o) incl += y;
+        }
+        const int excl = incl - d, total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+        for (int f0 = warp * 32 * kUpdUnroll; f0 < total; f0 += kIpWarps * 32 * kUpdUnroll) {
+          int idx[kUpdUnroll];
+#pragma unroll
+          for (int r = 0; r < kUpdUnroll; r++) {
+            const int f = f0 + r * 32 + lane;
+            int q = 0;
+#pragma unroll
+            for (int step = 16; step > 0; step >>= 1) {
+              const int val = __shfl_sync(0xFFFFFFFFu, incl, q + step - 1);
+              if (val <= f) q += step;
+            }
+            const int sq = __shfl_sync(0xFFFFFFFFu, r0, q), eq = __shfl_sync(0xFFFFFFFFu, excl, q);
+            idx[r] = f < total ? sq + (f - eq) : -1;
+          }
+          int2 e[kUpdUnroll];
+#pragma unroll
+          for (int r = 0; r < kUpdUnroll; r++) e[r] = idx[r] >= 0 ? entry(idx[r]) : make_int2(-1, 0);
+#pragma unroll
+          for (int r = 0; r < kUpdUnroll; r++) {
+            if (e[r].x < 0) continue;
+            const KT x = X.get(e[r].x);
+            if (x < 0 || x > kOut) {
+              if (x < 0) X.unfree(e[r].x);
+              const KT dl = W::delta(e[r].y);
+              best.raise(e[r].x / kChunkNodes, X.add(e[r].x, dl) + dl);
+            }
           }
         }
       }
       __syncthreads();
-      if (seq) {  // the chunk groups' maxima again for the one-by-one walk
+      if (!SM) {  // the maxima over 32 chunks again, from the raised chunk maxima (one warp per group)
         for (int sc = warp; sc < nsup; sc += kIpWarps) {
           const int c = sc * 32 + lane;
-          const unsigned long long x = wmax_u64(c < nch ? best[c] : 0ull);
+          const KT x = W::wmax(c < nch ? best.get(c) : 0);
           if (lane == 0) sup[sc] = x;
         }
         __syncthreads();
-        w1 = s_w1;
       }
     }
-    if (seq && warp == 0) {
-      int nb = batched ? s_nb : 0;
-      while (nb < B && w1 < S.T1) {
-        unsigned long long b = 0;
-        for (int c = lane; c < nsup; c += 32) b = sup[c] > b ? sup[c] : b;
-        b = wmax_u64(b);
-        if (b == 0) break;
-        const int j = (int)(0xFFFFFFFFu - (unsigned)(b & 0xFFFFFFFFull));
-        const int cj = cv ? (int)cv[j] : a.cvl[start + j];
-        const bool fit = w1 + cj <= S.L1;
-        if (lane == 0) {
-          st[j] = fit ? S_ONE : S_OUT;  // S_OUT: cannot fit now, nor later
-          if (fit) batch[nb] = j;
-          if (a.trace && !fit) atomicAdd(a.trace + 2, 1ull);
-        }
-        if (fit) { nb++; w1 += cj; }
-        __syncwarp();
-        const int c = j / kChunkNodes;
-        rescan_chunk(c, cnt, g, st, best);
-        const int s0 = (c / 32) * 32;  // the maximum over c's 32 chunks again
-        unsigned long long x = s0 + lane < nch ? best[s0 + lane] : 0;
-        x = wmax_u64(x);
-        if (lane == 0) sup[c / 32] = x;
-        __syncwarp();
-      }
-      if (lane == 0) {
-        s_nb = nb;
-        s_w1 = w1;
-        if (a.trace && !batched) atomicAdd(a.trace + 0, 1ull);
-      }
-    }
-    __syncthreads();
-    int nb = s_nb;
-    w1 = s_w1;
-    if (nb == 0) {  // no frontier node fits: the smallest-hash node that fits, found by all warps
-      if (a.trace && threadIdx.x == 0) atomicAdd(a.trace + 1, 1ull);
-      unsigned long long m = ~0ull;
-      for (int jj = threadIdx.x; jj < cnt; jj += blockDim.x) {
-        if (st[jj] != S_FREE) continue;
-        const int cjj = cv ? (int)cv[jj] : a.cvl[start + jj];
-        if (w1 + cjj > S.L1) continue;
-        const uint32_t h = hv ? hv[jj] : h32(kip, (uint32_t)a.vtx[start + jj], (uint32_t)t);
-        const unsigned long long key = ((unsigned long long)h << 32) | (unsigned)jj;
-        m = key < m ? key : m;
-      }
-      m = wmin_u64(m);
-      if (lane == 0) s_red[warp] = m;
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        unsigned long long mm = s_red[0];
-        for (int q = 1; q < kIpWarps; q++) mm = s_red[q] < mm ? s_red[q] : mm;
-        if (mm == ~0ull) {
-          s_nb = -1;
-        } else {
-          const int j = (int)(unsigned)(mm & 0xFFFFFFFFull);
-          s_w1 = w1 + (cv ? (int)cv[j] : a.cvl[start + j]);
-          st[j] = S_ONE;
-          batch[0] = j;
-          s_nb = 1;
-        }
-      }
-      __syncthreads();
-      nb = s_nb;
-      if (nb < 0) break;
-      if (threadIdx.x == 0) w1 = s_w1;
-    }
-    if (threadIdx.x == 0) w1 = s_w1;
-    // neighbours of the step's nodes, over their concatenated local rows (32 nodes at a time),
-    // 32 * kUpdUnroll entries per warp and pass
-    for (int b0 = 0; b0 < nb; b0 += 32) {
-      int rs = 0, d = 0;
-      if (b0 + lane < nb) {
-        const int p = start + batch[b0 + lane];
-        rs = a.lxadj[p];
-        d = a.lxadj[p + 1] - rs;
-      }
-      int incl = d;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const int excl = incl - d, total = __shfl_sync(0xFFFFFFFFu, incl, 31);
-      for (int f0 = warp * 32 * kUpdUnroll; f0 < total; f0 += kIpWarps * 32 * kUpdUnroll) {
-        int idx[kUpdUnroll];
-#pragma unroll
-        for (int r = 0; r < kUpdUnroll; r++) {
-          const int f = f0 + r * 32 + lane;
-          int q = 0;
-#pragma unroll
-          for (int step = 16; step > 0; step >>= 1) {
-            const int val = __shfl_sync(0xFFFFFFFFu, incl, q + step - 1);
-            if (val <= f) q += step;
-          }
-          const int sq = __shfl_sync(0xFFFFFFFFu, rs, q), eq = __shfl_sync(0xFFFFFFFFu, excl, q);
-          idx[r] = f < total ? sq + (f - eq) : -1;
-        }
-        int2 e[kUpdUnroll];
-#pragma unroll
-        for (int r = 0; r < kUpdUnroll; r++) e[r] = idx[r] >= 0 ? a.ladj[idx[r]] : make_int2(-1, 0);
-#pragma unroll
-        for (int r = 0; r < kUpdUnroll; r++) {
-          if (e[r].x < 0) continue;
-          const uint8_t su = st[e[r].x];
-          if (su == S_FREE || su == S_FRONT) {
-            const int ng = atomicAdd(&g[e[r].x], 2 * e[r].y) + 2 * e[r].y;
-            if (su == S_FREE) st[e[r].x] = S_FRONT;
-            atomicMax(&best[e[r].x / kChunkNodes], gain_key(ng, e[r].x));
-          }
-        }
-      }
-    }
-    __syncthreads();
-    // the maxima over 32 chunks again, from the raised chunk maxima (one warp per group); the
-    // batched selection reads the chunk maxima alone
-    for (int sc = warp; sc < (batched ? 0 : nsup); sc += kIpWarps) {
-      const int c = sc * 32 + lane;
-      const unsigned long long x = wmax_u64(c < nch ? best[c] : 0ull);
-      if (lane == 0) sup[sc] = x;
-    }
-    __syncthreads();
+  }
+  __syncthreads();
+  if (a.trace && threadIdx.x == 0) {
+    atomicAdd(a.trace + 0, steps);
+    atomicAdd(a.trace + 1, (unsigned long long)nfall);
+    atomicAdd(a.trace + 2, retired);
   }
   // cut of this trial inside the subproblem
   unsigned long long cut = 0;
-  for (int jj = threadIdx.x; jj < cnt; jj += blockDim.x) {
-    if (st[jj] != S_ONE) continue;
-    const int p = start + jj;
-    for (int e = a.lxadj[p]; e < a.lxadj[p + 1]; e++) {
-      const int2 x = a.ladj[e];
-      if (st[x.x] != S_ONE) cut += (unsigned long long)x.y;
+  for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
+    if (X.get(j) != kOne) continue;
+    const int e1 = row_begin(j + 1);
+    for (int e = row_begin(j); e < e1; e++) {
+      const int2 x = entry(e);
+      if (X.get(x.x) != kOne) cut += (unsigned long long)x.y;
     }
   }
   cut = warp_sum(cut);
@@ -532,55 +578,62 @@ __global__ void __launch_bounds__(32 * kIpWarps) k_ip_grow(IpArgs a) {
     for (int q = 0; q < kIpWarps; q++) c += s_red[q];
     a.trial_cut[blockIdx.x] = (int64_t)c;
   }
-  uint8_t *fl = a.flags + (int64_t)t * a.n + start;
-  for (int jj = threadIdx.x; jj < cnt; jj += blockDim.x) fl[jj] = st[jj] == S_ONE;
+  uint8_t *fl = a.flags + tpos;
+  for (int j = threadIdx.x; j < cnt; j += blockDim.x) fl[j] = X.get(j) == kOne;
 }
 
-__global__ void k_sub_count(const int32_t *sp, const int32_t *vwgt, int n, int32_t *cnt, long long *w) {
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-    const int s = sp[v];
-    if (s < 0) continue;
-    atomicAdd(&cnt[s], 1);
-    atomicAdd((unsigned long long *)&w[s], (unsigned long long)vwgt[v]);
-  }
-}
+// Totals of the graph: node weight, heaviest node, largest weighted degree; and the list of depth 0.
+struct IpTotals {
+  unsigned long long W;
+  int cmax;
+  int pad;
+  unsigned long long dmax;
+};
 
-// sort keys: live nodes by (subproblem, id) first, finished nodes after them
-__global__ void k_sub_keys(const int32_t *sp, int n, int ns, uint64_t *keys, uint32_t *vals) {
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-    const int s = sp[v];
-    keys[v] = ((uint64_t)(uint32_t)(s >= 0 ? s : ns) << 32) | (uint32_t)v;
-    vals[v] = 0;
-  }
-}
-
-__global__ void k_sub_lists(const uint64_t *keys, int n, int live, const int32_t *start, const int32_t *vwgt,
-                            int32_t *vtx, int32_t *cvl, int2 *splo) {
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
-    const int v = (int)(uint32_t)keys[p];
-    if (p < live) {
-      const int s = (int)(keys[p] >> 32);
-      vtx[p] = v;
-      cvl[p] = vwgt[v];
-      splo[v] = make_int2(s, p - start[s]);
-    } else {
-      splo[v] = make_int2(-1, 0);
+__global__ void k_ip_init(const int32_t *xadj, const int32_t *vwgt, const int32_t *adjwgt, int n, int32_t *vtx,
+                          int32_t *cvl, int32_t *sub, int2 *splo, IpTotals *o) {
+  const int lane = (int)lane_id();
+  const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int nw = (gridDim.x * blockDim.x) >> 5;
+  unsigned long long w = 0, dm = 0;
+  int cm = 0;
+  for (int v = wid; v < n; v += nw) {
+    unsigned long long d = 0;
+    const int e1 = xadj[v + 1];
+    for (int e = xadj[v] + lane; e < e1; e += 32) d += (unsigned)adjwgt[e];
+    d = warp_sum(d);
+    dm = d > dm ? d : dm;
+    if (lane == 0) {
+      const int c = vwgt[v];
+      w += (unsigned long long)c;
+      cm = c > cm ? c : cm;
+      vtx[v] = v;
+      cvl[v] = c;
+      sub[v] = 0;
+      splo[v] = make_int2(0, v);
     }
+  }
+  if (lane == 0) {
+    if (w) atomicAdd(&o->W, w);
+    if (cm) atomicMax(&o->cmax, cm);
+    if (dm) atomicMax(&o->dmax, dm);
   }
 }
 
 // deg'(v) (weight to nodes of the same subproblem) and the number of such
 // neighbours, one warp per listed node
 __global__ void k_sub_dp(const int32_t *xadj, const int32_t *adjncy, const int32_t *adjwgt, const int32_t *vtx,
-                         const int2 *splo, int live, int32_t *dpl, int32_t *lcnt) {
+                         const int32_t *sub, const int2 *splo, int live, int32_t *dpl, int32_t *lcnt) {
   const int lane = (int)lane_id();
   const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nw = (gridDim.x * blockDim.x) >> 5;
+  if (wid == 0 && lane == 0) lcnt[live] = 0;
   for (int p = wid; p < live; p += nw) {
     const int v = vtx[p];
-    const int s = splo[v].x;
+    const int s = sub[p];
     int sum = 0, c = 0;
-    for (int e = xadj[v] + lane; e < xadj[v + 1]; e += 32)
+    const int e1 = xadj[v + 1];
+    for (int e = xadj[v] + lane; e < e1; e += 32)
       if (splo[adjncy[e]].x == s) { sum += adjwgt[e]; c++; }
     sum = warp_sum(sum);
     c = warp_sum(c);
@@ -590,18 +643,19 @@ __global__ void k_sub_dp(const int32_t *xadj, const int32_t *adjncy, const int32
 
 // local rows: (local index, weight) of the internal neighbours of every listed node
 __global__ void k_sub_rows(const int32_t *xadj, const int32_t *adjncy, const int32_t *adjwgt, const int32_t *vtx,
-                           const int2 *splo, int live, const int32_t *lxadj, int2 *ladj) {
+                           const int32_t *sub, const int2 *splo, int live, const int32_t *lxadj, int2 *ladj) {
   const int lane = (int)lane_id();
   const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nw = (gridDim.x * blockDim.x) >> 5;
   for (int p = wid; p < live; p += nw) {
     const int v = vtx[p];
-    const int s = splo[v].x;
+    const int s = sub[p];
     int pos = lxadj[p];
-    for (int e0 = xadj[v]; e0 < xadj[v + 1]; e0 += 32) {
+    const int e1 = xadj[v + 1];
+    for (int e0 = xadj[v]; e0 < e1; e0 += 32) {
       const int e = e0 + lane;
       int2 sl = make_int2(-1, 0);
-      if (e < xadj[v + 1]) sl = splo[adjncy[e]];
+      if (e < e1) sl = splo[adjncy[e]];
       const bool in = sl.x == s;
       const unsigned m = __ballot_sync(0xFFFFFFFFu, in);
       if (in) ladj[pos + __popc(m & lanemask_lt())] = make_int2(sl.y, adjwgt[e]);
@@ -610,37 +664,60 @@ __global__ void k_sub_rows(const int32_t *xadj, const int32_t *adjncy, const int
   }
 }
 
-__global__ void k_ip_select(const int64_t *trial_cut, int nsubs, int trials, int32_t *best) {
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < nsubs; s += gridDim.x * blockDim.x) {
-    int bt = 0;
-    for (int t = 1; t < trials; t++)
-      if (trial_cut[s * trials + t] < trial_cut[s * trials + bt]) bt = t;
-    best[s] = bt;
+// Every subproblem's best trial (smallest cut, then lowest trial): the side of every listed node, and the
+// number and weight of its side-1 nodes.  One block per subproblem.
+struct Side1 {
+  long long count, weight;
+};
+
+__global__ void __launch_bounds__(256) k_ip_side(const int64_t *trial_cut, const Sub *subs, int trials, int n,
+                                                 const uint8_t *flags, const int32_t *cvl, int32_t *side,
+                                                 Side1 *out) {
+  __shared__ long long s_c[8], s_w[8];
+  const int s = blockIdx.x;
+  int bt = 0;
+  for (int t = 1; t < trials; t++)
+    if (trial_cut[s * trials + t] < trial_cut[s * trials + bt]) bt = t;
+  const Sub S = subs[s];
+  long long c = 0, w = 0;
+  for (int j = threadIdx.x; j < S.count; j += blockDim.x) {
+    const int f = flags[(int64_t)bt * n + S.start + j];
+    side[S.start + j] = f;
+    c += f;
+    w += f ? cvl[S.start + j] : 0;
+  }
+  c = warp_sum(c);
+  w = warp_sum(w);
+  if (lane_id() == 0) { s_c[threadIdx.x >> 5] = c; s_w[threadIdx.x >> 5] = w; }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < 8; q++) { c += s_c[q]; w += s_w[q]; }
+    out[s].count = c;
+    out[s].weight = w;
   }
 }
 
-// children: child[2 s + side] = new subproblem index, or -(1 + block) when final
-__global__ void k_ip_assign(int n, int live, const int32_t *vtx, const int2 *splo, const int32_t *best,
-                            const uint8_t *flags, const int32_t *child, int32_t *sp, int32_t *blocks) {
+// The next depth's lists, in the same order within each child (so lists stay sorted by id): child[2 s] is
+// side 1, child[2 s + 1] side 0; .x = the child's subproblem index, or -(1 + block) when it is final,
+// .y = its list start.  rank = number of side-1 nodes at smaller positions.
+__global__ void k_ip_split(int live, const int32_t *vtx, const int32_t *cvl, const int32_t *sub, const int32_t *side,
+                           const int32_t *rank, const Sub *subs, const int2 *child, int32_t *vtx2, int32_t *cvl2,
+                           int32_t *sub2, int2 *splo, int32_t *blocks) {
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < live; p += gridDim.x * blockDim.x) {
-    const int v = vtx[p];
-    const int s = splo[v].x;
-    const int side1 = flags[(int64_t)best[s] * n + p];
-    const int c = child[2 * s + (side1 ? 0 : 1)];
-    if (c < 0) {
-      blocks[v] = -(c + 1);
-      sp[v] = -1;
-    } else {
-      sp[v] = c;
+    const int v = vtx[p], s = sub[p], st = subs[s].start;
+    const int r1 = rank[p] - rank[st];
+    const int2 c = child[2 * s + (side[p] ? 0 : 1)];
+    if (c.x < 0) {
+      blocks[v] = -(c.x + 1);
+      splo[v] = make_int2(-1, 0);
+      continue;
     }
+    const int r = side[p] ? r1 : p - st - r1;
+    vtx2[c.y + r] = v;
+    cvl2[c.y + r] = cvl[p];
+    sub2[c.y + r] = c.x;
+    splo[v] = make_int2(c.x, r);
   }
-}
-
-__global__ void k_max_weight(const int32_t *w, int n, int *out) {
-  int m = 0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) m = w[i] > m ? w[i] : m;
-  m = warp_max(m);
-  if (lane_id() == 0 && m) atomicMax(out, m);
 }
 
 int32_t ceil_log2(int64_t k) {
@@ -650,8 +727,17 @@ int32_t ceil_log2(int64_t k) {
 }
 
 struct HostSub {
-  int32_t kk, b0, bid;
+  int32_t kk, b0, bid, count;
+  int64_t W;
 };
+
+template <typename KT, bool SM>
+void launch_grow(gp_ctx *ctx, const IpArgs &a, int nblocks, size_t smem) {
+  if (SM)
+    GP_CUDA(cudaFuncSetAttribute(k_ip_grow<KT, SM>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmemBytes));
+  k_ip_grow<KT, SM><<<nblocks, 32 * kIpWarps, smem, ctx->stream>>>(a);
+  GP_LAUNCH_CHECK();
+}
 
 }  // namespace
 
@@ -663,106 +749,102 @@ void initial_partition(gp_ctx *ctx, const DevGraph &g, int32_t k, int64_t eps_pp
   GP_CUDA(cudaMemsetAsync(blocks, 0, sizeof(int32_t) * (n > 0 ? n : 1), ctx->stream));
   if (k <= 1 || n == 0) return;
   const int grid = grid_for(n, 256, ctx->num_sms * 8);
-  DBuf<int32_t> sp(ctx, (size_t)n), vtx(ctx, (size_t)n), cvl(ctx, (size_t)n), dpl(ctx, (size_t)n),
-      lxadj(ctx, (size_t)n + 1);
+  const int wgrid = grid_for((int64_t)n * 32, 256, ctx->num_sms * 8);
+  // two sets of lists: this depth's and the next one's
+  DBuf<int32_t> lists(ctx, (size_t)6 * n), dpl(ctx, (size_t)n), lxadj(ctx, (size_t)n + 1), side(ctx, (size_t)n),
+      rank(ctx, (size_t)n);
+  int32_t *vtx = lists.get(), *cvl = vtx + n, *sub = cvl + n, *vtx2 = sub + n, *cvl2 = vtx2 + n, *sub2 = cvl2 + n;
   DBuf<int2> ladj(ctx, (size_t)(g.m2 > 0 ? g.m2 : 1));
-  DBuf<int> maxc(ctx, 1);
   DBuf<int2> splo(ctx, (size_t)n);
-  DBuf<uint64_t> keys(ctx, (size_t)n);
-  DBuf<uint32_t> vals(ctx, (size_t)n);
-  sp.zero();  // everybody in subproblem 0
-  const int64_t eps_l = eps_ppm / ceil_log2(k);
-  std::vector<HostSub> subs{{k, 0, 1}};
-  GP_CUDA(cudaFuncSetAttribute(k_ip_grow, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmemBytes));
-  maxc.zero();
-  k_max_weight<<<grid, 256, 0, ctx->stream>>>(g.vwgt, n, maxc.get());
+  DBuf<IpTotals> tot(ctx, 1);
+  tot.zero();
+  k_ip_init<<<wgrid, 256, 0, ctx->stream>>>(g.xadj, g.vwgt, g.adjwgt, n, vtx, cvl, sub, splo.get(), tot.get());
   GP_LAUNCH_CHECK();
-  const int cvmax = read_scalar(ctx, maxc.get());
+  IpTotals ht;
+  read_back(ctx, tot.get(), sizeof(ht), &ht);
+  const int64_t eps_l = eps_ppm / ceil_log2(k);
+  std::vector<HostSub> subs{{k, 0, 1, n, (int64_t)ht.W}};
   DBuf<uint8_t> flags(ctx, (size_t)trials * n);
+  DBuf<int32_t> fnext, fhead;
+  // per depth, at most k subproblems: their records, trial cuts, side totals, children
+  DBuf<Sub> dsub(ctx, (size_t)k);
+  DBuf<int64_t> tcut(ctx, (size_t)k * trials);
+  DBuf<Side1> dside(ctx, (size_t)k);
+  DBuf<int2> dchild(ctx, (size_t)2 * k);
+  std::vector<Sub> hsub;
+  std::vector<Side1> hside;
+  std::vector<int2> hchild;
+  int live = n;
+  const bool trace = getenv("GP_TRACE") != nullptr;
   while (!subs.empty()) {
     const int ns = (int)subs.size();
-    DBuf<int32_t> cnt(ctx, (size_t)ns), start(ctx, (size_t)ns + 1);
-    DBuf<long long> wsum(ctx, (size_t)ns);
-    cnt.zero(); wsum.zero();
-    k_sub_count<<<grid, 256, 0, ctx->stream>>>(sp.get(), g.vwgt, n, cnt.get(), wsum.get());
-    GP_LAUNCH_CHECK();
-    std::vector<int32_t> hc(ns);
-    std::vector<long long> hw(ns);
-    read_back(ctx, cnt.get(), sizeof(int32_t) * ns, hc.data());
-    read_back(ctx, wsum.get(), sizeof(long long) * ns, hw.data());
-    std::vector<int32_t> hs(ns + 1);
-    hs[0] = 0;
-    for (int i = 0; i < ns; i++) hs[i + 1] = hs[i] + hc[i];
-    const int live = hs[ns];
-    GP_CUDA(cudaMemcpyAsync(start.get(), hs.data(), sizeof(int32_t) * (ns + 1), cudaMemcpyHostToDevice,
-                            ctx->stream));
-    k_sub_keys<<<grid, 256, 0, ctx->stream>>>(sp.get(), n, ns, keys.get(), vals.get());
-    GP_LAUNCH_CHECK();
-    radix_sort_pairs(ctx, keys.get(), vals.get(), n, 32 + 1 + ceil_log2(ns + 1));
-    k_sub_lists<<<grid, 256, 0, ctx->stream>>>(keys.get(), n, live, start.get(), g.vwgt, vtx.get(), cvl.get(),
-                                                splo.get());
-    GP_LAUNCH_CHECK();
-    k_sub_dp<<<grid_for((int64_t)live * 32, 256, ctx->num_sms * 8), 256, 0, ctx->stream>>>(
-        g.xadj, g.adjncy, g.adjwgt, vtx.get(), splo.get(), live, dpl.get(), lxadj.get());
-    GP_LAUNCH_CHECK();
-    GP_CUDA(cudaMemsetAsync(lxadj.get() + live, 0, sizeof(int32_t), ctx->stream));
-    scan_exclusive_i32(ctx, lxadj.get(), lxadj.get(), live + 1, nullptr);
-    k_sub_rows<<<grid_for((int64_t)live * 32, 256, ctx->num_sms * 8), 256, 0, ctx->stream>>>(
-        g.xadj, g.adjncy, g.adjwgt, vtx.get(), splo.get(), live, lxadj.get(), ladj.get());
-    GP_LAUNCH_CHECK();
-    std::vector<Sub> hsub(ns);
-    int maxcnt = 0;
+    hsub.resize((size_t)ns);
+    int maxcnt = 0, pos = 0;
     for (int i = 0; i < ns; i++) {
       const int64_t kk = subs[i].kk, k1 = (kk + 1) / 2;
-      const int64_t W = hw[i];
-      hsub[i].start = hs[i];
-      hsub[i].count = hc[i];
-      hsub[i].bid = subs[i].bid;
-      hsub[i].pad = 0;
-      hsub[i].T1 = (W * k1 + kk - 1) / kk;
-      hsub[i].L1 = (int64_t)(((__int128)hsub[i].T1 * (1000000 + eps_l)) / 1000000);
-      maxcnt = std::max(maxcnt, hc[i]);
+      Sub &s = hsub[(size_t)i];
+      s.start = pos;
+      s.count = subs[i].count;
+      s.bid = subs[i].bid;
+      s.pad = 0;
+      s.T1 = (subs[i].W * k1 + kk - 1) / kk;
+      s.L1 = (int64_t)(((__int128)s.T1 * (1000000 + eps_l)) / 1000000);
+      pos += s.count;
+      maxcnt = std::max(maxcnt, s.count);
     }
-    DBuf<Sub> dsub(ctx, (size_t)ns);
     GP_CUDA(cudaMemcpyAsync(dsub.get(), hsub.data(), sizeof(Sub) * ns, cudaMemcpyHostToDevice, ctx->stream));
+    if (live > 0) {
+      k_sub_dp<<<grid_for((int64_t)live * 32, 256, ctx->num_sms * 8), 256, 0, ctx->stream>>>(
+          g.xadj, g.adjncy, g.adjwgt, vtx, sub, splo.get(), live, dpl.get(), lxadj.get());
+      GP_LAUNCH_CHECK();
+      scan_exclusive_i32(ctx, lxadj.get(), lxadj.get(), live + 1, nullptr);
+      k_sub_rows<<<grid_for((int64_t)live * 32, 256, ctx->num_sms * 8), 256, 0, ctx->stream>>>(
+          g.xadj, g.adjncy, g.adjwgt, vtx, sub, splo.get(), live, lxadj.get(), ladj.get());
+      GP_LAUNCH_CHECK();
+    } else {
+      lxadj.zero();
+    }
     const int nblocks = ns * trials;
-    DBuf<int64_t> tcut(ctx, (size_t)nblocks);
     IpArgs a{};
     a.lxadj = lxadj.get(); a.ladj = ladj.get();
-    a.vtx = vtx.get(); a.cvl = cvl.get(); a.dpl = dpl.get();
+    a.vtx = vtx; a.cvl = cvl; a.dpl = dpl.get();
     a.subs = dsub.get(); a.trials = trials; a.n = n; a.seed = seed;
-    a.cv16 = cvmax <= 65535 ? 1 : 0;
-    // shared-memory state: chunk maxima (8 B per 64 nodes) + gain (4 B) + weight (2 B, when it fits) +
-    // state (1 B) per node, and the fallback hash (4 B) when that still holds every subproblem of
-    // this depth
-    int per_node = a.cv16 ? 7 : 5;
-    auto cap_for = [&](int pn) { return (kMaxSmemBytes - 128) * kChunkNodes / (9 + pn * kChunkNodes); };
-    a.hv_smem = maxcnt <= cap_for(per_node + 4) ? 1 : 0;
-    if (a.hv_smem) per_node += 4;
-    const int smem_cap = cap_for(per_node);
-    a.smem_nodes = std::max(1, std::min(maxcnt, smem_cap));
-    const int mch = (a.smem_nodes + kChunkNodes - 1) / kChunkNodes;
-    const size_t smem_bytes = (size_t)(mch + (mch + 31) / 32) * 8 + (size_t)a.smem_nodes * per_node;
-    DBuf<int32_t> gg;
-    DBuf<uint8_t> gst;
-    DBuf<uint16_t> gcv;
-    DBuf<unsigned long long> gbest, gsup;
-    if (maxcnt > a.smem_nodes) {
-      a.gnodes = maxcnt;
-      a.gchunks = (maxcnt + kChunkNodes - 1) / kChunkNodes;
-      gg.reset(ctx, (size_t)nblocks * a.gnodes);
-      gst.reset(ctx, (size_t)nblocks * a.gnodes);
-      if (a.cv16) gcv.reset(ctx, (size_t)nblocks * a.gnodes);
-      gbest.reset(ctx, (size_t)nblocks * a.gchunks);
-      gsup.reset(ctx, (size_t)nblocks * ((a.gchunks + 31) / 32));
-      a.gg = gg.get(); a.gst = gst.get(); a.gcv = gcv.get(); a.gbest = gbest.get(); a.gsup = gsup.get();
-    }
+    a.cv16 = ht.cmax <= 65535 ? 1 : 0;
     a.trial_cut = tcut.get();
     a.flags = flags.get();
+    // 32-bit words: |gain| is at most the weighted degree
+    const bool narrow = maxcnt < kNarrowNodes && ht.dmax < (unsigned long long)kNarrowGain;
+    const int64_t wb = narrow ? 4 : 8;
+    const int64_t nch = (maxcnt + kChunkNodes - 1) / kChunkNodes;
+    const int64_t need = wb * (maxcnt + nch) + (a.cv16 ? 2 * (int64_t)maxcnt + 4 : 0);
+    const bool sm = need <= kMaxSmemBytes && nch <= 512;
+    // what the blocks that share an SM leave of its shared memory goes to row bounds and rows
+    const int per_sm = std::min(8, (nblocks + ctx->num_sms - 1) / ctx->num_sms);
+    const int64_t share = std::min<int64_t>(kMaxSmemBytes, kSmSmem / per_sm - 1024 - kStaticSmem);
+    const int64_t smem = sm ? std::max<int64_t>(need, share) : 0;
+    a.smem_bytes = (int)smem;
+    DBuf<long long> gx, gbest, gsup;
+    if (!sm) {
+      a.bstride = n / kChunkNodes + ns + 1;
+      a.sstride = n / (32 * kChunkNodes) + ns + 1;
+      gx.reset(ctx, (size_t)trials * n);
+      gbest.reset(ctx, (size_t)trials * a.bstride);
+      gsup.reset(ctx, (size_t)trials * a.sstride);
+      a.gx = gx.get(); a.gbest = gbest.get(); a.gsup = gsup.get();
+    }
+    if (sm) {
+      a.hstride = n / kChainNodes + k + 1;
+      if (!fnext.get()) {
+        fnext.reset(ctx, (size_t)trials * n);
+        fhead.reset(ctx, (size_t)(trials * a.hstride));
+      }
+      a.fnext = fnext.get();
+      a.fhead = fhead.get();
+    }
     a.batch_cap = 1 + maxcnt / 1024;
-    DBuf<int32_t> gbatch(ctx, (size_t)nblocks * a.batch_cap);
+    DBuf<int32_t> gbatch;
+    if (a.batch_cap > kSmemBatch) gbatch.reset(ctx, (size_t)nblocks * a.batch_cap);
     a.gbatch = gbatch.get();
-    const bool trace = getenv("GP_TRACE") != nullptr;
     DBuf<unsigned long long> tr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (trace) {
@@ -773,44 +855,60 @@ void initial_partition(gp_ctx *ctx, const DevGraph &g, int32_t k, int64_t eps_pp
       GP_CUDA(cudaEventCreate(&e1));
       GP_CUDA(cudaEventRecord(e0, ctx->stream));
     }
-    k_ip_grow<<<nblocks, 32 * kIpWarps, smem_bytes, ctx->stream>>>(a);
-    GP_LAUNCH_CHECK();
+    if (narrow && sm) launch_grow<int32_t, true>(ctx, a, nblocks, (size_t)smem);
+    else if (sm) launch_grow<long long, true>(ctx, a, nblocks, (size_t)smem);
+    else launch_grow<long long, false>(ctx, a, nblocks, 0);
     if (trace) {
       GP_CUDA(cudaEventRecord(e1, ctx->stream));
       unsigned long long h[3];
       read_back(ctx, tr.get(), sizeof(h), h);
       float ms = 0;
       GP_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-      fprintf(stderr, "[gp ip] subproblems=%d max_nodes=%d grow_ms=%.2f steps=%llu fallbacks=%llu retired=%llu\n",
-              ns, maxcnt, ms, h[0], h[1], h[2]);
+      fprintf(stderr,
+              "[gp ip] subproblems=%d max_nodes=%d word=%d shared=%lld grow_ms=%.2f steps=%llu fallbacks=%llu "
+              "retired=%llu\n",
+              ns, maxcnt, narrow && sm ? 32 : 64, (long long)smem, ms, h[0], h[1], h[2]);
       cudaEventDestroy(e0);
       cudaEventDestroy(e1);
     }
-    DBuf<int32_t> best(ctx, (size_t)ns), child(ctx, (size_t)2 * ns);
-    k_ip_select<<<grid_for(ns, 128, 1024), 128, 0, ctx->stream>>>(tcut.get(), ns, trials, best.get());
+    k_ip_side<<<ns, 256, 0, ctx->stream>>>(tcut.get(), dsub.get(), trials, n, flags.get(), cvl, side.get(),
+                                           dside.get());
     GP_LAUNCH_CHECK();
+    if (live > 0) scan_exclusive_i32(ctx, side.get(), rank.get(), live, nullptr);
+    hside.resize((size_t)ns);
+    read_back(ctx, dside.get(), sizeof(Side1) * ns, hside.data());
     // children of every subproblem (final when they hold a single block)
-    std::vector<int32_t> hchild(2 * ns);
+    hchild.resize((size_t)2 * ns);
     std::vector<HostSub> next;
+    int next_live = 0;
     for (int i = 0; i < ns; i++) {
       const int32_t kk = subs[i].kk, k1 = (kk + 1) / 2, k2 = kk - k1;
-      const HostSub c1{k1, subs[i].b0, 2 * subs[i].bid}, c2{k2, subs[i].b0 + k1, 2 * subs[i].bid + 1};
-      const HostSub cs[2] = {c1, c2};
-      for (int side = 0; side < 2; side++) {
-        if (cs[side].kk <= 1) {
-          hchild[2 * i + side] = -(cs[side].b0 + 1);
+      const Side1 &o = hside[(size_t)i];
+      const HostSub cs[2] = {{k1, subs[i].b0, 2 * subs[i].bid, (int32_t)o.count, o.weight},
+                             {k2, subs[i].b0 + k1, 2 * subs[i].bid + 1, subs[i].count - (int32_t)o.count,
+                              subs[i].W - o.weight}};
+      for (int q = 0; q < 2; q++) {
+        if (cs[q].kk <= 1) {
+          hchild[(size_t)(2 * i + q)] = make_int2(-(cs[q].b0 + 1), 0);
         } else {
-          hchild[2 * i + side] = (int32_t)next.size();
-          next.push_back(cs[side]);
+          hchild[(size_t)(2 * i + q)] = make_int2((int)next.size(), next_live);
+          next.push_back(cs[q]);
+          next_live += cs[q].count;
         }
       }
     }
-    GP_CUDA(cudaMemcpyAsync(child.get(), hchild.data(), sizeof(int32_t) * 2 * ns, cudaMemcpyHostToDevice,
-                            ctx->stream));
-    k_ip_assign<<<grid, 256, 0, ctx->stream>>>(n, live, vtx.get(), splo.get(), best.get(), flags.get(),
-                                                child.get(), sp.get(), blocks);
-    GP_LAUNCH_CHECK();
-    GP_CUDA(cudaStreamSynchronize(ctx->stream));  // host vectors above must outlive the copies
+    if (live > 0) {
+      GP_CUDA(cudaMemcpyAsync(dchild.get(), hchild.data(), sizeof(int2) * 2 * ns, cudaMemcpyHostToDevice,
+                              ctx->stream));
+      k_ip_split<<<grid, 256, 0, ctx->stream>>>(live, vtx, cvl, sub, side.get(), rank.get(), dsub.get(),
+                                                dchild.get(), vtx2, cvl2, sub2, splo.get(), blocks);
+      GP_LAUNCH_CHECK();
+      std::swap(vtx, vtx2);
+      std::swap(cvl, cvl2);
+      std::swap(sub, sub2);
+    }
+    live = next_live;
+    GP_CUDA(cudaStreamSynchronize(ctx->stream));  // the host vectors must outlive the copies
     subs.swap(next);
   }
 }

@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(256) k_mod_rows(const int32_t *xadj, const int
       int q[kModUnroll], Lq[kModUnroll], w[kModUnroll], v[kModUnroll];
 #pragma unroll
       for (int r = 0; r < kModUnroll; r++) {
-        q[r] = wk.owner(f0 + r * 32 + lane);
+        q[r] = wk.owner(f0 + r * 32);
         Lq[r] = __shfl_sync(FULL, Lu, q[r]);
       }
 #pragma unroll

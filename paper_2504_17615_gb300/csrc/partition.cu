@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(256) k_validate_entries(const int32_t *xadj, c
 #pragma unroll
       for (int r = 0; r < kValUnroll; r++) {
         e[r] = f0 + r * 32 + lane;
-        const int q = wk.owner(e[r]);
+        const int q = wk.owner(f0 + r * 32);
         row[r] = (int)(u0 + q);
         rs[r] = __shfl_sync(FULL, xs, q);
       }
@@ -81,7 +81,12 @@ __global__ void __launch_bounds__(256) k_validate_entries(const int32_t *xadj, c
         const bool in = e[r] < e1;
         v[r] = in ? adjncy[e[r]] : 0;
         w[r] = in ? adjwgt[e[r]] : 1;
-        pv[r] = in && e[r] > rs[r] ? adjncy[e[r] - 1] : -1;
+      }
+#pragma unroll
+      for (int r = 0; r < kValUnroll; r++) {  // the entry before: the lane before's, except in lane 0
+        pv[r] = __shfl_up_sync(FULL, v[r], 1);
+        if (lane == 0 && e[r] < e1 && e[r] > rs[r]) pv[r] = adjncy[e[r] - 1];
+        if (e[r] <= rs[r]) pv[r] = -1;
       }
 #pragma unroll
       for (int r = 0; r < kValUnroll; r++) {
@@ -136,7 +141,7 @@ __global__ void __launch_bounds__(256) k_cut(const int32_t *xadj, const int32_t 
 #pragma unroll
       for (int r = 0; r < R; r++) {
         e[r] = f0 + r * 32 + lane;
-        bo[r] = __shfl_sync(FULL, bu, wk.owner(e[r]));
+        bo[r] = __shfl_sync(FULL, bu, wk.owner(f0 + r * 32));
       }
 #pragma unroll
       for (int r = 0; r < R; r++) {

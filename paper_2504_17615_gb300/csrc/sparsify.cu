@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(256) k_keep(KeepArgs a) {
 #pragma unroll
       for (int r = 0; r < kKeepUnroll; r++) {
         e[r] = f0 + r * 32 + lane;
-        j[r] = wk.owner(e[r]);
+        j[r] = wk.owner(f0 + r * 32);
       }
 #pragma unroll
       for (int r = 0; r < kKeepUnroll; r++) {
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(256) k_hash_digit(HashHistArgs a) {
     const int e1 = wk.e1;
     for (int f0 = wk.e0; f0 < e1; f0 += 32) {
       const int e = f0 + lane;
-      const int q = wk.owner(e);
+      const int q = wk.owner(f0);
       if (e >= e1) continue;
       const int row = (int)(u0 + q), v = __ldcs(a.adjncy + e);
       if (row >= v || __ldcs(a.adjwgt + e) != a.wt) continue;
