@@ -10,9 +10,9 @@
 //           which write (coarse id of the neighbour, weight) into the owner's
 //           segment; entries inside the cluster are marked;
 //  merge  : each segment is summed by coarse neighbour in a hash table (a
-//           warp with a shared-memory table up to 256 entries, a block with
-//           a 4096-slot shared or a global table above) and written back in
-//           place, compacted;
+//           warp with a shared-memory table up to 128 entries, a block with
+//           a 4096-slot shared table up to 2048, many blocks with a table in
+//           global memory above) and written back in place, compacted;
 // and the merged rows are finally packed into the coarse CSR.  Row order
 // inside a coarse row is unspecified.
 #include "gp_internal.cuh"
@@ -28,6 +28,9 @@ constexpr int kWarpSlots = 256;
 constexpr int kWarpMaxUb = 128;
 constexpr int kBlockSmemSlots = 4096;
 constexpr int kMapUnroll = 8;
+constexpr int kHugeSeg = 2048;       // segments above this many entries are merged by many blocks
+constexpr int kSegChunk = 2048;      // their entries per block and step
+constexpr int kSegTabChunk = 4096;   // and table slots
 
 __device__ __forceinline__ unsigned slot_hash(int B, int bits) {
   return ((unsigned)B * 2654435761u) >> (32 - bits);
@@ -110,7 +113,8 @@ struct MergeArgs {
   int nc;
   int2 *temp;
   int32_t *rowcnt;
-  int32_t *large, *nlarge;
+  int32_t *large, *nlarge;  // segments for a block each, from the front; huge ones (nlarge[1]) from the back
+  int split_huge;           // 1: segments above kHugeSeg go to the huge list
   int32_t *gkeys, *gvals;
   int64_t gstride;
   unsigned long long *units;
@@ -131,7 +135,10 @@ __global__ void __launch_bounds__(kThreads) k_merge_warp(MergeArgs a) {
     const int s0 = a.tstart[A], s1 = a.tstart[A + 1];
     const int len = s1 - s0;
     if (len > kWarpMaxUb) {
-      if (lane == 0) a.large[atomicAdd(a.nlarge, 1)] = A;
+      if (lane == 0) {
+        if (a.split_huge && len > kHugeSeg) a.large[a.nc - atomicAdd(a.nlarge + 1, 1)] = A;
+        else a.large[atomicAdd(a.nlarge, 1)] = A;
+      }
       continue;
     }
     const int bits = table_bits(len), tsize = 1 << bits;
@@ -201,13 +208,193 @@ __global__ void __launch_bounds__(kThreads) k_merge_block(MergeArgs a) {
   if (a.units && threadIdx.x == 0) atomicAdd(a.units + 3, uout);
 }
 
-__global__ void k_max_i32(const int32_t *x, int n, int *out) {
-  int m = 0;
+// Longest segment, number of huge ones and table slots they need together.
+struct SegStats {
+  int longest, huge;
+  unsigned long long slots;
+};
+
+__device__ __forceinline__ int seg_slots(int len) { return len + len / 3 + 1; }
+
+__global__ void k_seg_stats(const int32_t *x, int n, SegStats *out) {
+  int m = 0, nh = 0;
+  unsigned long long ns = 0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    m = x[i] > m ? x[i] : m;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const int l = x[i];
+    m = l > m ? l : m;
+    if (l > kHugeSeg) { nh++; ns += (unsigned long long)seg_slots(l); }
+  }
   m = warp_max(m);
-  if (lane_id() == 0 && m) atomicMax(out, m);
+  if (lane_id() == 0 && m) atomicMax(&out->longest, m);
+  if (__any_sync(FULL, nh)) {
+    nh = warp_sum(nh);
+    ns = warp_sum(ns);
+    if (lane_id() == 0) { atomicAdd(&out->huge, nh); atomicAdd(&out->slots, ns); }
+  }
+}
+
+// ------------------------------------- huge segments: many blocks a segment
+//
+// A coarse node that holds a hub has a segment of up to several 1e5 entries; one block with a table in
+// global memory took milliseconds for it while the rest of the device waited (12 levels of the scale-24
+// R-MAT graph: 131 ms of contraction).  k_seg_plan lists the huge segments with the prefix sums of their
+// chunks, k_seg_insert sums 2048 entries at a time in a shared table and adds the sums to the segment's
+// table in global memory (4/3 slots an entry), and k_seg_extract writes the occupied slots back to the
+// segment.  Consecutive steps work on the same few tables, which stay in L2 meanwhile.
+
+struct Seg {
+  int A, s0, len, tsize;
+  long long toff;
+};
+
+struct SegArgs {
+  Seg *segs;
+  int *chunk0, *tchunk0;  // prefix sums of entry chunks and table chunks; [count] = totals
+  int2 *tab;              // (coarse neighbour, weight) slots
+};
+
+__global__ void __launch_bounds__(1024) k_seg_plan(MergeArgs a, SegArgs h) {
+  __shared__ long long s_w[3][32];
+  const int cnt = a.nlarge[1];
+  const int lane = (int)lane_id(), wp = threadIdx.x >> 5;
+  long long run[3] = {0, 0, 0};  // entry chunks, table chunks, table slots
+  for (int b = 0; b < cnt; b += 1024) {
+    const int i = b + (int)threadIdx.x;
+    Seg x{};
+    if (i < cnt) {
+      x.A = a.large[a.nc - i];
+      x.s0 = a.tstart[x.A];
+      x.len = a.tstart[x.A + 1] - x.s0;
+      x.tsize = seg_slots(x.len);
+    }
+    const long long val[3] = {(x.len + kSegChunk - 1) / kSegChunk, (x.tsize + kSegTabChunk - 1) / kSegTabChunk, x.tsize};
+    long long ex[3];
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      long long y = val[q];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const long long z = __shfl_up_sync(FULL, y, o);
+        if (lane >= o) y += z;
+      }
+      if (lane == 31) s_w[q][wp] = y;
+      ex[q] = y - val[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      long long before = run[q], total = run[q];
+      for (int w = 0; w < 32; w++) {
+        if (w < wp) before += s_w[q][w];
+        total += s_w[q][w];
+      }
+      ex[q] += before;
+      run[q] = total;
+    }
+    if (i < cnt) {
+      x.toff = ex[2];
+      h.segs[i] = x;
+      h.chunk0[i] = (int)ex[0];
+      h.tchunk0[i] = (int)ex[1];
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    h.chunk0[cnt] = (int)run[0];
+    h.tchunk0[cnt] = (int)run[1];
+  }
+}
+
+__device__ __forceinline__ int seg_of(const int *first, int cnt, int it) {
+  int lo = 0, hi = cnt;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (first[mid] <= it) lo = mid; else hi = mid;
+  }
+  return lo;
+}
+
+__global__ void k_seg_clear(int2 *tab, int64_t n) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    tab[i] = make_int2(-1, 0);
+}
+
+__global__ void __launch_bounds__(kThreads) k_seg_insert(MergeArgs a, SegArgs h) {
+  __shared__ int s_k[2 * kSegChunk];
+  __shared__ int s_v[2 * kSegChunk];
+  constexpr int BITS = 12;
+  static_assert((1 << BITS) == 2 * kSegChunk, "table size");
+  const int cnt = a.nlarge[1], items = h.chunk0[cnt];
+  for (int t = threadIdx.x; t < 2 * kSegChunk; t += blockDim.x) { s_k[t] = -1; s_v[t] = 0; }
+  for (int it = blockIdx.x; it < items; it += gridDim.x) {
+    const int si = seg_of(h.chunk0, cnt, it);
+    const Seg x = h.segs[si];
+    int2 *tab = h.tab + x.toff;
+    const int c0 = (it - h.chunk0[si]) * kSegChunk, c1 = min(x.len, c0 + kSegChunk);
+    constexpr int R = kSegChunk / kThreads;
+    int2 e[R];
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const int j = c0 + r * kThreads + (int)threadIdx.x;
+      e[r] = j < c1 ? __ldcs(a.temp + x.s0 + j) : make_int2(-1, 0);
+    }
+    __syncthreads();  // the shared table is empty
+#pragma unroll
+    for (int r = 0; r < R; r++)
+      if (e[r].x >= 0) table_add(s_k, s_v, 2 * kSegChunk - 1, BITS, e[r].x, e[r].y);
+    __syncthreads();
+    for (int t = threadIdx.x; t < 2 * kSegChunk; t += blockDim.x) {
+      const int B = s_k[t];
+      if (B < 0) continue;
+      const int w = s_v[t];
+      s_k[t] = -1;
+      s_v[t] = 0;
+      int s = (int)__umulhi((unsigned)B * 2654435761u, (unsigned)x.tsize);
+      for (int probe = 0; probe < x.tsize; probe++) {  // bounded: more slots than entries
+        const int prev = atomicCAS(&tab[s].x, -1, B);
+        if (prev == -1 || prev == B) { atomicAdd(&tab[s].y, w); break; }
+        s = s + 1 == x.tsize ? 0 : s + 1;
+      }
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kThreads) k_seg_extract(MergeArgs a, SegArgs h) {
+  const int cnt = a.nlarge[1], items = h.tchunk0[cnt];
+  unsigned long long uout = 0;
+  for (int it = blockIdx.x; it < items; it += gridDim.x) {
+    const int si = seg_of(h.tchunk0, cnt, it);
+    const Seg x = h.segs[si];
+    const int2 *tab = h.tab + x.toff;
+    const int t0 = (it - h.tchunk0[si]) * kSegTabChunk, t1 = min(x.tsize, t0 + kSegTabChunk);
+    constexpr int R = 8;
+    for (int b = t0 + (int)(threadIdx.x & ~31u); b < t1; b += kThreads * R) {  // a warp's R x 32 slots a step
+      int2 e[R];
+      unsigned m[R];
+      int n = 0;
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        const int t = b + r * kThreads + (int)lane_id();
+        e[r] = t < t1 ? __ldcs(tab + t) : make_int2(-1, 0);
+      }
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        m[r] = __ballot_sync(FULL, e[r].x >= 0);
+        n += __popc(m[r]);
+      }
+      int pos = 0;
+      if (lane_id() == 0 && n) pos = atomicAdd(&a.rowcnt[x.A], n);
+      pos = x.s0 + __shfl_sync(FULL, pos, 0);
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        if (e[r].x >= 0) a.temp[pos + __popc(m[r] & lanemask_lt())] = e[r];
+        pos += __popc(m[r]);
+      }
+      uout += (unsigned)n;
+    }
+  }
+  if (a.units && lane_id() == 0 && uout) atomicAdd(a.units + 3, uout);
 }
 
 // Packs the merged rows from the segment layout into the final CSR.
@@ -243,7 +430,7 @@ void contract_graph(gp_ctx *ctx, const DevGraph &g, const int32_t *cmap, int32_t
     scan_exclusive_i32(ctx, seg.get(), tstart.get(), nc + 1, nullptr);
   }
   DBuf<int2> temp(ctx, (size_t)(g.m2 > 0 ? g.m2 : 1));
-  DBuf<int32_t> rowcnt(ctx, (size_t)nc + 1), large(ctx, (size_t)nc + 1), nlarge(ctx, 1);
+  DBuf<int32_t> rowcnt(ctx, (size_t)nc + 1), large(ctx, (size_t)nc + 1), nlarge(ctx, 2);
   rowcnt.zero();
   nlarge.zero();
   MergeArgs a{};
@@ -251,17 +438,30 @@ void contract_graph(gp_ctx *ctx, const DevGraph &g, const int32_t *cmap, int32_t
   a.large = large.get(); a.nlarge = nlarge.get();
   unsigned long long *units = ctx->d_units ? ctx->d_units + PROF_CONTRACT * PROF_UNITS : nullptr;
   a.units = units;
-  // global tables when some coarse node needs more than the shared table
-  DBuf<int> maxseg(ctx, 1);
-  maxseg.zero();
-  k_max_i32<<<grid_for(nc, 256, ctx->num_sms * 8), 256, 0, ctx->stream>>>(seg.get(), nc, maxseg.get());
+  // segments beyond the shared tables: tables of their own, or, when those together would take more memory
+  // than the bound of table_blocks, per-block global tables
+  DBuf<SegStats> sstats(ctx, 1);
+  sstats.zero();
+  k_seg_stats<<<grid_for(nc, 256, ctx->num_sms * 8), 256, 0, ctx->stream>>>(seg.get(), nc, sstats.get());
   GP_LAUNCH_CHECK();
-  const int mseg = read_scalar(ctx, maxseg.get());
+  SegStats hs;
+  read_back(ctx, sstats.get(), sizeof(hs), &hs);
   int bits = 1;
-  while ((1 << bits) < 2 * mseg) bits++;
+  while ((1 << bits) < 2 * hs.longest) bits++;
   int lblocks = ctx->num_sms * 4;
   DBuf<int32_t> gk, gv;
-  if ((1 << bits) > kBlockSmemSlots) {
+  SegArgs sg{};
+  DBuf<Seg> segs;
+  DBuf<int> chunk0, tchunk0;
+  DBuf<int2> tab;
+  a.split_huge = hs.huge > 0 && 8 * (int64_t)hs.slots <= 8 * g.m2 + ((int64_t)16 << 20) ? 1 : 0;
+  if (a.split_huge) {
+    segs.reset(ctx, (size_t)hs.huge);
+    chunk0.reset(ctx, (size_t)hs.huge + 1);
+    tchunk0.reset(ctx, (size_t)hs.huge + 1);
+    tab.reset(ctx, (size_t)hs.slots);
+    sg = SegArgs{segs.get(), chunk0.get(), tchunk0.get(), tab.get()};
+  } else if ((1 << bits) > kBlockSmemSlots) {
     a.gstride = (int64_t)1 << bits;
     lblocks = table_blocks(g.m2, a.gstride, lblocks);
     gk.reset(ctx, (size_t)(a.gstride * lblocks));
@@ -278,8 +478,21 @@ void contract_graph(gp_ctx *ctx, const DevGraph &g, const int32_t *cmap, int32_t
     }
     k_merge_warp<<<grid_for((int64_t)nc * 32, kThreads, ctx->num_sms * 8), kThreads, 0, ctx->stream>>>(a);
     GP_LAUNCH_CHECK();
-    k_merge_block<<<lblocks, kThreads, 0, ctx->stream>>>(a);
-    GP_LAUNCH_CHECK();
+    if (hs.longest > kWarpMaxUb) {
+      k_merge_block<<<lblocks, kThreads, 0, ctx->stream>>>(a);
+      GP_LAUNCH_CHECK();
+    }
+    if (a.split_huge) {
+      k_seg_plan<<<1, 1024, 0, ctx->stream>>>(a, sg);
+      GP_LAUNCH_CHECK();
+      k_seg_clear<<<grid_for((int64_t)hs.slots, kThreads, ctx->num_sms * 8), kThreads, 0, ctx->stream>>>(
+          tab.get(), (int64_t)hs.slots);
+      GP_LAUNCH_CHECK();
+      k_seg_insert<<<ctx->num_sms * 6, kThreads, 0, ctx->stream>>>(a, sg);
+      GP_LAUNCH_CHECK();
+      k_seg_extract<<<ctx->num_sms * 8, kThreads, 0, ctx->stream>>>(a, sg);
+      GP_LAUNCH_CHECK();
+    }
   }
   DBuf<int32_t> total(ctx, 1);
   out.n = nc;

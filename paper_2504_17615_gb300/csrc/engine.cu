@@ -265,9 +265,55 @@ void engine_fill(gp_batch_item *items, const EngineJob &job, const std::vector<E
 
 }  // namespace
 
+namespace {
+
+// Without a tuning of the caller's the engine takes the items of up to kSplitFloor entries, and larger ones
+// up to the size at which the slower of the two paths, which run side by side, ends first.  An item is one
+// CTA's work from start to end, so one large item can outlast everything else: with all items of up to 2^22
+// entries on the engine a batch of 128 graphs of 1e3..1e5 nodes took 690 ms, 0.65 s of it in the CTA of the
+// largest R-MAT graph; split by this rule it takes SPLITNUM.  Costs in ms, measured on that mix (ER, grids,
+// R-MAT, k = 2..64): an item in its CTA takes 0.3-0.6 us per entry, up to 2.3 us where the bisection finds
+// many components, so kCtaPerEntry lies at the upper end; a graph on the per-graph path takes 1.7 ms (6k
+// entries), 4.5 (48k), 8.4 (195k), 13-15 (0.4-1.6M) with one worker, and the workers together get four times
+// one worker's rate (8 workers 0.41, 1.07, 2.2, 3.5-4.2 ms; 16 the same).
+constexpr int64_t kSplitFloor = 1 << 15;
+constexpr double kCtaPerEntry = 2.0e-3, kCtaBase = 4.0;
+constexpr double kPathBase = 1.6, kPathPerEntry = 5.0e-5, kPathMost = 14.0, kPathWorkers = 4.0;
+
+int64_t split_entries(const gp_batch_item *items, const std::vector<int32_t> &idx, int workers,
+                      const gp_batch_tuning &t, int ctas) {
+  std::vector<int64_t> m2;
+  double path = 0;
+  const double conc = std::min<double>(kPathWorkers, workers);
+  auto path_ms = [&](int64_t m) { return std::min(kPathMost, kPathBase + kPathPerEntry * (double)m) / conc; };
+  for (int32_t i : idx) {
+    path += path_ms(items[i].g.m2);
+    if (engine_item_ok(items[i], t)) m2.push_back(items[i].g.m2);
+  }
+  std::sort(m2.begin(), m2.end());
+  int64_t best = kSplitFloor;
+  double best_ms = -1, cta_sum = 0;
+  for (size_t j = 0; j < m2.size(); j++) {
+    const double item = kCtaBase + kCtaPerEntry * (double)m2[j];
+    cta_sum += item;
+    path -= path_ms(m2[j]);
+    const double ms = std::max(path, std::max(item, cta_sum / ctas));
+    if (m2[j] <= kSplitFloor || best_ms < 0 || ms < best_ms) {
+      best_ms = ms;
+      best = std::max(kSplitFloor, m2[j]);
+    }
+  }
+  return best;
+}
+
+}  // namespace
+
 void batch_run(gp_ctx *ctx, gp_batch_item *items, const std::vector<int32_t> &idx, int workers, const gp_config &cfg,
-               const gp_batch_tuning &t) {
+               const gp_batch_tuning &given) {
+  gp_batch_tuning t = given;
   const bool use = t.engine && engine_config_ok(cfg);
+  if (use && !ctx->tuning_given)
+    t.max_entries = std::min(t.max_entries, split_entries(items, idx, workers, t, ctx->num_sms));
   EngineJob job;
   std::vector<int32_t> rest;
   bool want_stats = false;
@@ -341,6 +387,7 @@ gp_status gp_batch_set_tuning(gp_ctx *ctx, const gp_batch_tuning *t) {
   }
   ctx->tuning = x;
   ctx->tuning_set = true;
+  ctx->tuning_given = true;
   return GP_OK;
 }
 
@@ -494,6 +541,7 @@ gp_status gp_batch_autotune(gp_ctx *ctx, const gp_batch_item *items, int32_t cou
   T.tune_ms = now_ms() - t0;
   ctx->tuning = T;
   ctx->tuning_set = true;
+  ctx->tuning_given = true;
   if (out) *out = T;
   return GP_OK;
 }

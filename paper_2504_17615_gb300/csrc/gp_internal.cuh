@@ -117,7 +117,8 @@ struct gp_ctx {
   int64_t wait_spins = 0;                        // limit of device-side waits (0: default)
   int device_share = 1;  // contexts sharing the device (batch / server workers): persistent grids shrink
   gp_batch_tuning tuning{};        // batched engine settings (gp_batch_set_tuning / gp_batch_autotune)
-  bool tuning_set = false;
+  bool tuning_set = false;         // tuning holds values (defaults or the caller's)
+  bool tuning_given = false;       // ... the caller's or the autotuner's: the engine's share is as they say
   cudaStream_t copy_streams[4] = {};  // host-to-device copies of large inputs
   cudaEvent_t copy_events[5] = {};
 };

@@ -729,6 +729,315 @@ __global__ void __launch_bounds__(kThreads) k_rate_large(RateArgs a) {
   add_units(a.units, ue, uv, uc, up, a.label8 != nullptr, a.adjwgt == nullptr);
 }
 
+// ------------------------------------------------- hubs: many blocks a node
+//
+// A node of more than kHubDeg neighbours is rated by as many blocks as its row has chunks.  With one block
+// a node, a sub-round waited for the block of the largest hub: 8 ms in every sub-round of the scale-24
+// R-MAT graph (4e5 neighbours, a 2^20-slot table in global memory walked by 256 threads), 330 ms for
+// level 1.  k_hub_plan lists the sub-round's hubs with the prefix sums of their chunks; then
+//  few labels (at most kHubDense: refinement): k_hub_dense counts a chunk per label in shared memory, adds
+//    it to the hub's counters, and the block that finishes a hub's last chunk chooses;
+//  many labels: k_hub_insert sums a chunk's labels in a shared table and adds the sums to the hub's table
+//    in global memory (4/3 slots per neighbour), k_hub_max walks the tables (4096 slots a block) for the
+//    largest admissible rating, and k_hub_pick walks them again for the smallest (hash, label) of that
+//    rating and leaves them empty.
+// The choice is the same as in the other kernels.
+
+constexpr int kHubChunk = 2048;    // row entries per block and step
+constexpr int kHubTabChunk = 4096; // table slots per block and step
+constexpr int kHubDense = 1024;    // labels up to which a hub's ratings are counted per label
+
+struct Hub {
+  int pos, v, st, deg, cv, own;  // list position, node, row offset, degree, weight, label
+  int tsize, done;               // table slots; blocks that finished (dense, pick)
+  long long toff;                // table offset
+  int rmax, ownr, rall, pad;     // ratings: largest admissible, own label's, largest of any other label
+  unsigned long long best;       // smallest (hash, label) of rating rmax
+};
+
+struct HubArgs {
+  Hub *hubs;
+  int *chunk0, *tchunk0;  // prefix sums of row chunks and of table chunks; [count] = totals
+  int2 *tab;              // (label, rating) slots, empty (-1, 0) between sub-rounds
+  int32_t *hist;          // dense: [hub][nlabels], zero between sub-rounds
+  int nlabels;
+};
+
+__device__ __forceinline__ int hub_slots(int deg) { return deg + deg / 3 + 1; }
+
+__global__ void __launch_bounds__(1024) k_hub_plan(RateArgs a, HubArgs h) {
+  __shared__ long long s_w[3][32];
+  if (a.stop && *a.stop) return;
+  const int begin = a.offs[a.key], cnt = list_end(a) - begin;
+  const int lane = (int)lane_id(), wp = threadIdx.x >> 5;
+  long long run[3] = {0, 0, 0};  // row chunks, table chunks, table slots
+  for (int b = 0; b < cnt; b += 1024) {
+    const int i = b + (int)threadIdx.x;
+    int deg = 0;
+    Hub x{};
+    if (i < cnt) {
+      const int4 rec = a.list[begin + i];
+      x.pos = begin + i; x.v = rec.x; x.st = rec.y; x.cv = rec.w;
+      deg = a.dirty && !a.dirty[rec.x] ? 0 : rec.z;  // clean: cannot move
+      if (deg == 0) a.prop[begin + i] = make_int2(-1, 0);
+      x.deg = deg;
+      x.own = label_of(a, rec.x);
+      x.tsize = deg > 0 ? hub_slots(deg) : 0;
+      x.rmax = -1;
+      x.best = ~0ull;
+    }
+    const long long val[3] = {(deg + kHubChunk - 1) / kHubChunk, (x.tsize + kHubTabChunk - 1) / kHubTabChunk, x.tsize};
+    long long ex[3];
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      long long y = val[q];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const long long z = __shfl_up_sync(FULL, y, o);
+        if (lane >= o) y += z;
+      }
+      if (lane == 31) s_w[q][wp] = y;
+      ex[q] = y - val[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      long long before = run[q], total = run[q];
+      for (int w = 0; w < 32; w++) {
+        if (w < wp) before += s_w[q][w];
+        total += s_w[q][w];
+      }
+      ex[q] += before;
+      run[q] = total;
+    }
+    if (i < cnt) {
+      x.toff = ex[2];
+      h.hubs[i] = x;
+      h.chunk0[i] = (int)ex[0];
+      h.tchunk0[i] = (int)ex[1];
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    h.chunk0[cnt] = (int)run[0];
+    h.tchunk0[cnt] = (int)run[1];
+  }
+}
+
+// The hub whose chunks hold item `it`: the last one with first[i] <= it.
+__device__ __forceinline__ int hub_of(const int *first, int cnt, int it) {
+  int lo = 0, hi = cnt;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (first[mid] <= it) lo = mid; else hi = mid;
+  }
+  return lo;
+}
+
+__device__ __forceinline__ void hub_emit(const RateArgs &a, const Hub &x, int rmax, int ownr, int rall,
+                                         unsigned long long best) {
+  if (a.dirty && rall <= ownr) a.dirty[x.v] = 0;
+  if (rmax < 0 || rmax <= ownr) a.prop[x.pos] = make_int2(-1, 0);
+  else emit<RATE_LP>(a, x.pos, x.v, (int)(uint32_t)best, x.cv, x.own);
+}
+
+__global__ void __launch_bounds__(kThreads) k_hub_dense(RateArgs a, HubArgs h) {
+  extern __shared__ int s_hist[];  // nlabels
+  __shared__ int s_ri[kWarpsPerBlock];
+  __shared__ uint64_t s_ru[kWarpsPerBlock];
+  __shared__ bool s_last;
+  if (a.stop && *a.stop) return;
+  const int cnt = list_end(a) - a.offs[a.key], items = h.chunk0[cnt];
+  for (int t = threadIdx.x; t < h.nlabels; t += blockDim.x) s_hist[t] = 0;
+  unsigned long long ue = 0, uv = 0;
+  for (int it = blockIdx.x; it < items; it += gridDim.x) {
+    const int hi = hub_of(h.chunk0, cnt, it);
+    const Hub x = h.hubs[hi];
+    const int c0 = (it - h.chunk0[hi]) * kHubChunk, c1 = min(x.deg, c0 + kHubChunk);
+    constexpr int R = kHubChunk / kThreads;
+    int u[R], w[R];
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const int j = c0 + r * kThreads + (int)threadIdx.x;
+      u[r] = j < c1 ? __ldcs(a.adjncy + x.st + j) : -1;
+      w[r] = j < c1 && a.adjwgt ? __ldcs(a.adjwgt + x.st + j) : 1;
+    }
+    __syncthreads();  // the counters are empty
+#pragma unroll
+    for (int r = 0; r < R; r++)
+      if (u[r] >= 0) atomicAdd(&s_hist[label_of(a, u[r])], w[r]);
+    __syncthreads();
+    int32_t *hist = h.hist + (int64_t)hi * h.nlabels;
+    for (int t = threadIdx.x; t < h.nlabels; t += blockDim.x) {
+      const int c = s_hist[t];
+      if (c) { atomicAdd(&hist[t], c); s_hist[t] = 0; }
+    }
+    __threadfence();
+    __syncthreads();
+    const int chunks = (x.deg + kHubChunk - 1) / kHubChunk;
+    if (threadIdx.x == 0) {
+      s_last = atomicAdd(&h.hubs[hi].done, 1) == chunks - 1;
+      ue += c1 - c0;
+    }
+    __syncthreads();
+    if (!s_last) continue;
+    __threadfence();
+    int rloc = -1, rall = 0;
+    const int ownr = *(volatile int32_t *)&hist[x.own];
+    for (int t = threadIdx.x; t < h.nlabels; t += blockDim.x) {
+      const int r = *(volatile int32_t *)&hist[t];
+      if (r == 0 || t == x.own) continue;
+      rall = r > rall ? r : rall;
+      if (r > rloc && (int64_t)a.weight[t] + x.cv <= a.bound) rloc = r;
+    }
+    const int rmax = block_max_i32(rloc, s_ri);
+    rall = block_max_i32(rall, s_ri);
+    uint64_t packed = ~0ull;
+    for (int t = threadIdx.x; t < h.nlabels; t += blockDim.x) {
+      const int r = *(volatile int32_t *)&hist[t];
+      if (r != 0 && r == rmax && t != x.own && (int64_t)a.weight[t] + x.cv <= a.bound) {
+        const uint64_t p = ((uint64_t)h32(a.ktie, (uint32_t)x.v, (uint32_t)t) << 32) | (uint32_t)t;
+        packed = p < packed ? p : packed;
+      }
+    }
+    packed = block_min_u64(packed, s_ru);
+    __syncthreads();  // every thread has read the own label's count
+    for (int t = threadIdx.x; t < h.nlabels; t += blockDim.x) hist[t] = 0;
+    if (threadIdx.x == 0) {
+      uv += 1;
+      hub_emit(a, x, rmax, ownr, rall, packed);
+    }
+  }
+  add_units(a.units, ue, uv, 0, 0, a.label8 != nullptr, a.adjwgt == nullptr);
+}
+
+__global__ void __launch_bounds__(kThreads) k_hub_insert(RateArgs a, HubArgs h) {
+  __shared__ int s_k[2 * kHubChunk];
+  __shared__ int s_v[2 * kHubChunk];
+  if (a.stop && *a.stop) return;
+  constexpr int BITS = 12;
+  static_assert((1 << BITS) == 2 * kHubChunk, "table size");
+  const int cnt = list_end(a) - a.offs[a.key], items = h.chunk0[cnt];
+  for (int t = threadIdx.x; t < 2 * kHubChunk; t += blockDim.x) { s_k[t] = -1; s_v[t] = 0; }
+  unsigned long long ue = 0;
+  for (int it = blockIdx.x; it < items; it += gridDim.x) {
+    const int hi = hub_of(h.chunk0, cnt, it);
+    const Hub &x = h.hubs[hi];
+    const int st = x.st, tsize = x.tsize;
+    int2 *tab = h.tab + x.toff;
+    const int c0 = (it - h.chunk0[hi]) * kHubChunk, c1 = min(x.deg, c0 + kHubChunk);
+    constexpr int R = kHubChunk / kThreads;
+    int L[R], w[R];
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const int j = c0 + r * kThreads + (int)threadIdx.x;
+      L[r] = j < c1 ? __ldcs(a.adjncy + st + j) : -1;
+      w[r] = j < c1 && a.adjwgt ? __ldcs(a.adjwgt + st + j) : 1;
+    }
+#pragma unroll
+    for (int r = 0; r < R; r++) L[r] = L[r] >= 0 ? label_of(a, L[r]) : -1;
+    __syncthreads();  // the shared table is empty
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      if (L[r] < 0) continue;
+      unsigned s = slot_hash(L[r], BITS);
+      for (int probe = 0; probe < 2 * kHubChunk; probe++) {  // bounded: at most half full
+        const int prev = atomicCAS(&s_k[s], -1, L[r]);
+        if (prev == -1 || prev == L[r]) { atomicAdd(&s_v[s], w[r]); break; }
+        s = (s + 1) & (2 * kHubChunk - 1);
+      }
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < 2 * kHubChunk; t += blockDim.x) {
+      const int K = s_k[t];
+      if (K < 0) continue;
+      const int sum = s_v[t];
+      s_k[t] = -1;
+      s_v[t] = 0;
+      int s = (int)__umulhi((unsigned)K * 2654435761u, (unsigned)tsize);
+      for (int probe = 0; probe < tsize; probe++) {  // bounded: more slots than neighbours
+        const int prev = atomicCAS(&tab[s].x, -1, K);
+        if (prev == -1 || prev == K) { atomicAdd(&tab[s].y, sum); break; }
+        s = s + 1 == tsize ? 0 : s + 1;
+      }
+    }
+    if (threadIdx.x == 0) ue += c1 - c0;
+  }
+  add_units(a.units, ue, 0, 0, 0, a.label8 != nullptr, a.adjwgt == nullptr);
+}
+
+template <bool PICK>
+__global__ void __launch_bounds__(kThreads) k_hub_table(RateArgs a, HubArgs h) {
+  __shared__ int s_ri[kWarpsPerBlock];
+  __shared__ uint64_t s_ru[kWarpsPerBlock];
+  if (a.stop && *a.stop) return;
+  const int cnt = list_end(a) - a.offs[a.key], items = h.tchunk0[cnt];
+  unsigned long long uv = 0, uc = 0;
+  for (int it = blockIdx.x; it < items; it += gridDim.x) {
+    const int hi = hub_of(h.tchunk0, cnt, it);
+    Hub *hp = &h.hubs[hi];
+    const int own = hp->own, cv = hp->cv, v = hp->v;
+    int2 *tab = h.tab + hp->toff;
+    const int t0 = (it - h.tchunk0[hi]) * kHubTabChunk, t1 = min(hp->tsize, t0 + kHubTabChunk);
+    constexpr int R = 8;
+    if (!PICK) {
+      int best = *(volatile int *)&hp->rmax, rall = 0;  // only ratings above what some block has found matter
+      const int floor0 = best;
+      for (int b = t0 + (int)threadIdx.x; b < t1; b += kThreads * R) {
+        int2 e[R];
+#pragma unroll
+        for (int r = 0; r < R; r++) e[r] = b + r * kThreads < t1 ? tab[b + r * kThreads] : make_int2(-1, 0);
+#pragma unroll
+        for (int r = 0; r < R; r++) {
+          if (e[r].x < 0) continue;
+          if (e[r].x == own) { hp->ownr = e[r].y; continue; }  // one slot holds the own label
+          uc++;
+          rall = e[r].y > rall ? e[r].y : rall;
+          if (e[r].y > best && (int64_t)a.weight[e[r].x] + cv <= a.bound) best = e[r].y;
+        }
+      }
+      best = block_max_i32(best, s_ri);
+      rall = block_max_i32(rall, s_ri);
+      if (threadIdx.x == 0) {
+        if (best > floor0) atomicMax(&hp->rmax, best);
+        if (rall > 0) atomicMax(&hp->rall, rall);
+      }
+    } else {
+      const int rmax = hp->rmax, ownr = hp->ownr;
+      const bool want = rmax >= 0 && rmax > ownr;
+      uint64_t packed = ~0ull;
+      for (int b = t0 + (int)threadIdx.x; b < t1; b += kThreads * R) {
+        int2 e[R];
+#pragma unroll
+        for (int r = 0; r < R; r++) e[r] = b + r * kThreads < t1 ? tab[b + r * kThreads] : make_int2(-1, 0);
+#pragma unroll
+        for (int r = 0; r < R; r++)
+          if (e[r].x >= 0) tab[b + r * kThreads] = make_int2(-1, 0);
+        if (!want) continue;
+#pragma unroll
+        for (int r = 0; r < R; r++) {
+          if (e[r].x < 0 || e[r].x == own || e[r].y != rmax || (int64_t)a.weight[e[r].x] + cv > a.bound) continue;
+          const uint64_t p = ((uint64_t)h32(a.ktie, (uint32_t)v, (uint32_t)e[r].x) << 32) | (uint32_t)e[r].x;
+          packed = p < packed ? p : packed;
+        }
+      }
+      packed = block_min_u64(packed, s_ru);
+      if (threadIdx.x == 0) {
+        if (packed != ~0ull) atomicMin(&hp->best, packed);
+        __threadfence();
+        const int chunks = (hp->tsize + kHubTabChunk - 1) / kHubTabChunk;
+        if (atomicAdd(&hp->done, 1) == chunks - 1) {
+          __threadfence();
+          uv += 1;
+          hub_emit(a, *hp, rmax, ownr, hp->rall, *(volatile unsigned long long *)&hp->best);
+        }
+      }
+    }
+    __syncthreads();
+  }
+  add_units(a.units, 0, uv, uc, 0, false, false);
+}
+
 // ----------------------------------------------------- per-round buckets
 
 struct BucketArgs {
@@ -1416,35 +1725,81 @@ __global__ void k_fill_i32(int32_t *a, int64_t n, int32_t v) {
     a[i] = v;
 }
 
-// Largest degree among nodes with more than kMediumMaxDeg neighbours.
-__global__ void k_max_degree(const int32_t *xadj, int n, int *out) {
-  int m = 0;
+// Largest degree, number of hubs and table slots they need together.
+struct DegStats {
+  int maxdeg, hubs;
+  unsigned long long slots;
+};
+
+__global__ void k_max_degree(const int32_t *xadj, int n, DegStats *out) {
+  int m = 0, nh = 0;
+  unsigned long long ns = 0;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x) {
     const int d = xadj[v + 1] - xadj[v];
     m = d > m ? d : m;
+    if (d > kHubDeg) { nh++; ns += (unsigned long long)hub_slots(d); }
   }
   m = warp_max(m);
-  if (lane_id() == 0 && m) atomicMax(out, m);
+  if (lane_id() == 0 && m) atomicMax(&out->maxdeg, m);
+  if (__any_sync(FULL, nh)) {
+    nh = warp_sum(nh);
+    ns = warp_sum(ns);
+    if (lane_id() == 0) { atomicAdd(&out->hubs, nh); atomicAdd(&out->slots, ns); }
+  }
+}
+
+__global__ void k_fill_slots(int2 *tab, int64_t n) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    tab[i] = make_int2(-1, 0);
 }
 
 struct RateTables {
   DBuf<int32_t> gkeys, gvals;
   int64_t stride = 0;
   int blocks = 0;
+  // hubs (HubArgs), when the graph has some and their tables stay within the bound of table_blocks
+  bool hubs = false;
+  DBuf<Hub> hub;
+  DBuf<int> chunk0, tchunk0;
+  DBuf<int2> tab;
+  DBuf<int32_t> hist;
 };
 
-// Global hash tables for the block-per-node kernel when some node needs more
-// than kLargeSmemSlots slots.
-void make_tables(gp_ctx *ctx, const DevGraph &g, RateTables &t) {
-  DBuf<int> md(ctx, 1);
-  md.zero();
-  k_max_degree<<<grid_for(g.n, 256, ctx->num_sms * 8), 256, 0, ctx->stream>>>(g.xadj, g.n, md.get());
+// What the kernels for nodes beyond the shared tables need: the hubs' plan and tables (nlabels > 0: label
+// propagation), or per-block hash tables in global memory (favourites, and graphs whose hubs' tables
+// together would take more memory than that).
+void make_tables(gp_ctx *ctx, const DevGraph &g, int64_t nlabels, RateTables &t) {
+  DBuf<DegStats> ds(ctx, 1);
+  ds.zero();
+  k_max_degree<<<grid_for(g.n, 256, ctx->num_sms * 8), 256, 0, ctx->stream>>>(g.xadj, g.n, ds.get());
   GP_LAUNCH_CHECK();
-  const int maxdeg = read_scalar(ctx, md.get());
+  DegStats h;
+  read_back(ctx, ds.get(), sizeof(h), &h);
+  const int maxdeg = h.maxdeg;
   int bits = 1;
   while ((1 << bits) < 2 * maxdeg) bits++;
   t.blocks = ctx->num_sms * 4;
+  if (nlabels > 0 && h.hubs > 0) {
+    const int64_t cap = (8 * g.m2 + ((int64_t)16 << 20)) / (int64_t)sizeof(int2);
+    const bool dense = nlabels <= kHubDense;
+    if (dense ? (int64_t)h.hubs * nlabels <= 2 * cap : (int64_t)h.slots <= cap) {
+      t.hubs = true;
+      t.hub.reset(ctx, (size_t)h.hubs);
+      t.chunk0.reset(ctx, (size_t)h.hubs + 1);
+      t.tchunk0.reset(ctx, (size_t)h.hubs + 1);
+      if (dense) {
+        t.hist.reset(ctx, (size_t)(h.hubs * nlabels));
+        t.hist.zero();
+      } else {
+        t.tab.reset(ctx, (size_t)h.slots);
+        k_fill_slots<<<grid_for((int64_t)h.slots, 256, ctx->num_sms * 8), 256, 0, ctx->stream>>>(t.tab.get(),
+                                                                                                (int64_t)h.slots);
+        GP_LAUNCH_CHECK();
+      }
+      return;
+    }
+  }
   if ((1 << bits) > kLargeSmemSlots) {
     t.stride = (int64_t)1 << bits;
     t.blocks = table_blocks(g.m2, t.stride, t.blocks);
@@ -1465,7 +1820,7 @@ inline int rate_grid(gp_ctx *ctx, int64_t count, int per_block, int cap) {
 template <int G, int U>
 constexpr int group_nodes_per_block() { return kWarpsPerBlock * (32 / G) * U; }
 
-// hcnt: the five bucket sizes of this sub-round when the host knows them (empty
+// hcnt: the bucket sizes of this sub-round when the host knows them (empty
 // buckets are then not launched), else nullptr
 template <int MODE, int LK>
 void launch_groups(gp_ctx *ctx, const RateArgs &a0, int bucket_key_base, const int *hcnt) {
@@ -1513,6 +1868,31 @@ void launch_rate(gp_ctx *ctx, RateArgs a, int bucket_key_base, const RateTables 
     k_rate_large<MODE><<<rate_grid(ctx, hcnt ? hcnt[4] : -1, 1, t.blocks), kThreads, 0, ctx->stream>>>(a);
     GP_LAUNCH_CHECK();
   }
+  if (hcnt && hcnt[5] == 0) return;
+  a.key = bucket_key_base + 5;
+  if (MODE == RATE_LP && t.hubs) {
+    HubArgs h{t.hub.get(), t.chunk0.get(), t.tchunk0.get(), t.tab.get(), t.hist.get(), (int)nlabels};
+    k_hub_plan<<<1, 1024, 0, ctx->stream>>>(a, h);
+    GP_LAUNCH_CHECK();
+    const int hgrid = ctx->num_sms * 6;
+    if (nlabels <= kHubDense) {
+      k_hub_dense<<<hgrid, kThreads, sizeof(int) * (size_t)nlabels, ctx->stream>>>(a, h);
+      GP_LAUNCH_CHECK();
+    } else {
+      k_hub_insert<<<hgrid, kThreads, 0, ctx->stream>>>(a, h);
+      GP_LAUNCH_CHECK();
+      k_hub_table<false><<<hgrid, kThreads, 0, ctx->stream>>>(a, h);
+      GP_LAUNCH_CHECK();
+      k_hub_table<true><<<hgrid, kThreads, 0, ctx->stream>>>(a, h);
+      GP_LAUNCH_CHECK();
+    }
+  } else {
+    a.gkeys = t.gkeys.get();
+    a.gvals = t.gvals.get();
+    a.gstride = t.stride;
+    k_rate_large<MODE><<<rate_grid(ctx, hcnt ? hcnt[5] : -1, 1, t.blocks), kThreads, 0, ctx->stream>>>(a);
+    GP_LAUNCH_CHECK();
+  }
 }
 
 }  // namespace
@@ -1525,8 +1905,10 @@ int bits_for(int64_t x) {
 
 LpResult lp_run(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *weight, int64_t nlabels, uint64_t seed, const LpParams &p, int64_t *nclusters_dev,
                 uint8_t *label8) {
-  if (lp_small_applicable(g, p)) return lp_run_small(ctx, g, label, weight, nlabels, seed, p, nclusters_dev, label8);
   LpResult res;
+  if (lp_small_applicable(g, p) &&
+      lp_run_small(ctx, g, label, weight, nlabels, seed, p, nclusters_dev, label8, res))
+    return res;
   const int n = g.n;
   const int S = p.subrounds;
   GP_REQUIRE(S >= 1 && S <= 64, GP_ERR_INVALID, "lp_subrounds must be in [1, 64]");
@@ -1583,7 +1965,7 @@ LpResult lp_run(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *weight,
   k_counters_init<<<1, 1, 0, ctx->stream>>>(C, ncl0);
   GP_LAUNCH_CHECK();
   RateTables tables;
-  make_tables(ctx, g, tables);
+  make_tables(ctx, g, nlabels, tables);
   unsigned long long *units_rate = ctx->d_units ? ctx->d_units + p.prof_rate * PROF_UNITS : nullptr;
 
   TraceTimer trace(ctx);
@@ -1813,7 +2195,7 @@ void favourites_bucketed(gp_ctx *ctx, const DevGraph &g, const int32_t *label, c
   k_fill_u64<<<grid_for(total, 256, grid), 256, 0, ctx->stream>>>(keys.get(), total, ~0ull);
   GP_LAUNCH_CHECK();
   RateTables tables;
-  make_tables(ctx, g, tables);
+  make_tables(ctx, g, 0, tables);
   RateArgs a{};
   a.xadj = g.xadj; a.adjncy = g.adjncy; a.adjwgt = g.unit_w ? nullptr : g.adjwgt; a.vwgt = g.vwgt;
   a.label = label; a.weight = nullptr; a.list = list.get(); a.offs = offs.get();

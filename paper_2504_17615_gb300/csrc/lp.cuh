@@ -7,13 +7,14 @@ namespace gp {
 
 // Degree classes of the rating kernels: <= 8, <= 16, <= 32 (8/16/32 lanes per
 // node, one neighbour per lane), <= 128 (a warp with a 256-slot shared table),
-// larger (a block with a shared table, or a global one beyond 2048).
-constexpr int kNumBuckets = 5;
+// <= 2048 (a block with a shared table), larger (hubs: many blocks a node).
+constexpr int kNumBuckets = 6;
 constexpr int kMediumMaxDeg = 128;
+constexpr int kHubDeg = 2048;
 constexpr int kLargeSmemSlots = 4096;
 
 __host__ __device__ __forceinline__ int degree_bucket(int deg) {
-  return deg <= 8 ? 0 : deg <= 16 ? 1 : deg <= 32 ? 2 : deg <= kMediumMaxDeg ? 3 : 4;
+  return deg <= 8 ? 0 : deg <= 16 ? 1 : deg <= 32 ? 2 : deg <= kMediumMaxDeg ? 3 : deg <= kHubDeg ? 4 : 5;
 }
 
 enum RateMode { RATE_LP = 0, RATE_FAV = 1 };
@@ -22,6 +23,11 @@ enum RateMode { RATE_LP = 0, RATE_FAV = 1 };
 // (gp_config.small_lp_nodes, default) and at most this many CSR entries.
 constexpr int32_t kLpSmallMaxNodes = 5 << 20;
 constexpr int64_t kLpSmallMaxEntries = (int64_t)1 << 26;
+// ... unless a node has more than kLpSmallMaxDeg neighbours and the graph more than kLpSmallHubEntries
+// entries: the persistent kernel rates a node with one block, the per-phase driver a hub with many, which
+// pays once the hub's rating outlasts the driver's launches (HUBNUM).
+constexpr int32_t kLpSmallMaxDeg = 8192;
+constexpr int64_t kLpSmallHubEntries = (int64_t)1 << 22;
 // iterations of a device-side wait before it gives up (about seconds)
 constexpr long long kDefaultWaitSpins = 1ll << 25;
 
@@ -66,9 +72,10 @@ void favourites_bucketed(gp_ctx *ctx, const DevGraph &g, const int32_t *label, c
 int bits_for(int64_t x);
 
 // The same LP run as lp_run as one cooperative persistent launch (lp_small.cu);
-// for graphs of at most p.small_nodes nodes and kLpSmallMaxEntries entries.
+// for graphs of at most p.small_nodes nodes and kLpSmallMaxEntries entries.  Returns false, with nothing
+// changed, when the graph's hubs make the per-phase driver the faster one.
 bool lp_small_applicable(const DevGraph &g, const LpParams &p);
-LpResult lp_run_small(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *weight, int64_t nlabels,
-                      uint64_t seed, const LpParams &p, int64_t *nclusters_dev, uint8_t *label8);
+bool lp_run_small(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *weight, int64_t nlabels,
+                  uint64_t seed, const LpParams &p, int64_t *nclusters_dev, uint8_t *label8, LpResult &res);
 
 }  // namespace gp

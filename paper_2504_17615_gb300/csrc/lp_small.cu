@@ -965,9 +965,9 @@ bool lp_small_applicable(const DevGraph &g, const LpParams &p) {
   return g.n > 0 && g.n <= p.small_nodes && g.m2 <= kLpSmallMaxEntries;
 }
 
-LpResult lp_run_small(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *weight, int64_t nlabels,
-                      uint64_t seed, const LpParams &p, int64_t *nclusters_dev, uint8_t *label8) {
-  LpResult res;
+bool lp_run_small(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *weight, int64_t nlabels,
+                  uint64_t seed, const LpParams &p, int64_t *nclusters_dev, uint8_t *label8, LpResult &res) {
+  res = LpResult{};
   const int n = g.n;
   GP_REQUIRE(p.subrounds >= 1 && p.subrounds <= 64, GP_ERR_INVALID, "lp_subrounds must be in [1, 64]");
   static bool attr_set[64] = {};
@@ -1023,6 +1023,7 @@ LpResult lp_run_small(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *w
   k_pmax_degree<<<grid_for(n, 256, ctx->num_sms * 8), 256, 0, ctx->stream>>>(g.xadj, n, md.get());
   GP_LAUNCH_CHECK();
   const int maxdeg = read_scalar(ctx, md.get());
+  if (maxdeg > kLpSmallMaxDeg && g.m2 > kLpSmallHubEntries) return false;
   int bits = 1;
   while ((1 << bits) < 2 * maxdeg) bits++;
   DBuf<int32_t> gtk, gtv;
@@ -1094,7 +1095,7 @@ LpResult lp_run_small(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *w
   if (p.count_clusters && nclusters_dev)
     GP_CUDA(cudaMemcpyAsync(nclusters_dev, &dc->out.nclusters, sizeof(int64_t), cudaMemcpyDeviceToDevice,
                             ctx->stream));
-  return res;
+  return true;
 }
 
 }  // namespace gp
