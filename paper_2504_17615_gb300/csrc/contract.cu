@@ -31,6 +31,7 @@ constexpr int kMapUnroll = 8;
 constexpr int kHugeSeg = 2048;       // segments above this many entries are merged by many blocks
 constexpr int kSegChunk = 2048;      // their entries per block and step
 constexpr int kSegTabChunk = 4096;   // and table slots
+constexpr unsigned long long kEmptySlot = 0xFFFFFFFFull;  // the slot (-1, 0): neighbour in the low half
 
 __device__ __forceinline__ unsigned slot_hash(int B, int bits) {
   return ((unsigned)B * 2654435761u) >> (32 - bits);
@@ -240,7 +241,7 @@ __global__ void k_seg_stats(const int32_t *x, int n, SegStats *out) {
 // global memory took milliseconds for it while the rest of the device waited (12 levels of the scale-24
 // R-MAT graph: 131 ms of contraction).  k_seg_plan lists the huge segments with the prefix sums of their
 // chunks, k_seg_insert sums 2048 entries at a time in a shared table and adds the sums to the segment's
-// table in global memory (4/3 slots an entry), and k_seg_extract writes the occupied slots back to the
+// table in global memory (4/3 slots an entry; one 64-bit exchange claims a slot), and k_seg_extract writes the occupied slots back to the
 // segment.  Consecutive steps work on the same few tables, which stay in L2 meanwhile.
 
 struct Seg {
@@ -352,8 +353,10 @@ __global__ void __launch_bounds__(kThreads) k_seg_insert(MergeArgs a, SegArgs h)
       s_v[t] = 0;
       int s = (int)__umulhi((unsigned)B * 2654435761u, (unsigned)x.tsize);
       for (int probe = 0; probe < x.tsize; probe++) {  // bounded: more slots than entries
-        const int prev = atomicCAS(&tab[s].x, -1, B);
-        if (prev == -1 || prev == B) { atomicAdd(&tab[s].y, w); break; }
+        const unsigned long long prev = atomicCAS((unsigned long long *)&tab[s], kEmptySlot,
+                                                  ((unsigned long long)(unsigned)w << 32) | (unsigned)B);
+        if (prev == kEmptySlot) break;
+        if ((int)(unsigned)prev == B) { atomicAdd(&tab[s].y, w); break; }
         s = s + 1 == x.tsize ? 0 : s + 1;
       }
     }

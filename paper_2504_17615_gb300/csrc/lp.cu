@@ -729,23 +729,143 @@ __global__ void __launch_bounds__(kThreads) k_rate_large(RateArgs a) {
   add_units(a.units, ue, uv, uc, up, a.label8 != nullptr, a.adjwgt == nullptr);
 }
 
+// ------------------- 128 < degree <= 18432: block/node, shared table
+//
+// The table has 4/3 slots per neighbour (a slot is the high half of hash x size, so any size will do) and
+// kBlockUnroll neighbours per thread are in flight.  Nodes of 2049 .. 18432 neighbours held 172M of the
+// 521M entries of the scale-24 R-MAT graph; their tables in shared memory take no global atomics, which
+// limited them to 7e9 entries/s (BLKNUM).
+
+constexpr int kBlockUnroll = 4;
+
+__host__ __device__ __forceinline__ int hub_slots(int deg) { return deg + deg / 3 + 1; }
+
+template <int NT>
+__device__ __forceinline__ int block_max_n(int v, int *s_red) {
+  v = __reduce_max_sync(FULL, v);
+  __syncthreads();
+  if (lane_id() == 0) s_red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  int r = s_red[0];
+#pragma unroll
+  for (int i = 1; i < NT / 32; i++) r = s_red[i] > r ? s_red[i] : r;
+  return r;
+}
+
+template <int NT>
+__device__ __forceinline__ uint64_t block_min_n(uint64_t v, uint64_t *s_red) {
+  v = warp_min(v);
+  __syncthreads();
+  if (lane_id() == 0) s_red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  uint64_t r = s_red[0];
+#pragma unroll
+  for (int i = 1; i < NT / 32; i++) r = s_red[i] < r ? s_red[i] : r;
+  return r;
+}
+
+template <int NT>
+__global__ void __launch_bounds__(NT) k_rate_block(RateArgs a, int slots) {
+  extern __shared__ int s_tab[];  // slots labels, slots ratings
+  __shared__ int s_ri[NT / 32], s_own;
+  __shared__ uint64_t s_ru[NT / 32];
+  if (a.stop && *a.stop) return;
+  int *tk = s_tab, *tv = s_tab + slots;
+  for (int t = threadIdx.x; t < slots; t += NT) { tk[t] = -1; tv[t] = 0; }
+  const int begin = a.offs[a.key], end = list_end(a);
+  unsigned long long ue = 0, uv = 0, uc = 0, up = 0;
+  for (int i = begin + (int)blockIdx.x; i < end; i += (int)gridDim.x) {
+    const int4 rec = a.list[i];
+    const int v = rec.x, start = rec.y, deg = rec.z, cv = rec.w;
+    if (a.dirty && !a.dirty[v]) {  // clean: cannot move (uniform in the block)
+      if (threadIdx.x == 0) a.prop[i] = make_int2(-1, 0);
+      continue;
+    }
+    const int own = label_of(a, v);
+    const int tsize = hub_slots(deg);
+    if (threadIdx.x == 0) s_own = 0;
+    __syncthreads();  // the table is empty, and the flag of the clean nodes was read before it may change
+    for (int j0 = threadIdx.x; j0 < deg; j0 += NT * kBlockUnroll) {
+      int L[kBlockUnroll], w[kBlockUnroll];
+#pragma unroll
+      for (int r = 0; r < kBlockUnroll; r++) {
+        const int j = j0 + r * NT;
+        L[r] = j < deg ? __ldcs(a.adjncy + start + j) : -1;
+        w[r] = j < deg && a.adjwgt ? __ldcs(a.adjwgt + start + j) : 1;
+      }
+#pragma unroll
+      for (int r = 0; r < kBlockUnroll; r++) L[r] = L[r] >= 0 ? label_of(a, L[r]) : -1;
+#pragma unroll
+      for (int r = 0; r < kBlockUnroll; r++) {
+        if (L[r] < 0) continue;
+        int s = (int)__umulhi((unsigned)L[r] * 2654435761u, (unsigned)tsize);
+        for (int probe = 0; probe < tsize; probe++) {  // bounded: more slots than neighbours
+          const int prev = atomicCAS(&tk[s], -1, L[r]);
+          if (prev == -1 || prev == L[r]) { atomicAdd(&tv[s], w[r]); break; }
+          s = s + 1 == tsize ? 0 : s + 1;
+        }
+      }
+    }
+    __syncthreads();
+    int rloc = -1, rall = 0, nc = 0;
+    for (int t = threadIdx.x; t < tsize; t += NT) {
+      const int L = tk[t];
+      if (L < 0) continue;
+      const int r = tv[t];
+      if (L == own) { s_own = r; continue; }
+      nc++;
+      rall = r > rall ? r : rall;
+      if (r > rloc && (int64_t)a.weight[L] + cv <= a.bound) rloc = r;  // only what beats the thread's best matters
+    }
+    const int rmax = block_max_n<NT>(rloc, s_ri);  // its barriers also publish s_own
+    const int own_r = s_own;
+    if (a.dirty) {
+      rall = block_max_n<NT>(rall, s_ri);
+      if (rall <= own_r && threadIdx.x == 0) a.dirty[v] = 0;
+    }
+    uc += nc;
+    const bool want = rmax >= 0 && rmax > own_r;
+    uint64_t packed = ~0ull;
+    for (int t = threadIdx.x; t < tsize; t += NT) {
+      const int L = tk[t];
+      if (L < 0) continue;
+      if (want && L != own && tv[t] == rmax && (int64_t)a.weight[L] + cv <= a.bound) {
+        const uint64_t p = ((uint64_t)h32(a.ktie, (uint32_t)v, (uint32_t)L) << 32) | (uint32_t)L;
+        packed = p < packed ? p : packed;
+      }
+      tk[t] = -1;
+      tv[t] = 0;
+    }
+    if (want) packed = block_min_n<NT>(packed, s_ru);
+    if (threadIdx.x == 0) {
+      ue += deg;
+      uv += 1;
+      if (want) { emit<RATE_LP>(a, i, v, (int)(uint32_t)packed, cv, own); up += 1; }
+      else a.prop[i] = make_int2(-1, 0);
+    }
+    __syncthreads();
+  }
+  add_units(a.units, ue, uv, uc, up, a.label8 != nullptr, a.adjwgt == nullptr);
+}
+
 // ------------------------------------------------- hubs: many blocks a node
 //
-// A node of more than kHubDeg neighbours is rated by as many blocks as its row has chunks.  With one block
-// a node, a sub-round waited for the block of the largest hub: 8 ms in every sub-round of the scale-24
-// R-MAT graph (4e5 neighbours, a 2^20-slot table in global memory walked by 256 threads), 330 ms for
-// level 1.  k_hub_plan lists the sub-round's hubs with the prefix sums of their chunks; then
+// A node of more neighbours than that (with few labels: of more than 2048) is rated by as many blocks as
+// its row has chunks.  With one block a node and a table in global memory, a sub-round waited for the
+// block of the largest hub: 8 ms in every sub-round of the scale-24 R-MAT graph (4e5 neighbours), 330 ms
+// for level 1.  k_hub_plan lists the sub-round's hubs with the prefix sums of their chunks; then
 //  few labels (at most kHubDense: refinement): k_hub_dense counts a chunk per label in shared memory, adds
 //    it to the hub's counters, and the block that finishes a hub's last chunk chooses;
 //  many labels: k_hub_insert sums a chunk's labels in a shared table and adds the sums to the hub's table
-//    in global memory (4/3 slots per neighbour), k_hub_max walks the tables (4096 slots a block) for the
-//    largest admissible rating, and k_hub_pick walks them again for the smallest (hash, label) of that
-//    rating and leaves them empty.
+//    in global memory (one 64-bit exchange claims a slot with its sum), k_hub_table walks the tables (4096
+//    slots a block) for the largest admissible rating, and then for the smallest (hash, label) of that
+//    rating, and leaves them empty.
 // The choice is the same as in the other kernels.
 
 constexpr int kHubChunk = 2048;    // row entries per block and step
 constexpr int kHubTabChunk = 4096; // table slots per block and step
 constexpr int kHubDense = 1024;    // labels up to which a hub's ratings are counted per label
+constexpr unsigned long long kEmptySlot = 0xFFFFFFFFull;  // the slot (-1, 0): label in the low half, rating in the high
 
 struct Hub {
   int pos, v, st, deg, cv, own;  // list position, node, row offset, degree, weight, label
@@ -762,8 +882,6 @@ struct HubArgs {
   int32_t *hist;          // dense: [hub][nlabels], zero between sub-rounds
   int nlabels;
 };
-
-__device__ __forceinline__ int hub_slots(int deg) { return deg + deg / 3 + 1; }
 
 __global__ void __launch_bounds__(1024) k_hub_plan(RateArgs a, HubArgs h) {
   __shared__ long long s_w[3][32];
@@ -956,8 +1074,10 @@ __global__ void __launch_bounds__(kThreads) k_hub_insert(RateArgs a, HubArgs h) 
       s_v[t] = 0;
       int s = (int)__umulhi((unsigned)K * 2654435761u, (unsigned)tsize);
       for (int probe = 0; probe < tsize; probe++) {  // bounded: more slots than neighbours
-        const int prev = atomicCAS(&tab[s].x, -1, K);
-        if (prev == -1 || prev == K) { atomicAdd(&tab[s].y, sum); break; }
+        const unsigned long long prev = atomicCAS((unsigned long long *)&tab[s], kEmptySlot,
+                                                  ((unsigned long long)(unsigned)sum << 32) | (unsigned)K);
+        if (prev == kEmptySlot) break;
+        if ((int)(unsigned)prev == K) { atomicAdd(&tab[s].y, sum); break; }
         s = s + 1 == tsize ? 0 : s + 1;
       }
     }
@@ -1078,16 +1198,27 @@ __global__ void __launch_bounds__(kThreads) k_bucket_count(BucketArgs b, int nke
     if (s_c[t]) atomicAdd(&cnt[t], s_c[t]);
 }
 
-__global__ void k_bucket_offsets(const int *cnt, int nkeys, int *offs, int *cursor, const int *stop) {
+// One block of kMaxKeys threads: a scan over the keys (one thread's loop over them took a dependent read
+// from memory each).
+__global__ void __launch_bounds__(kMaxKeys) k_bucket_offsets(const int *cnt, int nkeys, int *offs, int *cursor,
+                                                             const int *stop) {
+  __shared__ int s_w[kMaxKeys / 32];
   if (stop && *stop) return;
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    int run = 0;
-    for (int k = 0; k < nkeys; k++) {
-      offs[k] = run;
-      cursor[k] = run;
-      run += cnt[k];
-    }
-    offs[nkeys] = run;
+  const int t = threadIdx.x, lane = (int)lane_id();
+  const int x = t < nkeys ? cnt[t] : 0;
+  int y = x;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int z = __shfl_up_sync(FULL, y, o);
+    if (lane >= o) y += z;
+  }
+  if (lane == 31) s_w[t >> 5] = y;
+  __syncthreads();
+  for (int w = 0; w < (t >> 5); w++) y += s_w[w];
+  if (t < nkeys) {
+    offs[t] = y - x;
+    cursor[t] = y - x;
+    if (t == nkeys - 1) offs[nkeys] = y;
   }
 }
 
@@ -1725,9 +1856,9 @@ __global__ void k_fill_i32(int32_t *a, int64_t n, int32_t v) {
     a[i] = v;
 }
 
-// Largest degree, number of hubs and table slots they need together.
+// Largest degree, number of nodes above kBlockDeg0, and the table slots the hubs need together.
 struct DegStats {
-  int maxdeg, hubs;
+  int maxdeg, big;
   unsigned long long slots;
 };
 
@@ -1738,14 +1869,15 @@ __global__ void k_max_degree(const int32_t *xadj, int n, DegStats *out) {
        v += (int64_t)gridDim.x * blockDim.x) {
     const int d = xadj[v + 1] - xadj[v];
     m = d > m ? d : m;
-    if (d > kHubDeg) { nh++; ns += (unsigned long long)hub_slots(d); }
+    if (d > kBlockDeg0) nh++;
+    if (d > kHubDeg) ns += (unsigned long long)hub_slots(d);
   }
   m = warp_max(m);
   if (lane_id() == 0 && m) atomicMax(&out->maxdeg, m);
   if (__any_sync(FULL, nh)) {
     nh = warp_sum(nh);
     ns = warp_sum(ns);
-    if (lane_id() == 0) { atomicAdd(&out->hubs, nh); atomicAdd(&out->slots, ns); }
+    if (lane_id() == 0) { atomicAdd(&out->big, nh); atomicAdd(&out->slots, ns); }
   }
 }
 
@@ -1760,6 +1892,7 @@ struct RateTables {
   int blocks = 0;
   // hubs (HubArgs), when the graph has some and their tables stay within the bound of table_blocks
   bool hubs = false;
+  bool dense = false;  // few labels: nodes above kBlockDeg0 are counted per label
   DBuf<Hub> hub;
   DBuf<int> chunk0, tchunk0;
   DBuf<int2> tab;
@@ -1780,16 +1913,17 @@ void make_tables(gp_ctx *ctx, const DevGraph &g, int64_t nlabels, RateTables &t)
   int bits = 1;
   while ((1 << bits) < 2 * maxdeg) bits++;
   t.blocks = ctx->num_sms * 4;
-  if (nlabels > 0 && h.hubs > 0) {
+  if (nlabels > 0) {
     const int64_t cap = (8 * g.m2 + ((int64_t)16 << 20)) / (int64_t)sizeof(int2);
-    const bool dense = nlabels <= kHubDense;
-    if (dense ? (int64_t)h.hubs * nlabels <= 2 * cap : (int64_t)h.slots <= cap) {
-      t.hubs = true;
-      t.hub.reset(ctx, (size_t)h.hubs);
-      t.chunk0.reset(ctx, (size_t)h.hubs + 1);
-      t.tchunk0.reset(ctx, (size_t)h.hubs + 1);
-      if (dense) {
-        t.hist.reset(ctx, (size_t)(h.hubs * nlabels));
+    t.dense = nlabels <= kHubDense && (int64_t)h.big * nlabels <= 2 * cap;
+    const int64_t hubs = t.dense ? h.big : (int64_t)h.slots / kHubDeg;  // an upper bound
+    t.hubs = hubs > 0 && (t.dense || (int64_t)h.slots <= cap);
+    if (t.hubs) {
+      t.hub.reset(ctx, (size_t)hubs);
+      t.chunk0.reset(ctx, (size_t)hubs + 1);
+      t.tchunk0.reset(ctx, (size_t)hubs + 1);
+      if (t.dense) {
+        t.hist.reset(ctx, (size_t)(hubs * nlabels));
         t.hist.zero();
       } else {
         t.tab.reset(ctx, (size_t)h.slots);
@@ -1797,8 +1931,8 @@ void make_tables(gp_ctx *ctx, const DevGraph &g, int64_t nlabels, RateTables &t)
                                                                                                 (int64_t)h.slots);
         GP_LAUNCH_CHECK();
       }
-      return;
     }
+    if (t.hubs || maxdeg <= kHubDeg) return;
   }
   if ((1 << bits) > kLargeSmemSlots) {
     t.stride = (int64_t)1 << bits;
@@ -1846,6 +1980,16 @@ void launch_groups(gp_ctx *ctx, const RateArgs &a0, int bucket_key_base, const i
   }
 }
 
+template <int NT>
+void launch_block(gp_ctx *ctx, const RateArgs &a, int maxdeg, int grid) {
+  const int slots = hub_slots(maxdeg);
+  const size_t smem = 2 * sizeof(int) * (size_t)slots;
+  if (smem > 48 * 1024)
+    GP_CUDA(cudaFuncSetAttribute(k_rate_block<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k_rate_block<NT><<<grid, NT, smem, ctx->stream>>>(a, slots);
+  GP_LAUNCH_CHECK();
+}
+
 // nlabels: number of labels (chooses the narrow / dense group kernels when
 // a uint8 copy of the labels is present)
 template <int MODE>
@@ -1860,38 +2004,37 @@ void launch_rate(gp_ctx *ctx, RateArgs a, int bucket_key_base, const RateTables 
     k_rate_medium<MODE><<<rate_grid(ctx, hcnt ? hcnt[3] : -1, kWarpsPerBlock, cap), kThreads, 0, ctx->stream>>>(a);
     GP_LAUNCH_CHECK();
   }
-  if (!hcnt || hcnt[4] > 0) {
-    a.key = bucket_key_base + 4;
-    a.gkeys = t.gkeys.get();
-    a.gvals = t.gvals.get();
-    a.gstride = t.stride;
-    k_rate_large<MODE><<<rate_grid(ctx, hcnt ? hcnt[4] : -1, 1, t.blocks), kThreads, 0, ctx->stream>>>(a);
-    GP_LAUNCH_CHECK();
-  }
-  if (hcnt && hcnt[5] == 0) return;
-  a.key = bucket_key_base + 5;
-  if (MODE == RATE_LP && t.hubs) {
-    HubArgs h{t.hub.get(), t.chunk0.get(), t.tchunk0.get(), t.tab.get(), t.hist.get(), (int)nlabels};
-    k_hub_plan<<<1, 1024, 0, ctx->stream>>>(a, h);
-    GP_LAUNCH_CHECK();
-    const int hgrid = ctx->num_sms * 6;
-    if (nlabels <= kHubDense) {
-      k_hub_dense<<<hgrid, kThreads, sizeof(int) * (size_t)nlabels, ctx->stream>>>(a, h);
+  const int hgrid = ctx->num_sms * 6;
+  for (int b = 4; b < kNumBuckets; b++) {
+    const int c = hcnt ? hcnt[b] : -1;
+    if (c == 0) continue;
+    a.key = bucket_key_base + b;
+    if (MODE == RATE_LP && t.hubs && (b == 7 || (b > 4 && t.dense))) {
+      HubArgs h{t.hub.get(), t.chunk0.get(), t.tchunk0.get(), t.tab.get(), t.hist.get(), (int)nlabels};
+      k_hub_plan<<<1, 1024, 0, ctx->stream>>>(a, h);
       GP_LAUNCH_CHECK();
+      if (t.dense) {
+        k_hub_dense<<<hgrid, kThreads, sizeof(int) * (size_t)nlabels, ctx->stream>>>(a, h);
+        GP_LAUNCH_CHECK();
+      } else {
+        k_hub_insert<<<hgrid, kThreads, 0, ctx->stream>>>(a, h);
+        GP_LAUNCH_CHECK();
+        k_hub_table<false><<<hgrid, kThreads, 0, ctx->stream>>>(a, h);
+        GP_LAUNCH_CHECK();
+        k_hub_table<true><<<hgrid, kThreads, 0, ctx->stream>>>(a, h);
+        GP_LAUNCH_CHECK();
+      }
+    } else if (MODE == RATE_LP && b < 7) {
+      if (b == 4) launch_block<256>(ctx, a, kBlockDeg0, rate_grid(ctx, c, 1, ctx->num_sms * 6));
+      else if (b == 5) launch_block<512>(ctx, a, kBlockDeg1, rate_grid(ctx, c, 1, ctx->num_sms * 3));
+      else launch_block<1024>(ctx, a, kHubDeg, rate_grid(ctx, c, 1, ctx->num_sms));
     } else {
-      k_hub_insert<<<hgrid, kThreads, 0, ctx->stream>>>(a, h);
-      GP_LAUNCH_CHECK();
-      k_hub_table<false><<<hgrid, kThreads, 0, ctx->stream>>>(a, h);
-      GP_LAUNCH_CHECK();
-      k_hub_table<true><<<hgrid, kThreads, 0, ctx->stream>>>(a, h);
+      a.gkeys = t.gkeys.get();
+      a.gvals = t.gvals.get();
+      a.gstride = t.stride;
+      k_rate_large<MODE><<<rate_grid(ctx, c, 1, t.blocks), kThreads, 0, ctx->stream>>>(a);
       GP_LAUNCH_CHECK();
     }
-  } else {
-    a.gkeys = t.gkeys.get();
-    a.gvals = t.gvals.get();
-    a.gstride = t.stride;
-    k_rate_large<MODE><<<rate_grid(ctx, hcnt ? hcnt[5] : -1, 1, t.blocks), kThreads, 0, ctx->stream>>>(a);
-    GP_LAUNCH_CHECK();
   }
 }
 
@@ -1986,7 +2129,7 @@ LpResult lp_run(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *weight,
       cnt.zero();
       k_bucket_count<<<grid_for(n, kThreads, grid), kThreads, 0, ctx->stream>>>(b, nkeys, cnt.get());
       GP_LAUNCH_CHECK();
-      k_bucket_offsets<<<1, 1, 0, ctx->stream>>>(cnt.get(), nkeys, offs.get(), cursor.get(), &C->stop);
+      k_bucket_offsets<<<1, kMaxKeys, 0, ctx->stream>>>(cnt.get(), nkeys, offs.get(), cursor.get(), &C->stop);
       GP_LAUNCH_CHECK();
       k_bucket_scatter<<<grid_for(n, kChunk, grid), kThreads, 0, ctx->stream>>>(b, nkeys, cursor.get(),
                                                                                list.get());
@@ -2182,7 +2325,7 @@ void favourites_bucketed(gp_ctx *ctx, const DevGraph &g, const int32_t *label, c
   cnt.zero();
   k_bucket_count<<<grid_for(n, kThreads, grid), kThreads, 0, ctx->stream>>>(b, nkeys, cnt.get());
   GP_LAUNCH_CHECK();
-  k_bucket_offsets<<<1, 1, 0, ctx->stream>>>(cnt.get(), nkeys, offs.get(), cursor.get(), nullptr);
+  k_bucket_offsets<<<1, kMaxKeys, 0, ctx->stream>>>(cnt.get(), nkeys, offs.get(), cursor.get(), nullptr);
   GP_LAUNCH_CHECK();
   k_bucket_scatter<<<grid_for(n, kChunk, grid), kThreads, 0, ctx->stream>>>(b, nkeys, cursor.get(),
                                                                            list.get());

@@ -7,14 +7,16 @@ namespace gp {
 
 // Degree classes of the rating kernels: <= 8, <= 16, <= 32 (8/16/32 lanes per
 // node, one neighbour per lane), <= 128 (a warp with a 256-slot shared table),
-// <= 2048 (a block with a shared table), larger (hubs: many blocks a node).
-constexpr int kNumBuckets = 6;
+// <= 2048, <= 6144, <= 18432 (a block with a shared table of 4/3 slots per
+// neighbour at most: six, three and one block an SM), larger (hubs: many
+// blocks a node).
+constexpr int kNumBuckets = 8;
 constexpr int kMediumMaxDeg = 128;
-constexpr int kHubDeg = 2048;
+constexpr int kBlockDeg0 = 2048, kBlockDeg1 = 6144, kHubDeg = 18432;
 constexpr int kLargeSmemSlots = 4096;
 
 __host__ __device__ __forceinline__ int degree_bucket(int deg) {
-  return deg <= 8 ? 0 : deg <= 16 ? 1 : deg <= 32 ? 2 : deg <= kMediumMaxDeg ? 3 : deg <= kHubDeg ? 4 : 5;
+  return deg <= 8 ? 0 : deg <= 16 ? 1 : deg <= 32 ? 2 : deg <= kMediumMaxDeg ? 3 : deg <= kBlockDeg0 ? 4 : deg <= kBlockDeg1 ? 5 : deg <= kHubDeg ? 6 : 7;
 }
 
 enum RateMode { RATE_LP = 0, RATE_FAV = 1 };

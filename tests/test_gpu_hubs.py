@@ -1,6 +1,6 @@
-"""GPU vs CPU oracle, exact: nodes of more than 2048 neighbours in label propagation (rated by many
-blocks: counted per label up to 1024 labels, hash tables beyond; one block each when their tables
-together would take too much memory) and coarse nodes with long segments in contraction."""
+"""GPU vs CPU oracle, exact: nodes of more than 128 neighbours in label propagation (a block with a shared
+table each up to 18432; hubs by many blocks: counted per label up to 1024 labels, hash tables beyond)
+and coarse nodes with long segments in contraction."""
 from __future__ import annotations
 
 import numpy as np
@@ -39,10 +39,9 @@ def _clique(n):
     return gg.from_pairs(n, i, j)
 
 
-# 2048 neighbours are one block's, 2049 a hub's; 4096 entries end a chunk; the clique's hubs hold all
-# entries, so their tables would pass the memory bound
-GRAPHS = {"star": star(2049), "edges": _hubs(9000, [2047, 2048, 2049, 4096, 4097, 8000], 9000, 1),
-          "weighted": _hubs(30000, [29000, 12345, 2500, 2049], 20000, 50), "clique": _clique(3000)}
+# the classes end at 128, 2048, 6144 and 18432 neighbours; a hub's chunks have 2048 entries
+GRAPHS = {"star": star(2049), "edges": _hubs(9000, [128, 129, 2048, 2049, 6144, 6145, 8000], 9000, 1),
+          "weighted": _hubs(40000, [39000, 18433, 18432, 12345, 2500, 2049], 20000, 50), "clique": _clique(2500)}
 
 
 @pytest.mark.parametrize("name", sorted(GRAPHS))
