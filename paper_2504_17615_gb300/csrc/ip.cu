@@ -30,9 +30,10 @@
 //  * steps of up to kSoloB nodes run in one warp without block barriers.
 // A picked node that no longer fits is retired for good (side 1 only gets
 // heavier), which leaves the choice among the nodes that fit unchanged.
-// The fallback scans all nodes the first few times; after that, nodes are
-// chained by the top bits of their hash and a cursor walks the chains (a
-// node that left the free state or stopped fitting never comes back).
+// The fallback scans all nodes the first few times; after that, the nodes
+// still free are put in the order of the top bits of their hash (a counting
+// sort) and a cursor walks them, 32 at a time (a node that left the free state
+// or stopped fitting never comes back).
 //
 // Measured (20,480 nodes, 204,800 edges, k = 128, 8 trials; the whole initial partition): 17.0 ms with 64-bit
 // keys in separate arrays, block barriers in every step and a sort of the chunk maxima; 9.0 ms so.
@@ -49,8 +50,8 @@ constexpr int kSmemBatch = 64;  // the nodes of a growing step live in shared me
 constexpr int kChunkNodes = 64;
 constexpr int kIpWarps = 4;     // warps per (subproblem, trial)
 constexpr int kSoloB = 4;       // steps of up to this many nodes run in one warp
-constexpr int kScanFallbacks = 8;      // fallbacks found by a scan over all nodes before the chains are built
-constexpr int kChainNodes = 4;         // nodes per chain at least, on average
+constexpr int kScanFallbacks = 8;      // fallbacks found by a scan over all nodes before the order is made
+constexpr int kBucketNodes = 4;        // nodes per hash bucket of that order at least, on average
 constexpr int kNarrowNodes = 1 << 15;  // 32-bit words: subproblems below this many nodes ...
 constexpr int kNarrowGain = 1 << 15;   // ... and weighted degrees below this
 constexpr int kStaticSmem = 2048;      // room for the kernel's static shared variables
@@ -161,8 +162,9 @@ struct IpArgs {
   int32_t *gbatch;                 // per block: the nodes taken in the current step
   int batch_cap;
   int64_t bstride, sstride;        // their chunk maxima and maxima over 32 chunks, per trial
-  int32_t *fnext, *fhead;          // fallback chains (words in shared memory only): next node [trial][n],
-  int64_t hstride;                 // first node per bucket, hstride per trial
+  uint2 *ford;                     // [trial][n] fallback order (words in shared memory only): (hash, node)
+  int32_t *fcur;                   // and its buckets' places, hstride per trial
+  int64_t hstride;
   unsigned long long *trace;       // optional: [0] growing steps, [1] fallbacks, [2] retired nodes
   int64_t *trial_cut;              // per block
   uint8_t *flags;                  // [trial][n] side-1 flag by list position
@@ -261,11 +263,13 @@ __global__ void __launch_bounds__(32 * kIpWarps) k_ip_grow(IpArgs a) {
     x0 = W::wmax(x0);
     return x0 > kOut ? x0 : 0;
   };
-  int nfall = 0, cursor = 0;           // warp 0: fallbacks so far, bucket the chains are walked from
-  int bits = 0;                        // buckets: the hash's top bits, at most cnt / kChainNodes of them
-  while ((kChainNodes << (bits + 1)) <= cnt) bits++;
+  int nfall = 0, cursor = 0;           // warp 0: fallbacks so far, place in the order
+  int bits = 0;                        // buckets: the hash's top bits, at most cnt / kBucketNodes of them
+  while ((kBucketNodes << (bits + 1)) <= cnt) bits++;
   const int nbk = 1 << bits;
-  int32_t *const head = a.fhead + (int64_t)t * a.hstride + start / kChainNodes + si;
+  int32_t *const place = a.fcur + (int64_t)t * a.hstride + start / kBucketNodes + si;
+  uint2 *const order = a.ford + tpos;
+  __shared__ int s_free;               // nodes in the order
   auto hash_of = [&](int j) -> uint32_t { return h32(kip, (uint32_t)a.vtx[start + j], (uint32_t)t); };
   // one thread's share of a scan for the free node of smallest (hash, id) that fits
   auto scan_free = [&](int tid, int step, int64_t w1) -> unsigned long long {
@@ -277,30 +281,61 @@ __global__ void __launch_bounds__(32 * kIpWarps) k_ip_grow(IpArgs a) {
     }
     return m;
   };
-  auto chain_free = [&](int tid, int step) {  // chains of the nodes still free (heads cleared before)
+  auto bucket_of = [&](uint32_t h) -> int { return (int)((uint64_t)h >> (32 - bits)); };
+  // the order of the nodes still free, by one warp or the block (sync: its barrier); warp 0 scans the counts
+  auto make_order = [&](int tid, int step, auto sync) {
+    for (int b = tid; b < nbk; b += step) place[b] = 0;
+    sync();
     for (int j = tid; j < cnt; j += step)
-      if (X.get(j) < 0) a.fnext[tpos + j] = atomicExch(&head[(int)((uint64_t)hash_of(j) >> (32 - bits))], j);
-  };
-  // warp 0: the free node of smallest (hash, id) that fits, from the chains; -1 if none
-  auto walk_free = [&](int64_t w1) -> int {
-    while (cursor < nbk) {
-      unsigned long long m = ~0ull;
-      const int b = cursor + lane;
-      if (b < nbk)
-        for (int j = head[b]; j >= 0; j = a.fnext[tpos + j]) {
-          if (X.get(j) >= 0 || w1 + weight(j) > S.L1) continue;
-          const unsigned long long key = ((unsigned long long)hash_of(j) << 32) | (unsigned)j;
-          m = key < m ? key : m;
+      if (X.get(j) < 0) atomicAdd(&place[bucket_of(hash_of(j))], 1);
+    sync();
+    if (warp == 0) {
+      int run = 0;
+      for (int b0 = 0; b0 < nbk; b0 += 32) {
+        const int c = b0 + lane < nbk ? *(volatile int32_t *)&place[b0 + lane] : 0;
+        int y = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int z = __shfl_up_sync(0xFFFFFFFFu, y, o);
+          if (lane >= o) y += z;
         }
-      const unsigned any = __ballot_sync(0xFFFFFFFFu, m != ~0ull);
-      if (any) {
-        const int f = __ffs(any) - 1;
-        cursor += f;
-        return __shfl_sync(0xFFFFFFFFu, (int)(unsigned)m, f);
+        if (b0 + lane < nbk) place[b0 + lane] = run + y - c;
+        run += __shfl_sync(0xFFFFFFFFu, y, 31);
       }
-      cursor += 32;
+      if (lane == 0) s_free = run;
     }
-    return -1;
+    sync();
+    for (int j = tid; j < cnt; j += step) {
+      if (X.get(j) >= 0) continue;
+      const uint32_t h = hash_of(j);
+      order[atomicAdd(&place[bucket_of(h)], 1)] = make_uint2(h, (unsigned)j);
+    }
+    sync();
+  };
+  // warp 0: the free node of smallest (hash, id) that fits, from the order; -1 if none.  The first valid
+  // node's bucket holds the answer; it may go on past the 32 nodes looked at.
+  auto walk_free = [&](int64_t w1) -> int {
+    const int total = s_free;
+    int bucket = -1;
+    unsigned long long best = ~0ull;
+    for (int p = cursor; p < total; p += 32) {
+      const bool in = p + lane < total;
+      const uint2 x = in ? order[p + lane] : make_uint2(0, 0);
+      const bool ok = in && X.get((int)x.y) < 0 && w1 + weight((int)x.y) <= S.L1;
+      const unsigned m = __ballot_sync(0xFFFFFFFFu, ok);
+      if (bucket < 0) {
+        if (m == 0) { cursor = p + 32; continue; }
+        const int f = __ffs(m) - 1;
+        cursor = p + f;
+        bucket = bucket_of(__shfl_sync(0xFFFFFFFFu, x.x, f));
+      }
+      const bool same = in && bucket_of(x.x) == bucket;
+      const unsigned long long key = ok && same ? ((unsigned long long)x.x << 32) | x.y : ~0ull;
+      const unsigned long long k = wmin_u64(key);
+      best = k < best ? k : best;
+      if (!__shfl_sync(0xFFFFFFFFu, same, 31)) break;  // the bucket ends within these nodes
+    }
+    return best == ~0ull ? -1 : (int)(unsigned)best;
   };
 
   int64_t w1 = 0;
@@ -359,12 +394,7 @@ __global__ void __launch_bounds__(32 * kIpWarps) k_ip_grow(IpArgs a) {
       const unsigned long long m = wmin_u64(scan_free(lane, 32, w1));
       j = m == ~0ull ? -1 : (int)(unsigned)m;
     } else {
-      if (nfall == kScanFallbacks) {
-        for (int b = lane; b < nbk; b += 32) head[b] = -1;
-        __syncwarp();
-        chain_free(lane, 32);
-        __syncwarp();
-      }
+      if (nfall == kScanFallbacks) make_order(lane, 32, [] { __syncwarp(); });
       j = walk_free(w1);
     }
     nfall++;
@@ -473,12 +503,7 @@ __global__ void __launch_bounds__(32 * kIpWarps) k_ip_grow(IpArgs a) {
             s_fj = mm == ~0ull ? -1 : (int)(unsigned)mm;
           }
         } else {
-          if (nfall == kScanFallbacks) {
-            for (int b = threadIdx.x; b < nbk; b += blockDim.x) head[b] = -1;
-            __syncthreads();
-            chain_free(threadIdx.x, blockDim.x);
-            __syncthreads();
-          }
+          if (nfall == kScanFallbacks) make_order(threadIdx.x, blockDim.x, [] { __syncthreads(); });
           if (warp == 0) {
             const int j = walk_free(w1);
             if (lane == 0) s_fj = j;
@@ -765,7 +790,8 @@ void initial_partition(gp_ctx *ctx, const DevGraph &g, int32_t k, int64_t eps_pp
   const int64_t eps_l = eps_ppm / ceil_log2(k);
   std::vector<HostSub> subs{{k, 0, 1, n, (int64_t)ht.W}};
   DBuf<uint8_t> flags(ctx, (size_t)trials * n);
-  DBuf<int32_t> fnext, fhead;
+  DBuf<uint2> ford;
+  DBuf<int32_t> fcur;
   // per depth, at most k subproblems: their records, trial cuts, side totals, children
   DBuf<Sub> dsub(ctx, (size_t)k);
   DBuf<int64_t> tcut(ctx, (size_t)k * trials);
@@ -833,13 +859,13 @@ void initial_partition(gp_ctx *ctx, const DevGraph &g, int32_t k, int64_t eps_pp
       a.gx = gx.get(); a.gbest = gbest.get(); a.gsup = gsup.get();
     }
     if (sm) {
-      a.hstride = n / kChainNodes + k + 1;
-      if (!fnext.get()) {
-        fnext.reset(ctx, (size_t)trials * n);
-        fhead.reset(ctx, (size_t)(trials * a.hstride));
+      a.hstride = n / kBucketNodes + k + 1;
+      if (!ford.get()) {
+        ford.reset(ctx, (size_t)trials * n);
+        fcur.reset(ctx, (size_t)(trials * a.hstride));
       }
-      a.fnext = fnext.get();
-      a.fhead = fhead.get();
+      a.ford = ford.get();
+      a.fcur = fcur.get();
     }
     a.batch_cap = 1 + maxcnt / 1024;
     DBuf<int32_t> gbatch;

@@ -1,6 +1,6 @@
 """GPU vs CPU oracle, exact: the initial partition in every form its growing kernel takes -- 32-bit and
 64-bit node words, one-warp and four-warp steps, words in shared and in global memory, rows and row
-bounds in shared memory or not, and fallbacks found by scans and by the hash chains."""
+bounds in shared memory or not, and fallbacks found by scans and from the hash order."""
 from __future__ import annotations
 
 import numpy as np
@@ -37,7 +37,7 @@ def test_words_and_steps(ctx, n, wmax):
     _check(ctx, gg.with_node_weights(g, 5), 2 if n > 5000 else 5, n)
 
 
-# many components: most steps find no frontier node (the chains start at the ninth fallback of a trial)
+# many components: most steps find no frontier node (the hash order is made at the ninth fallback of a trial)
 @pytest.mark.parametrize("n,m", [(40, 5), (900, 150), (6000, 900)])
 @pytest.mark.parametrize("cmax", [1, 70000])
 def test_fallbacks(ctx, n, m, cmax):
