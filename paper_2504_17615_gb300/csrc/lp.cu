@@ -44,6 +44,7 @@ struct RateArgs {
   int32_t *gkeys, *gvals;  // large kernel global tables
   int64_t gstride;
   unsigned long long *units;
+  int64_t m2;           // CSR entries
   int wlabels;          // labels whose weights a launch may copy to shared memory (<= 256)
   uint8_t *dirty;       // optional: per node, 0 = cannot move until a neighbour moves (rating skipped)
   const int32_t *ccount;  // optional: the list holds ccount[key] records from offs[key] (compacted)
@@ -86,473 +87,159 @@ __device__ __forceinline__ void emit(const RateArgs &a, int i, int v, int best, 
   }
 }
 
-// ------------------------------------- degree <= 32: G lanes per node
+// ------------------------------------- degree <= 32: a thread per node
 //
-// A warp rates 32/G nodes side by side (one neighbour per lane of a G-lane
-// group) and keeps U such sets in flight, issuing the loads of all U*32/G
-// nodes phase by phase (offsets, neighbours, labels) so that independent
-// dependency chains overlap.  Equal labels within a group are summed in a
-// 2G-slot shared-memory table per group (the first lane to claim a slot is
-// the label's leader).  The choice is lazy in the label weights: candidates
-// are ranked by (rating, tie hash, label) without the bound, and only the
-// leading candidate's weight is fetched; if it does not fit, it is dropped
-// and the next one is tried.  This picks exactly the best admissible
-// candidate while reading one label weight per node in the usual case, and
-// none at all when no neighbouring label beats the node's own label.  With
-// one-byte labels (refinement: at most 255 labels) the label weights are
-// copied to shared memory once per launch and every candidate is checked
-// against the bound up front, so the first pass already picks the best
-// admissible label.
+// A thread loads its node's whole row (16 bytes a load where the arrays are aligned), gathers the labels,
+// and adds up equal labels by comparing all pairs in registers.  It is the gather of the labels that
+// should bound this step (about 300e9 random reads/s while the label array fits L2, 76e9/s from a 268 MB
+// array); with 8 or 16 lanes per node and tables in shared memory a node of 20 neighbours took 225-300
+// warp instructions, so that issue and latency bound it instead.  The pairs cost D (D - 1) / 2 x 3
+// instructions per 32 nodes, a tenth of that, and every label of the row is in flight at once.
+// THRNUM
+//
+// The choice is lazy in the label weights: candidates are ranked by (rating, tie hash, label) without the
+// bound, and only the best one's weight is read; if it does not fit, the weights of all that are rated
+// above the own label are read and those that do not fit dropped.  With one-byte labels (refinement: at
+// most 255 labels) the label weights are copied to shared memory once per block and every candidate is
+// checked up front.
 
-// Label kinds: LK_WIDE int32 labels summed in hash tables; LK_NARROW uint8
-// labels (fewer than 256) in hash tables; LK_DENSE uint8 labels below
-// kDenseLabels summed in a dense per-group array indexed by label.
-enum LabelKind { LK_WIDE = 0, LK_NARROW = 1, LK_DENSE = 2 };
-constexpr int kDenseLabels = 128;
+// Label kinds: LK_WIDE int32 labels, LK_NARROW uint8 labels (fewer than 256).
+enum LabelKind { LK_WIDE = 0, LK_NARROW = 1 };
 
-template <int MODE, int G, int U, int LK>
-__global__ void __launch_bounds__(kThreads, G == 32 ? 4 : 5) k_rate_group(RateArgs a) {
-  static_assert(G == 8 || G == 16 || G == 32, "group width");
-  constexpr int NV = 32 / G;
-  constexpr int PER = NV * U;
-  constexpr int TS = 2 * G;  // hash-table slots per group
-  constexpr int TW = LK == LK_DENSE ? U * NV * kDenseLabels : U * 64;  // table words per warp
-  __shared__ int s_tk[LK == LK_DENSE ? 1 : kWarpsPerBlock][LK == LK_DENSE ? 1 : U * 64];
-  __shared__ int s_tv[kWarpsPerBlock][TW];
-  constexpr bool kSmemW = MODE == RATE_LP && LK != LK_WIDE;
-  __shared__ int s_w[kSmemW ? 256 : 1];
-  if (a.stop && *a.stop) return;
-  if (kSmemW) {
-    for (int t = threadIdx.x; t < a.wlabels; t += blockDim.x) s_w[t] = a.weight[t];
-    __syncthreads();
-  }
-  const int lane = (int)lane_id(), wib = threadIdx.x >> 5;
-  const int grp = lane / G, gl = lane % G;
-  const unsigned gmask = G == 32 ? FULL : (((1u << G) - 1u) << (grp * G));
-  for (int t = lane; t < TW; t += 32) {
-    if (LK != LK_DENSE) s_tk[wib][t] = -1;
-    s_tv[wib][t] = 0;
-  }
-  __syncwarp();
-  const int begin = a.offs[a.key], end = list_end(a);
-  const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-  unsigned long long ue = 0, uv = 0, uc = 0, up = 0;
-  for (int base = begin + wid * PER; base < end; base += nw * PER) {
-    int v[U], st[U], deg[U], own[U], cv[U], L[U], w[U], u[U];
-    bool skip[U];
+template <int D>
+struct ThreadShape {
+  static constexpr int NT = D <= 16 ? 256 : 128;
+  static constexpr int PER_SM = D <= 8 ? 5 : D <= 16 ? 3 : 4;  // blocks an SM holds: 51, 85 and 128 registers
+};
+
+// x[q] = base[st + q] for q < deg, 0 beyond.  vec: base is 16-byte aligned; then 16 bytes a load, from the
+// last boundary before st, moved into place by two selects a word (lim: words that may be read).
+template <int D>
+__device__ __forceinline__ void load_row(const int32_t *base, int st, int deg, int64_t lim, bool vec, int (&x)[D]) {
+  if (vec) {
+    int w[D + 4];
+    const int off = st & 3, s0 = st - off;
 #pragma unroll
-    for (int q = 0; q < U; q++) {
-      const int i = base + q * NV + grp;
-      const int4 rec = i < end ? a.list[i] : make_int4(-1, 0, 0, 0);
-      v[q] = rec.x; st[q] = rec.y; deg[q] = rec.z; cv[q] = rec.w;
-    }
-#pragma unroll
-    for (int q = 0; q < U; q++) {
-      // a clean node cannot move: neither its neighbours' labels nor its own changed since it
-      // last found no label rated above its own
-      skip[q] = a.dirty && v[q] >= 0 && !a.dirty[v[q]];
-      if (skip[q]) { v[q] = -1; deg[q] = 0; }
-    }
-#pragma unroll
-    for (int q = 0; q < U; q++) {
-      const bool ok = v[q] >= 0;
-      own[q] = ok ? (LK == LK_WIDE ? a.label[v[q]] : (int)a.label8[v[q]]) : -2;
-    }
-#pragma unroll
-    for (int q = 0; q < U; q++) {
-      const bool ok = gl < deg[q];
-      u[q] = ok ? __ldcs(a.adjncy + st[q] + gl) : -1;  // rows are read once a round: evict first
-      w[q] = ok ? (a.adjwgt ? __ldcs(a.adjwgt + st[q] + gl) : 1) : 0;
-    }
-#pragma unroll
-    for (int q = 0; q < U; q++)
-      L[q] = u[q] >= 0 ? (LK == LK_WIDE ? a.label[u[q]] : (int)a.label8[u[q]]) : -1;
-    // sum equal labels per group in shared memory
-    int slot[U], own_r[U], sum[U];
-    bool lead[U];
-    if (LK == LK_DENSE) {
-#pragma unroll
-      for (int q = 0; q < U; q++) {
-        slot[q] = (q * NV + grp) * kDenseLabels;
-        if (u[q] >= 0) atomicAdd(&s_tv[wib][slot[q] + L[q]], w[q]);
-      }
-      __syncwarp();
-#pragma unroll
-      for (int q = 0; q < U; q++) {
-        sum[q] = u[q] >= 0 ? s_tv[wib][slot[q] + L[q]] : 0;
-        own_r[q] = v[q] >= 0 ? s_tv[wib][slot[q] + own[q]] : 0;
-        lead[q] = u[q] >= 0;  // duplicates of a label are harmless below
-      }
-      __syncwarp();
-#pragma unroll
-      for (int q = 0; q < U; q++)
-        if (u[q] >= 0) s_tv[wib][slot[q] + L[q]] = 0;
-      __syncwarp();
-    } else {
-#pragma unroll
-      for (int q = 0; q < U; q++) {
-        int *tk = &s_tk[wib][q * 64 + grp * TS];
-        slot[q] = -1;
-        lead[q] = false;
-        if (u[q] >= 0) {
-          unsigned sl = ((unsigned)L[q] * 2654435761u) >> (32 - (G == 8 ? 4 : G == 16 ? 5 : 6));
-          for (int p = 0; p < TS; p++) {  // bounded: a group has at most G labels in 2G slots
-            const int prev = atomicCAS(&tk[sl], -1, L[q]);
-            if (prev == -1) { lead[q] = true; break; }
-            if (prev == L[q]) break;
-            sl = (sl + 1) & (TS - 1);
-          }
-          slot[q] = q * 64 + grp * TS + (int)sl;
-          atomicAdd(&s_tv[wib][slot[q]], w[q]);
+    for (int g = 0; g < (D + 4) / 4; g++) {
+      const int idx = s0 + 4 * g;
+      int4 y = make_int4(0, 0, 0, 0);
+      if (idx < st + deg) {
+        if ((int64_t)idx + 4 <= lim) {
+          y = __ldcs(reinterpret_cast<const int4 *>(base + idx));
+        } else {  // the array's last words
+          y.x = base[idx];
+          if ((int64_t)idx + 1 < lim) y.y = base[idx + 1];
+          if ((int64_t)idx + 2 < lim) y.z = base[idx + 2];
         }
       }
-      __syncwarp();
-#pragma unroll
-      for (int q = 0; q < U; q++) sum[q] = slot[q] >= 0 ? s_tv[wib][slot[q]] : 0;
-      __syncwarp();
-#pragma unroll
-      for (int q = 0; q < U; q++)
-        if (lead[q]) { s_tk[wib][slot[q]] = -1; s_tv[wib][slot[q]] = 0; }
-      __syncwarp();
-#pragma unroll
-      for (int q = 0; q < U; q++)
-        own_r[q] = __reduce_max_sync(gmask, (lead[q] && L[q] == own[q]) ? sum[q] : 0);
-    }
-    // choose: all U sets advance together, so that the weight reads of their
-    // leading candidates are issued side by side.  When a group's leading
-    // candidate does not fit, the weights of all its remaining candidates are
-    // read at once on the next pass and the inadmissible ones dropped, so a
-    // node takes at most three passes.
-    bool alive[U], searching[U], eager[U];
-    unsigned best[U];
-    // no label rated above the own one, admissible or not: the node proposes nothing (so it skips
-    // the choice), and in refinement it stays clean until a neighbour moves
-    bool stay[U];
-#pragma unroll
-    for (int q = 0; q < U; q++) {
-      const int rall = (int)__reduce_max_sync(gmask, (lead[q] && L[q] != own[q]) ? (unsigned)sum[q] : 0u);
-      stay[q] = MODE == RATE_LP && rall <= own_r[q];
-      if (a.dirty && gl == 0 && v[q] >= 0 && stay[q]) a.dirty[v[q]] = 0;
+      w[4 * g] = y.x; w[4 * g + 1] = y.y; w[4 * g + 2] = y.z; w[4 * g + 3] = y.w;
     }
 #pragma unroll
-    for (int q = 0; q < U; q++) {
-      alive[q] = lead[q] && L[q] != own[q];
-      uc += alive[q];
-      if (kSmemW && alive[q]) alive[q] = (int64_t)s_w[L[q]] + cv[q] <= a.bound;
-      searching[q] = v[q] >= 0 && !stay[q];
-      eager[q] = kSmemW;
-      best[q] = 0xFFFFFFFFu;
-    }
-    for (int it = 0; it <= G; it++) {  // bounded: every pass drops one candidate per searching group
-      bool any = false;
+    for (int q = 0; q < D + 2; q++) w[q] = (off & 1) ? w[q + 1] : w[q];
 #pragma unroll
-      for (int q = 0; q < U; q++) any = any || searching[q];
-      if (!__any_sync(FULL, any)) break;
-      if (MODE == RATE_LP && !kSmemW) {
-        int we[U];
+    for (int q = 0; q < D; q++) x[q] = (off & 2) ? w[q + 2] : w[q];
+  } else {
 #pragma unroll
-        for (int q = 0; q < U; q++) we[q] = (eager[q] && searching[q] && alive[q]) ? a.weight[L[q]] : 0;
-#pragma unroll
-        for (int q = 0; q < U; q++)
-          if (eager[q] && searching[q] && alive[q] && (int64_t)we[q] + cv[q] > a.bound) alive[q] = false;
-      }
-      unsigned c[U];
-      bool holder[U];
-#pragma unroll
-      for (int q = 0; q < U; q++) {
-        const int r = __reduce_max_sync(gmask, (searching[q] && alive[q]) ? sum[q] : -1);
-        if (r < 0 || (MODE == RATE_LP && r <= own_r[q])) searching[q] = false;
-        const bool top = searching[q] && alive[q] && sum[q] == r;
-        const unsigned h = top ? h32(a.ktie, (uint32_t)v[q], (uint32_t)L[q]) : 0xFFFFFFFFu;
-        const unsigned hmin = __reduce_min_sync(gmask, h);
-        c[q] = __reduce_min_sync(gmask, (top && h == hmin) ? (unsigned)L[q] : 0xFFFFFFFFu);
-        holder[q] = top && h == hmin && (unsigned)L[q] == c[q];
-      }
-      if (MODE != RATE_LP || kSmemW) {
-#pragma unroll
-        for (int q = 0; q < U; q++)
-          if (searching[q]) { best[q] = c[q]; searching[q] = false; }
-      } else {
-        int wc[U];
-#pragma unroll
-        for (int q = 0; q < U; q++) wc[q] = (holder[q] && !eager[q]) ? a.weight[c[q]] : 0;
-#pragma unroll
-        for (int q = 0; q < U; q++) {
-          // after an eager pass every remaining candidate fits
-          const unsigned fits = holder[q] && (eager[q] || (int64_t)wc[q] + cv[q] <= a.bound) ? 1u : 0u;
-          if (__reduce_or_sync(gmask, fits) && searching[q]) { best[q] = c[q]; searching[q] = false; }
-          alive[q] = alive[q] && (unsigned)L[q] != c[q];
-          eager[q] = true;
-        }
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < U; q++) {
-      if (gl == 0 && v[q] >= 0) {
-        ue += deg[q];
-        uv += 1;
-        if (best[q] != 0xFFFFFFFFu) {
-          emit<MODE>(a, base + q * NV + grp, v[q], (int)best[q], cv[q], own[q]);
-          up += 1;
-        } else if (MODE == RATE_LP) {
-          a.prop[base + q * NV + grp] = make_int2(-1, 0);
-        }
-      } else if (gl == 0 && skip[q] && MODE == RATE_LP) {
-        a.prop[base + q * NV + grp] = make_int2(-1, 0);
-      }
-    }
+    for (int q = 0; q < D; q++) x[q] = q < deg ? __ldcs(base + st + q) : 0;
   }
-  add_units(a.units, ue, uv, uc, up, a.label8 != nullptr, a.adjwgt == nullptr);
 }
 
-// ----------------- degree <= 32 with E entries per lane: G lanes per node
-//
-// The same rating and choice as k_rate_group, with every lane of a G-lane group
-// holding up to E neighbours, so that a warp rates 32/G nodes of degree up to
-// G * E side by side and every group-wide reduction of the choice serves 32/G
-// nodes at once (nodes of degree 9-32 on 8 or 16 lanes instead of a whole warp).
-template <int MODE, int G, int E, int U, int LK>
-__global__ void __launch_bounds__(kThreads, 4) k_rate_multi(RateArgs a) {
-  static_assert(G == 8 || G == 16, "group width");
-  constexpr int NV = 32 / G;
-  constexpr int PER = NV * U;
-  constexpr int TS = 2 * G * E;  // hash-table slots per (set, group)
-  constexpr int TBITS = TS == 32 ? 5 : TS == 64 ? 6 : 7;
-  static_assert((1 << TBITS) == TS, "table size");
-  constexpr int TW = LK == LK_DENSE ? U * NV * kDenseLabels : U * NV * TS;  // table words per warp
-  __shared__ int s_tk[LK == LK_DENSE ? 1 : kWarpsPerBlock][LK == LK_DENSE ? 1 : TW];
-  __shared__ int s_tv[kWarpsPerBlock][TW];
+template <int MODE, int D, int LK>
+__global__ void __launch_bounds__(ThreadShape<D>::NT, ThreadShape<D>::PER_SM) k_rate_thread(RateArgs a) {
+  constexpr int NT = ThreadShape<D>::NT;
   constexpr bool kSmemW = MODE == RATE_LP && LK != LK_WIDE;
   __shared__ int s_w[kSmemW ? 256 : 1];
   if (a.stop && *a.stop) return;
   if (kSmemW) {
-    for (int t = threadIdx.x; t < a.wlabels; t += blockDim.x) s_w[t] = a.weight[t];
+    for (int t = threadIdx.x; t < a.wlabels; t += NT) s_w[t] = a.weight[t];
     __syncthreads();
   }
-  const int lane = (int)lane_id(), wib = threadIdx.x >> 5;
-  const int grp = lane / G, gl = lane % G;
-  const unsigned gmask = ((1u << G) - 1u) << (grp * G);
-  for (int t = lane; t < TW; t += 32) {
-    if (LK != LK_DENSE) s_tk[wib][t] = -1;
-    s_tv[wib][t] = 0;
-  }
-  __syncwarp();
+  const bool vec = (((uintptr_t)a.adjncy | (uintptr_t)a.adjwgt) & 15) == 0;
   const int begin = a.offs[a.key], end = list_end(a);
-  const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int nw = (int)((gridDim.x * blockDim.x) >> 5);
   unsigned long long ue = 0, uv = 0, uc = 0, up = 0;
-  for (int base = begin + wid * PER; base < end; base += nw * PER) {
-    int v[U], st[U], deg[U], own[U], cv[U];
-    int L[U][E], w[U][E], u[U][E];
-    bool skip[U];
+  for (int i0 = begin + (int)(blockIdx.x * NT); i0 < end; i0 += (int)(gridDim.x * NT)) {
+    const int i = i0 + (int)threadIdx.x;
+    int4 rec = i < end ? a.list[i] : make_int4(-1, 0, 0, 0);
+    const int v = rec.x, cv = rec.w;
+    // a clean node cannot move: neither its neighbours' labels nor its own changed since it last found no
+    // label rated above its own
+    const bool live = v >= 0 && !(a.dirty && !a.dirty[v]);
+    const int st = live ? rec.y : 0, deg = live ? rec.z : 0;
+    const int own = live ? (LK == LK_WIDE ? a.label[v] : (int)a.label8[v]) : -2;
+    int L[D], w[D];
+    load_row<D>(a.adjncy, st, deg, a.m2, vec, L);
 #pragma unroll
-    for (int q = 0; q < U; q++) {
-      const int i = base + q * NV + grp;
-      const int4 rec = i < end ? a.list[i] : make_int4(-1, 0, 0, 0);
-      v[q] = rec.x; st[q] = rec.y; deg[q] = rec.z; cv[q] = rec.w;
-    }
-#pragma unroll
-    for (int q = 0; q < U; q++) {
-      skip[q] = a.dirty && v[q] >= 0 && !a.dirty[v[q]];
-      if (skip[q]) { v[q] = -1; deg[q] = 0; }
-    }
-#pragma unroll
-    for (int q = 0; q < U; q++) {
-      const bool ok = v[q] >= 0;
-      own[q] = ok ? (LK == LK_WIDE ? a.label[v[q]] : (int)a.label8[v[q]]) : -2;
-    }
-#pragma unroll
-    for (int q = 0; q < U; q++)
-#pragma unroll
-      for (int e = 0; e < E; e++) {
-        const int j = gl + e * G;
-        const bool ok = j < deg[q];
-        u[q][e] = ok ? __ldcs(a.adjncy + st[q] + j) : -1;  // rows are read once a round: evict first
-        w[q][e] = ok ? (a.adjwgt ? __ldcs(a.adjwgt + st[q] + j) : 1) : 0;
-      }
-#pragma unroll
-    for (int q = 0; q < U; q++)
-#pragma unroll
-      for (int e = 0; e < E; e++)
-        L[q][e] = u[q][e] >= 0 ? (LK == LK_WIDE ? a.label[u[q][e]] : (int)a.label8[u[q][e]]) : -1;
-    int own_r[U], sum[U][E];
-    bool lead[U][E];
-    if (LK == LK_DENSE) {
-#pragma unroll
-      for (int q = 0; q < U; q++) {
-        const int sb = (q * NV + grp) * kDenseLabels;
-#pragma unroll
-        for (int e = 0; e < E; e++)
-          if (u[q][e] >= 0) atomicAdd(&s_tv[wib][sb + L[q][e]], w[q][e]);
-      }
-      __syncwarp();
-#pragma unroll
-      for (int q = 0; q < U; q++) {
-        const int sb = (q * NV + grp) * kDenseLabels;
-        own_r[q] = v[q] >= 0 ? s_tv[wib][sb + own[q]] : 0;
-#pragma unroll
-        for (int e = 0; e < E; e++) {
-          sum[q][e] = u[q][e] >= 0 ? s_tv[wib][sb + L[q][e]] : 0;
-          lead[q][e] = u[q][e] >= 0;  // duplicates of a label are harmless below
-        }
-      }
-      __syncwarp();
-#pragma unroll
-      for (int q = 0; q < U; q++) {
-        const int sb = (q * NV + grp) * kDenseLabels;
-#pragma unroll
-        for (int e = 0; e < E; e++)
-          if (u[q][e] >= 0) s_tv[wib][sb + L[q][e]] = 0;
-      }
-      __syncwarp();
+    for (int q = 0; q < D; q++) L[q] = q < deg ? (LK == LK_WIDE ? a.label[L[q]] : (int)a.label8[L[q]]) : -1;
+    if (a.adjwgt) {
+      load_row<D>(a.adjwgt, st, deg, a.m2, vec, w);
     } else {
-      int slot[U][E];
 #pragma unroll
-      for (int q = 0; q < U; q++) {
-        const int sb = (q * NV + grp) * TS;
-        int *tk = &s_tk[wib][sb];
-#pragma unroll
-        for (int e = 0; e < E; e++) {
-          slot[q][e] = -1;
-          lead[q][e] = false;
-          if (u[q][e] < 0) continue;
-          unsigned sl = ((unsigned)L[q][e] * 2654435761u) >> (32 - TBITS);
-          for (int p = 0; p < TS; p++) {  // bounded: a group holds at most G E labels in 2 G E slots
-            const int prev = atomicCAS(&tk[sl], -1, L[q][e]);
-            if (prev == -1) { lead[q][e] = true; break; }
-            if (prev == L[q][e]) break;
-            sl = (sl + 1) & (TS - 1);
-          }
-          slot[q][e] = sb + (int)sl;
-          atomicAdd(&s_tv[wib][slot[q][e]], w[q][e]);
-        }
-      }
-      __syncwarp();
-#pragma unroll
-      for (int q = 0; q < U; q++)
-#pragma unroll
-        for (int e = 0; e < E; e++) sum[q][e] = slot[q][e] >= 0 ? s_tv[wib][slot[q][e]] : 0;
-      __syncwarp();
-#pragma unroll
-      for (int q = 0; q < U; q++)
-#pragma unroll
-        for (int e = 0; e < E; e++)
-          if (lead[q][e]) { s_tk[wib][slot[q][e]] = -1; s_tv[wib][slot[q][e]] = 0; }
-      __syncwarp();
-#pragma unroll
-      for (int q = 0; q < U; q++) {
-        unsigned o = 0;
-#pragma unroll
-        for (int e = 0; e < E; e++)
-          if (lead[q][e] && L[q][e] == own[q]) o = max(o, (unsigned)sum[q][e]);
-        own_r[q] = (int)__reduce_max_sync(gmask, o);
-      }
+      for (int q = 0; q < D; q++) w[q] = 1;
     }
-    // choose (as k_rate_group): all U sets advance together; a group whose leading candidate does
-    // not fit reads the weights of all its remaining candidates on the next pass
-    bool alive[U][E], searching[U], eager[U];
-    unsigned best[U];
-    // no label rated above the own one, admissible or not: the node proposes nothing (so it skips
-    // the choice), and in refinement it stays clean until a neighbour moves
-    bool stay[U];
+    // equal labels: the first of them takes the sum, the others drop out (-1)
+    const int dm = __reduce_max_sync(FULL, deg);
 #pragma unroll
-    for (int q = 0; q < U; q++) {
-      unsigned ra = 0;
+    for (int p = 0; p < D - 1; p++) {
+      if (p >= dm) break;
 #pragma unroll
-      for (int e = 0; e < E; e++)
-        if (lead[q][e] && L[q][e] != own[q]) ra = max(ra, (unsigned)sum[q][e]);
-      const int rall = (int)__reduce_max_sync(gmask, ra);
-      stay[q] = MODE == RATE_LP && rall <= own_r[q];
-      if (a.dirty && gl == 0 && v[q] >= 0 && stay[q]) a.dirty[v[q]] = 0;
-    }
+      for (int b = p / 8 * 8; b < D; b += 8) {
+        if (b >= dm) break;
 #pragma unroll
-    for (int q = 0; q < U; q++) {
-#pragma unroll
-      for (int e = 0; e < E; e++) {
-        alive[q][e] = lead[q][e] && L[q][e] != own[q];
-        uc += alive[q][e];
-        if (kSmemW && alive[q][e]) alive[q][e] = (int64_t)s_w[L[q][e]] + cv[q] <= a.bound;
-      }
-      searching[q] = v[q] >= 0 && !stay[q];
-      eager[q] = kSmemW;
-      best[q] = 0xFFFFFFFFu;
-    }
-    for (int it = 0; it <= G * E; it++) {  // bounded: every pass drops one candidate per searching group
-      bool any = false;
-#pragma unroll
-      for (int q = 0; q < U; q++) any = any || searching[q];
-      if (!__any_sync(FULL, any)) break;
-      if (MODE == RATE_LP && !kSmemW) {
-#pragma unroll
-        for (int q = 0; q < U; q++)
-#pragma unroll
-          for (int e = 0; e < E; e++)
-            if (eager[q] && searching[q] && alive[q][e] && (int64_t)a.weight[L[q][e]] + cv[q] > a.bound)
-              alive[q][e] = false;
-      }
-      unsigned c[U];
-      bool holder[U];
-#pragma unroll
-      for (int q = 0; q < U; q++) {
-        int rl = -1;
-#pragma unroll
-        for (int e = 0; e < E; e++)
-          if (searching[q] && alive[q][e]) rl = max(rl, sum[q][e]);
-        const int r = __reduce_max_sync(gmask, rl);
-        if (r < 0 || (MODE == RATE_LP && r <= own_r[q])) searching[q] = false;
-        unsigned h[E], hl = 0xFFFFFFFFu;
-#pragma unroll
-        for (int e = 0; e < E; e++) {
-          const bool top = searching[q] && alive[q][e] && sum[q][e] == r;
-          h[e] = top ? h32(a.ktie, (uint32_t)v[q], (uint32_t)L[q][e]) : 0xFFFFFFFFu;
-          hl = min(hl, h[e]);
-        }
-        const unsigned hmin = __reduce_min_sync(gmask, hl);
-        unsigned cl = 0xFFFFFFFFu;
-#pragma unroll
-        for (int e = 0; e < E; e++)
-          if (searching[q] && alive[q][e] && sum[q][e] == r && h[e] == hmin) cl = min(cl, (unsigned)L[q][e]);
-        c[q] = __reduce_min_sync(gmask, cl);
-        holder[q] = false;
-#pragma unroll
-        for (int e = 0; e < E; e++)
-          holder[q] = holder[q] || (searching[q] && alive[q][e] && sum[q][e] == r && h[e] == hmin &&
-                                    (unsigned)L[q][e] == c[q]);
-      }
-      if (MODE != RATE_LP || kSmemW) {
-#pragma unroll
-        for (int q = 0; q < U; q++)
-          if (searching[q]) { best[q] = c[q]; searching[q] = false; }
-      } else {
-        int wc[U];
-#pragma unroll
-        for (int q = 0; q < U; q++) wc[q] = (holder[q] && !eager[q]) ? a.weight[c[q]] : 0;
-#pragma unroll
-        for (int q = 0; q < U; q++) {
-          // after an eager pass every remaining candidate fits
-          const unsigned fits = holder[q] && (eager[q] || (int64_t)wc[q] + cv[q] <= a.bound) ? 1u : 0u;
-          if (__reduce_or_sync(gmask, fits) && searching[q]) { best[q] = c[q]; searching[q] = false; }
-#pragma unroll
-          for (int e = 0; e < E; e++) alive[q][e] = alive[q][e] && (unsigned)L[q][e] != c[q];
-          eager[q] = true;
+        for (int q = b; q < b + 8; q++) {
+          if (q <= p) continue;
+          if (L[q] == L[p]) { w[p] += w[q]; L[q] = -1; }
         }
       }
     }
+    int own_r = 0, rall = 0, nc = 0;
 #pragma unroll
-    for (int q = 0; q < U; q++) {
-      if (gl == 0 && v[q] >= 0) {
-        ue += deg[q];
-        uv += 1;
-        if (best[q] != 0xFFFFFFFFu) {
-          emit<MODE>(a, base + q * NV + grp, v[q], (int)best[q], cv[q], own[q]);
-          up += 1;
-        } else if (MODE == RATE_LP) {
-          a.prop[base + q * NV + grp] = make_int2(-1, 0);
-        }
-      } else if (gl == 0 && skip[q] && MODE == RATE_LP) {
-        a.prop[base + q * NV + grp] = make_int2(-1, 0);
+    for (int q = 0; q < D; q++) {
+      if (L[q] == own) { own_r = w[q]; L[q] = -1; }
+      if (L[q] >= 0) { rall = w[q] > rall ? w[q] : rall; nc++; }
+    }
+    uc += nc;
+    // no label rated above the own one, admissible or not: the node proposes nothing, and in refinement it
+    // stays clean until a neighbour moves
+    const bool stay = MODE == RATE_LP && rall <= own_r;
+    if (a.dirty && live && stay) a.dirty[v] = 0;
+    int best = -1;
+    if (live && !stay) {
+      if (kSmemW) {
+#pragma unroll
+        for (int q = 0; q < D; q++)
+          if (L[q] >= 0 && (int64_t)s_w[L[q]] + cv > a.bound) L[q] = -1;
       }
+      for (int pass = 0; pass < 2; pass++) {
+        int r = -1;
+#pragma unroll
+        for (int q = 0; q < D; q++) r = L[q] >= 0 && w[q] > r ? w[q] : r;
+        if (r < 0 || (MODE == RATE_LP && r <= own_r)) break;
+        unsigned hb = 0xFFFFFFFFu;
+        int lb = 0x7FFFFFFF;
+#pragma unroll
+        for (int q = 0; q < D; q++) {
+          if (L[q] < 0 || w[q] != r) continue;
+          const unsigned h = h32(a.ktie, (uint32_t)v, (uint32_t)L[q]);
+          if (h < hb || (h == hb && L[q] < lb)) { hb = h; lb = L[q]; }
+        }
+        if (MODE != RATE_LP || kSmemW || pass == 1 || (int64_t)a.weight[lb] + cv <= a.bound) {
+          best = lb;
+          break;
+        }
+#pragma unroll
+        for (int q = 0; q < D; q++)
+          if (L[q] >= 0 && (w[q] <= own_r || (int64_t)a.weight[L[q]] + cv > a.bound)) L[q] = -1;
+      }
+    }
+    if (live) {
+      ue += deg;
+      uv += 1;
+    }
+    if (best >= 0) {
+      emit<MODE>(a, i, v, best, cv, own);
+      up += 1;
+    } else if (MODE == RATE_LP && v >= 0) {
+      a.prop[i] = make_int2(-1, 0);
     }
   }
   add_units(a.units, ue, uv, uc, up, a.label8 != nullptr, a.adjwgt == nullptr);
@@ -1951,33 +1638,25 @@ inline int rate_grid(gp_ctx *ctx, int64_t count, int per_block, int cap) {
   return grid_for(count, per_block, cap);
 }
 
-template <int G, int U>
-constexpr int group_nodes_per_block() { return kWarpsPerBlock * (32 / G) * U; }
+// One class of degree <= D; count < 0: unknown, the full grid.
+template <int MODE, int D, int LK>
+void launch_threads(gp_ctx *ctx, RateArgs a, int key, int count) {
+  if (count == 0) return;
+  a.key = key;
+  constexpr int NT = ThreadShape<D>::NT;
+  k_rate_thread<MODE, D, LK><<<rate_grid(ctx, count, NT, ctx->num_sms * ThreadShape<D>::PER_SM * 4), NT, 0,
+                               ctx->stream>>>(a);
+  GP_LAUNCH_CHECK();
+}
 
-// hcnt: the bucket sizes of this sub-round when the host knows them (empty
-// buckets are then not launched), else nullptr
+// hcnt: the bucket sizes of this sub-round when the host knows them (empty buckets are then not
+// launched), else nullptr
 template <int MODE, int LK>
-void launch_groups(gp_ctx *ctx, const RateArgs &a0, int bucket_key_base, const int *hcnt) {
-  const int cap = ctx->num_sms * 8;
-  RateArgs a = a0;
-  if (!hcnt || hcnt[0] > 0) {
-    a.key = bucket_key_base + 0;
-    k_rate_group<MODE, 8, 2, LK><<<rate_grid(ctx, hcnt ? hcnt[0] : -1, group_nodes_per_block<8, 2>(), cap),
-                                   kThreads, 0, ctx->stream>>>(a);
-    GP_LAUNCH_CHECK();
-  }
-  if (!hcnt || hcnt[1] > 0) {
-    a.key = bucket_key_base + 1;
-    k_rate_multi<MODE, 8, 2, 2, LK><<<rate_grid(ctx, hcnt ? hcnt[1] : -1, group_nodes_per_block<8, 2>(), cap),
-                                      kThreads, 0, ctx->stream>>>(a);
-    GP_LAUNCH_CHECK();
-  }
-  if (!hcnt || hcnt[2] > 0) {
-    a.key = bucket_key_base + 2;
-    k_rate_multi<MODE, 16, 2, 3, LK><<<rate_grid(ctx, hcnt ? hcnt[2] : -1, group_nodes_per_block<16, 3>(), cap),
-                                       kThreads, 0, ctx->stream>>>(a);
-    GP_LAUNCH_CHECK();
-  }
+void launch_groups(gp_ctx *ctx, const RateArgs &a, int base, const int *hcnt) {
+  launch_threads<MODE, 8, LK>(ctx, a, base + 0, hcnt ? hcnt[0] : -1);
+  launch_threads<MODE, 16, LK>(ctx, a, base + 1, hcnt ? hcnt[1] : -1);
+  launch_threads<MODE, 24, LK>(ctx, a, base + 2, hcnt ? hcnt[2] : -1);
+  launch_threads<MODE, 32, LK>(ctx, a, base + 3, hcnt ? hcnt[3] : -1);
 }
 
 template <int NT>
@@ -1990,26 +1669,25 @@ void launch_block(gp_ctx *ctx, const RateArgs &a, int maxdeg, int grid) {
   GP_LAUNCH_CHECK();
 }
 
-// nlabels: number of labels (chooses the narrow / dense group kernels when
-// a uint8 copy of the labels is present)
+// nlabels: number of labels
 template <int MODE>
 void launch_rate(gp_ctx *ctx, RateArgs a, int bucket_key_base, const RateTables &t, int64_t nlabels,
                  const int *hcnt) {
   const int cap = ctx->num_sms * 8;
-  if (MODE == RATE_LP && a.label8 && nlabels <= kDenseLabels) launch_groups<MODE, LK_DENSE>(ctx, a, bucket_key_base, hcnt);
-  else if (MODE == RATE_LP && a.label8) launch_groups<MODE, LK_NARROW>(ctx, a, bucket_key_base, hcnt);
+  if (MODE == RATE_LP && a.label8) launch_groups<MODE, LK_NARROW>(ctx, a, bucket_key_base, hcnt);
   else launch_groups<MODE, LK_WIDE>(ctx, a, bucket_key_base, hcnt);
-  if (!hcnt || hcnt[3] > 0) {
-    a.key = bucket_key_base + 3;
-    k_rate_medium<MODE><<<rate_grid(ctx, hcnt ? hcnt[3] : -1, kWarpsPerBlock, cap), kThreads, 0, ctx->stream>>>(a);
+  if (!hcnt || hcnt[kMediumBucket] > 0) {
+    a.key = bucket_key_base + kMediumBucket;
+    k_rate_medium<MODE><<<rate_grid(ctx, hcnt ? hcnt[kMediumBucket] : -1, kWarpsPerBlock, cap), kThreads, 0, ctx->stream>>>(a);
     GP_LAUNCH_CHECK();
   }
   const int hgrid = ctx->num_sms * 6;
-  for (int b = 4; b < kNumBuckets; b++) {
+  for (int q = 0; q < 4; q++) {  // the three block classes, the hubs
+    const int b = kMediumBucket + 1 + q;
     const int c = hcnt ? hcnt[b] : -1;
     if (c == 0) continue;
     a.key = bucket_key_base + b;
-    if (MODE == RATE_LP && t.hubs && (b == 7 || (b > 4 && t.dense))) {
+    if (MODE == RATE_LP && t.hubs && (q == 3 || (q > 0 && t.dense))) {
       HubArgs h{t.hub.get(), t.chunk0.get(), t.tchunk0.get(), t.tab.get(), t.hist.get(), (int)nlabels};
       k_hub_plan<<<1, 1024, 0, ctx->stream>>>(a, h);
       GP_LAUNCH_CHECK();
@@ -2024,9 +1702,9 @@ void launch_rate(gp_ctx *ctx, RateArgs a, int bucket_key_base, const RateTables 
         k_hub_table<true><<<hgrid, kThreads, 0, ctx->stream>>>(a, h);
         GP_LAUNCH_CHECK();
       }
-    } else if (MODE == RATE_LP && b < 7) {
-      if (b == 4) launch_block<256>(ctx, a, kBlockDeg0, rate_grid(ctx, c, 1, ctx->num_sms * 6));
-      else if (b == 5) launch_block<512>(ctx, a, kBlockDeg1, rate_grid(ctx, c, 1, ctx->num_sms * 3));
+    } else if (MODE == RATE_LP && q < 3) {
+      if (q == 0) launch_block<256>(ctx, a, kBlockDeg0, rate_grid(ctx, c, 1, ctx->num_sms * 6));
+      else if (q == 1) launch_block<512>(ctx, a, kBlockDeg1, rate_grid(ctx, c, 1, ctx->num_sms * 3));
       else launch_block<1024>(ctx, a, kHubDeg, rate_grid(ctx, c, 1, ctx->num_sms));
     } else {
       a.gkeys = t.gkeys.get();
@@ -2109,7 +1787,7 @@ LpResult lp_run(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *weight,
   GP_LAUNCH_CHECK();
   RateTables tables;
   make_tables(ctx, g, nlabels, tables);
-  unsigned long long *units_rate = ctx->d_units ? ctx->d_units + p.prof_rate * PROF_UNITS : nullptr;
+  unsigned long long *units_rate = ctx->profile && ctx->d_units ? ctx->d_units + p.prof_rate * PROF_UNITS : nullptr;
 
   TraceTimer trace(ctx);
   const int grid = ctx->num_sms * 8;
@@ -2146,7 +1824,7 @@ LpResult lp_run(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *weight,
       a.xadj = g.xadj; a.adjncy = g.adjncy; a.adjwgt = g.unit_w ? nullptr : g.adjwgt; a.vwgt = g.vwgt;
       a.label = label; a.weight = weight; a.list = list.get(); a.offs = offs.get();
       a.bound = p.bound; a.ktie = ktie; a.prop = prop.get(); a.incoming = incoming.get();
-      a.stop = &C->stop; a.units = units_rate; a.label8 = label8;
+      a.stop = &C->stop; a.units = units_rate; a.label8 = label8; a.m2 = g.m2;
       a.wlabels = label8 ? (int)nlabels : 0;
       a.dirty = dirty.get();
       if (use_dirty && r > 0) {  // in round 0 every node is still marked: the lists stay as they are
@@ -2342,7 +2020,7 @@ void favourites_bucketed(gp_ctx *ctx, const DevGraph &g, const int32_t *label, c
   RateArgs a{};
   a.xadj = g.xadj; a.adjncy = g.adjncy; a.adjwgt = g.unit_w ? nullptr : g.adjwgt; a.vwgt = g.vwgt;
   a.label = label; a.weight = nullptr; a.list = list.get(); a.offs = offs.get();
-  a.bound = U; a.ktie = kfav; a.fav_keys = keys.get(); a.stop = nullptr;
+  a.bound = U; a.ktie = kfav; a.fav_keys = keys.get(); a.stop = nullptr; a.m2 = g.m2;
   launch_rate<RATE_FAV>(ctx, a, 0, tables, 0, nullptr);
 }
 
