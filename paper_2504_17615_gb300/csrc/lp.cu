@@ -109,7 +109,7 @@ enum LabelKind { LK_WIDE = 0, LK_NARROW = 1 };
 template <int D>
 struct ThreadShape {
   static constexpr int NT = D <= 16 ? 256 : 128;
-  static constexpr int PER_SM = D <= 8 ? 5 : D <= 16 ? 3 : 4;  // blocks an SM holds: 51, 85 and 128 registers
+  static constexpr int PER_SM = D <= 8 ? 5 : D <= 16 ? 3 : D <= 24 ? 5 : 4;  // blocks an SM holds
 };
 
 // x[q] = base[st + q] for q < deg, 0 beyond.  vec: base is 16-byte aligned; then 16 bytes a load, from the
@@ -142,6 +142,13 @@ __device__ __forceinline__ void load_row(const int32_t *base, int st, int deg, i
 #pragma unroll
     for (int q = 0; q < D; q++) x[q] = q < deg ? __ldcs(base + st + q) : 0;
   }
+}
+
+// The largest label weight that leaves room for a node of weight cv under the bound (label weights are
+// below 2^31).
+__device__ __forceinline__ int room_of(int64_t bound, int cv) {
+  const int64_t r = bound - cv;
+  return r > 0x7FFFFFFF ? 0x7FFFFFFF : r < -1 ? -1 : (int)r;
 }
 
 template <int MODE, int D, int LK>
@@ -204,31 +211,39 @@ __global__ void __launch_bounds__(ThreadShape<D>::NT, ThreadShape<D>::PER_SM) k_
     if (a.dirty && live && stay) a.dirty[v] = 0;
     int best = -1;
     if (live && !stay) {
+      const int room = room_of(a.bound, cv);
       if (kSmemW) {
 #pragma unroll
         for (int q = 0; q < D; q++)
-          if (L[q] >= 0 && (int64_t)s_w[L[q]] + cv > a.bound) L[q] = -1;
+          if (L[q] >= 0 && s_w[L[q]] > room) L[q] = -1;
       }
       for (int pass = 0; pass < 2; pass++) {
-        int r = -1;
-#pragma unroll
-        for (int q = 0; q < D; q++) r = L[q] >= 0 && w[q] > r ? w[q] : r;
-        if (r < 0 || (MODE == RATE_LP && r <= own_r)) break;
-        unsigned hb = 0xFFFFFFFFu;
-        int lb = 0x7FFFFFFF;
+        int r = MODE == RATE_LP ? own_r : -1, lb = -1;
+        bool tie = false;
 #pragma unroll
         for (int q = 0; q < D; q++) {
-          if (L[q] < 0 || w[q] != r) continue;
-          const unsigned h = h32(a.ktie, (uint32_t)v, (uint32_t)L[q]);
-          if (h < hb || (h == hb && L[q] < lb)) { hb = h; lb = L[q]; }
+          if (L[q] < 0 || w[q] < r) continue;
+          tie = w[q] == r && lb >= 0;
+          if (w[q] > r) { r = w[q]; lb = L[q]; }
         }
-        if (MODE != RATE_LP || kSmemW || pass == 1 || (int64_t)a.weight[lb] + cv <= a.bound) {
+        if (lb < 0) break;
+        if (tie) {  // several labels of the best rating: the hashes decide
+          unsigned hb = 0xFFFFFFFFu;
+          lb = 0x7FFFFFFF;
+#pragma unroll
+          for (int q = 0; q < D; q++) {
+            if (L[q] < 0 || w[q] != r) continue;
+            const unsigned h = h32(a.ktie, (uint32_t)v, (uint32_t)L[q]);
+            if (h < hb || (h == hb && L[q] < lb)) { hb = h; lb = L[q]; }
+          }
+        }
+        if (MODE != RATE_LP || kSmemW || pass == 1 || a.weight[lb] <= room) {
           best = lb;
           break;
         }
 #pragma unroll
         for (int q = 0; q < D; q++)
-          if (L[q] >= 0 && (w[q] <= own_r || (int64_t)a.weight[L[q]] + cv > a.bound)) L[q] = -1;
+          if (L[q] >= 0 && (w[q] <= own_r || a.weight[L[q]] > room)) L[q] = -1;
       }
     }
     if (live) {
@@ -243,6 +258,104 @@ __global__ void __launch_bounds__(ThreadShape<D>::NT, ThreadShape<D>::PER_SM) k_
     }
   }
   add_units(a.units, ue, uv, uc, up, a.label8 != nullptr, a.adjwgt == nullptr);
+}
+
+// ------------- degree <= 32, unit weights, one-byte labels: counters per thread
+//
+// Refinement of an input with unit weights (level 1, the largest level): a rating is a count of at most
+// 32, so every thread counts its row in byte counters of its own, four to a word, in shared memory (word
+// [label / 4][thread]: no two lanes of a warp meet in a bank).  The pairs of k_rate_thread took 3100
+// instructions per 32 nodes of degree 17-24 and 106 registers (16 warps an SM, 80e9 entries/s); this takes
+// about a fifth of the instructions and half the registers.  BYTNUM
+
+template <int D>
+__global__ void __launch_bounds__(128, D <= 16 ? 8 : 6) k_rate_bytes(RateArgs a) {
+  constexpr int NT = 128;
+  extern __shared__ unsigned s_cnt[];  // (wlabels + 3) / 4 words a thread, then the label weights
+  if (a.stop && *a.stop) return;
+  const int words = (a.wlabels + 3) / 4;
+  int *s_w = reinterpret_cast<int *>(s_cnt + words * NT);
+  unsigned *cnt = s_cnt + threadIdx.x;
+  for (int t = 0; t < words; t++) cnt[t * NT] = 0;
+  for (int t = threadIdx.x; t < a.wlabels; t += NT) s_w[t] = a.weight[t];
+  __syncthreads();
+  const bool vec = ((uintptr_t)a.adjncy & 15) == 0;
+  const int begin = a.offs[a.key], end = list_end(a);
+  unsigned long long ue = 0, uv = 0, uc = 0, up = 0;
+  for (int i0 = begin + (int)(blockIdx.x * NT); i0 < end; i0 += (int)(gridDim.x * NT)) {
+    const int i = i0 + (int)threadIdx.x;
+    const int4 rec = i < end ? a.list[i] : make_int4(-1, 0, 0, 0);
+    const int v = rec.x, cv = rec.w;
+    const bool live = v >= 0 && !(a.dirty && !a.dirty[v]);
+    const int st = live ? rec.y : 0, deg = live ? rec.z : 0;
+    const int own = live ? (int)a.label8[v] : 0;
+    unsigned P[D / 4];  // the labels, four to a word
+    {
+      int u[D];
+      load_row<D>(a.adjncy, st, deg, a.m2, vec, u);
+#pragma unroll
+      for (int q = 0; q < D; q++) u[q] = q < deg ? (int)a.label8[u[q]] : 0;
+#pragma unroll
+      for (int q = 0; q < D / 4; q++)
+        P[q] = (unsigned)u[4 * q] | (unsigned)u[4 * q + 1] << 8 | (unsigned)u[4 * q + 2] << 16 | (unsigned)u[4 * q + 3] << 24;
+    }
+    auto label = [&](int q) -> int { return (int)((P[q / 4] >> (8 * (q & 3))) & 255u); };
+    const int dm = __reduce_max_sync(FULL, deg);
+#pragma unroll
+    for (int q = 0; q < D; q++) {
+      if (q >= dm) break;
+      const int L = label(q);
+      if (q < deg) cnt[(L >> 2) * NT] += 1u << ((L & 3) * 8);
+    }
+    const int own_r = (int)((cnt[(own >> 2) * NT] >> ((own & 3) * 8)) & 255u);
+    const int room = room_of(a.bound, cv);
+    int rall = 0, r = own_r, lb = -1, nc = 0;
+    bool tie = false;
+#pragma unroll
+    for (int q = 0; q < D; q++) {
+      if (q >= dm) break;
+      const int L = label(q);
+      if (q >= deg || L == own) continue;
+      const int c = (int)((cnt[(L >> 2) * NT] >> ((L & 3) * 8)) & 255u);
+      nc++;
+      rall = c > rall ? c : rall;
+      if (c > own_r && c >= r && s_w[L] <= room) {
+        if (c > r) { r = c; lb = L; tie = false; }
+        else if (L != lb) tie = true;
+      }
+    }
+    if (tie) {
+      unsigned hb = 0xFFFFFFFFu;
+      lb = 0x7FFFFFFF;
+#pragma unroll
+      for (int q = 0; q < D; q++) {
+        const int L = label(q);
+        if (q >= deg || L == own) continue;
+        const int c = (int)((cnt[(L >> 2) * NT] >> ((L & 3) * 8)) & 255u);
+        if (c != r || s_w[L] > room) continue;
+        const unsigned h = h32(a.ktie, (uint32_t)v, (uint32_t)L);
+        if (h < hb || (h == hb && L < lb)) { hb = h; lb = L; }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < D; q++) {
+      if (q >= dm) break;
+      if (q < deg) cnt[(label(q) >> 2) * NT] = 0;
+    }
+    if (a.dirty && live && rall <= own_r) a.dirty[v] = 0;
+    uc += nc;
+    if (live) {
+      ue += deg;
+      uv += 1;
+    }
+    if (lb >= 0) {
+      emit<RATE_LP>(a, i, v, lb, cv, own);
+      up += 1;
+    } else if (v >= 0) {
+      a.prop[i] = make_int2(-1, 0);
+    }
+  }
+  add_units(a.units, ue, uv, uc, up, true, true);
 }
 
 // --------------------------------------- degree <= 128: warp/node + table
@@ -1649,10 +1762,26 @@ void launch_threads(gp_ctx *ctx, RateArgs a, int key, int count) {
   GP_LAUNCH_CHECK();
 }
 
+template <int D>
+void launch_bytes(gp_ctx *ctx, RateArgs a, int key, int count) {
+  if (count == 0) return;
+  a.key = key;
+  const size_t smem = sizeof(int) * ((size_t)((a.wlabels + 3) / 4) * 128 + (size_t)a.wlabels);
+  k_rate_bytes<D><<<rate_grid(ctx, count, 128, ctx->num_sms * 16), 128, smem, ctx->stream>>>(a);
+  GP_LAUNCH_CHECK();
+}
+
 // hcnt: the bucket sizes of this sub-round when the host knows them (empty buckets are then not
 // launched), else nullptr
 template <int MODE, int LK>
 void launch_groups(gp_ctx *ctx, const RateArgs &a, int base, const int *hcnt) {
+  if (LK == LK_NARROW && a.adjwgt == nullptr && hcnt) {
+    launch_bytes<8>(ctx, a, base + 0, hcnt[0]);
+    launch_bytes<16>(ctx, a, base + 1, hcnt[1]);
+    launch_bytes<24>(ctx, a, base + 2, hcnt[2]);
+    launch_bytes<32>(ctx, a, base + 3, hcnt[3]);
+    return;
+  }
   launch_threads<MODE, 8, LK>(ctx, a, base + 0, hcnt ? hcnt[0] : -1);
   launch_threads<MODE, 16, LK>(ctx, a, base + 1, hcnt ? hcnt[1] : -1);
   launch_threads<MODE, 24, LK>(ctx, a, base + 2, hcnt ? hcnt[2] : -1);
