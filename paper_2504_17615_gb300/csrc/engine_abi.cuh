@@ -47,6 +47,43 @@ struct EArgs {
 };
 
 
+// The small end of one graph's hierarchy in one CTA (engine_tail.cu): the levels from `in` to the coarsest,
+// and back up from the coarsest graph's blocks to in's.
+struct EGraphRef {
+  const int32_t *xadj, *adjncy, *vwgt, *adjwgt;
+  int32_t n;
+  int64_t m2;
+};
+
+struct ELevel {
+  EGraphRef g;
+  int32_t *cmap;
+};
+
+struct TailOut {
+  int32_t status, levels;
+  EGraphRef coarsest;
+  int64_t arena_lo;  // end of the hierarchy in the arena
+  gp_level_stats st[GP_MAX_LEVELS];
+};
+
+struct TailArgs {
+  EGraphRef in;
+  int32_t level0, max_levels, k, pad;  // levels above `in`; levels left
+  int64_t U, Lmax;
+  uint64_t seed;
+  gp_config cfg;
+  unsigned char *arena;
+  int64_t arena_bytes;
+  ELevel *lv;  // GP_MAX_LEVELS + 1
+  TailOut *out;
+  int32_t *blk;  // up: the coarsest graph's blocks (refined in place when `in` is the coarsest)
+  int32_t *dst;  // up: in's blocks
+};
+
+void launch_tail_down(cudaStream_t stream, const TailArgs &a);
+void launch_tail_up(cudaStream_t stream, const TailArgs &a);
+
 // Launch entry points of the kernel instantiations (one translation unit each).
 struct Kernel {
   void (*launch)(int grid, size_t smem, cudaStream_t stream, const EArgs &a);

@@ -348,11 +348,7 @@ __device__ __forceinline__ int64_t lmax_of_dev(int64_t W, int k, int64_t eps_ppm
 
 // ---------------------------------------------------------------- context
 
-struct EGraph {
-  const int32_t *xadj, *adjncy, *vwgt, *adjwgt;
-  int32_t n;
-  int64_t m2;
-};
+using EGraph = EGraphRef;
 
 struct ECtx {
   Arena ar;
@@ -381,8 +377,9 @@ struct ELp {
 };
 
 struct ELpScr {
-  uint8_t *sr, *acc;
+  uint8_t *dirty, *acc;  // dirty: refinement, 0 = cannot move until a neighbour moves
   int32_t *pk, *list, *incoming, *P, *depw;
+  int32_t *off;          // starts of the round's lists by (sub-round, degree class)
   uint64_t *ovk, *ovk2, *dkey, *empt, *empt2;
   uint32_t *ovv, *ovv2, *ev, *ev2;
   int2 *gtab;   // the CTA's table for nodes of degree > kEWarpHeavy
@@ -390,6 +387,10 @@ struct ELpScr {
   int2 *wtab;   // per warp: a table of wbits^2 slots for nodes of degree in (kELight, kEWarpHeavy]
   int wbits;
 };
+
+constexpr int kEMaxLists = 254 * 5;  // sub-rounds x degree classes of a round (fits the CTA-wide table's keys)
+static_assert(kEMaxLists <= kEBlockSlots, "the list counters use the CTA-wide table");
+constexpr int kERankMax = 256;       // sets up to this size are ordered by counting, larger ones sorted
 
 // degree classes: lane groups of 8 / a warp with one or four entries per lane
 // (shared tables), a warp with a table in the arena, the CTA
@@ -404,7 +405,8 @@ __device__ int pow2_at_least(int64_t x) {
 }
 
 __device__ void lp_scratch(ECtx &c, int n, int64_t nlabels, int maxdeg, ELpScr &L) {
-  L.sr = c.ar.s<uint8_t>(n);
+  L.dirty = c.ar.s<uint8_t>(n);
+  L.off = c.ar.s<int32_t>(kEMaxLists + 1);
   L.acc = c.ar.s<uint8_t>(n);
   L.pk = c.ar.s<int32_t>(n);
   L.list = c.ar.s<int32_t>(n);
@@ -566,7 +568,8 @@ __device__ int rate_heavy(ECtx &c, const EGraph &g, const int32_t *label, const 
 // E entries per lane; LP mode proposes (pk, incoming), FAV mode writes fav.
 template <int G, int E, bool FAV>
 __device__ void rate_lanes(ECtx &c, const EGraph &g, const int32_t *list, int cnt, const int32_t *label,
-                           const int32_t *weight, int64_t bound, uint64_t ktie, int32_t *pk, int32_t *incoming) {
+                           const int32_t *weight, int64_t bound, uint64_t ktie, int32_t *pk, int32_t *incoming,
+                           uint8_t *dirty) {
   constexpr int NV = 32 / G;
   constexpr int TS = GroupTable<G, E>::TS;
   const int lane = (int)lane_id(), grp = lane / G, gl = lane % G;
@@ -575,7 +578,11 @@ __device__ void rate_lanes(ECtx &c, const EGraph &g, const int32_t *list, int cn
   int *tv = c.wtv + warp_idx() * kEWarpSlots + grp * TS;
   for (int i0 = warp_idx() * NV; i0 < cnt; i0 += nwarps() * NV) {
     const int i = i0 + grp;
-    const int v = i < cnt ? list[i] : -1;
+    int v = i < cnt ? list[i] : -1;
+    if (v >= 0 && dirty && !dirty[v]) {
+      if (gl == 0) pk[v] = -1;
+      v = -1;
+    }
     int st = 0, deg = 0, own = -2, cv = 0;
     if (v >= 0) {
       st = g.xadj[v];
@@ -588,6 +595,7 @@ __device__ void rate_lanes(ECtx &c, const EGraph &g, const int32_t *list, int cn
     const unsigned best = rate_group<G, E, FAV>(g.adjncy, g.adjwgt, label, nullptr, weight, nullptr, bound, ktie, v,
                                                 st, deg, own, cv, tk, tv, gmask, gl, false, nc, stable);
     if (gl == 0 && v >= 0) {
+      if (dirty && stable) dirty[v] = 0;
       if (FAV) {
         pk[v] = best == 0xFFFFFFFFu ? -1 : (int)best;
       } else {
@@ -603,11 +611,11 @@ __device__ void rate_lanes(ECtx &c, const EGraph &g, const int32_t *list, int cn
 template <bool FAV>
 __device__ void rate_all(ECtx &c, const EGraph &g, const int32_t *list, const int *off, const int32_t *label,
                          const int32_t *weight, int64_t bound, uint64_t ktie, int32_t *pk, int32_t *incoming,
-                         const ELpScr &L) {
+                         const ELpScr &L, uint8_t *dirty) {
   int2 *gtab = L.gtab;
-  rate_lanes<8, 1, FAV>(c, g, list + off[0], off[1] - off[0], label, weight, bound, ktie, pk, incoming);
-  rate_lanes<32, 1, FAV>(c, g, list + off[1], off[2] - off[1], label, weight, bound, ktie, pk, incoming);
-  rate_lanes<32, 4, FAV>(c, g, list + off[2], off[3] - off[2], label, weight, bound, ktie, pk, incoming);
+  rate_lanes<8, 1, FAV>(c, g, list + off[0], off[1] - off[0], label, weight, bound, ktie, pk, incoming, dirty);
+  rate_lanes<32, 1, FAV>(c, g, list + off[1], off[2] - off[1], label, weight, bound, ktie, pk, incoming, dirty);
+  rate_lanes<32, 4, FAV>(c, g, list + off[2], off[3] - off[2], label, weight, bound, ktie, pk, incoming, dirty);
   if (off[4] > off[3]) {
     int2 *tab = L.wtab + ((int64_t)warp_idx() << L.wbits);
     for (int i = off[3] + warp_idx(); i < off[4]; i += nwarps()) {
@@ -645,80 +653,143 @@ __device__ void e_lp(ECtx &c, const EGraph &g, int32_t *label, int32_t *weight, 
   fill_i32(L.incoming, nlabels, 0);
   fill_i32(L.depw, nlabels, 0);
   for (int64_t i = threadIdx.x; i < nlabels; i += blockDim.x) L.dkey[i] = 0;
+  uint8_t *dirty = P.count ? nullptr : L.dirty;
+  if (dirty)
+    for (int v = threadIdx.x; v < n; v += blockDim.x) dirty[v] = 1;
   __syncthreads();
   int subs = 0;
   int64_t total_moves = 0;
   bool stop = false;
   const int kbits = 32 + ebits(nlabels - 1);
+  const int nlists = P.S * 5;
   for (int r = 0; r < P.rounds && !stop; r++) {
     const uint64_t kact = stream_key(seed, P.tag_act, (uint32_t)P.level, (uint32_t)r);
     const uint64_t ktie = stream_key(seed, P.tag_tie, (uint32_t)P.level, (uint32_t)r);
     const uint64_t kprio = stream_key(seed, P.tag_prio, (uint32_t)P.level, (uint32_t)r);
+    if (P.count && ncl <= P.n_min) break;
+    if (P.dbg >= 0 && subs >= P.dbg) break;
+    // the round's nodes with neighbours by (sub-round, degree class): counted, then listed; the CTA-wide
+    // table holds the counters meanwhile and is left empty
+    int *hist = c.btk, *cursor = c.btv;
+    auto list_of = [&](int v) -> int {
+      const int deg = g.xadj[v + 1] - g.xadj[v];
+      return deg == 0 ? -1 : (int)(h32(kact, (uint32_t)v, 0) % (uint32_t)P.S) * 5 + deg_class(deg);
+    };
+    for (int t = threadIdx.x; t < nlists; t += blockDim.x) hist[t] = 0;
+    __syncthreads();
     for (int v = threadIdx.x; v < n; v += blockDim.x) {
-      const bool has = g.xadj[v + 1] > g.xadj[v];
-      L.sr[v] = has ? (uint8_t)(h32(kact, (uint32_t)v, 0) % (uint32_t)P.S) : (uint8_t)0xFF;
+      const int q = list_of(v);
+      if (q >= 0) atomicAdd(&hist[q], 1);
     }
+    __syncthreads();
+    if (warp_idx() == 0) {
+      int run = 0;
+      for (int b = 0; b < nlists; b += 32) {
+        const int t = b + (int)lane_id();
+        const int x = t < nlists ? hist[t] : 0;
+        int y = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int z = __shfl_up_sync(FULL, y, o);
+          if ((int)lane_id() >= o) y += z;
+        }
+        if (t < nlists) { L.off[t] = run + y - x; cursor[t] = run + y - x; }
+        run += __shfl_sync(FULL, y, 31);
+      }
+      if (lane_id() == 0) L.off[nlists] = run;
+    }
+    __syncthreads();
+    for (int v = threadIdx.x; v < n; v += blockDim.x) {
+      const int q = list_of(v);
+      if (q >= 0) L.list[atomicAdd(&cursor[q], 1)] = v;
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < nlists; t += blockDim.x) { hist[t] = -1; cursor[t] = 0; }
     __syncthreads();
     int64_t round_moves = 0;
     for (int sub = 0; sub < P.S; sub++) {
       if (P.count && ncl <= P.n_min) { stop = true; break; }
       if (P.dbg >= 0 && subs >= P.dbg) { stop = true; break; }
-      // the sub-round's nodes by degree class, each class in id order
-      auto cls = [&](int64_t v) -> int {
-        if (L.sr[v] != (uint8_t)sub) return -1;
-        return deg_class(g.xadj[v + 1] - g.xadj[v]);
-      };
-      blk_count_classes<5>(n, cls, 0, s);
       int off[6];
-      for (int q = 0; q < 5; q++) off[q] = s.off[q];
-      off[5] = s.off[4] + s.tot[4];
-      __syncthreads();
-      blk_classify<5>(n, cls, L.list, s);
-      const int nact = off[5];
+      for (int q = 0; q < 6; q++) off[q] = L.off[sub * 5 + q];
+      const int32_t *list = L.list + off[0];
+      const int nact = off[5] - off[0];
       // rate
-      rate_all<false>(c, g, L.list, off, label, weight, P.bound, ktie, L.pk, L.incoming, L);
+      rate_all<false>(c, g, L.list, off, label, weight, P.bound, ktie, L.pk, L.incoming, L, dirty);
       // decide: targets that take all their proposers
+      long long cnt = 0;  // proposals, and (<< 32) those of overflowing targets
       for (int i = threadIdx.x; i < nact; i += blockDim.x) {
-        const int v = L.list[i];
+        const int v = list[i];
         const int K = L.pk[v];
         if (K < 0) continue;
-        L.acc[v] = (int64_t)weight[K] + L.incoming[K] <= P.bound ? 1 : 2;
+        const bool fit = (int64_t)weight[K] + L.incoming[K] <= P.bound;
+        L.acc[v] = fit ? 1 : 2;
+        cnt += fit ? 1 : 1 + (1ll << 32);
       }
-      __syncthreads();
+      cnt = blk_sum(cnt, s);
+      const int nprop = (int)(cnt & 0xFFFFFFFF), nov = (int)(cnt >> 32);
+      if (nprop == 0) {  // nothing to order, cap or apply
+        subs++;
+        continue;
+      }
       // overflowing targets: proposers in (target, h32(PRIO), v) order, longest prefix
-      {
-        auto ovc = [&](int64_t v) -> int {
-          return (L.sr[v] == (uint8_t)sub && L.pk[v] >= 0 && L.acc[v] == 2) ? 0 : -1;
-        };
-        blk_count_classes<1>(n, ovc, 0, s);
-        const int nov = s.tot[0];
+      if (nov > 0) {
+        if (threadIdx.x == 0) s.cnt = 0;
         __syncthreads();
-        if (nov > 0) {
-          blk_classify<1>(n, ovc, reinterpret_cast<int32_t *>(L.ovv), s);
+        for (int i0 = 0; i0 < nact; i0 += blockDim.x) {
+          const int i = i0 + (int)threadIdx.x;
+          const int v = i < nact ? list[i] : -1;
+          const bool over = v >= 0 && L.pk[v] >= 0 && L.acc[v] == 2;
+          const int j = warp_append(&s.cnt, over);
+          if (over) {
+            L.ovv[j] = (uint32_t)v;
+            L.ovk[j] = ((uint64_t)(uint32_t)L.pk[v] << 32) | h32(kprio, (uint32_t)v, 0);
+          }
+        }
+        __syncthreads();
+        uint64_t *k1 = L.ovk, *k2 = L.ovk2;
+        uint32_t *v1 = L.ovv, *v2 = L.ovv2;
+        if (nov <= kERankMax) {  // placed by counting the proposers before each
           for (int i = threadIdx.x; i < nov; i += blockDim.x) {
-            const int v = (int)L.ovv[i];
-            L.ovk[i] = ((uint64_t)(uint32_t)L.pk[v] << 32) | h32(kprio, (uint32_t)v, 0);
+            const uint64_t k = k1[i];
+            const uint32_t v = v1[i];
+            int rank = 0;
+            for (int j = 0; j < nov; j++) rank += k1[j] < k || (k1[j] == k && v1[j] < v) ? 1 : 0;
+            k2[rank] = k;
+            v2[rank] = v;
           }
           __syncthreads();
-          uint64_t *k1 = L.ovk, *k2 = L.ovk2;
-          uint32_t *v1 = L.ovv, *v2 = L.ovv2;
+          k1 = L.ovk2;
+          v1 = L.ovv2;
+        } else {
           blk_sort(k1, v1, k2, v2, nov, kbits, c.btk, s);
-          blk_scan<int>(
-              nov, [&](int64_t i) { return g.vwgt[v1[i]]; }, [&](int64_t i, int p) { L.P[i] = p + g.vwgt[v1[i]]; },
-              s);
-          for (int i = threadIdx.x; i < nov; i += blockDim.x) {
-            const int K = (int)(k1[i] >> 32);
-            const int st = lower_bound_u64(k1, nov, (uint64_t)(uint32_t)K << 32);
-            const int pre = L.P[i] - (st > 0 ? L.P[st - 1] : 0);
-            L.acc[v1[i]] = (int64_t)weight[K] + pre <= P.bound ? 1 : 0;
+          for (int i = threadIdx.x; i < nov; i += blockDim.x) {  // runs of equal keys by node
+            if ((i > 0 && k1[i - 1] == k1[i]) || i + 1 >= nov || k1[i + 1] != k1[i]) continue;
+            for (int a = i + 1; a < nov && k1[a] == k1[i]; a++) {
+              const uint32_t x = v1[a];
+              int b = a - 1;
+              while (b >= i && v1[b] > x) { v1[b + 1] = v1[b]; b--; }
+              v1[b + 1] = x;
+            }
           }
           __syncthreads();
         }
+        blk_scan<int>(
+            nov, [&](int64_t i) { return g.vwgt[v1[i]]; }, [&](int64_t i, int p) { L.P[i] = p + g.vwgt[v1[i]]; },
+            s);
+        for (int i = threadIdx.x; i < nov; i += blockDim.x) {
+          const int K = (int)(k1[i] >> 32);
+          const int st = lower_bound_u64(k1, nov, (uint64_t)(uint32_t)K << 32);
+          const int pre = L.P[i] - (st > 0 ? L.P[st - 1] : 0);
+          L.acc[v1[i]] = (int64_t)weight[K] + pre <= P.bound ? 1 : 0;
+        }
+        __syncthreads();
       }
       // the 2.5x cap (R8): at most D = ncl - n_min clusters may be emptied
-      if (P.count) {
+      const int64_t D = ncl - P.n_min;
+      if (P.count && nprop > D) {
         for (int i = threadIdx.x; i < nact; i += blockDim.x) {
-          const int v = L.list[i];
+          const int v = list[i];
           if (L.pk[v] < 0 || L.acc[v] != 1) continue;
           const int own = label[v];
           atomicAdd(&L.depw[own], g.vwgt[v]);
@@ -732,7 +803,7 @@ __device__ void e_lp(ECtx &c, const EGraph &g, int32_t *label, int32_t *weight, 
           bool e = false;
           uint64_t kv = 0;
           if (i < nact) {
-            const int v = L.list[i];
+            const int v = list[i];
             if (L.pk[v] >= 0 && L.acc[v] == 1) {
               const int own = label[v];
               kv = ((uint64_t)h32(kprio, (uint32_t)v, 0) << 32) | (uint32_t)v;
@@ -744,17 +815,29 @@ __device__ void e_lp(ECtx &c, const EGraph &g, int32_t *label, int32_t *weight, 
         }
         __syncthreads();
         const int64_t E = s.cnt;
-        const int64_t D = ncl - P.n_min;
         __syncthreads();
         if (E > D) {
-          for (int i = threadIdx.x; i < E; i += blockDim.x) L.ev[i] = 0;
-          __syncthreads();
-          uint64_t *k1 = L.empt, *k2 = L.empt2;
-          uint32_t *v1 = L.ev, *v2 = L.ev2;
-          blk_sort(k1, v1, k2, v2, (int)E, 64, c.btk, s);
-          const uint64_t cutoff = k1[D];
+          uint64_t cutoff;
+          if (E <= kERankMax) {  // keys are distinct
+            for (int i = threadIdx.x; i < E; i += blockDim.x) {
+              const uint64_t k = L.empt[i];
+              int below = 0;
+              for (int j = 0; j < E; j++) below += L.empt[j] < k ? 1 : 0;
+              if (below == D) s.u[0] = k;
+            }
+            __syncthreads();
+            cutoff = s.u[0];
+            __syncthreads();
+          } else {
+            for (int i = threadIdx.x; i < E; i += blockDim.x) L.ev[i] = 0;
+            __syncthreads();
+            uint64_t *k1 = L.empt, *k2 = L.empt2;
+            uint32_t *v1 = L.ev, *v2 = L.ev2;
+            blk_sort(k1, v1, k2, v2, (int)E, 64, c.btk, s);
+            cutoff = k1[D];
+          }
           for (int i = threadIdx.x; i < nact; i += blockDim.x) {
-            const int v = L.list[i];
+            const int v = list[i];
             if (L.pk[v] < 0 || L.acc[v] != 1) continue;
             const uint64_t kv = ((uint64_t)h32(kprio, (uint32_t)v, 0) << 32) | (uint32_t)v;
             if (kv >= cutoff) L.acc[v] = 0;
@@ -762,7 +845,7 @@ __device__ void e_lp(ECtx &c, const EGraph &g, int32_t *label, int32_t *weight, 
           __syncthreads();
         }
         for (int i = threadIdx.x; i < nact; i += blockDim.x) {
-          const int v = L.list[i];
+          const int v = list[i];
           if (L.pk[v] < 0) continue;
           const int own = label[v];
           L.depw[own] = 0;
@@ -773,7 +856,7 @@ __device__ void e_lp(ECtx &c, const EGraph &g, int32_t *label, int32_t *weight, 
       // apply; the cluster count follows the weight transitions 0 <-> non-0
       long long moved = 0, delta = 0;
       for (int i = threadIdx.x; i < nact; i += blockDim.x) {
-        const int v = L.list[i];
+        const int v = list[i];
         const int K = L.pk[v];
         if (K < 0) continue;
         if (L.acc[v] == 1) {
@@ -785,8 +868,18 @@ __device__ void e_lp(ECtx &c, const EGraph &g, int32_t *label, int32_t *weight, 
         }
         L.incoming[K] = 0;
       }
-      moved = blk_sum(moved, s);
-      delta = blk_sum(delta, s);
+      if (dirty) {  // every applied move marks its node and the node's neighbours, a warp per move
+        for (int i = warp_idx(); i < nact; i += nwarps()) {
+          const int v = list[i];
+          if (L.pk[v] < 0 || L.acc[v] != 1) continue;
+          if (lane_id() == 0) dirty[v] = 1;
+          for (int e = g.xadj[v] + (int)lane_id(); e < g.xadj[v + 1]; e += 32) dirty[g.adjncy[e]] = 1;
+        }
+      }
+      // |delta| <= 2 moved, so one sum carries both
+      const long long both = blk_sum(moved + (delta << 32), s);
+      moved = both & 0xFFFFFFFF;
+      delta = (both - moved) >> 32;
       if (P.count) ncl += delta;
       round_moves += moved;
       subs++;
@@ -899,7 +992,7 @@ __device__ void e_cluster(ECtx &c, const EGraph &g, int64_t U, int level, uint64
     __syncthreads();
     blk_classify<5>(n, cand, L.list, s);
     const uint64_t kfav = stream_key(seed, TAG_FAV, (uint32_t)level, 0);
-    rate_all<true>(c, g, L.list, off, label, cw, U, kfav, fav, nullptr, L);
+    rate_all<true>(c, g, L.list, off, label, cw, U, kfav, fav, nullptr, L, nullptr);
     // (fav, v) keys of the candidates with a favourite (all of them: a singleton's
     // neighbours lie in other clusters), sorted
     auto hasfav = [&](int64_t v) -> int { return (cand(v) >= 0 && fav[v] >= 0) ? 0 : -1; };
@@ -1696,10 +1789,70 @@ __device__ int e_maxdeg(ECtx &c, const EGraph &g) {
 
 // ------------------------------------------------------------ one item
 
-struct ELevel {
-  EGraph g;
-  int32_t *cmap;
-};
+// The level loop of Alg. 1 from lv[0].g (level level0 of its hierarchy: levels are numbered from there) to
+// the coarsest graph, in lv; false when the arena is too small.
+__device__ bool e_coarsen(ECtx &c, int64_t U, int k, uint64_t seed, int level0, int maxl, ELevel *lv,
+                          gp_level_stats *lvo, int &levels) {
+  const gp_config &cfg = *c.cfg;
+  int L = 0;
+  while ((int64_t)lv[L].g.n > (int64_t)cfg.coarsest_factor * k && L < maxl) {
+    const EGraph cur = lv[L].g;
+    const int64_t hmark = c.ar.lo;
+    int32_t *cmap = c.ar.h<int32_t>(cur.n);
+    const int64_t smark = c.ar.hi;
+    int32_t *label = c.ar.s<int32_t>(cur.n);
+    if (c.ar.fail) return false;
+    const int maxdeg = e_maxdeg(c, cur);
+    ECluster cl{};
+    e_cluster(c, cur, U, level0 + L + 1, seed, label, maxdeg, cl);
+    phase(c, EP_CLUSTER);
+    if (c.ar.fail) return false;
+    const int nc = e_relabel(c, cur.n, label, cmap);
+    c.ar.hi = smark;
+    phase(c, EP_RELABEL);
+    if (c.ar.fail) return false;
+    EGraph gc{};
+    e_contract(c, cur, cmap, nc, gc);
+    phase(c, EP_CONTRACT);
+    if (c.ar.fail) return false;
+    gp_level_stats ls{};
+    ls.n = cur.n;
+    ls.n_next = nc;
+    ls.m = cur.m2 / 2;
+    ls.m_coarse = gc.m2 / 2;
+    ls.lp_subrounds = cl.subs;
+    ls.lp_moves = cl.moves;
+    ls.clusters_lp = cl.ncl_lp;
+    ls.clusters_2hop = cl.ncl_2hop;
+    ls.clusters_final = cl.ncl_final;
+    if ((int64_t)nc * cfg.min_shrink_num > (int64_t)cur.n * cfg.min_shrink_den) {
+      c.ar.lo = hmark;
+      break;
+    }
+    const int64_t a = (int64_t)muldiv_u64((uint64_t)ls.m, (uint64_t)cfg.tau_e_num, (uint64_t)cfg.tau_e_den);
+    const int64_t b = (int64_t)muldiv_u64((uint64_t)ls.m * (uint64_t)nc, (uint64_t)cfg.tau_d_num,
+                                          (uint64_t)cfg.tau_d_den * (uint64_t)cur.n);
+    ls.m_hat = a < b ? a : b;
+    ls.triggered = cfg.sparsifier != GP_SPARSIFY_NONE &&
+                   (uint64_t)ls.m_coarse * (uint64_t)cfg.rho_den > (uint64_t)cfg.rho_num * (uint64_t)ls.m_hat;
+    if (ls.triggered) {
+      e_sparsify(c, gc, ls.m_hat, level0 + L + 2, seed, cfg.sparsifier, ls);
+      phase(c, EP_SPARSIFY);
+      if (c.ar.fail) return false;
+    }
+    ls.m_next = gc.m2 / 2;
+    if (threadIdx.x == 0) {
+      if (lvo) lvo[L] = ls;
+      lv[L].cmap = cmap;
+      lv[L + 1].g = gc;
+      lv[L + 1].cmap = nullptr;
+    }
+    L++;
+    __syncthreads();
+  }
+  levels = L;
+  return true;
+}
 
 __device__ void e_item(ECtx &c, const EItem &it, EOut &o, gp_level_stats *lvo, ELevel *lv) {
   const gp_config &cfg = *c.cfg;
@@ -1732,61 +1885,7 @@ __device__ void e_item(ECtx &c, const EItem &it, EOut &o, gp_level_stats *lvo, E
   __syncthreads();
   int L = 0;
   const int maxl = cfg.max_levels < GP_MAX_LEVELS ? cfg.max_levels : GP_MAX_LEVELS;
-  while ((int64_t)lv[L].g.n > (int64_t)cfg.coarsest_factor * k && L < maxl) {
-    const EGraph cur = lv[L].g;
-    const int64_t hmark = c.ar.lo;
-    int32_t *cmap = c.ar.h<int32_t>(cur.n);
-    const int64_t smark = c.ar.hi;
-    int32_t *label = c.ar.s<int32_t>(cur.n);
-    if (c.ar.fail) { o.status = kERetry; return; }
-    const int maxdeg = e_maxdeg(c, cur);
-    ECluster cl{};
-    e_cluster(c, cur, U, L + 1, it.seed, label, maxdeg, cl);
-    phase(c, EP_CLUSTER);
-    if (c.ar.fail) { o.status = kERetry; return; }
-    const int nc = e_relabel(c, cur.n, label, cmap);
-    c.ar.hi = smark;
-    phase(c, EP_RELABEL);
-    if (c.ar.fail) { o.status = kERetry; return; }
-    EGraph gc{};
-    e_contract(c, cur, cmap, nc, gc);
-    phase(c, EP_CONTRACT);
-    if (c.ar.fail) { o.status = kERetry; return; }
-    gp_level_stats ls{};
-    ls.n = cur.n;
-    ls.n_next = nc;
-    ls.m = cur.m2 / 2;
-    ls.m_coarse = gc.m2 / 2;
-    ls.lp_subrounds = cl.subs;
-    ls.lp_moves = cl.moves;
-    ls.clusters_lp = cl.ncl_lp;
-    ls.clusters_2hop = cl.ncl_2hop;
-    ls.clusters_final = cl.ncl_final;
-    if ((int64_t)nc * cfg.min_shrink_num > (int64_t)cur.n * cfg.min_shrink_den) {
-      c.ar.lo = hmark;
-      break;
-    }
-    const int64_t a = (int64_t)muldiv_u64((uint64_t)ls.m, (uint64_t)cfg.tau_e_num, (uint64_t)cfg.tau_e_den);
-    const int64_t b = (int64_t)muldiv_u64((uint64_t)ls.m * (uint64_t)nc, (uint64_t)cfg.tau_d_num,
-                                          (uint64_t)cfg.tau_d_den * (uint64_t)cur.n);
-    ls.m_hat = a < b ? a : b;
-    ls.triggered = cfg.sparsifier != GP_SPARSIFY_NONE &&
-                   (uint64_t)ls.m_coarse * (uint64_t)cfg.rho_den > (uint64_t)cfg.rho_num * (uint64_t)ls.m_hat;
-    if (ls.triggered) {
-      e_sparsify(c, gc, ls.m_hat, L + 2, it.seed, cfg.sparsifier, ls);
-      phase(c, EP_SPARSIFY);
-      if (c.ar.fail) { o.status = kERetry; return; }
-    }
-    ls.m_next = gc.m2 / 2;
-    if (threadIdx.x == 0) {
-      if (lvo) lvo[L] = ls;
-      lv[L].cmap = cmap;
-      lv[L + 1].g = gc;
-      lv[L + 1].cmap = nullptr;
-    }
-    L++;
-    __syncthreads();
-  }
+  if (!e_coarsen(c, U, k, it.seed, 0, maxl, lv, lvo, L)) { o.status = kERetry; return; }
   o.levels = L;
   o.n_coarsest = lv[L].g.n;
   // buffers of the uncoarsening: block ids per level (two alternating), LP scratch for the largest level
@@ -1827,17 +1926,12 @@ __device__ void e_item(ECtx &c, const EItem &it, EOut &o, gp_level_stats *lvo, E
   o.status = GP_OK;
 }
 
-template <int NT>
-__global__ void __launch_bounds__(NT) k_engine(EArgs a) {
-  extern __shared__ __align__(16) unsigned char esm[];
-  __shared__ ESmem s;
-  __shared__ ELevel lv[GP_MAX_LEVELS + 1];
-  __shared__ int s_item;
+// The context's shared tables, carved out of esm and emptied.
+__device__ void e_context(ECtx &c, unsigned char *esm, ESmem &s, const gp_config &cfg, bool prof) {
   const int nw = nwarps();
-  ECtx c;
   c.s = &s;
-  c.cfg = &a.cfg;
-  c.prof = a.profile != 0;
+  c.cfg = &cfg;
+  c.prof = prof;
   c.wtk = reinterpret_cast<int *>(esm);
   c.wtv = c.wtk + nw * kEWarpSlots;
   c.btk = c.wtv + nw * kEWarpSlots;
@@ -1845,6 +1939,16 @@ __global__ void __launch_bounds__(NT) k_engine(EArgs a) {
   for (int t = threadIdx.x; t < nw * kEWarpSlots; t += blockDim.x) { c.wtk[t] = -1; c.wtv[t] = 0; }
   for (int t = threadIdx.x; t < kEBlockSlots; t += blockDim.x) { c.btk[t] = -1; c.btv[t] = 0; }
   __syncthreads();
+}
+
+template <int NT>
+__global__ void __launch_bounds__(NT) k_engine(EArgs a) {
+  extern __shared__ __align__(16) unsigned char esm[];
+  __shared__ ESmem s;
+  __shared__ ELevel lv[GP_MAX_LEVELS + 1];
+  __shared__ int s_item;
+  ECtx c;
+  e_context(c, esm, s, a.cfg, a.profile != 0);
   for (;;) {
     if (threadIdx.x == 0) s_item = atomicAdd(a.head, 1);
     __syncthreads();

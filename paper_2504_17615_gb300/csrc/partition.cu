@@ -1,5 +1,6 @@
 // partition.cu -- input validation, projection, cut, LP refinement and the
 // multilevel driver (Sec. 2, Alg. 1, Sec. 4.3).
+#include "engine_abi.cuh"
 #include "lp.cuh"
 
 #include <memory>
@@ -341,6 +342,76 @@ struct Timer {
   }
 };
 
+// Graphs of at most kTailNodes nodes and kTailEntries entries go through the rest of their hierarchy in
+// one CTA (engine_tail.cu), unless the configuration asks for what that code does not do, or for no
+// persistent launches.
+#ifndef GP_TAIL_NODES
+#define GP_TAIL_NODES 4608
+#endif
+#ifndef GP_TAIL_ENTRIES
+#define GP_TAIL_ENTRIES 49152
+#endif
+constexpr int32_t kTailNodes = GP_TAIL_NODES;
+constexpr int64_t kTailEntries = GP_TAIL_ENTRIES;
+
+bool tail_takes(const gp_config &cfg, const DevGraph &g) {
+  return g.n <= kTailNodes && g.m2 <= kTailEntries && g.n <= cfg.small_lp_nodes && cfg.lp_subrounds <= 64 &&
+         engine_config_ok(cfg);
+}
+
+// The tail of a hierarchy: its buffers from the way down to the way up.
+struct Tail {
+  DBuf<unsigned char> arena;
+  DBuf<eng::ELevel> lv;
+  DBuf<eng::TailOut> out;
+  eng::TailArgs a{};
+  DevGraph coarsest;  // a view of arena memory (or of the graph itself)
+  int levels = 0;
+};
+
+// The levels below g (level `level` of its hierarchy); false: the arena was too small, nothing is kept.
+bool tail_down(gp_ctx *ctx, const DevGraph &g, int level, int32_t k, int64_t U, int64_t Lmax, uint64_t seed,
+               const gp_config &cfg, gp_level_stats *st, Tail &t) {
+  ProfScope ps(ctx, PROF_LP_SMALL);
+  const int64_t bytes = 160 * (int64_t)g.n + 40 * g.m2 + 64 * (int64_t)k + ((int64_t)4 << 20);
+  t.arena.reset(ctx, (size_t)bytes);
+  t.lv.reset(ctx, GP_MAX_LEVELS + 1);
+  t.out.reset(ctx, 1);
+  t.a.in = eng::EGraphRef{g.xadj, g.adjncy, g.vwgt, g.adjwgt, g.n, g.m2};
+  t.a.level0 = level;
+  t.a.max_levels = std::min<int>(cfg.max_levels, GP_MAX_LEVELS) - level;
+  t.a.k = k;
+  t.a.U = U;
+  t.a.Lmax = Lmax;
+  t.a.seed = seed;
+  t.a.cfg = cfg;
+  t.a.arena = t.arena.get();
+  t.a.arena_bytes = bytes;
+  t.a.lv = t.lv.get();
+  t.a.out = t.out.get();
+  eng::launch_tail_down(ctx->stream, t.a);
+  eng::TailOut h;
+  static_assert(sizeof(h) <= 4096 * sizeof(int64_t), "read through the staging area");
+  read_back(ctx, t.out.get(), sizeof(h), &h);
+  if (h.status != GP_OK) return false;
+  t.levels = h.levels;
+  for (int i = 0; i < h.levels; i++) st[i] = h.st[i];
+  gp_graph v;
+  v.n = h.coarsest.n; v.m2 = h.coarsest.m2;
+  v.xadj = const_cast<int32_t *>(h.coarsest.xadj); v.adjncy = const_cast<int32_t *>(h.coarsest.adjncy);
+  v.vwgt = const_cast<int32_t *>(h.coarsest.vwgt); v.adjwgt = const_cast<int32_t *>(h.coarsest.adjwgt);
+  t.coarsest = DevGraph::wrap(v);
+  return true;
+}
+
+// Refines the coarsest graph's blocks and carries them up to g's (dst).
+void tail_up(gp_ctx *ctx, Tail &t, int32_t *blk, int32_t *dst) {
+  ProfScope ps(ctx, PROF_REF_SMALL);
+  t.a.blk = blk;
+  t.a.dst = dst;
+  eng::launch_tail_up(ctx->stream, t.a);
+}
+
 void partition_impl(gp_ctx *ctx, const DevGraph &input, int32_t k, double eps, uint64_t seed,
                     const gp_config &cfg, int32_t *blocks, int64_t *cut_out, gp_partition_stats *st) {
   GP_REQUIRE(k >= 1, GP_ERR_INVALID, "k must be >= 1");
@@ -377,8 +448,15 @@ void partition_impl(gp_ctx *ctx, const DevGraph &input, int32_t k, double eps, u
   G.push_back(std::make_unique<DevGraph>(DevGraph::wrap(input.view())));
   G[0]->unit_w = tot.unit_w;
   int L = 0;
+  std::unique_ptr<Tail> tail;
   while ((int64_t)G[L]->n > (int64_t)cfg.coarsest_factor * k && L < cfg.max_levels) {
     const DevGraph &cur = *G[L];
+    if (tail_takes(cfg, cur)) {
+      NvtxRange r("tail", L + 1);
+      tail = std::make_unique<Tail>();
+      if (tail_down(ctx, cur, L, k, U, Lmax, seed, cfg, S.lv + L, *tail)) break;
+      tail.reset();
+    }
     DBuf<int32_t> cmap(ctx, (size_t)cur.n);
     LevelOut lo;
     {
@@ -413,19 +491,25 @@ void partition_impl(gp_ctx *ctx, const DevGraph &input, int32_t k, double eps, u
     G.push_back(std::move(Gc));
     L++;
   }
-  S.levels = L;
-  S.n_coarsest = G[L]->n;
+  S.levels = L + (tail ? tail->levels : 0);
+  const DevGraph &coarsest = tail ? tail->coarsest : *G[L];
+  S.n_coarsest = coarsest.n;
   tm.mark(1);
   // initial partition of the coarsest graph
-  DBuf<int32_t> blk(ctx, (size_t)G[L]->n);
+  DBuf<int32_t> blk(ctx, (size_t)coarsest.n);
   {
     NvtxRange r("initial");
-    initial_partition(ctx, *G[L], k, eps_ppm, seed, cfg.ip_trials, blk.get());
-    cut_and_weights(ctx, *G[L], blk.get(), k, &S.ip_cut, nullptr);
-    S.rebalance_moves = rebalance_blocks(ctx, *G[L], k, Lmax, blk.get());
+    initial_partition(ctx, coarsest, k, eps_ppm, seed, cfg.ip_trials, blk.get());
+    cut_and_weights(ctx, coarsest, blk.get(), k, &S.ip_cut, nullptr);
+    S.rebalance_moves = rebalance_blocks(ctx, coarsest, k, Lmax, blk.get());
   }
   tm.mark(2);
-  {
+  if (tail) {
+    NvtxRange r("tail refine", L + 1);
+    DBuf<int32_t> fine(ctx, (size_t)G[L]->n);
+    tail_up(ctx, *tail, blk.get(), fine.get());
+    blk = std::move(fine);
+  } else {
     NvtxRange r("refine", L + 1);
     refine_blocks(ctx, *G[L], k, Lmax, L + 1, seed, cfg, blk.get());
   }
