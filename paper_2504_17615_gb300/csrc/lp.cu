@@ -16,6 +16,7 @@
 //            labels of positive weight) are counted; the stop flag is raised
 //            when that count reaches n_min or a round moved nothing.
 #include "lp.cuh"
+#include "lp_rate.cuh"
 
 #include <chrono>
 
@@ -112,45 +113,6 @@ struct ThreadShape {
   static constexpr int PER_SM = D <= 8 ? 5 : D <= 16 ? 3 : D <= 24 ? 5 : 4;  // blocks an SM holds
 };
 
-// x[q] = base[st + q] for q < deg, 0 beyond.  vec: base is 16-byte aligned; then 16 bytes a load, from the
-// last boundary before st, moved into place by two selects a word (lim: words that may be read).
-template <int D>
-__device__ __forceinline__ void load_row(const int32_t *base, int st, int deg, int64_t lim, bool vec, int (&x)[D]) {
-  if (vec) {
-    int w[D + 4];
-    const int off = st & 3, s0 = st - off;
-#pragma unroll
-    for (int g = 0; g < (D + 4) / 4; g++) {
-      const int idx = s0 + 4 * g;
-      int4 y = make_int4(0, 0, 0, 0);
-      if (idx < st + deg) {
-        if ((int64_t)idx + 4 <= lim) {
-          y = __ldcs(reinterpret_cast<const int4 *>(base + idx));
-        } else {  // the array's last words
-          y.x = base[idx];
-          if ((int64_t)idx + 1 < lim) y.y = base[idx + 1];
-          if ((int64_t)idx + 2 < lim) y.z = base[idx + 2];
-        }
-      }
-      w[4 * g] = y.x; w[4 * g + 1] = y.y; w[4 * g + 2] = y.z; w[4 * g + 3] = y.w;
-    }
-#pragma unroll
-    for (int q = 0; q < D + 2; q++) w[q] = (off & 1) ? w[q + 1] : w[q];
-#pragma unroll
-    for (int q = 0; q < D; q++) x[q] = (off & 2) ? w[q + 2] : w[q];
-  } else {
-#pragma unroll
-    for (int q = 0; q < D; q++) x[q] = q < deg ? __ldcs(base + st + q) : 0;
-  }
-}
-
-// The largest label weight that leaves room for a node of weight cv under the bound (label weights are
-// below 2^31).
-__device__ __forceinline__ int room_of(int64_t bound, int cv) {
-  const int64_t r = bound - cv;
-  return r > 0x7FFFFFFF ? 0x7FFFFFFF : r < -1 ? -1 : (int)r;
-}
-
 template <int MODE, int D, int LK>
 __global__ void __launch_bounds__(ThreadShape<D>::NT, ThreadShape<D>::PER_SM) k_rate_thread(RateArgs a) {
   constexpr int NT = ThreadShape<D>::NT;
@@ -183,69 +145,12 @@ __global__ void __launch_bounds__(ThreadShape<D>::NT, ThreadShape<D>::PER_SM) k_
 #pragma unroll
       for (int q = 0; q < D; q++) w[q] = 1;
     }
-    // equal labels: the first of them takes the sum, the others drop out (-1)
-    const int dm = __reduce_max_sync(FULL, deg);
-#pragma unroll
-    for (int p = 0; p < D - 1; p++) {
-      if (p >= dm) break;
-#pragma unroll
-      for (int b = p / 8 * 8; b < D; b += 8) {
-        if (b >= dm) break;
-#pragma unroll
-        for (int q = b; q < b + 8; q++) {
-          if (q <= p) continue;
-          if (L[q] == L[p]) { w[p] += w[q]; L[q] = -1; }
-        }
-      }
-    }
-    int own_r = 0, rall = 0, nc = 0;
-#pragma unroll
-    for (int q = 0; q < D; q++) {
-      if (L[q] == own) { own_r = w[q]; L[q] = -1; }
-      if (L[q] >= 0) { rall = w[q] > rall ? w[q] : rall; nc++; }
-    }
+    bool stay;
+    int nc;
+    const int best = choose_row<D, MODE == RATE_FAV>(L, w, deg, live, v, own, cv, a.bound, a.ktie,
+                                                     kSmemW ? s_w : nullptr, a.weight, stay, nc);
     uc += nc;
-    // no label rated above the own one, admissible or not: the node proposes nothing, and in refinement it
-    // stays clean until a neighbour moves
-    const bool stay = MODE == RATE_LP && rall <= own_r;
     if (a.dirty && live && stay) a.dirty[v] = 0;
-    int best = -1;
-    if (live && !stay) {
-      const int room = room_of(a.bound, cv);
-      if (kSmemW) {
-#pragma unroll
-        for (int q = 0; q < D; q++)
-          if (L[q] >= 0 && s_w[L[q]] > room) L[q] = -1;
-      }
-      for (int pass = 0; pass < 2; pass++) {
-        int r = MODE == RATE_LP ? own_r : -1, lb = -1;
-        bool tie = false;
-#pragma unroll
-        for (int q = 0; q < D; q++) {
-          if (L[q] < 0 || w[q] < r) continue;
-          tie = w[q] == r && lb >= 0;
-          if (w[q] > r) { r = w[q]; lb = L[q]; }
-        }
-        if (lb < 0) break;
-        if (tie) {  // several labels of the best rating: the hashes decide
-          unsigned hb = 0xFFFFFFFFu;
-          lb = 0x7FFFFFFF;
-#pragma unroll
-          for (int q = 0; q < D; q++) {
-            if (L[q] < 0 || w[q] != r) continue;
-            const unsigned h = h32(a.ktie, (uint32_t)v, (uint32_t)L[q]);
-            if (h < hb || (h == hb && L[q] < lb)) { hb = h; lb = L[q]; }
-          }
-        }
-        if (MODE != RATE_LP || kSmemW || pass == 1 || a.weight[lb] <= room) {
-          best = lb;
-          break;
-        }
-#pragma unroll
-        for (int q = 0; q < D; q++)
-          if (L[q] >= 0 && (w[q] <= own_r || a.weight[L[q]] > room)) L[q] = -1;
-      }
-    }
     if (live) {
       ue += deg;
       uv += 1;

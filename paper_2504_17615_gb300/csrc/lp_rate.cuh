@@ -13,6 +13,9 @@
 // weight is read, and the remaining candidates' weights only when it does not
 // fit.  In favourite mode (2-hop clustering, Sec. 4.1) the bound and the own
 // label's rating play no part.
+//
+// choose_row is the same choice by one thread that holds a whole row of at
+// most D labels and weights in registers.
 #pragma once
 #include "gp_internal.cuh"
 
@@ -48,7 +51,7 @@ __device__ __forceinline__ unsigned rate_group(const int32_t *__restrict__ adjnc
     int u = 0;
     if (ok) {
       u = stream_rows ? __ldcs(adjncy + st + j) : adjncy[st + j];
-      w[e] = stream_rows ? __ldcs(adjwgt + st + j) : adjwgt[st + j];
+      w[e] = !adjwgt ? 1 : stream_rows ? __ldcs(adjwgt + st + j) : adjwgt[st + j];
     } else {
       w[e] = 0;
     }
@@ -143,6 +146,112 @@ __device__ __forceinline__ unsigned rate_group(const int32_t *__restrict__ adjnc
     }
   }
   return best;
+}
+
+// x[q] = base[st + q] for q < deg, 0 beyond.  vec: base is 16-byte aligned; then 16 bytes a load, from the
+// last boundary before st, moved into place by two selects a word (lim: words that may be read).
+template <int D>
+__device__ __forceinline__ void load_row(const int32_t *base, int st, int deg, int64_t lim, bool vec, int (&x)[D]) {
+  if (vec) {
+    int w[D + 4];
+    const int off = st & 3, s0 = st - off;
+#pragma unroll
+    for (int g = 0; g < (D + 4) / 4; g++) {
+      const int idx = s0 + 4 * g;
+      int4 y = make_int4(0, 0, 0, 0);
+      if (idx < st + deg) {
+        if ((int64_t)idx + 4 <= lim) {
+          y = __ldcs(reinterpret_cast<const int4 *>(base + idx));
+        } else {  // the array's last words
+          y.x = base[idx];
+          if ((int64_t)idx + 1 < lim) y.y = base[idx + 1];
+          if ((int64_t)idx + 2 < lim) y.z = base[idx + 2];
+        }
+      }
+      w[4 * g] = y.x; w[4 * g + 1] = y.y; w[4 * g + 2] = y.z; w[4 * g + 3] = y.w;
+    }
+#pragma unroll
+    for (int q = 0; q < D + 2; q++) w[q] = (off & 1) ? w[q + 1] : w[q];
+#pragma unroll
+    for (int q = 0; q < D; q++) x[q] = (off & 2) ? w[q + 2] : w[q];
+  } else {
+#pragma unroll
+    for (int q = 0; q < D; q++) x[q] = q < deg ? __ldcs(base + st + q) : 0;
+  }
+}
+
+// The largest label weight that leaves room for a node of weight cv under the bound (label weights are
+// below 2^31).
+__device__ __forceinline__ int room_of(int64_t bound, int cv) {
+  const int64_t r = bound - cv;
+  return r > 0x7FFFFFFF ? 0x7FFFFFFF : r < -1 ? -1 : (int)r;
+}
+
+// The choice of one thread's node from its row: L[q] the labels (-1 beyond deg), w[q] the edge weights; both
+// are used up.  Returns the label to propose or -1.  s_w: label weights in shared memory (every candidate
+// is checked against the bound at once), or null: only the best candidate's weight is read from weight,
+// and the other candidates' when that one does not fit.  stay: no label rated above the own one,
+// admissible or not.  nc: labels other than own.  All lanes of the warp call it together.
+template <int D, bool FAV>
+__device__ __forceinline__ int choose_row(int (&L)[D], int (&w)[D], int deg, bool live, int v, int own, int cv,
+                                          int64_t bound, uint64_t ktie, const int *s_w, const int32_t *weight,
+                                          bool &stay, int &nc) {
+  // equal labels: the first of them takes the sum, the others drop out (-1)
+  const int dm = __reduce_max_sync(0xFFFFFFFFu, deg);
+#pragma unroll
+  for (int p = 0; p < D - 1; p++) {
+    if (p >= dm) break;
+#pragma unroll
+    for (int b = p / 8 * 8; b < D; b += 8) {
+      if (b >= dm) break;
+#pragma unroll
+      for (int q = b; q < b + 8; q++) {
+        if (q <= p) continue;
+        if (L[q] == L[p]) { w[p] += w[q]; L[q] = -1; }
+      }
+    }
+  }
+  int own_r = 0, rall = 0;
+  nc = 0;
+#pragma unroll
+  for (int q = 0; q < D; q++) {
+    if (L[q] == own) { own_r = w[q]; L[q] = -1; }
+    if (L[q] >= 0) { rall = w[q] > rall ? w[q] : rall; nc++; }
+  }
+  stay = !FAV && rall <= own_r;
+  if (!live || stay) return -1;
+  const int room = room_of(bound, cv);
+  if (s_w) {
+#pragma unroll
+    for (int q = 0; q < D; q++)
+      if (L[q] >= 0 && s_w[L[q]] > room) L[q] = -1;
+  }
+  for (int pass = 0; pass < 2; pass++) {
+    int r = FAV ? -1 : own_r, lb = -1;
+    bool tie = false;
+#pragma unroll
+    for (int q = 0; q < D; q++) {
+      if (L[q] < 0 || w[q] < r) continue;
+      tie = w[q] == r && lb >= 0;
+      if (w[q] > r) { r = w[q]; lb = L[q]; }
+    }
+    if (lb < 0) return -1;
+    if (tie) {  // several labels of the best rating: the hashes decide
+      unsigned hb = 0xFFFFFFFFu;
+      lb = 0x7FFFFFFF;
+#pragma unroll
+      for (int q = 0; q < D; q++) {
+        if (L[q] < 0 || w[q] != r) continue;
+        const unsigned h = h32(ktie, (uint32_t)v, (uint32_t)L[q]);
+        if (h < hb || (h == hb && L[q] < lb)) { hb = h; lb = L[q]; }
+      }
+    }
+    if (FAV || s_w || pass == 1 || weight[lb] <= room) return lb;
+#pragma unroll
+    for (int q = 0; q < D; q++)
+      if (L[q] >= 0 && (w[q] <= own_r || weight[L[q]] > room)) L[q] = -1;
+  }
+  return -1;
 }
 
 }  // namespace gp

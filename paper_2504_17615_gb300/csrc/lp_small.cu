@@ -13,10 +13,11 @@
 //
 // Per round, the nodes with neighbours are listed by (sub-round, degree
 // class) in two passes (count, scatter).  Per sub-round:
-//   rate    nodes of degree <= 8 are rated by 8-lane groups, <= 32 by a warp
-//           with one entry per lane, <= 128 by a warp with four entries per
-//           lane (equal labels summed in a small shared table, read back only
-//           by the lane that claimed the label's slot), larger ones by a block
+//   rate    nodes of degree <= 32 are rated by a thread each with the row in
+//           registers when there are many, else by groups of 8, 16 or 32
+//           lanes; <= 128 by a warp with four entries per lane (equal labels
+//           summed in a small shared table, read back only by the lane that
+//           claimed the label's slot); larger ones by a block
 //   decide  a target whose snapshot weight plus all incoming weight fits the
 //           bound accepts its proposers outright; the others are resolved in
 //           (target, h32(PRIO), node) order, longest prefix (R7)
@@ -58,19 +59,27 @@ constexpr int kPCross = 1024;       // few-label overflow: crossing-bucket entri
 // sorted by one block in shared memory
 constexpr int kPFewLabels = 1024;
 constexpr int kPSortOne = 1024;
+// with the label weights in shared memory, a sub-round of at most this many proposals is decided by every
+// block for itself (the same decisions from the same snapshot), which saves two grid barriers
+constexpr int kPLocal = 1024;
 // 2.5x cap: digits of the radix select (11 bits from the top), and the keys left at which the
 // remaining ones are listed and ranked directly
 constexpr int kPCapBits = 11;
 constexpr int kPCapBins = 1 << kPCapBits;
 constexpr int kPCapPasses = 6;
 constexpr int kPCapList = 256;
+constexpr size_t kLocalBytes = (sizeof(uint64_t) + sizeof(uint32_t) + sizeof(int32_t) + sizeof(long long) + 1) * kPLocal;
+// a class's list longer than this many nodes per warp is rated by a thread per node, a shorter one by lane
+// groups: a thread's whole row takes 1.5 to 4 us, a pass of lane groups (4, 2 or 1 nodes a warp) about 1 us
+constexpr int kPRows8 = 16, kPRows16 = 6, kPRows32 = 8;
 constexpr int kPPropBuf = 32;       // proposals a warp collects before it takes list slots for them
 constexpr int kPAggLabels = 4096;   // labels up to this count: weight updates aggregated per block
 constexpr int kPWeightSmem = 1024;  // refinement with labels up to this count: weights in shared memory
-constexpr int kPKeys = 64 * 4;      // (sub-round, degree class) lists of a round
+constexpr int kPClasses = 5;        // degree classes
+constexpr int kPKeys = 64 * kPClasses;  // (sub-round, degree class) lists of a round
 // resident blocks per SM of the persistent grid, and the pause between polls of a grid-wide wait
 #ifndef GP_PLP_BLOCKS_PER_SM
-#define GP_PLP_BLOCKS_PER_SM 3
+#define GP_PLP_BLOCKS_PER_SM 2
 #endif
 #ifndef GP_PLP_POLL_NS
 #define GP_PLP_POLL_NS 128
@@ -91,8 +100,9 @@ struct PResult {
 };
 
 struct PArgs {
-  const int32_t *xadj, *adjncy, *adjwgt, *vwgt;
+  const int32_t *xadj, *adjncy, *adjwgt, *vwgt;  // adjwgt may be null: every weight is 1
   int n;
+  int64_t m2;
   int32_t *label, *weight;
   uint8_t *label8;
   uint8_t *dirty;        // refinement: per node, 0 = cannot move until a neighbour moves (may be null)
@@ -104,11 +114,11 @@ struct PArgs {
   int64_t ncl0;
   // scratch
   int4 *prop;            // [n] (node, target, own label, weight)
-  int32_t *incoming;     // [nlabels], zero between sub-rounds
+  int32_t *incoming;     // [nlabels], zero between sub-rounds; two such arrays in turn when two_inc
+  int two_inc;
   uint8_t *acc;          // [n] per proposal: accepted
-  int32_t *blist;        // [n] the round's nodes by (sub-round, degree class)
+  int4 *blist;           // [n] the round's nodes (node, row offset, degree, weight) by (sub-round, degree class)
   int32_t *bcnt, *bfill; // [2][kPKeys] list sizes and fill cursors (by round parity)
-  int32_t *boffs;        // [2][kPKeys + 1] list offsets
   uint64_t *ovk;         // [cap2] (target << 32 | priority)
   uint32_t *ovv;         // [cap2] node
   int32_t *ovi;          // [cap2] proposal index
@@ -191,16 +201,16 @@ __device__ __forceinline__ uint64_t pkey(uint64_t kprio, int v) {
 
 // Adds a proposal's weight to its target.  The additions to a target see every partial total, the last
 // one the full one, so the sub-round's overflow flag is raised iff some target's total does not fit.
-__device__ __forceinline__ void add_incoming(const PArgs &a, PCount *c, int K, int cv, int wK) {
-  const int before = atomicAdd(&a.incoming[K], cv);
+__device__ __forceinline__ void add_incoming(const PArgs &a, PCount *c, int32_t *inc, int K, int cv, int wK) {
+  const int before = atomicAdd(&inc[K], cv);
   if ((int64_t)wK + before + cv > a.bound) *(volatile int *)&c->over = 1;
 }
 
 // Appends one proposal (thread 0 of the rating block).
-__device__ __forceinline__ void propose(const PArgs &a, PCount *c, int v, int K, int own, int cv) {
+__device__ __forceinline__ void propose(const PArgs &a, PCount *c, int32_t *inc, int v, int K, int own, int cv) {
   const int i = atomicAdd(&c->nprop, 1);
   a.prop[i] = make_int4(v, K, own, cv);
-  add_incoming(a, c, K, cv, a.weight[K]);
+  add_incoming(a, c, inc, K, cv, a.weight[K]);
 }
 
 // A warp's proposals are collected in shared memory and take their places in the list 32 at a time:
@@ -327,10 +337,61 @@ __device__ void bitonic(uint64_t *k, uint32_t *v, int32_t *ix, int P) {
   }
 }
 
+// The warp's proposals (prop: this lane has one), into its buffer.
+__device__ __forceinline__ void buffer_props(const PArgs &a, PCount *c, int32_t *inc, PropBuf &pb, bool prop, int v,
+                                             int best, int own, int cv, const int *s_wl) {
+  const unsigned pm = __ballot_sync(FULL, prop);
+  if (!pm) return;
+  if (pb.cnt + __popc(pm) > kPPropBuf) flush_props(a, c, pb);
+  if (prop) {
+    pb.buf[pb.cnt + __popc(pm & lanemask_lt())] = make_int4(v, best, own, cv);
+    add_incoming(a, c, inc, best, cv, s_wl ? s_wl[best] : a.weight[best]);
+  }
+  pb.cnt += __popc(pm);
+}
+
+// Rates the nodes list[0 .. count) of degree <= D, a thread each (choose_row of lp_rate.cuh), and proposes
+// the moves.
+template <int D>
+__device__ __forceinline__ void rate_rows(const PArgs &a, PCount *c, int32_t *inc, const int4 *list, int count, int gt,
+                                          int gthreads, uint64_t ktie, const int *s_wl, PropBuf &pb,
+                                          unsigned long long &ue, unsigned long long &uv) {
+  const int lane = (int)lane_id();
+  const bool vec = (((uintptr_t)a.adjncy | (uintptr_t)a.adjwgt) & 15) == 0;
+  for (int i0 = gt - lane; i0 < count; i0 += gthreads) {
+    const int i = i0 + lane;
+    const int4 rec = i < count ? list[i] : make_int4(-1, 0, 0, 0);
+    const int v = rec.x, cv = rec.w;
+    const bool live = v >= 0 && !(a.dirty && !a.dirty[v]);  // clean: cannot move until a neighbour moves
+    const int st = live ? rec.y : 0, deg = live ? rec.z : 0;
+    const int own = live ? plabel(a, v) : -2;
+    int L[D], w[D];
+    load_row<D>(a.adjncy, st, deg, a.m2, vec, L);
+#pragma unroll
+    for (int q = 0; q < D; q++) L[q] = q < deg ? plabel(a, L[q]) : -1;
+    if (a.adjwgt) {
+      load_row<D>(a.adjwgt, st, deg, a.m2, vec, w);
+    } else {
+#pragma unroll
+      for (int q = 0; q < D; q++) w[q] = 1;
+    }
+    bool stay;
+    int nc;
+    const int best = choose_row<D, false>(L, w, deg, live, v, own, cv, a.bound, ktie, s_wl, a.weight, stay, nc);
+    if (a.dirty && live && stay) a.dirty[v] = 0;
+    __syncwarp();
+    buffer_props(a, c, inc, pb, best >= 0, v, best, own, cv, s_wl);
+    if (live) {
+      ue += deg;
+      uv += 1;
+    }
+  }
+}
+
 // Rates the nodes list[0 .. count), one node per G-lane group with up to E
 // entries per lane (rate_group of lp_rate.cuh), and proposes the moves.
 template <int G, int E>
-__device__ __forceinline__ void rate_list(const PArgs &a, PCount *c, const int32_t *list, int count, int gw,
+__device__ __forceinline__ void rate_list(const PArgs &a, PCount *c, int32_t *inc, const int4 *list, int count, int gw,
                                           int nw, int *tk, int *tv, uint64_t ktie, const int *s_wl,
                                           PropBuf &pb, unsigned long long &ue, unsigned long long &uv) {
   constexpr int NV = 32 / G;
@@ -340,14 +401,15 @@ __device__ __forceinline__ void rate_list(const PArgs &a, PCount *c, const int32
   const unsigned gmask = G == 32 ? FULL : (((1u << G) - 1u) << (grp * G));
   for (int i0 = gw * NV; i0 < count; i0 += nw * NV) {
     const int i = i0 + grp;
-    int v = i < count ? list[i] : -1;
+    const int4 rec = i < count ? list[i] : make_int4(-1, 0, 0, 0);
+    int v = rec.x;
     if (v >= 0 && a.dirty && !a.dirty[v]) v = -1;  // cannot move until a neighbour moves
     int st = 0, deg = 0, own = -2, cv = 0;
     if (v >= 0) {
-      st = a.xadj[v];
-      deg = a.xadj[v + 1] - st;
+      st = rec.y;
+      deg = rec.z;
       own = plabel(a, v);
-      cv = a.vwgt[v];
+      cv = rec.w;
     }
     int nc = 0;
     bool stable = false;
@@ -355,16 +417,7 @@ __device__ __forceinline__ void rate_list(const PArgs &a, PCount *c, const int32
                                                   ktie, v, st, deg, own, cv, tk + grp * TS, tv + grp * TS, gmask,
                                                   gl, false, nc, stable);
     const bool mine = gl == 0 && v >= 0;
-    const bool prop = mine && best != 0xFFFFFFFFu;
-    const unsigned pm = __ballot_sync(FULL, prop);
-    if (pm) {
-      if (pb.cnt + __popc(pm) > kPPropBuf) flush_props(a, c, pb);
-      if (prop) {
-        pb.buf[pb.cnt + __popc(pm & lanemask_lt())] = make_int4(v, (int)best, own, cv);
-        add_incoming(a, c, (int)best, cv, s_wl ? s_wl[best] : a.weight[best]);
-      }
-      pb.cnt += __popc(pm);
-    }
+    buffer_props(a, c, inc, pb, mine && best != 0xFFFFFFFFu, v, (int)best, own, cv, s_wl);
     if (mine) {
       ue += deg;
       uv += 1;
@@ -373,14 +426,16 @@ __device__ __forceinline__ void rate_list(const PArgs &a, PCount *c, const int32
   }
 }
 
-// degree classes of the per-round lists: <= 8 (8 lanes per node), <= 32 (a
-// warp, one entry per lane), <= 128 (a warp, four entries per lane), larger
-// (a block)
-__device__ __forceinline__ int deg_class(int deg) { return deg <= 8 ? 0 : deg <= 32 ? 1 : deg <= kPLight ? 2 : 3; }
+// degree classes of the per-round lists: <= 8, <= 16, <= 32 (a thread or 8, 16
+// or 32 lanes per node), <= 128 (a warp, four entries per lane), larger (a
+// block)
+__device__ __forceinline__ int deg_class(int deg) {
+  return deg <= 8 ? 0 : deg <= 16 ? 1 : deg <= 32 ? 2 : deg <= kPLight ? 3 : 4;
+}
 
 // ---------------------------------------------------------- the kernel
 
-__global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
+__global__ void __launch_bounds__(kPThreads, GP_PLP_BLOCKS_PER_SM) k_lp_persistent(PArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   // per-warp rating tables, then a phase-shared area
   int *wtk = reinterpret_cast<int *>(smem);                 // [kPWarps][kPSlots]
@@ -422,10 +477,9 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
     if (a.dbg_max >= 0 && subs >= a.dbg_max) break;
     // the round's lists: nodes with neighbours by (sub-round, degree class), in two passes
     {
-      const int nkeys = a.S * 4;
+      const int nkeys = a.S * kPClasses;
       int32_t *cnt = a.bcnt + (r & 1) * kPKeys;
       int32_t *fill = a.bfill + (r & 1) * kPKeys;
-      int32_t *offs = a.boffs + (r & 1) * (kPKeys + 1);
       if (blockIdx.x == 0) {  // the other parity's counters, for the next round
         for (int t = threadIdx.x; t < kPKeys; t += blockDim.x) {
           a.bcnt[((r + 1) & 1) * kPKeys + t] = 0;
@@ -438,32 +492,42 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
         const int deg = a.xadj[v + 1] - a.xadj[v];
         if (deg == 0) continue;
         const int sr = (int)(h32(kact, (uint32_t)v, 0) % (uint32_t)a.S);
-        atomicAdd(&s_bc[sr * 4 + deg_class(deg)], 1);
+        atomicAdd(&s_bc[sr * kPClasses + deg_class(deg)], 1);
       }
       __syncthreads();
       for (int t = threadIdx.x; t < nkeys; t += blockDim.x)
         if (s_bc[t]) atomicAdd(&cnt[t], s_bc[t]);
       if (!grid_sync(a)) return;
       // offsets (every block computes the same prefix), then the scatter in chunks
-      if (threadIdx.x == 0) {
+      if (wib == 0) {
         int run = 0;
-        for (int t = 0; t < nkeys; t++) { s_bo[t] = run; run += cnt[t]; }
-        s_bo[nkeys] = run;
+        for (int b = 0; b < nkeys; b += 32) {
+          const int x = b + lane < nkeys ? *(volatile int32_t *)&cnt[b + lane] : 0;
+          int y = x;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const int z = __shfl_up_sync(FULL, y, o);
+            if (lane >= o) y += z;
+          }
+          if (b + lane < nkeys) s_bo[b + lane] = run + y - x;
+          run += __shfl_sync(FULL, y, 31);
+        }
+        if (lane == 0) s_bo[nkeys] = run;
       }
       __syncthreads();
-      if (blockIdx.x == 0)
-        for (int t = threadIdx.x; t <= nkeys; t += blockDim.x) offs[t] = s_bo[t];
       for (int c0 = blockIdx.x * kPThreads * 4; c0 < n; c0 += gridDim.x * kPThreads * 4) {
         for (int t = threadIdx.x; t < nkeys; t += blockDim.x) s_bc[t] = 0;
         __syncthreads();
-        int key[4];
+        int key[4], vst[4], vdeg[4];
 #pragma unroll
         for (int q = 0; q < 4; q++) {
           const int v = c0 + q * kPThreads + (int)threadIdx.x;
           key[q] = -1;
           if (v < n) {
-            const int deg = a.xadj[v + 1] - a.xadj[v];
-            if (deg > 0) key[q] = (int)(h32(kact, (uint32_t)v, 0) % (uint32_t)a.S) * 4 + deg_class(deg);
+            vst[q] = a.xadj[v];
+            vdeg[q] = a.xadj[v + 1] - vst[q];
+            if (vdeg[q] > 0)
+              key[q] = (int)(h32(kact, (uint32_t)v, 0) % (uint32_t)a.S) * kPClasses + deg_class(vdeg[q]);
           }
           if (key[q] >= 0) atomicAdd(&s_bc[key[q]], 1);
         }
@@ -477,7 +541,7 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
         for (int q = 0; q < 4; q++) {
           if (key[q] < 0) continue;
           const int v = c0 + q * kPThreads + (int)threadIdx.x;
-          a.blist[s_bb[key[q]] + atomicAdd(&s_bc[key[q]], 1)] = v;
+          a.blist[s_bb[key[q]] + atomicAdd(&s_bc[key[q]], 1)] = make_int4(v, vst[q], vdeg[q], a.vwgt[v]);
         }
         __syncthreads();
       }
@@ -493,7 +557,14 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
         nx->delta = 0; nx->moved = 0; nx->over = 0; nx->nleft = 0;
       }
       // ---------------------------------------------------------- rate
-      const int32_t *lo = a.boffs + (r & 1) * (kPKeys + 1) + s * 4;  // this sub-round's four lists
+      const int *lo = s_bo + s * kPClasses;  // this sub-round's lists
+      // with two arrays of incoming weights the other one is cleared meanwhile: its last readers are past the
+      // barrier that ended the sub-round before
+      int32_t *inc = a.incoming + (a.two_inc ? (int64_t)(subs & 1) * a.nlabels : 0);
+      if (a.two_inc && blockIdx.x == gridDim.x - 1) {
+        int32_t *other = a.incoming + (int64_t)((subs + 1) & 1) * a.nlabels;
+        for (int t = threadIdx.x; t < (int)a.nlabels; t += blockDim.x) other[t] = 0;
+      }
       if (few_w) {
         for (int t = threadIdx.x; t < (int)a.nlabels; t += blockDim.x) s_wl[t] = a.weight[t];
         __syncthreads();
@@ -502,26 +573,27 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
       {
         int *htk = reinterpret_cast<int *>(area);
         int *htv = htk + kPHeavySlots;
-        const int h0 = lo[3], h1 = lo[4];
+        const int h0 = lo[4], h1 = lo[5];
         if (h1 > h0) {
           for (int t = threadIdx.x; t < kPHeavySlots; t += blockDim.x) { htk[t] = -1; htv[t] = 0; }
           __syncthreads();
         }
         for (int h = h0 + blockIdx.x; h < h1 && (int)blockIdx.x < a.hblocks; h += a.hblocks) {
-          const int v = a.blist[h];
+          const int4 rec = a.blist[h];
+          const int v = rec.x;
           // read by every thread before thread 0 may clear it below (barriers in between)
           if (a.dirty && !a.dirty[v]) continue;
-          const int st = a.xadj[v], deg = a.xadj[v + 1] - st;
+          const int st = rec.y, deg = rec.z;
           int bits = 1;
           while ((1 << bits) < 2 * deg) bits++;
           const int tsize = 1 << bits;
           const bool sm = tsize <= kPHeavySlots;
           int *k2 = sm ? htk : a.gtk + (int64_t)blockIdx.x * a.gstride;
           int *v2 = sm ? htv : a.gtv + (int64_t)blockIdx.x * a.gstride;
-          const int own = plabel(a, v), cv = a.vwgt[v];
+          const int own = plabel(a, v), cv = rec.w;
           for (int j = threadIdx.x; j < deg; j += blockDim.x) {
             const int L = plabel(a, a.adjncy[st + j]);
-            const int w = a.adjwgt[st + j];
+            const int w = a.adjwgt ? a.adjwgt[st + j] : 1;
             unsigned sl = ((unsigned)L * 2654435761u) >> (32 - bits);
             for (int probe = 0; probe < tsize; probe++) {  // bounded: the table never fills
               const int prev = atomicCAS(&k2[sl], -1, L);
@@ -538,7 +610,7 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
           if (threadIdx.x == 0) {
             ue += deg;
             uv += 1;
-            if (best != ~0ull) propose(a, c, v, (int)(uint32_t)best, own, cv);
+            if (best != ~0ull) propose(a, c, inc, v, (int)(uint32_t)best, own, cv);
             if (stable) a.dirty[v] = 0;
           }
           __syncthreads();
@@ -550,9 +622,19 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
         const int *wl = few_w ? s_wl : nullptr;
         // the proposal buffers lie behind the heavy nodes' tables in the shared area
         PropBuf pb{reinterpret_cast<int4 *>(area + sizeof(int) * 2 * kPHeavySlots) + wib * kPPropBuf, 0};
-        rate_list<32, 4>(a, c, a.blist + lo[2], lo[3] - lo[2], gw, nw, tk, tv, ktie, wl, pb, ue, uv);
-        rate_list<32, 1>(a, c, a.blist + lo[1], lo[2] - lo[1], gw, nw, tk, tv, ktie, wl, pb, ue, uv);
-        rate_list<8, 1>(a, c, a.blist + lo[0], lo[1] - lo[0], gw, nw, tk, tv, ktie, wl, pb, ue, uv);
+        rate_list<32, 4>(a, c, inc, a.blist + lo[3], lo[4] - lo[3], gw, nw, tk, tv, ktie, wl, pb, ue, uv);
+        if (lo[3] - lo[2] > kPRows32 * nw)
+          rate_rows<32>(a, c, inc, a.blist + lo[2], lo[3] - lo[2], gt, gthreads, ktie, wl, pb, ue, uv);
+        else
+          rate_list<32, 1>(a, c, inc, a.blist + lo[2], lo[3] - lo[2], gw, nw, tk, tv, ktie, wl, pb, ue, uv);
+        if (lo[2] - lo[1] > kPRows16 * nw)
+          rate_rows<16>(a, c, inc, a.blist + lo[1], lo[2] - lo[1], gt, gthreads, ktie, wl, pb, ue, uv);
+        else
+          rate_list<16, 1>(a, c, inc, a.blist + lo[1], lo[2] - lo[1], gw, nw, tk, tv, ktie, wl, pb, ue, uv);
+        if (lo[1] - lo[0] > kPRows8 * nw)
+          rate_rows<8>(a, c, inc, a.blist + lo[0], lo[1] - lo[0], gt, gthreads, ktie, wl, pb, ue, uv);
+        else
+          rate_list<8, 1>(a, c, inc, a.blist + lo[0], lo[1] - lo[0], gw, nw, tk, tv, ktie, wl, pb, ue, uv);
         flush_props(a, c, pb);
       }
       if (!grid_sync(a)) return;
@@ -564,14 +646,68 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
       // -------------------------------------------------------- decide
       // when no target overflows every proposal is accepted, and there is nothing to decide
       const bool over_any = *(volatile int *)&c->over != 0;
-      if (over_any) {
+      // few proposals, and the label weights of the sub-round's start in shared memory: every block decides
+      // all of them from those and the incoming weights, into its own flags, and applies its share
+      const bool local = over_any && few_w && nprop <= kPLocal;
+      uint64_t *lk = reinterpret_cast<uint64_t *>(area);               // [kPLocal] overflow keys
+      uint32_t *lv = reinterpret_cast<uint32_t *>(lk + kPLocal);       // [kPLocal] nodes
+      int32_t *lx = reinterpret_cast<int32_t *>(lv + kPLocal);         // [kPLocal] proposal indices
+      long long *lp = reinterpret_cast<long long *>(lx + kPLocal);     // [kPLocal] running weights
+      uint8_t *lacc = reinterpret_cast<uint8_t *>(lp + kPLocal);       // [kPLocal] accepted
+      int nov = 0;
+      if (local) {
+        __shared__ int s_no;
+        if (threadIdx.x == 0) s_no = 0;
+        __syncthreads();
+        for (int i = threadIdx.x; i < nprop; i += blockDim.x) {
+          const int4 p = a.prop[i];
+          const bool fit = (int64_t)s_wl[p.y] + *(volatile int32_t *)&inc[p.y] <= a.bound;
+          lacc[i] = fit ? 1 : 0;
+          if (!fit) {
+            const int j = atomicAdd(&s_no, 1);
+            lk[j] = ((uint64_t)(uint32_t)p.y << 32) | h32(kprio, (uint32_t)p.x, 0);
+            lv[j] = (uint32_t)p.x;
+            lx[j] = i;
+          }
+        }
+        __syncthreads();
+        nov = s_no;
+        int P = 1;
+        while (P < nov) P <<= 1;
+        for (int i = nov + threadIdx.x; i < P; i += blockDim.x) { lk[i] = ~0ull; lv[i] = 0xFFFFFFFFu; lx[i] = -1; }
+        __syncthreads();
+        bitonic(lk, lv, lx, P);
+        long long carry = 0;
+        for (int c0 = 0; c0 < nov; c0 += blockDim.x) {
+          const int i = c0 + (int)threadIdx.x;
+          const long long x = i < nov ? (long long)a.vwgt[lv[i]] : 0;
+          long long tot;
+          const long long incl = block_incl_scan(x, s_ll, tot);
+          if (i < nov) lp[i] = carry + incl;
+          carry += tot;
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < nov; i += blockDim.x) {
+          const uint64_t seg = lk[i] & 0xFFFFFFFF00000000ull;
+          int l0 = 0, l1 = i;
+          while (l0 < l1) {
+            const int mid = (l0 + l1) >> 1;
+            if (lk[mid] < seg) l0 = mid + 1; else l1 = mid;
+          }
+          const long long w = lp[i] - (l0 > 0 ? lp[l0 - 1] : 0);
+          lacc[lx[i]] = (int64_t)s_wl[(int)(lk[i] >> 32)] + w <= a.bound ? 1 : 0;
+        }
+        __syncthreads();
+      }
+      const uint8_t *acc = local ? lacc : a.acc;
+      if (over_any && !local) {
       for (int b0 = blockIdx.x * blockDim.x; b0 < nprop; b0 += gthreads) {
         const int i = b0 + (int)threadIdx.x;
         bool over = false;
         int4 p = make_int4(0, 0, 0, 0);
         if (i < nprop) {
           p = a.prop[i];
-          const bool fit = (int64_t)a.weight[p.y] + a.incoming[p.y] <= a.bound;
+          const bool fit = (int64_t)a.weight[p.y] + inc[p.y] <= a.bound;
           a.acc[i] = fit ? 1 : 0;
           over = !fit;
         }
@@ -585,8 +721,8 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
       if (!grid_sync(a)) return;
       }
       // ------------------------------------------------------ overflow
-      const int nov = over_any ? *(volatile int *)&c->nov : 0;
-      if (nov > 0) {
+      if (over_any && !local) {
+        nov = *(volatile int *)&c->nov;
         if (few && nov > kPSortOne) {
           // per target: weighted histogram over the top 12 priority bits finds the
           // bucket where the running weight passes the room; only that bucket's
@@ -856,7 +992,7 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
         }
       }
       // --------------------------------------------------------- apply
-      int *s_dw = reinterpret_cast<int *>(area);
+      int *s_dw = reinterpret_cast<int *>(area + kLocalBytes);
       if (agg) {
         for (int q = threadIdx.x; q < (int)a.nlabels; q += blockDim.x) s_dw[q] = 0;
         __syncthreads();
@@ -864,8 +1000,8 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
       long long moved = 0, delta = 0;
       for (int i = gt; i < nprop; i += gthreads) {
         const int4 p = a.prop[i];
-        a.incoming[p.y] = 0;
-        if (over_any && !a.acc[i]) continue;
+        if (!a.two_inc) inc[p.y] = 0;
+        if (over_any && !acc[i]) continue;
         if (cutoff != ~0ull && pkey(kprio, p.x) >= cutoff) continue;
         a.label[p.x] = p.y;
         if (a.label8) a.label8[p.x] = (uint8_t)p.y;
@@ -886,7 +1022,7 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
       }
       if (a.dirty) {  // every applied move marks its node and the node's neighbours, a warp per move
         for (int i = gw; i < nprop; i += nw) {
-          if (over_any && !a.acc[i]) continue;
+          if (over_any && !acc[i]) continue;
           const int v = a.prop[i].x;
           if (cutoff != ~0ull && pkey(kprio, v) >= cutoff) continue;
           const int e0 = a.xadj[v], e1 = a.xadj[v + 1];
@@ -918,6 +1054,7 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
     if (lane == 0) {
       if (ue) atomicAdd(a.units + 0, ue);
       if (ue && a.label8) atomicAdd(a.units + 4, ue);
+      if (ue && !a.adjwgt) atomicAdd(a.units + 5, ue);
       if (uv) atomicAdd(a.units + 1, uv);
     }
   }
@@ -933,12 +1070,13 @@ __global__ void __launch_bounds__(kPThreads) k_lp_persistent(PArgs a) {
 }
 
 constexpr size_t kAreaBytes() {
+  // (the aggregated weight changes lie behind the locally decided sub-round's arrays)
   // the largest phase use of the shared area
   size_t heavy = sizeof(int) * 2 * kPHeavySlots + sizeof(int4) * kPWarps * kPPropBuf;
   size_t cap = sizeof(unsigned) * kPCapBins;
   size_t sort = (sizeof(uint64_t) + sizeof(uint32_t) + sizeof(int32_t) + sizeof(long long)) * kPSortSmem;
   size_t fewb = sizeof(long long) * kPBuckets + (sizeof(uint64_t) + 2 * sizeof(int)) * kPCross;
-  size_t aggb = sizeof(int) * kPAggLabels;
+  size_t aggb = kLocalBytes + sizeof(int) * kPAggLabels;
   size_t m = heavy;
   m = sort > m ? sort : m;
   m = fewb > m ? fewb : m;
@@ -988,9 +1126,10 @@ bool lp_run_small(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *weigh
   if (p.count_clusters && nclusters_dev) read_back(ctx, nclusters_dev, sizeof(int64_t), &ncl0);
   int64_t cap2 = 1;
   while (cap2 < n) cap2 <<= 1;
-  DBuf<int4> prop(ctx, (size_t)n);
-  DBuf<int32_t> incoming(ctx, (size_t)nlabels), blist(ctx, (size_t)n), ovi(ctx, (size_t)cap2);
-  DBuf<int32_t> bcnt(ctx, 2 * (size_t)kPKeys), bfill(ctx, 2 * (size_t)kPKeys), boffs(ctx, 2 * ((size_t)kPKeys + 1));
+  const bool two_inc = !p.count_clusters && nlabels <= kPWeightSmem;
+  DBuf<int4> prop(ctx, (size_t)n), blist(ctx, (size_t)n);
+  DBuf<int32_t> incoming(ctx, (size_t)nlabels * (two_inc ? 2 : 1)), ovi(ctx, (size_t)cap2);
+  DBuf<int32_t> bcnt(ctx, 2 * (size_t)kPKeys), bfill(ctx, 2 * (size_t)kPKeys);
   bcnt.zero();
   bfill.zero();
   DBuf<uint8_t> acc(ctx, (size_t)n);
@@ -1049,7 +1188,8 @@ bool lp_run_small(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *weigh
   Ctl *dc = ctl.get();
 
   PArgs a{};
-  a.xadj = g.xadj; a.adjncy = g.adjncy; a.adjwgt = g.adjwgt; a.vwgt = g.vwgt; a.n = n;
+  a.xadj = g.xadj; a.adjncy = g.adjncy; a.adjwgt = g.unit_w ? nullptr : g.adjwgt; a.vwgt = g.vwgt; a.n = n;
+  a.m2 = g.m2; a.two_inc = two_inc ? 1 : 0;
   a.label = label; a.weight = weight; a.label8 = label8; a.nlabels = nlabels;
   a.dirty = p.count_clusters ? nullptr : dirty.get();
   a.bound = p.bound; a.n_min = p.n_min; a.count_clusters = p.count_clusters ? 1 : 0;
@@ -1057,7 +1197,7 @@ bool lp_run_small(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *weigh
   a.seed = seed; a.tag_act = p.tag_act; a.tag_tie = p.tag_tie; a.tag_prio = p.tag_prio;
   a.ncl0 = ncl0;
   a.prop = prop.get(); a.incoming = incoming.get(); a.acc = acc.get(); a.blist = blist.get();
-  a.bcnt = bcnt.get(); a.bfill = bfill.get(); a.boffs = boffs.get();
+  a.bcnt = bcnt.get(); a.bfill = bfill.get();
   a.ovk = ovk.get(); a.ovv = ovv.get(); a.ovi = ovi.get(); a.ovps = ovps.get(); a.cap2 = cap2;
   a.depw = depw.get(); a.dkey = dkey.get(); a.ekeys = ekeys.get(); a.chist = chist.get();
   a.cleft = cleft.get();
