@@ -27,7 +27,12 @@
 //  * rows are copied to shared memory where they fit (below the first depths
 //    only a subproblem's internal edges are left); the row bounds of a taken
 //    node are fetched while the next one is being chosen.
-//  * steps of up to kSoloB nodes run in one warp without block barriers.
+//  * steps of up to kSoloB nodes run in one warp without block barriers;
+//  * steps of kBatchB nodes or more select them together: a histogram of the
+//    chunk maxima's gains gives the gain of the B-th largest maximum, the nodes
+//    of at least that gain in the (at most B) chunks that can hold the step's
+//    nodes are ranked by counting, and one warp walks them in order.  One pick
+//    after another is a chain of some 460 cycles each.
 // A picked node that no longer fits is retired for good (side 1 only gets
 // heavier), which leaves the choice among the nodes that fit unchanged.
 // The fallback scans all nodes the first few times; after that, the nodes
@@ -36,7 +41,8 @@
 // or stopped fitting never comes back).
 //
 // Measured (20,480 nodes, 204,800 edges, k = 128, 8 trials; the whole initial partition): 17.0 ms with 64-bit
-// keys in separate arrays, block barriers in every step and a sort of the chunk maxima; 9.0 ms so.
+// keys in separate arrays, block barriers in every step and a sort of the chunk maxima; 9.0 ms with the
+// words, one pick after another everywhere; 7.8 ms with the steps of kBatchB nodes selected together.
 #include "gp_internal.cuh"
 
 #include <algorithm>
@@ -48,13 +54,16 @@ namespace {
 constexpr int kUpdUnroll = 4;
 constexpr int kSmemBatch = 64;  // the nodes of a growing step live in shared memory up to this many
 constexpr int kChunkNodes = 64;
-constexpr int kIpWarps = 4;     // warps per (subproblem, trial)
+constexpr int kIpWarps = 8;     // warps per (subproblem, trial)
 constexpr int kSoloB = 4;       // steps of up to this many nodes run in one warp
+constexpr int kBatchB = 8;      // steps of at least this many select them together
+constexpr int kBins = 512;      // gains below the largest one that the selection tells apart
+constexpr int kCands = 256;     // nodes ranked per selection; more: picked one by one
 constexpr int kScanFallbacks = 8;      // fallbacks found by a scan over all nodes before the order is made
 constexpr int kBucketNodes = 4;        // nodes per hash bucket of that order at least, on average
 constexpr int kNarrowNodes = 1 << 15;  // 32-bit words: subproblems below this many nodes ...
 constexpr int kNarrowGain = 1 << 15;   // ... and weighted degrees below this
-constexpr int kStaticSmem = 2048;      // room for the kernel's static shared variables
+constexpr int kStaticSmem = 8192;      // room for the kernel's static shared variables
 constexpr int kSmSmem = 228 * 1024;    // shared memory of an SM; every resident block reserves another 1 KiB
 constexpr int kMaxSmemBytes = 227 * 1024 - kStaticSmem;
 
@@ -74,6 +83,7 @@ template <> struct Word<int32_t> {
   __device__ static int32_t make(int64_t gain, int j) {
     return ((int32_t)(gain + kNarrowGain) << 15) | (kNarrowNodes - 1 - j);
   }
+  __device__ static int64_t gain(int32_t x) { return x >> 15; }  // plus a constant
   __device__ static int node(int32_t x) { return kNarrowNodes - 1 - (x & (kNarrowNodes - 1)); }
   __device__ static int32_t delta(int w) { return (int32_t)((uint32_t)(2 * w) << 15); }  // connection + w
   __device__ static int32_t wmax(int32_t x) { return __reduce_max_sync(0xFFFFFFFFu, x); }
@@ -83,6 +93,7 @@ template <> struct Word<long long> {
   __device__ static long long make(int64_t gain, int j) {
     return ((gain + 2147483648ll) << 31) | (2147483647 - j);
   }
+  __device__ static int64_t gain(long long x) { return x >> 31; }
   __device__ static int node(long long x) { return 2147483647 - (int)(x & 2147483647ll); }
   __device__ static long long delta(int w) { return (long long)w << 32; }
   __device__ static long long wmax(long long x) {
@@ -194,7 +205,9 @@ __global__ void __launch_bounds__(32 * kIpWarps) k_ip_grow(IpArgs a) {
   __shared__ long long s_w1;
   __shared__ unsigned long long s_red[kIpWarps];
   __shared__ int32_t s_batch[kSmemBatch];
-  __shared__ int s_rs[32], s_re[32];
+  __shared__ int s_rs[kSmemBatch], s_re[kSmemBatch];
+  __shared__ int s_hist[kBins], s_wsum[2][kIpWarps], s_list[kSmemBatch], s_nlist, s_ncand, s_bin, s_need;
+  __shared__ KT s_wmax[kIpWarps], s_cand[kCands], s_rank[kCands], s_tau;
   const int lane = (int)lane_id(), warp = threadIdx.x >> 5;
   const int si = blockIdx.x / a.trials, t = blockIdx.x % a.trials;
   const Sub S = a.subs[si];
@@ -457,14 +470,189 @@ __global__ void __launch_bounds__(32 * kIpWarps) k_ip_grow(IpArgs a) {
       }
     }
   } else {
-    const bool rows_async = SM && !lx && B <= 32;
+    const bool rows_async = SM && !lx && B <= kSmemBatch;
     int32_t *batch = B <= kSmemBatch ? s_batch : a.gbatch + (int64_t)blockIdx.x * a.batch_cap;
+    const bool batched = SM && B >= kBatchB && B <= kSmemBatch;
+    // One selection of up to `want` nodes by the whole block, appended to batch from nb0 on; returns 0 when no
+    // frontier node is left, -1 when they must be picked one by one (gains too far apart, or too many
+    // equal ones), else 1; s_nb and s_w1 are the new number and weight (warp 0 keeps w1).
+    auto select = [&](int nb0) -> int {
+      if constexpr (!SM) {
+        return -1;
+      } else {
+        const int want = B - nb0;
+        constexpr int PER = 512 / (32 * kIpWarps);  // chunks per thread
+        static_assert(PER >= 1 && PER <= 2, "two chunk maxima a thread at most");
+        KT x[PER], mx = 0;
+#pragma unroll
+        for (int i = 0; i < PER; i++) {
+          const int c = (int)threadIdx.x + i * 32 * kIpWarps;
+          x[i] = c < nch ? best.get(c) : 0;
+          mx = x[i] > mx ? x[i] : mx;
+        }
+        mx = W::wmax(mx);
+        if (lane == 0) s_wmax[warp] = mx;
+        for (int t2 = threadIdx.x; t2 < kBins; t2 += blockDim.x) s_hist[t2] = 0;
+        if (threadIdx.x == 0) { s_nlist = 0; s_ncand = 0; s_bin = -1; }
+        __syncthreads();
+        mx = s_wmax[0];
+#pragma unroll
+        for (int w = 1; w < kIpWarps; w++) mx = s_wmax[w] > mx ? s_wmax[w] : mx;
+        if (mx <= kOut) return 0;
+        const int64_t top = W::gain(mx);
+        int bin[PER];
+#pragma unroll
+        for (int i = 0; i < PER; i++) {
+          const int64_t d = top - W::gain(x[i]);
+          bin[i] = x[i] > kOut && d < kBins ? (int)d : kBins;
+          if (bin[i] < kBins) atomicAdd(&s_hist[bin[i]], 1);
+        }
+        const int present = __syncthreads_count(x[0] > kOut) + (PER > 1 ? __syncthreads_count(x[PER - 1] > kOut) : 0);
+        const int q = want < present ? want : present;  // chunks that can hold the step's nodes
+        // the bin of the q-th largest maximum, and how many of its maxima belong to the q
+        if (warp == 0) {
+          constexpr int PB = kBins / 32;
+          int loc = 0;
+#pragma unroll
+          for (int i = 0; i < PB; i++) loc += s_hist[lane * PB + i];
+          int incl = loc;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= o) incl += y;
+          }
+          int run = incl - loc;
+          if (run < q && q <= incl) {
+#pragma unroll
+            for (int i = 0; i < PB; i++) {
+              const int h = s_hist[lane * PB + i];
+              if (run < q && q <= run + h) { s_bin = lane * PB + i; s_need = q - run; }
+              run += h;
+            }
+          }
+        }
+        __syncthreads();
+        const int cutbin = s_bin, need = s_need;
+        if (cutbin < 0) return -1;  // the gains lie further apart than the bins
+        // the q largest maxima: those above the cut bin, and the first `need` of it in id order (of equal gains
+        // the smaller id goes first).  The smallest of them, tau, is reached by at least q nodes, and all
+        // nodes that reach it lie in those q chunks
+#pragma unroll
+        for (int i = 0; i < PER; i++) {
+          const unsigned m = __ballot_sync(0xFFFFFFFFu, bin[i] == cutbin);
+          if (lane == 0) s_wsum[i][warp] = __popc(m);
+        }
+        __syncthreads();
+        int before = 0;
+#pragma unroll
+        for (int i = 0; i < PER; i++) {
+          int at = before;
+#pragma unroll
+          for (int w = 0; w < kIpWarps; w++) {
+            const int v = s_wsum[i][w];
+            at += w < warp ? v : 0;
+            before += v;
+          }
+          const unsigned m = __ballot_sync(0xFFFFFFFFu, bin[i] == cutbin);
+          at += __popc(m & lanemask_lt());
+          if (bin[i] < cutbin || (bin[i] == cutbin && at < need))
+            s_list[atomicAdd(&s_nlist, 1)] = (int)threadIdx.x + i * 32 * kIpWarps;
+          if (bin[i] == cutbin && at == need - 1) s_tau = x[i];
+        }
+        __syncthreads();
+        const KT tau = s_tau;
+        const int nl = s_nlist;  // q chunks
+        for (int l = warp; l < nl; l += kIpWarps) {
+          const int j0 = s_list[l] * kChunkNodes + lane, j1 = j0 + 32;
+          const KT a0 = j0 < cnt ? X.get(j0) : 0, a1 = j1 < cnt ? X.get(j1) : 0;
+          const bool in0 = a0 >= tau, in1 = a1 >= tau;  // tau > kOut
+          const unsigned m0 = __ballot_sync(0xFFFFFFFFu, in0), m1 = __ballot_sync(0xFFFFFFFFu, in1);
+          int at = 0;
+          if (lane == 0) at = atomicAdd(&s_ncand, __popc(m0) + __popc(m1));
+          at = __shfl_sync(0xFFFFFFFFu, at, 0);
+          const int p0 = at + __popc(m0 & lanemask_lt()), p1 = at + __popc(m0) + __popc(m1 & lanemask_lt());
+          if (in0 && p0 < kCands) s_cand[p0] = a0;
+          if (in1 && p1 < kCands) s_cand[p1] = a1;
+        }
+        __syncthreads();
+        const int C = s_ncand;
+        if (C > kCands) return -1;
+        for (int t2 = threadIdx.x; t2 < C; t2 += blockDim.x) {  // words are distinct: rank = place
+          const KT mine = s_cand[t2];
+          int r = 0;
+#pragma unroll 4
+          for (int u = 0; u < C; u++) r += s_cand[u] > mine ? 1 : 0;
+          s_rank[r] = mine;
+        }
+        __syncthreads();
+        if (warp == 0) {
+          int nb = nb0, i0 = 0;
+          while (i0 < C) {
+            const int i = i0 + lane;
+            const int j = i < C ? W::node(s_rank[i]) : -1;
+            const long long c = i < C ? weight(j) : 0;
+            long long pre = c;  // weight of lanes 0 .. lane
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+              const long long y = __shfl_up_sync(0xFFFFFFFFu, pre, o);
+              if (lane >= o) pre += y;
+            }
+            // a lane is reached iff every earlier one was taken
+            const bool considered = i < C && nb + lane < B && w1 + (pre - c) < S.T1;
+            const bool fits = w1 + pre <= S.L1;
+            const unsigned bad = __ballot_sync(0xFFFFFFFFu, !(considered && fits));
+            const int f = bad ? __ffs(bad) - 1 : 32;
+            if (lane < f) {
+              X.set(j, kOne);
+              batch[nb + lane] = j;
+              if (rows_async) {  // the row's bounds come while the chunks are looked over again
+                copy_async4(&s_rs[nb + lane], a.lxadj + start + j);
+                copy_async4(&s_re[nb + lane], a.lxadj + start + j + 1);
+              }
+            }
+            const long long wf = __shfl_sync(0xFFFFFFFFu, pre, f > 0 ? f - 1 : 0);
+            const bool cf = __shfl_sync(0xFFFFFFFFu, considered, f < 32 ? f : 0);
+            if (f > 0) w1 += wf;
+            nb += f;
+            if (f == 32) { i0 += 32; continue; }
+            if (i0 + f >= C || !cf) break;  // list used up, or the step is complete
+            if (lane == f) X.set(j, kOut);  // reached and does not fit: retired
+            retired++;
+            i0 += f + 1;
+          }
+          if (lane == 0) { s_nb = nb; s_w1 = w1; }
+        }
+        __syncthreads();
+        for (int l = warp; l < nl; l += kIpWarps) {  // the listed chunks' maxima again
+          const int c = s_list[l];
+          const KT nm = chunk_max(c, -1);
+          if (lane == 0) best.set(c, nm);
+        }
+        if (rows_async && warp == 0) copy_async_wait();
+        __syncthreads();
+        return 1;
+      }
+    };
     for (;;) {
+      int got = 0;     // batched: nodes selected so far
+      bool one_by_one = !batched;
+      if (batched) {
+        if (threadIdx.x == 0) { s_w1 = w1; s_nb = 0; }
+        __syncthreads();
+        if (s_w1 >= S.T1) break;
+        if (warp == 0) steps++;
+        while (got < B && s_w1 < S.T1) {
+          const int r = select(got);
+          if (r <= 0) { one_by_one = r < 0; break; }
+          got = s_nb;
+        }
+      }
+      if (one_by_one) {
       if (warp == 0) {
         int nb = -2;  // done
         if (w1 < S.T1) {
-          nb = 0;
-          steps++;
+          nb = got;
+          if (!batched) steps++;
           constexpr int kN = SM ? 16 : 1;
           constexpr IntC<kN> N{};
           KT r[kN];
@@ -487,6 +675,7 @@ __global__ void __launch_bounds__(32 * kIpWarps) k_ip_grow(IpArgs a) {
         if (lane == 0) { s_nb = nb; s_w1 = w1; }
       }
       __syncthreads();
+      }
       int nb = s_nb;
       if (nb == -2) break;
       bool fell = false;
@@ -524,8 +713,8 @@ __global__ void __launch_bounds__(32 * kIpWarps) k_ip_grow(IpArgs a) {
         int r0 = 0, d = 0;
         if (b0 + lane < nb) {
           if (rows_async && !fell) {
-            r0 = s_rs[lane] - base;
-            d = s_re[lane] - base - r0;
+            r0 = s_rs[b0 + lane] - base;
+            d = s_re[b0 + lane] - base - r0;
           } else {
             const int j = batch[b0 + lane];
             r0 = row_begin(j);
