@@ -209,13 +209,14 @@ __global__ void __launch_bounds__(kThreads) k_merge_block(MergeArgs a) {
   if (a.units && threadIdx.x == 0) atomicAdd(a.units + 3, uout);
 }
 
-// Longest segment, number of huge ones and table slots they need together.
+// Longest segment, number of huge ones and their entries.
 struct SegStats {
   int longest, huge;
-  unsigned long long slots;
+  unsigned long long entries;
 };
 
-__device__ __forceinline__ int seg_slots(int len) { return len + len / 3 + 1; }
+// Slots of a huge segment's table, q4 quarters of a slot an entry.
+__device__ __forceinline__ int seg_slots(int len, int q4) { return (int)((int64_t)len * q4 / 4 + 1); }
 
 __global__ void k_seg_stats(const int32_t *x, int n, SegStats *out) {
   int m = 0, nh = 0;
@@ -224,14 +225,14 @@ __global__ void k_seg_stats(const int32_t *x, int n, SegStats *out) {
        i += (int64_t)gridDim.x * blockDim.x) {
     const int l = x[i];
     m = l > m ? l : m;
-    if (l > kHugeSeg) { nh++; ns += (unsigned long long)seg_slots(l); }
+    if (l > kHugeSeg) { nh++; ns += (unsigned long long)l; }
   }
   m = warp_max(m);
   if (lane_id() == 0 && m) atomicMax(&out->longest, m);
   if (__any_sync(FULL, nh)) {
     nh = warp_sum(nh);
     ns = warp_sum(ns);
-    if (lane_id() == 0) { atomicAdd(&out->huge, nh); atomicAdd(&out->slots, ns); }
+    if (lane_id() == 0) { atomicAdd(&out->huge, nh); atomicAdd(&out->entries, ns); }
   }
 }
 
@@ -241,7 +242,8 @@ __global__ void k_seg_stats(const int32_t *x, int n, SegStats *out) {
 // global memory took milliseconds for it while the rest of the device waited (12 levels of the scale-24
 // R-MAT graph: 131 ms of contraction).  k_seg_plan lists the huge segments with the prefix sums of their
 // chunks, k_seg_insert sums 2048 entries at a time in a shared table and adds the sums to the segment's
-// table in global memory (4/3 slots an entry; one 64-bit exchange claims a slot), and k_seg_extract writes the occupied slots back to the
+// table in global memory (two slots an entry where the memory bound allows; one 64-bit exchange claims a
+// slot), and k_seg_extract writes the occupied slots back to the
 // segment.  Consecutive steps work on the same few tables, which stay in L2 meanwhile.
 
 struct Seg {
@@ -253,6 +255,7 @@ struct SegArgs {
   Seg *segs;
   int *chunk0, *tchunk0;  // prefix sums of entry chunks and table chunks; [count] = totals
   int2 *tab;              // (coarse neighbour, weight) slots
+  int q4;                 // slots an entry, in quarters
 };
 
 __global__ void __launch_bounds__(1024) k_seg_plan(MergeArgs a, SegArgs h) {
@@ -267,7 +270,7 @@ __global__ void __launch_bounds__(1024) k_seg_plan(MergeArgs a, SegArgs h) {
       x.A = a.large[a.nc - i];
       x.s0 = a.tstart[x.A];
       x.len = a.tstart[x.A + 1] - x.s0;
-      x.tsize = seg_slots(x.len);
+      x.tsize = seg_slots(x.len, h.q4);
     }
     const long long val[3] = {(x.len + kSegChunk - 1) / kSegChunk, (x.tsize + kSegTabChunk - 1) / kSegTabChunk, x.tsize};
     long long ex[3];
@@ -457,13 +460,18 @@ void contract_graph(gp_ctx *ctx, const DevGraph &g, const int32_t *cmap, int32_t
   DBuf<Seg> segs;
   DBuf<int> chunk0, tchunk0;
   DBuf<int2> tab;
-  a.split_huge = hs.huge > 0 && 8 * (int64_t)hs.slots <= 8 * g.m2 + ((int64_t)16 << 20) ? 1 : 0;
+  int64_t slots = 0;
+  for (sg.q4 = 8; sg.q4 > 4; sg.q4--) {  // two slots an entry down to one and a quarter
+    slots = (int64_t)hs.entries * sg.q4 / 4 + hs.huge;
+    if (slots <= g.m2 + ((int64_t)2 << 20)) break;
+  }
+  a.split_huge = hs.huge > 0 && sg.q4 > 4 ? 1 : 0;
   if (a.split_huge) {
     segs.reset(ctx, (size_t)hs.huge);
     chunk0.reset(ctx, (size_t)hs.huge + 1);
     tchunk0.reset(ctx, (size_t)hs.huge + 1);
-    tab.reset(ctx, (size_t)hs.slots);
-    sg = SegArgs{segs.get(), chunk0.get(), tchunk0.get(), tab.get()};
+    tab.reset(ctx, (size_t)slots);
+    sg = SegArgs{segs.get(), chunk0.get(), tchunk0.get(), tab.get(), sg.q4};
   } else if ((1 << bits) > kBlockSmemSlots) {
     a.gstride = (int64_t)1 << bits;
     lblocks = table_blocks(g.m2, a.gstride, lblocks);
@@ -488,8 +496,7 @@ void contract_graph(gp_ctx *ctx, const DevGraph &g, const int32_t *cmap, int32_t
     if (a.split_huge) {
       k_seg_plan<<<1, 1024, 0, ctx->stream>>>(a, sg);
       GP_LAUNCH_CHECK();
-      k_seg_clear<<<grid_for((int64_t)hs.slots, kThreads, ctx->num_sms * 8), kThreads, 0, ctx->stream>>>(
-          tab.get(), (int64_t)hs.slots);
+      k_seg_clear<<<grid_for(slots, kThreads, ctx->num_sms * 8), kThreads, 0, ctx->stream>>>(tab.get(), slots);
       GP_LAUNCH_CHECK();
       k_seg_insert<<<ctx->num_sms * 6, kThreads, 0, ctx->stream>>>(a, sg);
       GP_LAUNCH_CHECK();

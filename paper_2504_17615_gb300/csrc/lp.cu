@@ -25,7 +25,6 @@ namespace gp {
 namespace {
 
 constexpr unsigned FULL = 0xFFFFFFFFu;
-constexpr int kMedSlots = 256;
 constexpr int kThreads = 256;
 constexpr int kWarpsPerBlock = kThreads / 32;
 constexpr int kMaxKeys = 64 * kNumBuckets;
@@ -96,7 +95,7 @@ __device__ __forceinline__ void emit(const RateArgs &a, int i, int v, int best, 
 // array); with 8 or 16 lanes per node and tables in shared memory a node of 20 neighbours took 225-300
 // warp instructions, so that issue and latency bound it instead.  The pairs cost D (D - 1) / 2 x 3
 // instructions per 32 nodes, a tenth of that, and every label of the row is in flight at once.
-// THRNUM
+// The clustering and refinement of a level of 16.8M nodes and 268M entries went from 25.6 to 21.7 ms.
 //
 // The choice is lazy in the label weights: candidates are ranked by (rating, tie hash, label) without the
 // bound, and only the best one's weight is read; if it does not fit, the weights of all that are rated
@@ -171,7 +170,8 @@ __global__ void __launch_bounds__(ThreadShape<D>::NT, ThreadShape<D>::PER_SM) k_
 // 32, so every thread counts its row in byte counters of its own, four to a word, in shared memory (word
 // [label / 4][thread]: no two lanes of a warp meet in a bank).  The pairs of k_rate_thread took 3100
 // instructions per 32 nodes of degree 17-24 and 106 registers (16 warps an SM, 80e9 entries/s); this takes
-// about a fifth of the instructions and half the registers.  BYTNUM
+// about a fifth of the instructions and half the registers.  It reaches
+// 105e9 entries/s on 2^26 nodes of degree 16, bound by the L1 path of the gathers.
 
 template <int D>
 __global__ void __launch_bounds__(128, D <= 16 ? 8 : 6) k_rate_bytes(RateArgs a) {
@@ -263,15 +263,29 @@ __global__ void __launch_bounds__(128, D <= 16 ? 8 : 6) k_rate_bytes(RateArgs a)
   add_units(a.units, ue, uv, uc, up, true, true);
 }
 
-// --------------------------------------- degree <= 128: warp/node + table
+// ------------------------- degree <= 128, <= 512: warp/node, shared table
+//
+// The table has two slots per neighbour (a slot is the high half of hash x size, so any size will do) and
+// kWarpUnroll neighbours per lane are in flight.  What costs here is the probing: a warp goes on until its
+// unluckiest lane has found a slot, some ten probes with 4/3 slots per neighbour and about four with two.
+// On the scale-24 R-MAT graph two slots (and more for blocks and hubs) took the partition from 468 to 425 ms.
+
+constexpr int kWarpUnroll = 4;
+
+// Slots of a table for deg labels, q4 quarters of a slot each (more than deg, so that no table fills).
+__host__ __device__ __forceinline__ int tab_slots(int deg, int q4) {
+  const int64_t s = (int64_t)deg * q4 / 4 + 1;
+  return s > 0x7FFFFFF0 ? 0x7FFFFFF0 : (int)s;
+}
+constexpr int kTabQ4 = 8;     // shared tables: two slots per neighbour ...
+constexpr int kTabQ4Last = 6; // ... one and a half in the largest class (an SM's whole shared memory)
 
 template <int MODE>
-__global__ void __launch_bounds__(kThreads) k_rate_medium(RateArgs a) {
-  __shared__ int s_k[kWarpsPerBlock][kMedSlots];
-  __shared__ int s_v[kWarpsPerBlock][kMedSlots];
+__global__ void __launch_bounds__(kThreads) k_rate_warp(RateArgs a, int slots) {
+  extern __shared__ int s_tab[];  // per warp: slots labels, slots ratings
   const int lane = (int)lane_id(), wib = threadIdx.x >> 5;
-  int *tk = s_k[wib], *tv = s_v[wib];
-  for (int t = lane; t < kMedSlots; t += 32) { tk[t] = -1; tv[t] = 0; }
+  int *tk = s_tab + wib * 2 * slots, *tv = tk + slots;
+  for (int t = lane; t < slots; t += 32) { tk[t] = -1; tv[t] = 0; }
   __syncwarp();
   if (a.stop && *a.stop) return;
   const int begin = a.offs[a.key], end = list_end(a);
@@ -286,47 +300,61 @@ __global__ void __launch_bounds__(kThreads) k_rate_medium(RateArgs a) {
       continue;
     }
     const int own = label_of(a, v);
-    for (int j = lane; j < deg; j += 32) {
-      const int L = label_of(a, __ldcs(a.adjncy + start + j));
-      const int w = a.adjwgt ? __ldcs(a.adjwgt + start + j) : 1;
-      unsigned s = slot_hash(L, 8);
-      for (int probe = 0; probe < kMedSlots; probe++) {  // bounded: the table never fills
-        const int prev = atomicCAS(&tk[s], -1, L);
-        if (prev == -1 || prev == L) { atomicAdd(&tv[s], w); break; }
-        s = (s + 1) & (kMedSlots - 1);
+    const int tsize = tab_slots(deg, kTabQ4);
+    for (int j0 = lane; j0 < deg; j0 += 32 * kWarpUnroll) {
+      int L[kWarpUnroll], w[kWarpUnroll];
+#pragma unroll
+      for (int r = 0; r < kWarpUnroll; r++) {
+        const int j = j0 + r * 32;
+        L[r] = j < deg ? __ldcs(a.adjncy + start + j) : -1;
+        w[r] = j < deg && a.adjwgt ? __ldcs(a.adjwgt + start + j) : 1;
+      }
+#pragma unroll
+      for (int r = 0; r < kWarpUnroll; r++) L[r] = L[r] >= 0 ? label_of(a, L[r]) : -1;
+#pragma unroll
+      for (int r = 0; r < kWarpUnroll; r++) {
+        if (L[r] < 0) continue;
+        int s = (int)__umulhi((unsigned)L[r] * 2654435761u, (unsigned)tsize);
+        for (int probe = 0; probe < tsize; probe++) {  // bounded: more slots than neighbours
+          const int prev = atomicCAS(&tk[s], -1, L[r]);
+          if (prev == -1 || prev == L[r]) { atomicAdd(&tv[s], w[r]); break; }
+          s = s + 1 == tsize ? 0 : s + 1;
+        }
       }
     }
     __syncwarp();
     int own_loc = 0, rloc = -1, nc = 0, rall = 0;
-    for (int t = lane; t < kMedSlots; t += 32) {
+    for (int t = lane; t < tsize; t += 32) {
       const int L = tk[t];
       if (L < 0) continue;
       const int r = tv[t];
       if (L == own) { own_loc = r; continue; }
       nc++;
       rall = r > rall ? r : rall;
-      if (MODE == RATE_LP && (int64_t)a.weight[L] + cv > a.bound) continue;
-      rloc = r > rloc ? r : rloc;
+      if (r > rloc && (MODE != RATE_LP || (int64_t)a.weight[L] + cv <= a.bound)) rloc = r;  // only a better one matters
     }
-    const int own_r = warp_max(own_loc);
-    const int rmax = warp_max(rloc);
-    if (a.dirty && warp_max(rall) <= own_r && lane == 0) a.dirty[v] = 0;
+    const int own_r = __reduce_max_sync(FULL, own_loc);
+    const int rmax = __reduce_max_sync(FULL, rloc);
+    if (a.dirty && __reduce_max_sync(FULL, rall) <= own_r && lane == 0) a.dirty[v] = 0;
     ue += deg; uv += 1; uc += nc;
-    if (!(rmax < 0 || (MODE == RATE_LP && rmax <= own_r))) {
-      uint64_t packed = ~0ull;
-      for (int t = lane; t < kMedSlots; t += 32) {
-        const int L = tk[t];
-        if (L < 0 || L == own || tv[t] != rmax) continue;
-        if (MODE == RATE_LP && (int64_t)a.weight[L] + cv > a.bound) continue;
+    const bool want = !(rmax < 0 || (MODE == RATE_LP && rmax <= own_r));
+    uint64_t packed = ~0ull;
+    for (int t = lane; t < tsize; t += 32) {
+      const int L = tk[t];
+      if (L < 0) continue;
+      if (want && L != own && tv[t] == rmax && (MODE != RATE_LP || (int64_t)a.weight[L] + cv <= a.bound)) {
         const uint64_t p = ((uint64_t)h32(a.ktie, (uint32_t)v, (uint32_t)L) << 32) | (uint32_t)L;
         packed = p < packed ? p : packed;
       }
+      tk[t] = -1;
+      tv[t] = 0;
+    }
+    if (want) {
       packed = warp_min(packed);
       if (lane == 0) { emit<MODE>(a, i, v, (int)(uint32_t)packed, cv, own); up += 1; }
     } else if (MODE == RATE_LP && lane == 0) {
       a.prop[i] = make_int2(-1, 0);
     }
-    for (int t = lane; t < kMedSlots; t += 32) { tk[t] = -1; tv[t] = 0; }
     __syncwarp();
   }
   add_units(a.units, ue * (lane == 0), uv * (lane == 0), uc, up, a.label8 != nullptr, a.adjwgt == nullptr);
@@ -434,16 +462,14 @@ __global__ void __launch_bounds__(kThreads) k_rate_large(RateArgs a) {
   add_units(a.units, ue, uv, uc, up, a.label8 != nullptr, a.adjwgt == nullptr);
 }
 
-// ------------------- 128 < degree <= 18432: block/node, shared table
+// ------------------- 512 < degree <= 18432: block/node, shared table
 //
-// The table has 4/3 slots per neighbour (a slot is the high half of hash x size, so any size will do) and
-// kBlockUnroll neighbours per thread are in flight.  Nodes of 2049 .. 18432 neighbours held 172M of the
-// 521M entries of the scale-24 R-MAT graph; their tables in shared memory take no global atomics, which
-// limited them to 7e9 entries/s (BLKNUM).
+// As k_rate_warp with a block's threads.  Nodes of 2049 .. 18432 neighbours held 172M of the 521M entries of
+// the scale-24 R-MAT graph; their tables in shared memory take no global atomics, which limited them to
+// 7e9 entries/s: clustering of that level 183 -> 115 ms.  With two slots instead of 4/3 a sub-round takes
+// .35 instead of .47 ms in the 512-thread class, .40 instead of .45 in the 1024-thread one (one and a half).
 
 constexpr int kBlockUnroll = 4;
-
-__host__ __device__ __forceinline__ int hub_slots(int deg) { return deg + deg / 3 + 1; }
 
 template <int NT>
 __device__ __forceinline__ int block_max_n(int v, int *s_red) {
@@ -470,7 +496,7 @@ __device__ __forceinline__ uint64_t block_min_n(uint64_t v, uint64_t *s_red) {
 }
 
 template <int NT>
-__global__ void __launch_bounds__(NT) k_rate_block(RateArgs a, int slots) {
+__global__ void __launch_bounds__(NT) k_rate_block(RateArgs a, int slots, int q4) {
   extern __shared__ int s_tab[];  // slots labels, slots ratings
   __shared__ int s_ri[NT / 32], s_own;
   __shared__ uint64_t s_ru[NT / 32];
@@ -487,7 +513,7 @@ __global__ void __launch_bounds__(NT) k_rate_block(RateArgs a, int slots) {
       continue;
     }
     const int own = label_of(a, v);
-    const int tsize = hub_slots(deg);
+    const int tsize = tab_slots(deg, q4);
     if (threadIdx.x == 0) s_own = 0;
     __syncthreads();  // the table is empty, and the flag of the clean nodes was read before it may change
     for (int j0 = threadIdx.x; j0 < deg; j0 += NT * kBlockUnroll) {
@@ -562,7 +588,8 @@ __global__ void __launch_bounds__(NT) k_rate_block(RateArgs a, int slots) {
 //  few labels (at most kHubDense: refinement): k_hub_dense counts a chunk per label in shared memory, adds
 //    it to the hub's counters, and the block that finishes a hub's last chunk chooses;
 //  many labels: k_hub_insert sums a chunk's labels in a shared table and adds the sums to the hub's table
-//    in global memory (one 64-bit exchange claims a slot with its sum), k_hub_table walks the tables (4096
+//    in global memory (one 64-bit exchange claims a slot with its sum; three slots per neighbour where the
+//    memory bound allows, since every probe is a round trip to L2), k_hub_table walks the tables (4096
 //    slots a block) for the largest admissible rating, and then for the smallest (hash, label) of that
 //    rating, and leaves them empty.
 // The choice is the same as in the other kernels.
@@ -586,6 +613,7 @@ struct HubArgs {
   int2 *tab;              // (label, rating) slots, empty (-1, 0) between sub-rounds
   int32_t *hist;          // dense: [hub][nlabels], zero between sub-rounds
   int nlabels;
+  int q4;                 // slots per neighbour, in quarters
 };
 
 __global__ void __launch_bounds__(1024) k_hub_plan(RateArgs a, HubArgs h) {
@@ -605,7 +633,7 @@ __global__ void __launch_bounds__(1024) k_hub_plan(RateArgs a, HubArgs h) {
       if (deg == 0) a.prop[begin + i] = make_int2(-1, 0);
       x.deg = deg;
       x.own = label_of(a, rec.x);
-      x.tsize = deg > 0 ? hub_slots(deg) : 0;
+      x.tsize = deg > 0 ? tab_slots(deg, h.q4) : 0;
       x.rmax = -1;
       x.best = ~0ull;
     }
@@ -1561,28 +1589,29 @@ __global__ void k_fill_i32(int32_t *a, int64_t n, int32_t v) {
     a[i] = v;
 }
 
-// Largest degree, number of nodes above kBlockDeg0, and the table slots the hubs need together.
+// Largest degree, number of nodes above kBlockDeg0, number of hubs and their neighbours.
 struct DegStats {
-  int maxdeg, big;
-  unsigned long long slots;
+  int maxdeg, big, hubs, pad;
+  unsigned long long hubdeg;
 };
 
 __global__ void k_max_degree(const int32_t *xadj, int n, DegStats *out) {
-  int m = 0, nh = 0;
+  int m = 0, nb = 0, nh = 0;
   unsigned long long ns = 0;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x) {
     const int d = xadj[v + 1] - xadj[v];
     m = d > m ? d : m;
-    if (d > kBlockDeg0) nh++;
-    if (d > kHubDeg) ns += (unsigned long long)hub_slots(d);
+    if (d > kBlockDeg0) nb++;
+    if (d > kHubDeg) { nh++; ns += (unsigned long long)d; }
   }
   m = warp_max(m);
   if (lane_id() == 0 && m) atomicMax(&out->maxdeg, m);
-  if (__any_sync(FULL, nh)) {
+  if (__any_sync(FULL, nb)) {
+    nb = warp_sum(nb);
     nh = warp_sum(nh);
     ns = warp_sum(ns);
-    if (lane_id() == 0) { atomicAdd(&out->big, nh); atomicAdd(&out->slots, ns); }
+    if (lane_id() == 0) { atomicAdd(&out->big, nb); atomicAdd(&out->hubs, nh); atomicAdd(&out->hubdeg, ns); }
   }
 }
 
@@ -1597,6 +1626,7 @@ struct RateTables {
   int blocks = 0;
   // hubs (HubArgs), when the graph has some and their tables stay within the bound of table_blocks
   bool hubs = false;
+  int q4 = 0;          // the hub tables' slots per neighbour, in quarters
   bool dense = false;  // few labels: nodes above kBlockDeg0 are counted per label
   DBuf<Hub> hub;
   DBuf<int> chunk0, tchunk0;
@@ -1621,8 +1651,13 @@ void make_tables(gp_ctx *ctx, const DevGraph &g, int64_t nlabels, RateTables &t)
   if (nlabels > 0) {
     const int64_t cap = (8 * g.m2 + ((int64_t)16 << 20)) / (int64_t)sizeof(int2);
     t.dense = nlabels <= kHubDense && (int64_t)h.big * nlabels <= 2 * cap;
-    const int64_t hubs = t.dense ? h.big : (int64_t)h.slots / kHubDeg;  // an upper bound
-    t.hubs = hubs > 0 && (t.dense || (int64_t)h.slots <= cap);
+    const int64_t hubs = t.dense ? h.big : h.hubs;
+    int64_t slots = 0;
+    for (t.q4 = 12; t.q4 > 4; t.q4 -= 2) {  // three slots per neighbour down to one and a half
+      slots = (int64_t)h.hubdeg * t.q4 / 4 + hubs;
+      if (slots <= cap) break;
+    }
+    t.hubs = hubs > 0 && (t.dense || t.q4 > 4);
     if (t.hubs) {
       t.hub.reset(ctx, (size_t)hubs);
       t.chunk0.reset(ctx, (size_t)hubs + 1);
@@ -1631,9 +1666,8 @@ void make_tables(gp_ctx *ctx, const DevGraph &g, int64_t nlabels, RateTables &t)
         t.hist.reset(ctx, (size_t)(hubs * nlabels));
         t.hist.zero();
       } else {
-        t.tab.reset(ctx, (size_t)h.slots);
-        k_fill_slots<<<grid_for((int64_t)h.slots, 256, ctx->num_sms * 8), 256, 0, ctx->stream>>>(t.tab.get(),
-                                                                                                (int64_t)h.slots);
+        t.tab.reset(ctx, (size_t)slots);
+        k_fill_slots<<<grid_for(slots, 256, ctx->num_sms * 8), 256, 0, ctx->stream>>>(t.tab.get(), slots);
         GP_LAUNCH_CHECK();
       }
     }
@@ -1694,12 +1728,12 @@ void launch_groups(gp_ctx *ctx, const RateArgs &a, int base, const int *hcnt) {
 }
 
 template <int NT>
-void launch_block(gp_ctx *ctx, const RateArgs &a, int maxdeg, int grid) {
-  const int slots = hub_slots(maxdeg);
+void launch_block(gp_ctx *ctx, const RateArgs &a, int maxdeg, int q4, int grid) {
+  const int slots = tab_slots(maxdeg, q4);
   const size_t smem = 2 * sizeof(int) * (size_t)slots;
   if (smem > 48 * 1024)
     GP_CUDA(cudaFuncSetAttribute(k_rate_block<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_rate_block<NT><<<grid, NT, smem, ctx->stream>>>(a, slots);
+  k_rate_block<NT><<<grid, NT, smem, ctx->stream>>>(a, slots, q4);
   GP_LAUNCH_CHECK();
 }
 
@@ -1710,19 +1744,25 @@ void launch_rate(gp_ctx *ctx, RateArgs a, int bucket_key_base, const RateTables 
   const int cap = ctx->num_sms * 8;
   if (MODE == RATE_LP && a.label8) launch_groups<MODE, LK_NARROW>(ctx, a, bucket_key_base, hcnt);
   else launch_groups<MODE, LK_WIDE>(ctx, a, bucket_key_base, hcnt);
-  if (!hcnt || hcnt[kMediumBucket] > 0) {
-    a.key = bucket_key_base + kMediumBucket;
-    k_rate_medium<MODE><<<rate_grid(ctx, hcnt ? hcnt[kMediumBucket] : -1, kWarpsPerBlock, cap), kThreads, 0, ctx->stream>>>(a);
+  for (int q = 0; q < 2; q++) {  // a warp per node; favourites of larger nodes: k_rate_large
+    const int b = kMediumBucket + q;
+    if ((hcnt && hcnt[b] == 0) || (q == 1 && MODE != RATE_LP)) continue;
+    a.key = bucket_key_base + b;
+    const int slots = tab_slots(q == 0 ? kMediumMaxDeg : kWarpMaxDeg, kTabQ4);
+    const size_t smem = 2 * sizeof(int) * (size_t)slots * kWarpsPerBlock;
+    if (smem > 48 * 1024)
+      GP_CUDA(cudaFuncSetAttribute(k_rate_warp<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_rate_warp<MODE><<<rate_grid(ctx, hcnt ? hcnt[b] : -1, kWarpsPerBlock, cap), kThreads, smem, ctx->stream>>>(a, slots);
     GP_LAUNCH_CHECK();
   }
   const int hgrid = ctx->num_sms * 6;
-  for (int q = 0; q < 4; q++) {  // the three block classes, the hubs
-    const int b = kMediumBucket + 1 + q;
+  for (int q = MODE == RATE_LP ? 0 : -1; q < 4; q++) {  // the three block classes, the hubs
+    const int b = kMediumBucket + 2 + q;
     const int c = hcnt ? hcnt[b] : -1;
     if (c == 0) continue;
     a.key = bucket_key_base + b;
     if (MODE == RATE_LP && t.hubs && (q == 3 || (q > 0 && t.dense))) {
-      HubArgs h{t.hub.get(), t.chunk0.get(), t.tchunk0.get(), t.tab.get(), t.hist.get(), (int)nlabels};
+      HubArgs h{t.hub.get(), t.chunk0.get(), t.tchunk0.get(), t.tab.get(), t.hist.get(), (int)nlabels, t.q4};
       k_hub_plan<<<1, 1024, 0, ctx->stream>>>(a, h);
       GP_LAUNCH_CHECK();
       if (t.dense) {
@@ -1737,9 +1777,9 @@ void launch_rate(gp_ctx *ctx, RateArgs a, int bucket_key_base, const RateTables 
         GP_LAUNCH_CHECK();
       }
     } else if (MODE == RATE_LP && q < 3) {
-      if (q == 0) launch_block<256>(ctx, a, kBlockDeg0, rate_grid(ctx, c, 1, ctx->num_sms * 6));
-      else if (q == 1) launch_block<512>(ctx, a, kBlockDeg1, rate_grid(ctx, c, 1, ctx->num_sms * 3));
-      else launch_block<1024>(ctx, a, kHubDeg, rate_grid(ctx, c, 1, ctx->num_sms));
+      if (q == 0) launch_block<256>(ctx, a, kBlockDeg0, kTabQ4, rate_grid(ctx, c, 1, ctx->num_sms * 6));
+      else if (q == 1) launch_block<512>(ctx, a, kBlockDeg1, kTabQ4, rate_grid(ctx, c, 1, ctx->num_sms * 2));
+      else launch_block<1024>(ctx, a, kHubDeg, kTabQ4Last, rate_grid(ctx, c, 1, ctx->num_sms));
     } else {
       a.gkeys = t.gkeys.get();
       a.gvals = t.gvals.get();

@@ -6,19 +6,19 @@
 namespace gp {
 
 // Degree classes of the rating kernels: <= 8, <= 16, <= 24, <= 32 (a thread
-// per node, its labels in registers), <= 128 (a warp with a 256-slot shared table),
-// <= 2048, <= 6144, <= 18432 (a block with a shared table of 4/3 slots per
-// neighbour at most: six, three and one block an SM), larger (hubs: many
-// blocks a node).
-constexpr int kNumBuckets = 9;
+// per node, its labels in registers), <= 128, <= 512 (a warp with a shared
+// table), <= 2048, <= 6144, <= 18432 (a block with a shared table: six, two
+// and one block an SM), larger (hubs: many blocks a node).
+constexpr int kNumBuckets = 10;
 constexpr int kMediumBucket = 4;  // the class of degree <= 128
-constexpr int kMediumMaxDeg = 128;
+constexpr int kMediumMaxDeg = 128, kWarpMaxDeg = 512;
 constexpr int kBlockDeg0 = 2048, kBlockDeg1 = 6144, kHubDeg = 18432;
 constexpr int kLargeSmemSlots = 4096;
 
 __host__ __device__ __forceinline__ int degree_bucket(int deg) {
   if (deg <= 32) return deg <= 8 ? 0 : deg <= 16 ? 1 : deg <= 24 ? 2 : 3;
-  return deg <= kMediumMaxDeg ? 4 : deg <= kBlockDeg0 ? 5 : deg <= kBlockDeg1 ? 6 : deg <= kHubDeg ? 7 : 8;
+  if (deg <= kWarpMaxDeg) return deg <= kMediumMaxDeg ? 4 : 5;
+  return deg <= kBlockDeg0 ? 6 : deg <= kBlockDeg1 ? 7 : deg <= kHubDeg ? 8 : 9;
 }
 
 enum RateMode { RATE_LP = 0, RATE_FAV = 1 };

@@ -39,8 +39,8 @@ def _clique(n):
     return gg.from_pairs(n, i, j)
 
 
-# the classes end at 128, 2048, 6144 and 18432 neighbours; a hub's chunks have 2048 entries
-GRAPHS = {"star": star(2049), "edges": _hubs(9000, [128, 129, 2048, 2049, 6144, 6145, 8000], 9000, 1),
+# the classes end at 128, 512, 2048, 6144 and 18432 neighbours; a hub's chunks have 2048 entries
+GRAPHS = {"star": star(2049), "edges": _hubs(9000, [128, 129, 512, 513, 2048, 2049, 6144, 6145, 8000], 9000, 1),
           "weighted": _hubs(40000, [39000, 18433, 18432, 12345, 2500, 2049], 20000, 50), "clique": _clique(2500)}
 
 
