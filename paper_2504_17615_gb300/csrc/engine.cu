@@ -267,40 +267,55 @@ void engine_fill(gp_batch_item *items, const EngineJob &job, const std::vector<E
 
 namespace {
 
-// Without a tuning of the caller's the engine takes the items of up to kSplitFloor entries, and larger ones
-// up to the size at which the slower of the two paths, which run side by side, ends first.  An item is one
-// CTA's work from start to end, so one large item can outlast everything else: with all items of up to 2^22
-// entries on the engine a batch of 128 graphs of 1e3..1e5 nodes took 690 ms, 0.65 s of it in the CTA of the
-// largest R-MAT graph; split by this rule it takes SPLITNUM.  Costs in ms, measured on that mix (ER, grids,
-// R-MAT, k = 2..64): an item in its CTA takes 0.3-0.6 us per entry, up to 2.3 us where the bisection finds
-// many components, so kCtaPerEntry lies at the upper end; a graph on the per-graph path takes 1.7 ms (6k
-// entries), 4.5 (48k), 8.4 (195k), 13-15 (0.4-1.6M) with one worker, and the workers together get four times
-// one worker's rate (8 workers 0.41, 1.07, 2.2, 3.5-4.2 ms; 16 the same).
+// Without a tuning of the caller's the engine takes the items of up to kSplitFloor entries, and others up to
+// the predicted time in a CTA at which the slower of the two paths, which run side by side, ends first.  An
+// item is one CTA's work from start to end, so one large item can outlast everything else: with all items of
+// up to 2^22 entries on the engine a batch of 128 graphs of 1e3..1e5 nodes took 690 ms (400 with the growing
+// trials of today), nearly all of it in the CTA of the largest R-MAT graph; split by this rule it takes
+// 107, a batch of 512 197.
+// Costs in ms, measured on that mix (ER, grids, R-MAT, k = 2..64), 512 threads:
+//  * in a CTA: coarsening and refinement 0.7e-4 (ER), 1.6e-4 (grids) to 2e-4 (R-MAT) an entry, and 1.6 us for
+//    each node that the growing trials take one after another: half the coarsest graph's nodes (some 200 k of
+//    them) at the first bisection, where a warp has one trial at most, and trials / warps of that at each
+//    depth below;
+//  * on the per-graph path: 1.4 (6k entries), 4 (48k), 7 (195k), 8-14 (0.5M), 27-30 (1.9M, R-MAT) with one
+//    worker; the workers together get four times one worker's rate.
 constexpr int64_t kSplitFloor = 1 << 15;
-constexpr double kCtaPerEntry = 2.0e-3, kCtaBase = 4.0;
-constexpr double kPathBase = 1.6, kPathPerEntry = 5.0e-5, kPathMost = 14.0, kPathWorkers = 4.0;
+constexpr double kCtaBase = 1.5, kCtaPerEntry = 2.0e-4, kCtaPerTake = 1.6e-3;
+constexpr double kPathBase = 1.6, kPathPerEntry = 5.0e-5, kPathMost = 10.0, kPathPerBigEntry = 8.0e-6,
+                 kPathWorkers = 4.0;
 
-int64_t split_entries(const gp_batch_item *items, const std::vector<int32_t> &idx, int workers,
-                      const gp_batch_tuning &t, int ctas) {
-  std::vector<int64_t> m2;
+double cta_ms(const gp_batch_item &it, const gp_config &cfg, int threads) {
+  const double nc = std::min((double)it.g.n, 200.0 * it.k);
+  int depths = 0;
+  while ((1ll << depths) < it.k) depths++;
+  const double takes = nc / 2 * (1 + std::max(0, depths - 1) * (double)cfg.ip_trials / (threads / 32));
+  return kCtaBase + kCtaPerEntry * (double)it.g.m2 + kCtaPerTake * takes;
+}
+
+// The predicted time in a CTA up to which an item goes to the engine.
+double split_ms(const gp_batch_item *items, const std::vector<int32_t> &idx, int workers, const gp_config &cfg,
+                const gp_batch_tuning &t, int ctas) {
+  std::vector<std::pair<double, int32_t>> order;
   double path = 0;
   const double conc = std::min<double>(kPathWorkers, workers);
-  auto path_ms = [&](int64_t m) { return std::min(kPathMost, kPathBase + kPathPerEntry * (double)m) / conc; };
+  auto path_ms = [&](int32_t i) {
+    const double m = (double)items[i].g.m2;
+    return std::min(kPathMost + kPathPerBigEntry * m, kPathBase + kPathPerEntry * m) / conc;
+  };
   for (int32_t i : idx) {
-    path += path_ms(items[i].g.m2);
-    if (engine_item_ok(items[i], t)) m2.push_back(items[i].g.m2);
+    path += path_ms(i);
+    if (engine_item_ok(items[i], t)) order.emplace_back(cta_ms(items[i], cfg, t.threads), i);
   }
-  std::sort(m2.begin(), m2.end());
-  int64_t best = kSplitFloor;
-  double best_ms = -1, cta_sum = 0;
-  for (size_t j = 0; j < m2.size(); j++) {
-    const double item = kCtaBase + kCtaPerEntry * (double)m2[j];
-    cta_sum += item;
-    path -= path_ms(m2[j]);
-    const double ms = std::max(path, std::max(item, cta_sum / ctas));
-    if (m2[j] <= kSplitFloor || best_ms < 0 || ms < best_ms) {
+  std::sort(order.begin(), order.end());
+  double best = 0, best_ms = path, sum = 0;
+  for (const auto &o : order) {
+    sum += o.first;
+    path -= path_ms(o.second);
+    const double ms = std::max(path, std::max(o.first, sum / ctas));
+    if (ms < best_ms) {
       best_ms = ms;
-      best = std::max(kSplitFloor, m2[j]);
+      best = o.first;
     }
   }
   return best;
@@ -312,13 +327,15 @@ void batch_run(gp_ctx *ctx, gp_batch_item *items, const std::vector<int32_t> &id
                const gp_batch_tuning &given) {
   gp_batch_tuning t = given;
   const bool use = t.engine && engine_config_ok(cfg);
-  if (use && !ctx->tuning_given)
-    t.max_entries = std::min(t.max_entries, split_entries(items, idx, workers, t, ctx->num_sms));
+  const bool split = use && !ctx->tuning_given;
+  const double most = split ? split_ms(items, idx, workers, cfg, t, ctx->num_sms) : 0;
   EngineJob job;
   std::vector<int32_t> rest;
   bool want_stats = false;
   for (int32_t i : idx) {
-    if (!use || !engine_item_ok(items[i], t)) { rest.push_back(i); continue; }
+    const bool take = use && engine_item_ok(items[i], t) &&
+                      (!split || items[i].g.m2 <= kSplitFloor || cta_ms(items[i], cfg, t.threads) <= most);
+    if (!take) { rest.push_back(i); continue; }
     job.items.push_back(to_eitem(items[i]));
     job.owner.push_back(i);
     job.stats.push_back(items[i].stats);

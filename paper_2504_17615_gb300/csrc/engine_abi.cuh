@@ -95,7 +95,7 @@ Kernel kernel_512();
 Kernel kernel_1024();
 
 // dynamic shared memory of the kernel with `threads` threads per CTA
-inline size_t smem_bytes(int threads) {
+__host__ __device__ constexpr size_t smem_bytes(int threads) {
   return (size_t)(2 * kEBlockSlots + 2 * (threads / 32) * kEWarpSlots) * sizeof(int);
 }
 

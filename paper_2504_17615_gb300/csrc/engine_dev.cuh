@@ -30,6 +30,7 @@
 // with a retry status and the host runs it on the per-graph path.
 #pragma once
 #include "engine_abi.cuh"
+#include "ip_words.cuh"
 #include "lp.cuh"
 #include "lp_rate.cuh"
 
@@ -1420,123 +1421,197 @@ struct ESub {
 struct EBis {
   int32_t start, count, kk, b0;
   uint32_t bid;
-  int32_t pad;
+  int32_t maxd;  // largest deg'
   int64_t T1, L1, B;
 };
 
-__device__ __forceinline__ unsigned long long egain_key(int64_t gain, int j) {
-  return ((unsigned long long)(gain + 2147483648ll) << 32) | (0xFFFFFFFFu - (unsigned)j);
-}
+// Node words in the arena, private to the warp that runs the trial (plain accesses: its own stores come back
+// from L1).
+template <typename T> struct EWords {
+  T *p;
+  __device__ T get(int i) const { return p[i]; }
+  __device__ void set(int i, T x) const { p[i] = x; }
+};
 
-// States of a node in a growing trial.
-enum : uint8_t { T_FREE = 0, T_FRONT = 1, T_ONE = 2, T_OUT = 3 };
+// What a trial reads of its subproblem, by list position, and its fallback order's scratch.
+struct ETrial {
+  const int32_t *V, *cw, *Dp;
+  const int2 *rows;  // bounds of the internal rows in adj
+  const int2 *adj;   // (list position, weight)
+  uint2 *ford;       // b.count
+  int32_t *fcur;     // b.count / kBucketNodes + 1
+  int32_t *tkn;      // b.B
+};
 
-// One greedy-growing trial of bisection b (R18) by one warp.  Each step takes,
-// in order of their gains at the start of the step, up to B frontier nodes
-// that still fit; the node of largest key (gain, -index) comes from per-chunk
-// maxima of 64 keys.  A node that no longer fits when it comes up is retired
-// for good (side 1 only gets heavier), which leaves the choice among the
-// nodes that fit as it is.  The neighbour updates of the nodes a step takes
-// are applied after the step, so the step ranks by the gains at its start.
-// With no frontier node that fits, the step takes the free node of smallest
-// (h32(key(IP, 0, bid), v, t), index) that fits.  Writes the side-1 flags and
-// returns the cut.
-__device__ long long ip_trial(const EGraph &g, const int32_t *V, const int32_t *cw, const int32_t *Dp,
-                              const int32_t *mark, const int32_t *loc, const EBis &b, int t, uint64_t kip,
-                              int32_t *conn, uint64_t *key, uint8_t *st, uint64_t *cmax, int32_t *tkn,
-                              uint8_t *side) {
+// One greedy-growing trial of bisection b (R18) by one warp.  Each step takes, in order of their gains at the
+// start of the step, up to B frontier nodes that still fit.  A node that no longer fits when it comes up is
+// retired for good (side 1 only gets heavier), which leaves the choice among the nodes that fit as it is.  The
+// neighbour updates of the nodes a step takes are applied after the step, so the step ranks by the gains at
+// its start.  With no frontier node that fits, the step takes the free node of smallest
+// (h32(key(IP, 0, bid), v, t), index) that fits: by a scan the first few times, then from the nodes put in the
+// order of their hashes.  Writes the side-1 flags and returns the cut.
+//
+// A trial is one chain of dependent steps in one warp, bound by latency.  State, gain and id of a node are one
+// word (ip_words.cuh), so the choice is a maximum over words and a neighbour's update one read and one write;
+// the words and the maxima of 64-node chunks lie in shared memory where they fit, the internal rows are listed
+// once per depth, and the cut is summed from the gains at which nodes are taken.  With 64-bit keys, states and
+// connections in separate arrays of the arena and two walks over the whole rows per step, growing took 65-90 %
+// of the engine's time: 9.4 and 18.3 million cycles an item of up to 16384 and 65536 entries (k = 2..64), now 4.3
+// and 8.0.  Four row loads in flight per lane instead of one: 18 % slower, rows are mostly shorter than 32.
+template <typename T, class XW, class BW>
+__device__ __noinline__ long long ip_trial(XW X, BW best, const ETrial a, const EBis &b, int t, uint64_t kip,
+                                           uint8_t *side) {
+  using W = Word<T>;
   const int lane = (int)lane_id();
-  const int nv = b.count, nch = (nv + 63) >> 6;
-  const int32_t bid = (int32_t)b.bid;
-  for (int j = lane; j < nv; j += 32) { conn[j] = 0; key[j] = 0; st[j] = T_FREE; }
-  for (int q = lane; q < nch; q += 32) cmax[q] = 0;
+  const int nv = b.count, nch = (nv + kChunkNodes - 1) / kChunkNodes;
+  const int64_t T1 = b.T1, L1 = b.L1, B = b.B;
+  for (int j = lane; j < nv; j += 32) X.set(j, W::make(-(int64_t)a.Dp[j], j) | W::kFree);
+  for (int q = lane; q < nch; q += 32) best.set(q, 0);
   __syncwarp();
-  auto rescan = [&](int ch) {
-    const int j0 = ch << 6;
-    const uint64_t a0 = j0 + lane < nv ? key[j0 + lane] : 0;
-    const uint64_t a1 = j0 + 32 + lane < nv ? key[j0 + 32 + lane] : 0;
-    const uint64_t m = wmax64(a0 > a1 ? a0 : a1);
-    if (lane == 0) cmax[ch] = m;
+  int bits = 0;  // buckets of the fallback order: the hash's top bits, at most nv / kBucketNodes of them
+  while ((kBucketNodes << (bits + 1)) <= nv) bits++;
+  auto hash_of = [&](int j) -> uint32_t { return h32(kip, (uint32_t)a.V[j], (uint32_t)t); };
+  auto bucket_of = [&](uint32_t h) -> int { return (int)((uint64_t)h >> (32 - bits)); };
+  int nfall = 0, cursor = 0, total = 0;
+  int64_t w1 = 0;
+  auto fallback = [&]() -> int {
+    if (nfall < kScanFallbacks) {
+      nfall++;
+      unsigned long long m = ~0ull;
+      for (int j = lane; j < nv; j += 32) {
+        if (X.get(j) >= 0 || w1 + a.cw[j] > L1) continue;
+        const unsigned long long key = ((unsigned long long)hash_of(j) << 32) | (unsigned)j;
+        m = key < m ? key : m;
+      }
+      m = wmin_u64(m);
+      return m == ~0ull ? -1 : (int)(unsigned)m;
+    }
+    volatile int32_t *place = a.fcur;
+    if (nfall == kScanFallbacks) {  // a counting sort of the nodes still free
+      nfall++;
+      const int nbk = 1 << bits;
+      for (int q = lane; q < nbk; q += 32) place[q] = 0;
+      __syncwarp();
+      for (int j = lane; j < nv; j += 32)
+        if (X.get(j) < 0) atomicAdd(a.fcur + bucket_of(hash_of(j)), 1);
+      __syncwarp();
+      for (int b0 = 0; b0 < nbk; b0 += 32) {
+        const int x = b0 + lane < nbk ? place[b0 + lane] : 0;
+        int y = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int z = __shfl_up_sync(FULL, y, o);
+          if (lane >= o) y += z;
+        }
+        if (b0 + lane < nbk) place[b0 + lane] = total + y - x;
+        total += __shfl_sync(FULL, y, 31);
+      }
+      __syncwarp();
+      for (int j = lane; j < nv; j += 32) {
+        if (X.get(j) >= 0) continue;
+        const uint32_t h = hash_of(j);
+        a.ford[atomicAdd(a.fcur + bucket_of(h), 1)] = make_uint2(h, (unsigned)j);
+      }
+      __syncwarp();
+    }
+    // the first node of the order that is free and fits; its bucket holds the answer and may go on past
+    // the 32 nodes looked at
+    int bucket = -1;
+    unsigned long long m = ~0ull;
+    for (int p = cursor; p < total; p += 32) {
+      const bool in = p + lane < total;
+      const uint2 x = in ? a.ford[p + lane] : make_uint2(0, 0);
+      const bool ok = in && X.get((int)x.y) < 0 && w1 + a.cw[x.y] <= L1;
+      const unsigned bal = __ballot_sync(FULL, ok);
+      if (bucket < 0) {
+        if (bal == 0) { cursor = p + 32; continue; }
+        const int f = __ffs(bal) - 1;
+        cursor = p + f;
+        bucket = bucket_of(__shfl_sync(FULL, x.x, f));
+      }
+      const bool same = in && bucket_of(x.x) == bucket;
+      const unsigned long long k = wmin_u64(ok && same ? ((unsigned long long)x.x << 32) | x.y : ~0ull);
+      m = k < m ? k : m;
+      if (!__shfl_sync(FULL, same, 31)) break;
+    }
+    return m == ~0ull ? -1 : (int)(unsigned)m;
+  };
+  const int64_t zero_gain = W::gain(W::make(0, 0));
+  long long cut = 0;   // minus the gains of the nodes taken (uniform) ...
+  long long twice = 0; // ... minus the edges inside a step, seen from both ends (per lane)
+  auto update = [&](int2 r) {
+    for (int e = r.x + lane; e < r.y; e += 32) {
+      const int2 y = a.adj[e];
+      const T x = X.get(y.x);
+      if (x == kStep) twice += y.y;
+      if (x >= 0 && x <= kStep) continue;
+      const T z = (x & ~W::kFree) + W::delta(y.y);
+      X.set(y.x, z);
+      best.raise(y.x / kChunkNodes, z);
+    }
     __syncwarp();
   };
-  int64_t w1 = 0;
-  while (w1 < b.T1) {
-    int ntk = 0;
-    int64_t taken = 0;
-    while (taken < b.B && w1 < b.T1) {
-      uint64_t m = 0;
-      for (int q = lane; q < nch; q += 32) m = cmax[q] > m ? cmax[q] : m;
-      m = wmax64(m);
-      if (m == 0) break;
-      const int j = (int)(0xFFFFFFFFu - (uint32_t)m);
-      const int cj = cw[j];
-      const bool fits = w1 + cj <= b.L1;
+  while (w1 < T1) {
+    int ntk = 0, j = -1;
+    int2 rw = make_int2(0, 0);
+    while (ntk < B && w1 < T1) {
+      T m = 0;
+      for (int q = lane; q < nch; q += 32) { const T x = best.get(q); m = x > m ? x : m; }
+      m = W::wmax(m);
+      if (m <= kOut) break;
+      j = W::node(m);
+      const int2 rj = a.rows[j];
+      const int cj = a.cw[j];
+      const int j0 = (j / kChunkNodes) * kChunkNodes + lane, j1 = j0 + 32;
+      const T x0 = j0 < nv && j0 != j ? X.get(j0) : 0, x1 = j1 < nv && j1 != j ? X.get(j1) : 0;
+      const T nm = W::wmax(x0 > x1 ? x0 : x1);
+      const bool fits = w1 + cj <= L1;
       if (lane == 0) {
-        key[j] = 0;
-        st[j] = fits ? T_ONE : T_OUT;
-        if (fits) tkn[ntk] = j;
+        X.set(j, fits ? kOne : kOut);
+        best.set(j / kChunkNodes, nm > kOut ? nm : 0);
+        if (fits && B > 1) a.tkn[ntk] = j;
       }
       __syncwarp();
-      rescan(j >> 6);
       if (!fits) continue;  // no longer fits (nor ever will)
+      rw = rj;
       ntk++;
-      taken++;
       w1 += cj;
+      cut -= W::gain(m) - zero_gain;
     }
-    if (taken == 0) {
-      unsigned long long fb = ~0ull;
-      for (int j = lane; j < nv; j += 32) {
-        if (st[j] != T_FREE || w1 + cw[j] > b.L1) continue;
-        const unsigned long long h = ((unsigned long long)h32(kip, (uint32_t)V[j], (uint32_t)t) << 32) | (uint32_t)j;
-        fb = h < fb ? h : fb;
-      }
-      fb = wmin64(fb);
-      if (fb == ~0ull) break;
-      const int j = (int)(uint32_t)fb;
-      if (lane == 0) { st[j] = T_ONE; tkn[0] = j; }
+    if (ntk == 0) {
+      j = fallback();
+      if (j < 0) break;
+      rw = a.rows[j];
+      w1 += a.cw[j];
+      cut += a.Dp[j];
+      __syncwarp();
+      if (lane == 0) X.set(j, kOne);
       ntk = 1;
-      w1 += cw[j];
       __syncwarp();
     }
-    // neighbour updates of the nodes taken in this step, then their keys
-    for (int q = 0; q < ntk; q++) {
-      const int v = V[tkn[q]];
-      for (int e = g.xadj[v] + lane; e < g.xadj[v + 1]; e += 32) {
-        const int u = g.adjncy[e];
-        if (mark[u] == bid) atomicAdd(&conn[loc[u]], g.adjwgt[e]);
-      }
+    // neighbours of the step's nodes, row by row (a row has no neighbour twice)
+    if (ntk == 1) {
+      update(rw);
+      continue;
     }
+    // several: the nodes taken are told from side 1 (kStep) until the edges among them are counted
+    for (int q = lane; q < ntk; q += 32) X.set(a.tkn[q], kStep);
     __syncwarp();
-    for (int q = 0; q < ntk; q++) {
-      const int v = V[tkn[q]];
-      for (int e = g.xadj[v] + lane; e < g.xadj[v + 1]; e += 32) {
-        const int u = g.adjncy[e];
-        if (mark[u] != bid) continue;
-        const int lu = loc[u];
-        const uint8_t su = st[lu];
-        if (su != T_FREE && su != T_FRONT) continue;
-        const uint64_t nk = egain_key(2 * (int64_t)conn[lu] - Dp[lu], lu);
-        key[lu] = nk;
-        st[lu] = T_FRONT;
-        atomicMax((unsigned long long *)&cmax[lu >> 6], (unsigned long long)nk);
-      }
-    }
+    for (int q = 0; q < ntk; q++) update(a.rows[a.tkn[q]]);
+    for (int q = lane; q < ntk; q += 32) X.set(a.tkn[q], kOne);
     __syncwarp();
   }
-  long long cut = 0;
-  for (int j = lane; j < nv; j += 32) {
-    const bool one = st[j] == T_ONE;
-    side[j] = one ? 1 : 0;
-    if (!one) continue;
-    const int v = V[j];
-    for (int e = g.xadj[v]; e < g.xadj[v + 1]; e++) {
-      const int u = g.adjncy[e];
-      if (mark[u] == bid && st[loc[u]] != T_ONE) cut += g.adjwgt[e];
-    }
-  }
-  cut = warp_sum(cut);
+  for (int j = lane; j < nv; j += 32) side[j] = X.get(j) == kOne ? 1 : 0;
+  cut -= warp_sum(twice);
   __syncwarp();
   return cut;
+}
+
+__device__ void e_clear_tables(ECtx &c) {
+  __syncthreads();
+  for (int t = threadIdx.x; t < nwarps() * kEWarpSlots; t += blockDim.x) { c.wtk[t] = -1; c.wtv[t] = 0; }
+  for (int t = threadIdx.x; t < kEBlockSlots; t += blockDim.x) { c.btk[t] = -1; c.btv[t] = 0; }
+  __syncthreads();
 }
 
 // Recursive bisection of the coarsest graph (Sec. 4.3, R18), depth by depth:
@@ -1544,6 +1619,7 @@ __device__ long long ip_trial(const EGraph &g, const int32_t *V, const int32_t *
 // the CTA take, largest subproblems first; the smallest cut wins (ties:
 // lowest trial), and each subproblem splits into side 1 and the rest, in
 // list order.
+// (The trials' words take the shared tables, which are left empty.)
 __device__ void e_initial(ECtx &c, const EGraph &g, int k, int64_t eps_ppm, uint64_t seed, int trials,
                           int32_t *blk) {
   ESmem &s = *c.s;
@@ -1560,6 +1636,8 @@ __device__ void e_initial(ECtx &c, const EGraph &g, int k, int64_t eps_ppm, uint
   ESub *sb = c.ar.s<ESub>(k + 1);
   EBis *bis = c.ar.s<EBis>(k + 1);
   int32_t *ord = c.ar.s<int32_t>(k + 1);
+  int2 *rows = c.ar.s<int2>(n);
+  int2 *adj = c.ar.s<int2>(g.m2);
   long long *res = c.ar.s<long long>((int64_t)(k + 1) * trials);
   uint8_t *side = c.ar.s<uint8_t>((int64_t)n * trials);
   if (c.ar.fail) return;
@@ -1597,7 +1675,7 @@ __device__ void e_initial(ECtx &c, const EGraph &g, int k, int64_t eps_ppm, uint
       if (threadIdx.x == 0) {
         const int k1 = (sub.kk + 1) / 2;
         EBis x;
-        x.start = sub.start; x.count = nv; x.kk = sub.kk; x.b0 = sub.b0; x.bid = sub.bid; x.pad = 0;
+        x.start = sub.start; x.count = nv; x.kk = sub.kk; x.b0 = sub.b0; x.bid = sub.bid; x.maxd = 0;
         x.T1 = (Ws * k1 + sub.kk - 1) / sub.kk;
         x.L1 = (int64_t)muldiv_u64((uint64_t)x.T1, (uint64_t)(1000000 + eps_l), 1000000ull);
         x.B = 1 + nv / 1024;
@@ -1610,17 +1688,40 @@ __device__ void e_initial(ECtx &c, const EGraph &g, int k, int64_t eps_ppm, uint
     const int nb = s.cnt, nvmax = s.flag;
     __syncthreads();
     if (nb == 0) break;
-    // deg' inside the subproblem, per list position
+    // the internal rows by list position, each where its node's whole row lies in g, and deg'
     for (int bi = 0; bi < nb; bi++) {
-      const EBis b = bis[bi];
-      for (int j = warp_idx(); j < b.count; j += NW) {
-        const int v = cl[b.start + j];
+      const int start = bis[bi].start, count = bis[bi].count;
+      const int32_t bid = (int32_t)bis[bi].bid;
+      int maxd = 0;
+      for (int j = warp_idx(); j < count; j += NW) {
+        const int v = cl[start + j];
+        const int r0 = g.xadj[v], r1 = g.xadj[v + 1];
+        int at = r0;
         long long d = 0;
-        for (int e = g.xadj[v] + (int)lane_id(); e < g.xadj[v + 1]; e += 32)
-          if (mark[g.adjncy[e]] == (int32_t)b.bid) d += g.adjwgt[e];
+        for (int e0 = r0; e0 < r1; e0 += 32) {
+          const int e = e0 + (int)lane_id();
+          int u = 0, w = 0;
+          bool in = false;
+          if (e < r1) {
+            u = g.adjncy[e];
+            w = g.adjwgt[e];
+            in = mark[u] == bid;
+          }
+          const unsigned m = __ballot_sync(FULL, in);
+          if (in) {
+            adj[at + __popc(m & lanemask_lt())] = make_int2(loc[u], w);
+            d += w;
+          }
+          at += __popc(m);
+        }
         d = warp_sum(d);
-        if (lane_id() == 0) Dp[b.start + j] = (int32_t)d;
+        maxd = max(maxd, (int)d);
+        if (lane_id() == 0) {
+          Dp[start + j] = (int32_t)d;
+          rows[start + j] = make_int2(r0, at);
+        }
       }
+      if (lane_id() == 0) atomicMax(&bis[bi].maxd, maxd);
     }
     // work order: subproblems by size, largest first
     if (threadIdx.x == 0) {
@@ -1636,13 +1737,18 @@ __device__ void e_initial(ECtx &c, const EGraph &g, int k, int64_t eps_ppm, uint
     const int slots = items < NW ? items : NW;
     const int64_t dmark = c.ar.hi;
     const int nchmax = (nvmax + 63) >> 6;
-    int32_t *conn = c.ar.s<int32_t>((int64_t)slots * nvmax);
-    uint64_t *key = c.ar.s<uint64_t>((int64_t)slots * nvmax);
-    uint8_t *st = c.ar.s<uint8_t>((int64_t)slots * nvmax);
-    uint64_t *cmax = c.ar.s<uint64_t>((int64_t)slots * nchmax);
-    int32_t *tkn = c.ar.s<int32_t>((int64_t)slots * (1 + nvmax / 1024));
-    if (c.ar.fail) return;
+    // each warp's share of the shared tables holds its trial's words and chunk maxima if they fit, else the
+    // maxima alone if they do (32-bit ones always: at most 512 of them)
     const int w = warp_idx();
+    const int64_t share = (int64_t)smem_bytes((int)blockDim.x) / slots & ~(int64_t)15;
+    unsigned char *const sm = reinterpret_cast<unsigned char *>(c.wtk) + (w < slots ? w : 0) * share;
+    const bool outside = 8 * ((int64_t)nvmax + nchmax) > share;  // some trial may need the arena
+    long long *gx = c.ar.s<long long>(outside ? (int64_t)slots * nvmax : 1);
+    long long *gbest = c.ar.s<long long>(outside ? (int64_t)slots * nchmax : 1);
+    uint2 *ford = c.ar.s<uint2>((int64_t)slots * nvmax);
+    int32_t *fcur = c.ar.s<int32_t>((int64_t)slots * (nvmax / kBucketNodes + 1));
+    int32_t *tkn = c.ar.s<int32_t>((int64_t)slots * (1 + nvmax / 1024));
+    if (c.ar.fail) { e_clear_tables(c); return; }
     if (w < slots) {
       for (;;) {
         int it = 0;
@@ -1652,11 +1758,30 @@ __device__ void e_initial(ECtx &c, const EGraph &g, int k, int64_t eps_ppm, uint
         const int bi = ord[it / trials], t = it % trials;
         const EBis b = bis[bi];
         const uint64_t kip = stream_key(seed, TAG_IP, 0, b.bid);
-        const long long cut =
-            ip_trial(g, cl + b.start, cw + b.start, Dp + b.start, mark, loc, b, t, kip,
-                     conn + (int64_t)w * nvmax, key + (int64_t)w * nvmax, st + (int64_t)w * nvmax,
-                     cmax + (int64_t)w * nchmax, tkn + (int64_t)w * (1 + nvmax / 1024),
-                     side + (int64_t)t * n + b.start);
+        const ETrial tr{cl + b.start, cw + b.start, Dp + b.start, rows + b.start, adj,
+                        ford + (int64_t)w * nvmax, fcur + (int64_t)w * (nvmax / kBucketNodes + 1),
+                        tkn + (int64_t)w * (1 + nvmax / 1024)};
+        uint8_t *const sd = side + (int64_t)t * n + b.start;
+        const int nch = (b.count + kChunkNodes - 1) / kChunkNodes;
+        const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(sm);
+        long long cut;
+        if (b.count < kNarrowNodes && b.maxd < kNarrowGain) {
+          const Words<int32_t, true> best{s0};
+          if (4 * ((int64_t)b.count + nch) <= share)
+            cut = ip_trial<int32_t>(Words<int32_t, true>{s0 + 4 * nch}, best, tr, b, t, kip, sd);
+          else
+            cut = ip_trial<int32_t>(EWords<int32_t>{reinterpret_cast<int32_t *>(gx + (int64_t)w * nvmax)}, best, tr, b,
+                                    t, kip, sd);
+        } else {
+          const Words<long long, true> best{s0};
+          const EWords<long long> X{gx + (int64_t)w * nvmax};
+          if (8 * ((int64_t)b.count + nch) <= share)
+            cut = ip_trial<long long>(Words<long long, true>{s0 + 8 * nch}, best, tr, b, t, kip, sd);
+          else if (8 * (int64_t)nch <= share)
+            cut = ip_trial<long long>(X, best, tr, b, t, kip, sd);
+          else
+            cut = ip_trial<long long>(X, Words<long long, false>{gbest + (int64_t)w * nchmax}, tr, b, t, kip, sd);
+        }
         if (lane_id() == 0) res[bi * trials + t] = cut;
       }
     }
@@ -1695,7 +1820,7 @@ __device__ void e_initial(ECtx &c, const EGraph &g, int k, int64_t eps_ppm, uint
     ESub *ts = cs; cs = ns; ns = ts;
   }
   c.ar.hi = smark;
-  __syncthreads();
+  e_clear_tables(c);
 }
 
 // R19: while a block exceeds L_max, move from the heaviest block A to the
@@ -1936,9 +2061,7 @@ __device__ void e_context(ECtx &c, unsigned char *esm, ESmem &s, const gp_config
   c.wtv = c.wtk + nw * kEWarpSlots;
   c.btk = c.wtv + nw * kEWarpSlots;
   c.btv = c.btk + kEBlockSlots;
-  for (int t = threadIdx.x; t < nw * kEWarpSlots; t += blockDim.x) { c.wtk[t] = -1; c.wtv[t] = 0; }
-  for (int t = threadIdx.x; t < kEBlockSlots; t += blockDim.x) { c.btk[t] = -1; c.btv[t] = 0; }
-  __syncthreads();
+  e_clear_tables(c);
 }
 
 template <int NT>
