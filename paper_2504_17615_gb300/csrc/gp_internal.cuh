@@ -361,6 +361,16 @@ __device__ __forceinline__ int row_of(const int32_t *xadj, int n, int64_t e) {
   return lo;
 }
 
+// Slot of a key in a table of 2^bits slots that takes a part of a row.  The rows of a contracted graph lie in
+// the slot order of the tables that merged them (a multiplicative hash), so a part of such a row shares its
+// hash's high bits: with the same hash the keys of a 2048-entry part crowd into a few slots and probe hundreds
+// of each other.  The product is therefore folded and multiplied once more.
+__device__ __forceinline__ unsigned part_slot(int key, int bits) {
+  unsigned h = (unsigned)key * 2654435761u;
+  h ^= h >> 15;
+  return (h * 739982445u) >> (32 - bits);
+}
+
 // A walk of one warp over its share of a graph's CSR entries, 32 consecutive rows (a window) at a
 // time.  The entries are split evenly over the warps, not the rows: with 32 rows per warp step one warp
 // walked a hub's whole row (4e5 entries of the scale-24 R-MAT graph) while the rest of the device

@@ -791,7 +791,7 @@ __global__ void __launch_bounds__(kThreads) k_hub_insert(RateArgs a, HubArgs h) 
 #pragma unroll
     for (int r = 0; r < R; r++) {
       if (L[r] < 0) continue;
-      unsigned s = slot_hash(L[r], BITS);
+      unsigned s = part_slot(L[r], BITS);
       for (int probe = 0; probe < 2 * kHubChunk; probe++) {  // bounded: at most half full
         const int prev = atomicCAS(&s_k[s], -1, L[r]);
         if (prev == -1 || prev == L[r]) { atomicAdd(&s_v[s], w[r]); break; }
