@@ -77,9 +77,11 @@ int bits_for(int64_t x);
 
 // The same LP run as lp_run as one cooperative persistent launch (lp_small.cu);
 // for graphs of at most p.small_nodes nodes and kLpSmallMaxEntries entries.  Returns false, with nothing
-// changed, when the graph's hubs make the per-phase driver the faster one.
+// changed, when the graph's hubs make the per-phase driver the faster one.  full (clustering; may be null):
+// nodes that no cluster can have room for.
 bool lp_small_applicable(const DevGraph &g, const LpParams &p);
 bool lp_run_small(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *weight, int64_t nlabels,
-                  uint64_t seed, const LpParams &p, int64_t *nclusters_dev, uint8_t *label8, LpResult &res);
+                  uint64_t seed, const LpParams &p, int64_t *nclusters_dev, uint8_t *label8, const uint8_t *full,
+                  LpResult &res);
 
 }  // namespace gp

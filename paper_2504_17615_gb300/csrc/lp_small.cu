@@ -105,6 +105,7 @@ struct PArgs {
   int64_t m2;
   int32_t *label, *weight;
   uint8_t *label8;
+  const uint8_t *full;   // clustering: nodes that no cluster can have room for, not listed (may be null)
   uint8_t *dirty;        // refinement: per node, 0 = cannot move until a neighbour moves (may be null)
   int64_t nlabels;
   int64_t bound, n_min;
@@ -490,7 +491,7 @@ __global__ void __launch_bounds__(kPThreads, GP_PLP_BLOCKS_PER_SM) k_lp_persiste
       __syncthreads();
       for (int v = gt; v < n; v += gthreads) {
         const int deg = a.xadj[v + 1] - a.xadj[v];
-        if (deg == 0) continue;
+        if (deg == 0 || (a.full && a.full[v])) continue;
         const int sr = (int)(h32(kact, (uint32_t)v, 0) % (uint32_t)a.S);
         atomicAdd(&s_bc[sr * kPClasses + deg_class(deg)], 1);
       }
@@ -526,7 +527,7 @@ __global__ void __launch_bounds__(kPThreads, GP_PLP_BLOCKS_PER_SM) k_lp_persiste
           if (v < n) {
             vst[q] = a.xadj[v];
             vdeg[q] = a.xadj[v + 1] - vst[q];
-            if (vdeg[q] > 0)
+            if (vdeg[q] > 0 && !(a.full && a.full[v]))
               key[q] = (int)(h32(kact, (uint32_t)v, 0) % (uint32_t)a.S) * kPClasses + deg_class(vdeg[q]);
           }
           if (key[q] >= 0) atomicAdd(&s_bc[key[q]], 1);
@@ -1104,7 +1105,8 @@ bool lp_small_applicable(const DevGraph &g, const LpParams &p) {
 }
 
 bool lp_run_small(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *weight, int64_t nlabels,
-                  uint64_t seed, const LpParams &p, int64_t *nclusters_dev, uint8_t *label8, LpResult &res) {
+                  uint64_t seed, const LpParams &p, int64_t *nclusters_dev, uint8_t *label8,
+                  const uint8_t *skip, LpResult &res) {
   res = LpResult{};
   const int n = g.n;
   GP_REQUIRE(p.subrounds >= 1 && p.subrounds <= 64, GP_ERR_INVALID, "lp_subrounds must be in [1, 64]");
@@ -1191,6 +1193,7 @@ bool lp_run_small(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *weigh
   a.xadj = g.xadj; a.adjncy = g.adjncy; a.adjwgt = g.unit_w ? nullptr : g.adjwgt; a.vwgt = g.vwgt; a.n = n;
   a.m2 = g.m2; a.two_inc = two_inc ? 1 : 0;
   a.label = label; a.weight = weight; a.label8 = label8; a.nlabels = nlabels;
+  a.full = skip;
   a.dirty = p.count_clusters ? nullptr : dirty.get();
   a.bound = p.bound; a.n_min = p.n_min; a.count_clusters = p.count_clusters ? 1 : 0;
   a.rounds = p.rounds; a.S = p.subrounds; a.dbg_max = p.dbg_max_subrounds; a.level = p.level;

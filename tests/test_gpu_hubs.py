@@ -3,6 +3,8 @@ table each up to 18432; hubs by many blocks: counted per label up to 1024 labels
 and coarse nodes with long segments in contraction."""
 from __future__ import annotations
 
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -52,6 +54,22 @@ def test_clustering_with_hubs(ctx, name, U):
     cmap, nc, st = ctx.gp_coarsen(gp.DeviceGraph.from_host(g), U, 1, 5, gp.default_config(**HOST_PATH))
     ocmap, onc, ost = orc.coarsen(g, U, 1, 5)
     assert nc == onc and np.array_equal(cmap.cpu().numpy(), ocmap)
+
+
+# nodes that no cluster can have room for are left out: weights around the bound and around half of it, with
+# and without light nodes to take in; the per-phase and the persistent path
+@pytest.mark.parametrize("cfg", [HOST_PATH, {}])
+@pytest.mark.parametrize("weights", [(1, 2, 20, 21, 38, 39, 40), (20, 21, 40), (21, 39, 40), (40,)])
+def test_clustering_with_full_nodes(ctx, weights, cfg):
+    import paper_2504_17615_gb300 as gp
+    for name in ("edges", "star"):
+        g = GRAPHS[name]
+        vw = np.random.default_rng(len(weights)).choice(np.array(weights, dtype=g.vwgt.dtype), g.n)
+        g = dataclasses.replace(g, vwgt=vw)
+        cmap, nc, st = ctx.gp_coarsen(gp.DeviceGraph.from_host(g), 40, 1, 5, gp.default_config(**cfg))
+        ocmap, onc, ost = orc.coarsen(g, 40, 1, 5)
+        assert nc == onc and np.array_equal(cmap.cpu().numpy(), ocmap)
+        assert (st.lp_moves, st.lp_subrounds, st.clusters_lp) == (ost.lp_moves, ost.lp_subrounds, ost.clusters_lp)
 
 
 @pytest.mark.parametrize("name", sorted(GRAPHS))
