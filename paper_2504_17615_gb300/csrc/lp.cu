@@ -901,7 +901,8 @@ __global__ void __launch_bounds__(kThreads) k_hub_table(RateArgs a, HubArgs h) {
 constexpr int kFullUnroll = 8;
 
 __global__ void __launch_bounds__(kThreads) k_mark_full(const int32_t *xadj, const int32_t *adjncy,
-                                                        const int32_t *vwgt, int n, int64_t bound, uint8_t *full) {
+                                                        const int32_t *vwgt, int n, int64_t bound,
+                                                        uint8_t *full) {  // full: zero on entry
   const int lane = (int)lane_id();
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int64_t step = ((int64_t)n + 31) / 32;  // a warp's nodes lie this far apart: hubs have neighbouring ids
@@ -929,7 +930,7 @@ __global__ void __launch_bounds__(kThreads) k_mark_full(const int32_t *xadj, con
       }
       if (lane == l) mark = !fits;
     }
-    if (v < n) full[v] = mark ? 1 : 0;
+    if (mark) full[v] = 1;
   }
 }
 
@@ -1849,6 +1850,7 @@ LpResult lp_run(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *weight,
   if (p.count_clusters && n > 0) {
     ProfScope ps(ctx, PROF_ROUND_SETUP);
     full.reset(ctx, (size_t)n);
+    full.zero();
     k_mark_full<<<grid_for(n, kThreads, ctx->num_sms * 8), kThreads, 0, ctx->stream>>>(g.xadj, g.adjncy, g.vwgt, n,
                                                                                        p.bound, full.get());
     GP_LAUNCH_CHECK();

@@ -64,3 +64,19 @@ def test_fallbacks(ctx, cmax):
             g = gg.with_node_weights(g, cmax)
         graphs += [(g, k, k) for k in (2, 3, 7)]
     _check(ctx, graphs, 512)
+
+
+# without a tuning: small items on the engine, large ones by the predicted time in a CTA, results as single calls
+def test_untuned_split():
+    import paper_2504_17615_gb300 as gp
+    c = gp.Context(0)
+    graphs = [(gp.DeviceGraph.from_host(gg.er(n, 10 * n, n)), k, 0.03, n)
+              for n in (1000, 1638, 1639, 4000, 30000, 60000) for k in (2, 64)]
+    graphs.append((gp.DeviceGraph.from_host(gg.rmat(16, 16, seed=2)), 8, 0.03, 1))
+    res = c.gp_partition_batch(graphs, details=True)
+    assert all(r[2] for r, j in zip(res, graphs) if j[0].m2 <= 1 << 15)
+    assert not all(r[2] for r in res)
+    for (blocks, cut, _, _), (g, k, eps, seed) in zip(res, graphs):
+        want, want_cut, _ = c.gp_partition(g, k, eps, seed)
+        assert cut == want_cut and np.array_equal(blocks.cpu().numpy(), want.cpu().numpy())
+    c.close()
