@@ -391,7 +391,7 @@ struct EntryWalk {
     const int64_t per = (((hi - lo + nw - 1) / nw) + 31) & ~(int64_t)31;
     pos = lo + per * wid;
     end = pos + per < hi ? pos + per : hi;
-    row = pos < end ? find(pos) : 0;
+    row = pos < end ? first(lo, hi) : 0;
     u0 = 0; e0 = e1 = xe = 0; no_empty = false;
   }
   __device__ __forceinline__ bool next() {
@@ -414,6 +414,14 @@ struct EntryWalk {
       return true;
     }
     return false;
+  }
+  // Row of entry pos: where even degrees would put it, else by the search.
+  __device__ __forceinline__ int64_t first(int64_t lo, int64_t hi) const {
+    int64_t g = (int64_t)((float)(pos - lo) / (float)(hi - lo) * (float)n) - 16;
+    g = g < 0 ? 0 : g > n ? n : g;
+    const int64_t p = g + lane_id();
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, p < n && (int64_t)xadj[p] <= pos);
+    return (m & 1) && m != 0xFFFFFFFFu ? g + __popc(m) - 1 : find(pos);
   }
   // Row of entry e (xadj[0] <= e < xadj[n]); the whole warp asks for the same e.
   __device__ __forceinline__ int64_t find(int64_t e) const {
@@ -447,9 +455,15 @@ struct EntryWalk {
   }
 };
 
-// Blocks of 256 threads for an EntryWalk over m2 entries: at least 2048 entries a warp, so that the
-// search for its first row stays a small part, and at most 16 blocks an SM.
-inline int walk_grid(int64_t m2, int num_sms) { return grid_for(m2, 8 * 2048, num_sms * 16); }
+// Blocks of 256 threads for an EntryWalk over m2 entries: 96 entries a warp (the 32 rows of a mesh hold 128) until
+// every SM holds four blocks, then more entries a warp up to 512, then more blocks up to 16 an SM.  With
+// 2048 entries a warp throughout, small graphs kept a few SMs busy with chains of a dozen steps (a drawn
+// scoring case 334 us, ER partition of 65,536 nodes 7.69 ms, now 7.5); with 128 to 512 entries a warp small meshes'
+// kernels took a second window's chain, some 3 us each.
+inline int walk_grid(int64_t m2, int num_sms) {
+  const int64_t b = m2 / (8 * 96) < 4 * (int64_t)num_sms ? m2 / (8 * 96) : 4 * (int64_t)num_sms;
+  return grid_for(b * 256 > m2 / 16 ? b * 256 : m2 / 16, 256, num_sms * 16);
+}
 
 // ---------------------------------------------------------- primitives
 

@@ -124,8 +124,10 @@ void modularity(gp_ctx *ctx, const DevGraph &g, const int32_t *labels, int32_t n
   vol.zero();
   o.zero();
   if (g.n > 0) {
-    const int nsh = nlabels <= kModShared ? nlabels : 0;
-    k_mod_rows<<<walk_grid(g.m2, ctx->num_sms), 256, sizeof(unsigned long long) * nsh, ctx->stream>>>(
+    // per-block volumes pay when a block has several rows a cluster; small graphs add directly
+    const int grid = walk_grid(g.m2, ctx->num_sms);
+    const int nsh = nlabels <= kModShared && g.n / grid >= 2 * nlabels ? nlabels : 0;
+    k_mod_rows<<<grid, 256, sizeof(unsigned long long) * nsh, ctx->stream>>>(
         g.xadj, g.adjncy, g.adjwgt, labels, g.n, nlabels, nsh, vol.get(), o.get());
     GP_LAUNCH_CHECK();
   }
