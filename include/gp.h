@@ -127,7 +127,8 @@ gp_status gp_create(gp_ctx **ctx, int device, void *stream, const gp_allocator *
 void gp_destroy(gp_ctx *ctx);
 /*
  * Upper bound on the iterations of every grid-wide wait inside the library's
- * persistent kernels (the small-graph label propagation).  A wait that runs
+ * persistent kernels (the small-graph label propagation; graphs of a few
+ * thousand nodes run in one block, without such waits).  A wait that runs
  * out makes the call return GP_ERR_TIMEOUT; the context stays usable and the
  * call's outputs are undefined.  spins = 0 restores the default (several
  * seconds of waiting); spins < 0 makes every wait give up at once (tests).
@@ -322,7 +323,10 @@ gp_status gp_partition_batch(gp_ctx *ctx, gp_batch_item *items, int32_t count, i
  * readings as gp_partition, so the results are identical -- with its hierarchy
  * and scratch in a per-CTA arena.  The other items, and engine items whose
  * hierarchy outgrows the arena, run on the per-graph path (the worker
- * contexts above), after the engine.  The configuration must use a sparsifier
+ * contexts above), beside the engine or (the latter) after it.  Until a tuning
+ * is set or measured, the defaults are narrowed per batch: beyond 2^15 entries
+ * the engine takes only the items up to a predicted time in their CTA, chosen
+ * so that the slower of the two paths ends first.  The configuration must use a sparsifier
  * other than GP_SPARSIFY_TWEIGHT_EXACT, at most 254 sub-rounds and at least one
  * bisection trial; otherwise every item takes the per-graph path.
  *
