@@ -107,13 +107,6 @@ __device__ __forceinline__ unsigned long long wmin64(unsigned long long x) {
   return ((unsigned long long)mh << 32) | ml;
 }
 
-__device__ __forceinline__ unsigned long long wmax64(unsigned long long x) {
-  const unsigned hi = (unsigned)(x >> 32);
-  const unsigned mh = __reduce_max_sync(FULL, hi);
-  const unsigned ml = __reduce_max_sync(FULL, hi == mh ? (unsigned)x : 0u);
-  return ((unsigned long long)mh << 32) | ml;
-}
-
 __device__ unsigned long long blk_min_u64(unsigned long long x, ESmem &s) {
   x = wmin64(x);
   __syncthreads();

@@ -457,8 +457,8 @@ struct EntryWalk {
 
 // Blocks of 256 threads for an EntryWalk over m2 entries: 96 entries a warp (the 32 rows of a mesh hold 128) until
 // every SM holds four blocks, then more entries a warp up to 512, then more blocks up to 16 an SM.  With
-// 2048 entries a warp throughout, small graphs kept a few SMs busy with chains of a dozen steps (a drawn
-// scoring case 334 us, ER partition of 65,536 nodes 7.69 ms, now 7.5); with 128 to 512 entries a warp small meshes'
+// 2048 entries a warp throughout, small graphs kept a few SMs busy with chains of a dozen steps (a small
+// graph's scoring took 334 us against 201 with a warp per 32 rows; ER partition of 65,536 nodes 7.69 -> 7.5 ms); with 128 to 512 entries a warp small meshes'
 // kernels took a second window's chain, some 3 us each.
 inline int walk_grid(int64_t m2, int num_sms) {
   const int64_t b = m2 / (8 * 96) < 4 * (int64_t)num_sms ? m2 / (8 * 96) : 4 * (int64_t)num_sms;
