@@ -37,20 +37,17 @@ __device__ __forceinline__ unsigned slot_hash(int B, int bits) {
   return ((unsigned)B * 2654435761u) >> (32 - bits);
 }
 
-__device__ __forceinline__ void table_add(int *tk, int *tv, int mask, int bits, int B, int w) {
+__device__ __forceinline__ void table_add(int *tk, int *tv, unsigned mask, int bits, int B, int w) {
   unsigned s = slot_hash(B, bits);
-  for (int probe = 0; probe <= mask; probe++) {  // bounded: the table never fills
+  for (unsigned probe = 0; probe <= mask; probe++) {  // bounded: more slots than keys
     const int prev = atomicCAS(&tk[s], -1, B);
     if (prev == -1 || prev == B) { atomicAdd(&tv[s], w); return; }
-    s = (s + 1) & (unsigned)mask;
+    s = (s + 1) & mask;
   }
 }
 
-__device__ __forceinline__ int table_bits(int entries) {
-  int bits = 5;
-  while ((1 << bits) < 2 * entries) bits++;
-  return bits;
-}
+// Distinct neighbours that a segment of len entries can have: no more than there are coarse nodes.
+__host__ __device__ __forceinline__ int seg_keys(int len, int nc) { return len < nc ? len : nc; }
 
 // Segment length (the member rows' total length) and weight of every coarse
 // node; moff[v] = offset of v's row inside its coarse node's segment.
@@ -142,7 +139,7 @@ __global__ void __launch_bounds__(kThreads) k_merge_warp(MergeArgs a) {
       }
       continue;
     }
-    const int bits = table_bits(len), tsize = 1 << bits;
+    const int bits = table_bits(len, 5), tsize = 1 << bits;
     for (int i0 = s0; i0 < s1; i0 += 64) {  // two entries per lane in flight
       const int i1 = i0 + lane, i2 = i0 + 32 + lane;
       const int2 x1 = i1 < s1 ? __ldcs(a.temp + i1) : make_int2(-1, 0);
@@ -183,11 +180,12 @@ __global__ void __launch_bounds__(kThreads) k_merge_block(MergeArgs a) {
   for (int li = blockIdx.x; li < nl; li += gridDim.x) {
     const int A = a.large[li];
     const int s0 = a.tstart[A], s1 = a.tstart[A + 1];
-    const int bits = table_bits(s1 - s0), tsize = 1 << bits;
+    const int bits = table_bits(seg_keys(s1 - s0, a.nc), 5);
+    const unsigned tsize = 1u << bits;
     const bool in_smem = tsize <= kBlockSmemSlots;
     int *tk = in_smem ? s_k : gk;
     int *tv = in_smem ? s_v : gv;
-    for (int t = threadIdx.x; t < tsize; t += blockDim.x) { tk[t] = -1; tv[t] = 0; }
+    for (unsigned t = threadIdx.x; t < tsize; t += blockDim.x) { tk[t] = -1; tv[t] = 0; }
     if (threadIdx.x == 0) s_cnt = 0;
     __syncthreads();
     for (int i = s0 + threadIdx.x; i < s1; i += blockDim.x) {
@@ -195,7 +193,7 @@ __global__ void __launch_bounds__(kThreads) k_merge_block(MergeArgs a) {
       if (x.x >= 0) table_add(tk, tv, tsize - 1, bits, x.x, x.y);
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < tsize; t += blockDim.x) {
+    for (unsigned t = threadIdx.x; t < tsize; t += blockDim.x) {
       const int key = tk[t];
       if (key >= 0) a.temp[s0 + atomicAdd(&s_cnt, 1)] = make_int2(key, tv[t]);
     }
@@ -209,14 +207,11 @@ __global__ void __launch_bounds__(kThreads) k_merge_block(MergeArgs a) {
   if (a.units && threadIdx.x == 0) atomicAdd(a.units + 3, uout);
 }
 
-// Longest segment, number of huge ones and their entries.
+// Longest segment, number of huge ones and the keys their tables have to hold.
 struct SegStats {
   int longest, huge;
-  unsigned long long entries;
+  unsigned long long keys;
 };
-
-// Slots of a huge segment's table, q4 quarters of a slot an entry.
-__device__ __forceinline__ int seg_slots(int len, int q4) { return (int)((int64_t)len * q4 / 4 + 1); }
 
 __global__ void k_seg_stats(const int32_t *x, int n, SegStats *out) {
   int m = 0, nh = 0;
@@ -225,14 +220,14 @@ __global__ void k_seg_stats(const int32_t *x, int n, SegStats *out) {
        i += (int64_t)gridDim.x * blockDim.x) {
     const int l = x[i];
     m = l > m ? l : m;
-    if (l > kHugeSeg) { nh++; ns += (unsigned long long)l; }
+    if (l > kHugeSeg) { nh++; ns += (unsigned long long)seg_keys(l, n); }
   }
   m = warp_max(m);
   if (lane_id() == 0 && m) atomicMax(&out->longest, m);
   if (__any_sync(FULL, nh)) {
     nh = warp_sum(nh);
     ns = warp_sum(ns);
-    if (lane_id() == 0) { atomicAdd(&out->huge, nh); atomicAdd(&out->entries, ns); }
+    if (lane_id() == 0) { atomicAdd(&out->huge, nh); atomicAdd(&out->keys, ns); }
   }
 }
 
@@ -242,7 +237,8 @@ __global__ void k_seg_stats(const int32_t *x, int n, SegStats *out) {
 // global memory took milliseconds for it while the rest of the device waited (12 levels of the scale-24
 // R-MAT graph: 131 ms of contraction).  k_seg_plan lists the huge segments with the prefix sums of their
 // chunks, k_seg_insert sums 2048 entries at a time in a shared table and adds the sums to the segment's
-// table in global memory (two slots an entry where the memory bound allows; one 64-bit exchange claims a
+// table in global memory (two slots a key where the memory bound allows, a key being an entry or, if there are
+// fewer of them, a coarse node; one 64-bit exchange claims a
 // slot), and k_seg_extract writes the occupied slots back to the
 // segment.  Consecutive steps work on the same few tables, which stay in L2 meanwhile.
 
@@ -255,7 +251,7 @@ struct SegArgs {
   Seg *segs;
   int *chunk0, *tchunk0;  // prefix sums of entry chunks and table chunks; [count] = totals
   int2 *tab;              // (coarse neighbour, weight) slots
-  int q4;                 // slots an entry, in quarters
+  int q4;                 // slots a key, in quarters
 };
 
 __global__ void __launch_bounds__(1024) k_seg_plan(MergeArgs a, SegArgs h) {
@@ -270,9 +266,9 @@ __global__ void __launch_bounds__(1024) k_seg_plan(MergeArgs a, SegArgs h) {
       x.A = a.large[a.nc - i];
       x.s0 = a.tstart[x.A];
       x.len = a.tstart[x.A + 1] - x.s0;
-      x.tsize = seg_slots(x.len, h.q4);
+      x.tsize = tab_slots(seg_keys(x.len, a.nc), h.q4);
     }
-    const long long val[3] = {(x.len + kSegChunk - 1) / kSegChunk, (x.tsize + kSegTabChunk - 1) / kSegTabChunk, x.tsize};
+    const long long val[3] = {chunks_of(x.len, kSegChunk), chunks_of(x.tsize, kSegTabChunk), x.tsize};
     long long ex[3];
 #pragma unroll
     for (int q = 0; q < 3; q++) {
@@ -335,13 +331,14 @@ __global__ void __launch_bounds__(kThreads) k_seg_insert(MergeArgs a, SegArgs h)
     const int si = seg_of(h.chunk0, cnt, it);
     const Seg x = h.segs[si];
     int2 *tab = h.tab + x.toff;
-    const int c0 = (it - h.chunk0[si]) * kSegChunk, c1 = min(x.len, c0 + kSegChunk);
+    const int c0 = (it - h.chunk0[si]) * kSegChunk, left = min(x.len - c0, kSegChunk);
+    const int2 *in = a.temp + x.s0 + c0;
     constexpr int R = kSegChunk / kThreads;
     int2 e[R];
 #pragma unroll
     for (int r = 0; r < R; r++) {
-      const int j = c0 + r * kThreads + (int)threadIdx.x;
-      e[r] = j < c1 ? __ldcs(a.temp + x.s0 + j) : make_int2(-1, 0);
+      const int j = r * kThreads + (int)threadIdx.x;
+      e[r] = j < left ? __ldcs(in + j) : make_int2(-1, 0);
     }
     __syncthreads();  // the shared table is empty
 #pragma unroll
@@ -355,7 +352,7 @@ __global__ void __launch_bounds__(kThreads) k_seg_insert(MergeArgs a, SegArgs h)
       s_k[t] = -1;
       s_v[t] = 0;
       int s = (int)__umulhi((unsigned)B * 2654435761u, (unsigned)x.tsize);
-      for (int probe = 0; probe < x.tsize; probe++) {  // bounded: more slots than entries
+      for (int probe = 0; probe < x.tsize; probe++) {  // bounded: more slots than keys
         const unsigned long long prev = atomicCAS((unsigned long long *)&tab[s], kEmptySlot,
                                                   ((unsigned long long)(unsigned)w << 32) | (unsigned)B);
         if (prev == kEmptySlot) break;
@@ -452,8 +449,6 @@ void contract_graph(gp_ctx *ctx, const DevGraph &g, const int32_t *cmap, int32_t
   GP_LAUNCH_CHECK();
   SegStats hs;
   read_back(ctx, sstats.get(), sizeof(hs), &hs);
-  int bits = 1;
-  while ((1 << bits) < 2 * hs.longest) bits++;
   int lblocks = ctx->num_sms * 4;
   DBuf<int32_t> gk, gv;
   SegArgs sg{};
@@ -461,8 +456,8 @@ void contract_graph(gp_ctx *ctx, const DevGraph &g, const int32_t *cmap, int32_t
   DBuf<int> chunk0, tchunk0;
   DBuf<int2> tab;
   int64_t slots = 0;
-  for (sg.q4 = 8; sg.q4 > 4; sg.q4--) {  // two slots an entry down to one and a quarter
-    slots = (int64_t)hs.entries * sg.q4 / 4 + hs.huge;
+  for (sg.q4 = 8; sg.q4 > 4; sg.q4--) {  // two slots a key down to one and a quarter
+    slots = (int64_t)hs.keys * sg.q4 / 4 + hs.huge;
     if (slots <= g.m2 + ((int64_t)2 << 20)) break;
   }
   a.split_huge = hs.huge > 0 && sg.q4 > 4 ? 1 : 0;
@@ -472,7 +467,7 @@ void contract_graph(gp_ctx *ctx, const DevGraph &g, const int32_t *cmap, int32_t
     tchunk0.reset(ctx, (size_t)hs.huge + 1);
     tab.reset(ctx, (size_t)slots);
     sg = SegArgs{segs.get(), chunk0.get(), tchunk0.get(), tab.get(), sg.q4};
-  } else if ((1 << bits) > kBlockSmemSlots) {
+  } else if (const int bits = table_bits(seg_keys(hs.longest, nc), 5); ((int64_t)1 << bits) > kBlockSmemSlots) {
     a.gstride = (int64_t)1 << bits;
     lblocks = table_blocks(g.m2, a.gstride, lblocks);
     gk.reset(ctx, (size_t)(a.gstride * lblocks));

@@ -272,11 +272,6 @@ __global__ void __launch_bounds__(128, D <= 16 ? 8 : 6) k_rate_bytes(RateArgs a)
 
 constexpr int kWarpUnroll = 4;
 
-// Slots of a table for deg labels, q4 quarters of a slot each (more than deg, so that no table fills).
-__host__ __device__ __forceinline__ int tab_slots(int deg, int q4) {
-  const int64_t s = (int64_t)deg * q4 / 4 + 1;
-  return s > 0x7FFFFFF0 ? 0x7FFFFFF0 : (int)s;
-}
 constexpr int kTabQ4 = 8;     // shared tables: two slots per neighbour ...
 constexpr int kTabQ4Last = 6; // ... one and a half in the largest class (an SM's whole shared memory)
 
