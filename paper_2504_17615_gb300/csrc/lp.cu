@@ -400,9 +400,8 @@ __global__ void __launch_bounds__(kThreads) k_rate_large(RateArgs a) {
       continue;
     }
     const int own = label_of(a, v);
-    int bits = 1;
-    while ((1 << bits) < 2 * deg) bits++;
-    const int tsize = 1 << bits;
+    const int bits = table_bits(deg, 1);
+    const unsigned tsize = 1u << bits;
     const bool in_smem = tsize <= kLargeSmemSlots;
     int *tk = in_smem ? s_k : gk;
     int *tv = in_smem ? s_v : gv;
@@ -410,15 +409,15 @@ __global__ void __launch_bounds__(kThreads) k_rate_large(RateArgs a) {
       const int L = label_of(a, __ldcs(a.adjncy + start + j));
       const int w = a.adjwgt ? __ldcs(a.adjwgt + start + j) : 1;
       unsigned s = slot_hash(L, bits);
-      for (int probe = 0; probe < tsize; probe++) {  // bounded: the table never fills
+      for (unsigned probe = 0; probe < tsize; probe++) {  // bounded: the table never fills
         const int prev = atomicCAS(&tk[s], -1, L);
         if (prev == -1 || prev == L) { atomicAdd(&tv[s], w); break; }
-        s = (s + 1) & (unsigned)(tsize - 1);
+        s = (s + 1) & (tsize - 1);
       }
     }
     __syncthreads();
     int own_loc = 0, rloc = -1, nc = 0, rall = 0;
-    for (int t = threadIdx.x; t < tsize; t += blockDim.x) {
+    for (unsigned t = threadIdx.x; t < tsize; t += blockDim.x) {
       const int L = tk[t];
       if (L < 0) continue;
       const int r = tv[t];
@@ -438,7 +437,7 @@ __global__ void __launch_bounds__(kThreads) k_rate_large(RateArgs a) {
     if (threadIdx.x == 0) { ue += deg; uv += 1; }
     if (!(rmax < 0 || (MODE == RATE_LP && rmax <= own_r))) {
       uint64_t packed = ~0ull;
-      for (int t = threadIdx.x; t < tsize; t += blockDim.x) {
+      for (unsigned t = threadIdx.x; t < tsize; t += blockDim.x) {
         const int L = tk[t];
         if (L < 0 || L == own || tv[t] != rmax) continue;
         if (MODE == RATE_LP && (int64_t)a.weight[L] + cv > a.bound) continue;
@@ -451,7 +450,7 @@ __global__ void __launch_bounds__(kThreads) k_rate_large(RateArgs a) {
       a.prop[i] = make_int2(-1, 0);
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < tsize; t += blockDim.x) { tk[t] = -1; tv[t] = 0; }
+    for (unsigned t = threadIdx.x; t < tsize; t += blockDim.x) { tk[t] = -1; tv[t] = 0; }
     __syncthreads();
   }
   add_units(a.units, ue, uv, uc, up, a.label8 != nullptr, a.adjwgt == nullptr);
@@ -632,7 +631,7 @@ __global__ void __launch_bounds__(1024) k_hub_plan(RateArgs a, HubArgs h) {
       x.rmax = -1;
       x.best = ~0ull;
     }
-    const long long val[3] = {(deg + kHubChunk - 1) / kHubChunk, (x.tsize + kHubTabChunk - 1) / kHubTabChunk, x.tsize};
+    const long long val[3] = {chunks_of(deg, kHubChunk), chunks_of(x.tsize, kHubTabChunk), x.tsize};
     long long ex[3];
 #pragma unroll
     for (int q = 0; q < 3; q++) {
@@ -720,7 +719,7 @@ __global__ void __launch_bounds__(kThreads) k_hub_dense(RateArgs a, HubArgs h) {
     }
     __threadfence();
     __syncthreads();
-    const int chunks = (x.deg + kHubChunk - 1) / kHubChunk;
+    const int chunks = chunks_of(x.deg, kHubChunk);
     if (threadIdx.x == 0) {
       s_last = atomicAdd(&h.hubs[hi].done, 1) == chunks - 1;
       ue += c1 - c0;
@@ -873,7 +872,7 @@ __global__ void __launch_bounds__(kThreads) k_hub_table(RateArgs a, HubArgs h) {
       if (threadIdx.x == 0) {
         if (packed != ~0ull) atomicMin(&hp->best, packed);
         __threadfence();
-        const int chunks = (hp->tsize + kHubTabChunk - 1) / kHubTabChunk;
+        const int chunks = chunks_of(hp->tsize, kHubTabChunk);
         if (atomicAdd(&hp->done, 1) == chunks - 1) {
           __threadfence();
           uv += 1;
@@ -1684,8 +1683,6 @@ void make_tables(gp_ctx *ctx, const DevGraph &g, int64_t nlabels, RateTables &t)
   DegStats h;
   read_back(ctx, ds.get(), sizeof(h), &h);
   const int maxdeg = h.maxdeg;
-  int bits = 1;
-  while ((1 << bits) < 2 * maxdeg) bits++;
   t.blocks = ctx->num_sms * 4;
   if (nlabels > 0) {
     const int64_t cap = (8 * g.m2 + ((int64_t)16 << 20)) / (int64_t)sizeof(int2);
@@ -1712,7 +1709,8 @@ void make_tables(gp_ctx *ctx, const DevGraph &g, int64_t nlabels, RateTables &t)
     }
     if (t.hubs || maxdeg <= kHubDeg) return;
   }
-  if ((1 << bits) > kLargeSmemSlots) {
+  const int bits = table_bits(maxdeg, 1);
+  if (((int64_t)1 << bits) > kLargeSmemSlots) {
     t.stride = (int64_t)1 << bits;
     t.blocks = table_blocks(g.m2, t.stride, t.blocks);
     t.gkeys.reset(ctx, (size_t)(t.stride * t.blocks));

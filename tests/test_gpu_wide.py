@@ -45,3 +45,22 @@ def test_contraction_to_few_nodes(ctx, ring, parts):
     rows = [i for i in range(nc) for _ in range(nc - 1)]
     assert sorted(zip(rows, got.adjncy.tolist())) == [(i, j) for i in range(nc) for j in range(nc) if i != j]
     assert got.adjwgt.tolist() == [2 * cross if nc == 2 else cross] * len(rows)
+
+
+# the centre's row, 2^29 + 2 entries, is rated within the eight sub-rounds; a cluster holds two nodes
+def test_clustering_of_a_wide_star(ctx):
+    import torch
+    import paper_2504_17615_gb300 as gp
+    leaves = (1 << 29) + 2
+    n = leaves + 1
+    adj = torch.zeros(2 * leaves, dtype=torch.int32, device="cuda")
+    adj[:leaves] = torch.arange(1, n, dtype=torch.int32, device="cuda")
+    xadj = torch.arange(leaves - 1, leaves + n, dtype=torch.int32, device="cuda")
+    xadj[0] = 0
+    one = torch.ones(2 * leaves, dtype=torch.int32, device="cuda")
+    g = gp.DeviceGraph(n, 2 * leaves, xadj, adj, one[:n], one)
+    cmap, nc, st = ctx.gp_coarsen(g, 2, 1, 5, gp.default_config(dbg_max_subrounds=8, two_hop=0))
+    size = torch.zeros(nc, dtype=torch.int32, device="cuda").scatter_add_(0, cmap.long(), one[:n])
+    assert st.lp_subrounds == 8 and 0 < st.lp_moves <= 16  # each sub-round: a leaf to the centre, the centre to a leaf
+    assert int(size.min()) >= 1 and int(size.max()) == 2
+    assert st.clusters_lp == st.clusters_final == nc and n - 9 <= nc < n
