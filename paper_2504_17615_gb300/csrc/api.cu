@@ -77,6 +77,9 @@ void gp_set_wait_limit(gp_ctx *ctx, int64_t spins) {
   if (ctx) ctx->wait_spins = spins;
 }
 
+// For tests, not part of the C-ABI (gp.h): the context's Limits.
+void gp_test_limits(gp_ctx *ctx, int32_t hash_collect) { ctx->limits.hash_collect = hash_collect; }
+
 const char *gp_version(void) { return "gp-gb300 1.0 (sm_103a)"; }
 
 int64_t gp_launch_count(void) { return gp::g_launch_count.load(); }

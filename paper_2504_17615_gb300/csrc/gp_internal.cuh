@@ -94,6 +94,16 @@ struct ProfRecord {
 
 // ------------------------------------------------------------------ context
 
+namespace gp {
+
+// Sizes at which a context changes its way of working, never its results; gp_test_limits lowers them, so that
+// small graphs reach what otherwise only very large ones do.
+struct Limits {
+  int32_t hash_collect = 16384;  // exact sampler: edges fetched and ordered on the host
+};
+
+}  // namespace gp
+
 struct gp_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -119,6 +129,7 @@ struct gp_ctx {
   gp_batch_tuning tuning{};        // batched engine settings (gp_batch_set_tuning / gp_batch_autotune)
   bool tuning_set = false;         // tuning holds values (defaults or the caller's)
   bool tuning_given = false;       // ... the caller's or the autotuner's: the engine's share is as they say
+  gp::Limits limits;
   cudaStream_t copy_streams[4] = {};  // host-to-device copies of large inputs
   cudaEvent_t copy_events[5] = {};
 };

@@ -195,11 +195,9 @@ __global__ void __launch_bounds__(256) k_hash_digit(HashHistArgs a) {
 // The r-th smallest (1-based) 64-bit hash among the edges of weight wt, and the
 // edge that closes the kept prefix when several edges share that hash.  After
 // a digit, the edges that share the prefix are as a rule few (a 2048th of
-// them): once at most kHashCollect are left they are fetched and ordered on the
+// them): once at most 16384 (Limits) are left they are fetched and ordered on the
 // host, two passes over the entries instead of six (a level of 299,993 weighted
 // nodes 2.29 -> 1.91 ms).
-constexpr int kHashCollect = 16384;
-
 void exact_boundary(gp_ctx *ctx, const DevGraph &g, int32_t wt, uint64_t key, int64_t r, uint64_t *t_out,
                     uint32_t *blo, uint32_t *bhi) {
   const int digits[6][2] = {{53, 11}, {42, 11}, {31, 11}, {20, 11}, {10, 10}, {0, 10}};  // (shift, bits)
@@ -210,7 +208,7 @@ void exact_boundary(gp_ctx *ctx, const DevGraph &g, int32_t wt, uint64_t key, in
   uint64_t prefix = 0;
   int64_t below = 0, equal = 0;  // edges below the prefix, edges that have it
   int bits = 0;
-  for (int d = 0; d < 6 && (d == 0 || equal > kHashCollect); d++) {
+  for (int d = 0; d < 6 && (d == 0 || equal > ctx->limits.hash_collect); d++) {
     a.shift = digits[d][0];
     a.nbits = digits[d][1];
     a.prefix = prefix;
