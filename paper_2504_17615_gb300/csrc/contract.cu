@@ -6,7 +6,7 @@
 //  reserve: every fine node reserves room for its row inside its coarse
 //           node's segment (an atomic add on the segment length returns the
 //           node's offset) and adds its weight to the coarse node;
-//  map    : the fine entries are split evenly over the warps (EntryWalk),
+//  map    : rows and entries are split evenly over the warps (EntryWalk),
 //           which write (coarse id of the neighbour, weight) into the owner's
 //           segment; entries inside the cluster are marked;
 //  merge  : each segment is summed by coarse neighbour in a hash table (a
@@ -76,28 +76,29 @@ __global__ void __launch_bounds__(kThreads) k_map(const int32_t *xadj, const int
     int A = -2, base = 0;
     if (u < n) {
       A = cmap[u];
-      base = tstart[A] + moff[u] - xadj[u];
+      base = tstart[A] + moff[u] - wk.xs;
     }
-    const int e0 = wk.e0, e1 = wk.e1;
-    if (lane == 0) ue += (unsigned long long)(e1 - e0);
+    const int e1 = wk.e1;
+    if (lane == 0) ue += (unsigned long long)(e1 - wk.e0);
     // kMapUnroll entries per lane in flight: ids, then coarse ids, then the writes
-    for (int f0 = e0; f0 < e1; f0 += 32 * kMapUnroll) {
-      int e[kMapUnroll], bj[kMapUnroll], Aj[kMapUnroll], nb[kMapUnroll];
+    walk_entries<kMapUnroll>(wk.e0, e1, [&](auto steps, int f0) {
+      constexpr int R = decltype(steps)::value;
+      int e[R], bj[R], Aj[R], nb[R];
 #pragma unroll
-      for (int r = 0; r < kMapUnroll; r++) {
+      for (int r = 0; r < R; r++) {
         e[r] = f0 + r * 32 + lane;
         const int j = wk.owner(f0 + r * 32);
         bj[r] = __shfl_sync(FULL, base, j);
         Aj[r] = __shfl_sync(FULL, A, j);
       }
 #pragma unroll
-      for (int r = 0; r < kMapUnroll; r++) nb[r] = e[r] < e1 ? __ldcs(adjncy + e[r]) : 0;  // read once: evict first
+      for (int r = 0; r < R; r++) nb[r] = e[r] < e1 ? __ldcs(adjncy + e[r]) : 0;  // read once: evict first
 #pragma unroll
-      for (int r = 0; r < kMapUnroll; r++) nb[r] = e[r] < e1 ? cmap[nb[r]] : 0;
+      for (int r = 0; r < R; r++) nb[r] = e[r] < e1 ? cmap[nb[r]] : 0;
 #pragma unroll
-      for (int r = 0; r < kMapUnroll; r++)
+      for (int r = 0; r < R; r++)
         if (e[r] < e1) temp[bj[r] + e[r]] = nb[r] == Aj[r] ? make_int2(-1, 0) : make_int2(nb[r], adjwgt ? __ldcs(adjwgt + e[r]) : 1);
-    }
+    });
   }
   ue = warp_sum(ue);
   if (units && lane == 0) {
@@ -478,7 +479,7 @@ void contract_graph(gp_ctx *ctx, const DevGraph &g, const int32_t *cmap, int32_t
   {
     ProfScope ps(ctx, PROF_CONTRACT);
     if (g.m2 > 0) {
-      k_map<<<walk_grid(g.m2, ctx->num_sms), kThreads, 0, ctx->stream>>>(
+      k_map<<<walk_grid(n, g.m2, ctx->num_sms, 5), kThreads, 0, ctx->stream>>>(
           g.xadj, g.adjncy, g.unit_w ? nullptr : g.adjwgt, cmap, moff.get(), tstart.get(), n, temp.get(), units);
       GP_LAUNCH_CHECK();
     }

@@ -18,7 +18,7 @@ struct ModOut {
 __device__ __forceinline__ bool in_range(int L, int nl) { return L >= 0 && L < nl; }
 
 // The weight of entries whose endpoints share a label, the total weight, and every row's weight added
-// to its node's cluster volume.  The entries are split evenly over the warps (EntryWalk), kModUnroll
+// to its node's cluster volume.  Rows and entries are split evenly over the warps (EntryWalk), kModUnroll
 // per lane in flight.  Row weights are summed in shared memory (32 bits hold them: the validation
 // bounds the total edge weight by 2^31 - 1); with at most kModShared clusters (nsh > 0) the volumes are
 // summed per block too, the rows of one cluster in a window added up first: direct adds to a few dozen
@@ -47,21 +47,22 @@ __global__ void __launch_bounds__(256) k_mod_rows(const int32_t *xadj, const int
     const int e1 = wk.e1;
     s_deg[wib][lane] = 0;
     __syncwarp();
-    for (int f0 = wk.e0; f0 < e1; f0 += 32 * kModUnroll) {
-      int q[kModUnroll], Lq[kModUnroll], w[kModUnroll], v[kModUnroll];
+    walk_entries<kModUnroll>(wk.e0, e1, [&](auto steps, int f0) {
+      constexpr int R = decltype(steps)::value;
+      int q[R], Lq[R], w[R], v[R];
 #pragma unroll
-      for (int r = 0; r < kModUnroll; r++) {
+      for (int r = 0; r < R; r++) {
         q[r] = wk.owner(f0 + r * 32);
         Lq[r] = __shfl_sync(FULL, Lu, q[r]);
       }
 #pragma unroll
-      for (int r = 0; r < kModUnroll; r++) {
+      for (int r = 0; r < R; r++) {
         const int e = f0 + r * 32 + lane;
         v[r] = e < e1 ? __ldcs(adjncy + e) : -1;
         w[r] = e < e1 ? __ldcs(adjwgt + e) : 0;
       }
 #pragma unroll
-      for (int r = 0; r < kModUnroll; r++) {
+      for (int r = 0; r < R; r++) {
         if (v[r] < 0) continue;
         const int Lv = label[v[r]];
         if (!in_range(Lv, nl)) bad = 1;
@@ -69,7 +70,7 @@ __global__ void __launch_bounds__(256) k_mod_rows(const int32_t *xadj, const int
         if (Lv == Lq[r]) win += (unsigned long long)w[r];
         atomicAdd(&s_deg[wib][q[r]], (unsigned)w[r]);
       }
-    }
+    });
     __syncwarp();
     const unsigned d = s_deg[wib][lane];
     if (nsh > 0) {
@@ -125,7 +126,7 @@ void modularity(gp_ctx *ctx, const DevGraph &g, const int32_t *labels, int32_t n
   o.zero();
   if (g.n > 0) {
     // per-block volumes pay when a block has several rows a cluster; small graphs add directly
-    const int grid = walk_grid(g.m2, ctx->num_sms);
+    const int grid = walk_grid(g.n, g.m2, ctx->num_sms, 6);
     const int nsh = nlabels <= kModShared && g.n / grid >= 2 * nlabels ? nlabels : 0;
     k_mod_rows<<<grid, 256, sizeof(unsigned long long) * nsh, ctx->stream>>>(
         g.xadj, g.adjncy, g.adjwgt, labels, g.n, nlabels, nsh, vol.get(), o.get());

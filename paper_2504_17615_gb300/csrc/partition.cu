@@ -55,7 +55,7 @@ __device__ __forceinline__ unsigned long long pair_hash(uint32_t lo, uint32_t hi
 // 2^-64 collision).  Bound by the instructions of the hash, so one is taken
 // per entry and added with the entry's sign, whichever side it lies on (scoring
 // 8.4M nodes 2.21 -> 2.13 ms).  Runs after the row offsets were checked.  The
-// entries are split evenly over the warps (EntryWalk).
+// rows and entries are split evenly over the warps (EntryWalk).
 constexpr int kValUnroll = 4;
 
 __global__ void __launch_bounds__(256) k_validate_entries(const int32_t *xadj, const int32_t *adjncy,
@@ -68,34 +68,31 @@ __global__ void __launch_bounds__(256) k_validate_entries(const int32_t *xadj, c
   unsigned long long ws = 0, hd = 0;
   int nd = 0;
   for (EntryWalk wk(xadj, n, wid, nw); wk.next();) {
-    const int64_t u0 = wk.u0;
-    const int e0 = wk.e0, e1 = wk.e1;
-    // lane i's row start: the previous row's end
-    const int up = __shfl_up_sync(FULL, wk.xe, 1);
-    const int xs = lane == 0 ? xadj[u0] : up;
-    for (int f0 = e0; f0 < e1; f0 += 32 * kValUnroll) {
-      int e[kValUnroll], row[kValUnroll], rs[kValUnroll], v[kValUnroll], w[kValUnroll], pv[kValUnroll];
+    const int e1 = wk.e1;
+    walk_entries<kValUnroll>(wk.e0, e1, [&](auto steps, int f0) {
+      constexpr int R = decltype(steps)::value;
+      int e[R], row[R], rs[R], v[R], w[R], pv[R];
 #pragma unroll
-      for (int r = 0; r < kValUnroll; r++) {
+      for (int r = 0; r < R; r++) {
         e[r] = f0 + r * 32 + lane;
         const int q = wk.owner(f0 + r * 32);
-        row[r] = (int)(u0 + q);
-        rs[r] = __shfl_sync(FULL, xs, q);
+        row[r] = (int)(wk.u0 + q);
+        rs[r] = __shfl_sync(FULL, wk.xs, q);
       }
 #pragma unroll
-      for (int r = 0; r < kValUnroll; r++) {
+      for (int r = 0; r < R; r++) {
         const bool in = e[r] < e1;
         v[r] = in ? adjncy[e[r]] : 0;
         w[r] = in ? adjwgt[e[r]] : 1;
       }
 #pragma unroll
-      for (int r = 0; r < kValUnroll; r++) {  // the entry before: the lane before's, except in lane 0
+      for (int r = 0; r < R; r++) {  // the entry before: the lane before's, except in lane 0
         pv[r] = __shfl_up_sync(FULL, v[r], 1);
         if (lane == 0 && e[r] < e1 && e[r] > rs[r]) pv[r] = adjncy[e[r] - 1];
         if (e[r] <= rs[r]) pv[r] = -1;
       }
 #pragma unroll
-      for (int r = 0; r < kValUnroll; r++) {
+      for (int r = 0; r < R; r++) {
         if (e[r] >= e1) continue;
         if (v[r] < 0 || v[r] >= n) { err |= VE_RANGE; continue; }
         if (v[r] == row[r]) err |= VE_LOOP;
@@ -108,7 +105,7 @@ __global__ void __launch_bounds__(256) k_validate_entries(const int32_t *xadj, c
         hd += above ? h : 0ull - h;
         nd += above ? 1 : -1;
       }
-    }
+    });
   }
   ws = warp_sum(ws);
   hd = warp_sum(hd);
@@ -129,14 +126,12 @@ __global__ void k_project(int n, const int32_t *cmap, const int32_t *coarse, int
 }
 
 // cut = 1/2 sum over CSR entries whose endpoints lie in different blocks: the
-// entries are split evenly over the warps (EntryWalk); a warp finds each
-// entry's row among its lanes by a shuffle search, and keeps four entries per
-// lane in flight.
+// rows and entries are split evenly over the warps (EntryWalk); a warp finds each
+// entry's row among its lanes and keeps four entries per lane in flight.
 template <typename B>
 __global__ void __launch_bounds__(256) k_cut(const int32_t *xadj, const int32_t *adjncy,
                                              const int32_t *adjwgt, const B *blk, int n,
                                              unsigned long long *cut) {
-  constexpr int R = 4;
   const int lane = (int)lane_id();
   const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int nw = (int)((gridDim.x * blockDim.x) >> 5);
@@ -144,8 +139,9 @@ __global__ void __launch_bounds__(256) k_cut(const int32_t *xadj, const int32_t 
   for (EntryWalk wk(xadj, n, wid, nw); wk.next();) {
     const int64_t u = wk.u0 + lane;
     const int bu = u < n ? (int)blk[u] : -1;
-    const int e0 = wk.e0, e1 = wk.e1;
-    for (int f0 = e0; f0 < e1; f0 += 32 * R) {
+    const int e1 = wk.e1;
+    walk_entries<4>(wk.e0, e1, [&](auto steps, int f0) {
+      constexpr int R = decltype(steps)::value;
       int e[R], bo[R], v[R], w[R];
 #pragma unroll
       for (int r = 0; r < R; r++) {
@@ -161,7 +157,7 @@ __global__ void __launch_bounds__(256) k_cut(const int32_t *xadj, const int32_t 
 #pragma unroll
       for (int r = 0; r < R; r++)
         if (e[r] < e1 && (int)blk[v[r]] != bo[r]) s += (unsigned long long)w[r];
-    }
+    });
   }
   s = warp_sum(s);
   if (lane == 0 && s) atomicAdd(cut, s);
@@ -236,7 +232,7 @@ GraphTotals validate_graph(gp_ctx *ctx, const DevGraph &g, bool full) {
   GP_REQUIRE(h.csum <= 0x7FFFFFFFull, GP_ERR_OVERFLOW, "total node weight exceeds 2^31 - 1");
   prof_bytes(ctx, PROF_VALIDATE, 8.0 * g.n + 8.0 * g.m2);  // offsets, node weights, ids, edge weights
   if (g.m2 > 0) {
-    k_validate_entries<<<walk_grid(g.m2, ctx->num_sms), 256, 0, ctx->stream>>>(
+    k_validate_entries<<<walk_grid(g.n, g.m2, ctx->num_sms, 4), 256, 0, ctx->stream>>>(
         g.xadj, g.adjncy, g.adjwgt, g.n, g.m2, o.get());
     GP_LAUNCH_CHECK();
     read_back(ctx, o.get(), sizeof(ValOut), &h);
@@ -266,7 +262,7 @@ void cut_and_weights(gp_ctx *ctx, const DevGraph &g, const int32_t *blocks, int3
   DBuf<unsigned long long> c(ctx, 1);
   c.zero();
   if (g.m2 > 0) {
-    const int grid = walk_grid(g.m2, ctx->num_sms);
+    const int grid = walk_grid(g.n, g.m2, ctx->num_sms, 8);
     if (k <= 255) {
       DBuf<uint8_t> b8(ctx, (size_t)g.n);
       k_narrow<<<grid_for(g.n, 256, ctx->num_sms * 8), 256, 0, ctx->stream>>>(blocks, g.n, b8.get());

@@ -12,7 +12,7 @@
 // its hash is below floor(m_hat 2^32 / m).  Both CSR directions of an edge
 // see the same hash, so the result stays symmetric.
 //
-// Two passes over the entries, split evenly over the warps (EntryWalk): the
+// Two passes over rows and entries, split evenly over the warps (EntryWalk): the
 // first counts the kept entries of every row and of every warp's share, prefix
 // sums turn the counts into the new row offsets and into each share's place in
 // the output (kept entries stay in order), and the second takes the same keep
@@ -91,23 +91,24 @@ __global__ void __launch_bounds__(256) k_keep(KeepArgs a) {
   int out = WRITE ? a.share[wid] : 0;
   for (EntryWalk wk(a.xadj, a.n, wid, nw); wk.next();) {
     const int64_t u0 = wk.u0, u = u0 + lane;
-    const int e0 = wk.e0, e1 = wk.e1;
+    const int e1 = wk.e1;
     if (!WRITE) s_cnt[wib][lane] = 0;
     __syncwarp();
-    for (int f0 = e0; f0 < e1; f0 += 32 * kKeepUnroll) {
-      int e[kKeepUnroll], j[kKeepUnroll], v[kKeepUnroll], x[kKeepUnroll];
+    walk_entries<kKeepUnroll>(wk.e0, e1, [&](auto steps, int f0) {
+      constexpr int R = decltype(steps)::value;
+      int e[R], j[R], v[R], x[R];
 #pragma unroll
-      for (int r = 0; r < kKeepUnroll; r++) {
+      for (int r = 0; r < R; r++) {
         e[r] = f0 + r * 32 + lane;
         j[r] = wk.owner(f0 + r * 32);
       }
 #pragma unroll
-      for (int r = 0; r < kKeepUnroll; r++) {
+      for (int r = 0; r < R; r++) {
         v[r] = e[r] < e1 ? __ldcs(a.adjncy + e[r]) : 0;
         x[r] = e[r] < e1 ? __ldcs(a.adjwgt + e[r]) : 0;
       }
 #pragma unroll
-      for (int r = 0; r < kKeepUnroll; r++) {
+      for (int r = 0; r < R; r++) {
         const bool k = e[r] < e1 && keep_entry(a, (int)(u0 + j[r]), v[r], x[r]);
         if (WRITE) {
           const unsigned m = __ballot_sync(FULL, k);
@@ -121,7 +122,7 @@ __global__ void __launch_bounds__(256) k_keep(KeepArgs a) {
           atomicAdd(&s_cnt[wib][j[r]], 1);
         }
       }
-    }
+    });
     if (!WRITE) {
       __syncwarp();
       const int c = s_cnt[wib][lane];
@@ -204,7 +205,7 @@ void exact_boundary(gp_ctx *ctx, const DevGraph &g, int32_t wt, uint64_t key, in
   DBuf<unsigned long long> hist(ctx, 2048);
   std::vector<unsigned long long> h(2048);
   HashHistArgs a{g.xadj, g.adjncy, g.adjwgt, g.n, wt, key, 0, 0, 0, 0, hist.get(), nullptr, nullptr, 0};
-  const int grid = walk_grid(g.m2, ctx->num_sms);
+  const int grid = walk_grid(g.n, g.m2, ctx->num_sms, 8);
   uint64_t prefix = 0;
   int64_t below = 0, equal = 0;  // edges below the prefix, edges that have it
   int bits = 0;
@@ -344,7 +345,7 @@ void sparsify_graph(gp_ctx *ctx, const DevGraph &g, int64_t m_hat, int32_t level
     exact_boundary(ctx, g, wt, key, m_hat - ng, &T, &blo, &bhi);
   }
   KeepArgs a{g.xadj, g.adjncy, g.adjwgt, n, kmode, wt, T, key, blo, bhi, nullptr, nullptr, nullptr, nullptr};
-  const int kgrid = walk_grid(m2, ctx->num_sms);
+  const int kgrid = walk_grid(n, m2, ctx->num_sms, 8);
   DBuf<int32_t> cnt(ctx, (size_t)n + 1), total(ctx, 1), share(ctx, (size_t)kgrid * 8);
   cnt.zero();
   if (m2 > 0) {

@@ -1,5 +1,6 @@
 // EntryWalk on the CPU: every entry is handed out once, in order, with its row; on offsets that decrease
-// somewhere the walk ends and stays within the offsets' range.
+// somewhere the walk ends and stays within the offsets' range; and the work is even over the warps, also
+// where entries or rows lie unevenly.
 #include "warp.h"
 
 #include "walk.cuh"
@@ -36,7 +37,47 @@ static int walk(const std::vector<int32_t> &xadj, int nw, bool monotone) {
   return bad;
 }
 
+// Most collectives a warp of a walk takes to go over its share.
+static int most(const std::vector<int32_t> &xadj, int nw) {
+  const int n = (int)xadj.size() - 1;
+  int m = 0;
+  for (int w = 0; w < nw; w++) {
+    warp::run([&] {
+      for (gp::EntryWalk wk(xadj.data(), n, w, nw); wk.next();)
+        for (int f = wk.e0; f < wk.e1; f += 32) wk.owner(f);
+    });
+    m = warp::turn[0] > m ? warp::turn[0] : m;
+  }
+  return m;
+}
+
+static int even() {
+  int bad = 0;
+  const int n = 1 << 17, sms = 8;
+  for (int kind = 0; kind < 6; kind++) {
+    std::vector<int32_t> x(n + 1);
+    for (int i = 0; i < n; i++) {  // few entries anywhere | at one end | one hub | even | none | a dense end
+      const int deg = kind == 0 ? i % 9973 == 17 : kind == 1 ? i < 16 : kind == 2 ? (i == 70000 ? 100000 : i % 64 == 0)
+                    : kind == 3 ? 2 : kind == 4 ? 0 : i < 4096 ? 64 : i % 1024 == 3;
+      x[i + 1] = x[i] + deg;
+    }
+    const int blocks = gp::walk_grid(n, x[n], sms, 8), nw = blocks * 8;
+    // a warp takes the search, a window's five collectives per 32 units and an owner's seven per 32 entries
+    const int64_t units = (int64_t)n + x[n], per = units / nw + 1;
+    const int got = most(x, nw), allowed = 40 + (int)(per * (5.0 / 32 + 7.0 / 32));
+    if (got > allowed) {
+      printf("kind=%d blocks=%d: %d collectives, %d allowed\n", kind, blocks, got, allowed);
+      bad = 32;
+    }
+    if (blocks < (units < 8 * 576 * 4 * sms ? 1 : 4 * sms)) bad |= 64;
+  }
+  // millions of nodes fill the device whatever the entries
+  if (gp::walk_grid(8 << 20, 0, 152, 8) < 152 * 8 || gp::walk_grid(1, 0, 152, 8) != 1) bad |= 64;
+  return bad;
+}
+
 int main(int argc, char **argv) {
+  if (argc > 1 && argv[1][0] == 'e') return even();
   const bool monotone = argc > 1 && argv[1][0] == 'm';
   int bad = 0;
   if (monotone) {

@@ -64,6 +64,7 @@ inline void run(std::function<void()> f) {
 inline unsigned lane_id() { return (unsigned)warp::lane; }
 inline unsigned lanemask_lt() { return (1u << warp::lane) - 1u; }
 inline int __popc(unsigned x) { return __builtin_popcount(x); }
+inline int __ffs(unsigned x) { return __builtin_ffs((int)x); }
 inline int __shfl_sync(unsigned, int x, int from) { return (int)warp::exchange((uint32_t)x)[from & 31]; }
 inline int __shfl_up_sync(unsigned, int x, int d) {
   const uint32_t *v = warp::exchange((uint32_t)x);

@@ -23,8 +23,9 @@ def walk_check(tmp_path_factory):
     return build_host(tmp_path_factory.mktemp("walk"), "walk_check")
 
 
-# "any": offsets that decrease somewhere, which not every caller checks for; the walk has to end
-@pytest.mark.parametrize("offsets", ["monotone", "any"])
+# "any": offsets that decrease somewhere, which not every caller checks for; the walk has to end.  "even": no warp
+# has far more to do than the others
+@pytest.mark.parametrize("offsets", ["monotone", "any", "even"])
 def test_walk(walk_check, offsets):
     r = subprocess.run([walk_check, offsets], capture_output=True, text=True, timeout=30)
     assert r.returncode == 0, r.stdout
