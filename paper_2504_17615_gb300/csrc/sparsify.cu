@@ -13,10 +13,11 @@
 // see the same hash, so the result stays symmetric.
 //
 // Two passes over rows and entries, split evenly over the warps (EntryWalk): the
-// first counts the kept entries of every row and of every warp's share, prefix
-// sums turn the counts into the new row offsets and into each share's place in
-// the output (kept entries stay in order), and the second takes the same keep
-// decisions again and writes each share's kept entries contiguously.
+// first counts the kept entries of every row, a prefix sum turns the counts into
+// the new row offsets, and the second takes the same keep decisions again and
+// writes each share's kept entries contiguously from its first row's offset
+// (kept entries stay in order).  A share that begins inside a long row adds what
+// the shares before it keep of that row, which the first pass leaves behind.
 #include "gp_internal.cuh"
 
 #include <algorithm>
@@ -60,9 +61,12 @@ struct KeepArgs {
   uint64_t T;   // modes 1, 2: 32-bit hash threshold; mode 4: the last kept 64-bit hash
   uint64_t key;
   uint32_t blo, bhi;  // mode 4: the last kept edge among those whose hash equals T
-  int32_t *cnt;         // count pass: kept entries per row (zeroed before: a row may lie in two shares)
-  int32_t *share;       // per warp: kept entries of its share (count pass), their place (write pass)
+  int32_t *cnt;         // count pass: kept entries per row (zeroed before)
+  int32_t *part;        // per warp: kept entries of the row that goes on in the next warp's share, as ~x if this
+                        // share lies in that row from its beginning on
+  const int32_t *nxadj; // write pass: new row offsets
   int32_t *oadj, *ow;
+  unsigned room;          // entries that oadj and ow hold
 };
 
 constexpr int kKeepUnroll = 4;
@@ -81,17 +85,34 @@ __device__ __forceinline__ bool keep_entry(const KeepArgs &a, int row, int v, in
   return x > a.wt || (x == a.wt && h < a.T);
 }
 
-// WRITE = false: kept entries per row; WRITE = true: the kept entries, compacted.
+// WRITE = false: kept entries per row; WRITE = true: the kept entries, compacted.  Bound by the instructions of the
+// hash and of the walk (three quarters of the issue slots).  Against a warp per 32 rows, uniform mode: scale-21
+// R-MAT 5.8 -> .31 ms, meshes and random graphs of up to some million entries 3 to 20 % slower (216,000-node mesh
+// .064 -> .076 ms, 1M nodes and 21M entries .175 -> .195), 268M and 537M entries 3 %: every warp begins with a
+// search.
 template <bool WRITE>
-__global__ void __launch_bounds__(256) k_keep(KeepArgs a) {
+__global__ void __launch_bounds__(256, 7) k_keep(KeepArgs a) {
   __shared__ int s_cnt[8][32];
   const int lane = (int)lane_id(), wib = threadIdx.x >> 5;
   const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-  int out = WRITE ? a.share[wid] : 0;
-  for (EntryWalk wk(a.xadj, a.n, wid, nw); wk.next();) {
-    const int64_t u0 = wk.u0, u = u0 + lane;
-    const int e1 = wk.e1;
+  EntryWalk wk(a.xadj, a.n, wid, nw);
+  const unsigned r0 = wk.row;
+  const bool inside = wk.pos > wk.start;  // the share begins inside row r0
+  int out = 0;
+  if (WRITE && r0 < (unsigned)a.n) {
+    out = a.nxadj[r0];
+    for (int w = wid - 1; inside; w -= 32) {  // what the shares before this one keep of the row
+      const int x = w - lane >= 0 ? a.part[w - lane] : 0;
+      const unsigned first = __ballot_sync(FULL, x >= 0);  // the share in which the row begins
+      const int f = first ? __ffs(first) - 1 : 32;
+      out += warp_sum(lane <= f ? (x < 0 ? ~x : x) : 0);
+      if (first) break;
+    }
+  }
+  while (wk.next()) {
+    const unsigned u = wk.u0 + lane;
+    const int u0 = (int)wk.u0, e1 = wk.e1;
     if (!WRITE) s_cnt[wib][lane] = 0;
     __syncwarp();
     walk_entries<kKeepUnroll>(wk.e0, e1, [&](auto steps, int f0) {
@@ -109,13 +130,15 @@ __global__ void __launch_bounds__(256) k_keep(KeepArgs a) {
       }
 #pragma unroll
       for (int r = 0; r < R; r++) {
-        const bool k = e[r] < e1 && keep_entry(a, (int)(u0 + j[r]), v[r], x[r]);
+        const bool k = e[r] < e1 && keep_entry(a, u0 + j[r], v[r], x[r]);
         if (WRITE) {
           const unsigned m = __ballot_sync(FULL, k);
           if (k) {
-            const int pos = out + __popc(m & lanemask_lt());
-            a.oadj[pos] = v[r];
-            a.ow[pos] = x[r];
+            const unsigned pos = (unsigned)(out + __popc(m & lanemask_lt()));
+            if (pos < a.room) {  // always, unless offsets decrease somewhere
+              a.oadj[pos] = v[r];
+              a.ow[pos] = x[r];
+            }
           }
           out += __popc(m);
         } else if (k) {
@@ -126,14 +149,14 @@ __global__ void __launch_bounds__(256) k_keep(KeepArgs a) {
     if (!WRITE) {
       __syncwarp();
       const int c = s_cnt[wib][lane];
-      if (c) atomicAdd(&a.cnt[u], c);
-      out += c;
+      if (wk.split < 0 && !inside) {
+        if (c) a.cnt[u] = c;
+      } else {  // rows that lie in several shares
+        if (c) atomicAdd(&a.cnt[u], c);
+        if (lane == wk.split) a.part[wid] = inside && u == r0 ? ~c : c;
+      }
       __syncwarp();
     }
-  }
-  if (!WRITE) {
-    out = warp_sum(out);
-    if (lane == 0) a.share[wid] = out;
   }
 }
 
@@ -166,13 +189,12 @@ __global__ void __launch_bounds__(256) k_hash_digit(HashHistArgs a) {
   const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int nw = (int)((gridDim.x * blockDim.x) >> 5);
   for (EntryWalk wk(a.xadj, a.n, wid, nw); wk.next();) {
-    const int64_t u0 = wk.u0;
-    const int e1 = wk.e1;
+    const int u0 = (int)wk.u0, e1 = wk.e1;
     for (int f0 = wk.e0; f0 < e1; f0 += 32) {
       const int e = f0 + lane;
       const int q = wk.owner(f0);
       if (e >= e1) continue;
-      const int row = (int)(u0 + q), v = __ldcs(a.adjncy + e);
+      const int row = u0 + q, v = __ldcs(a.adjncy + e);
       if (row >= v || __ldcs(a.adjwgt + e) != a.wt) continue;
       const uint64_t h = h64(a.key, (uint32_t)row, (uint32_t)v);
       if (COLLECT) {
@@ -344,22 +366,23 @@ void sparsify_graph(gp_ctx *ctx, const DevGraph &g, int64_t m_hat, int32_t level
     kmode = 4;
     exact_boundary(ctx, g, wt, key, m_hat - ng, &T, &blo, &bhi);
   }
-  KeepArgs a{g.xadj, g.adjncy, g.adjwgt, n, kmode, wt, T, key, blo, bhi, nullptr, nullptr, nullptr, nullptr};
-  const int kgrid = walk_grid(n, m2, ctx->num_sms, 8);
-  DBuf<int32_t> cnt(ctx, (size_t)n + 1), total(ctx, 1), share(ctx, (size_t)kgrid * 8);
-  cnt.zero();
+  KeepArgs a{g.xadj, g.adjncy, g.adjwgt, n, kmode, wt, T, key, blo, bhi, nullptr, nullptr, nullptr, nullptr, nullptr, 0};
+  const int kgrid = walk_grid(n, m2, ctx->num_sms, 16);
+  // the rows' counts, their total, the parts of rows in several shares
+  DBuf<int32_t> cnt(ctx, (size_t)n + 2 + (size_t)kgrid * 8);
+  int32_t *const total = cnt.get() + n + 1;
+  GP_CUDA(cudaMemsetAsync(cnt.get(), 0, sizeof(int32_t) * ((size_t)n + 1), ctx->stream));
   if (m2 > 0) {
     a.cnt = cnt.get();
-    a.share = share.get();
+    a.part = total + 1;
     k_keep<false><<<kgrid, 256, 0, ctx->stream>>>(a);
     GP_LAUNCH_CHECK();
   }
   out.n = n;
   out.bx.reset(ctx, (size_t)n + 1);
   out.xadj = out.bx.get();
-  scan_exclusive_i32(ctx, cnt.get(), out.xadj, n + 1, total.get());
-  if (m2 > 0) scan_exclusive_i32(ctx, share.get(), share.get(), (int64_t)kgrid * 8, nullptr);
-  const int32_t m2_out = read_scalar(ctx, total.get());
+  scan_exclusive_i32(ctx, cnt.get(), out.xadj, n + 1, total);
+  const int32_t m2_out = read_scalar(ctx, total);
   out.m2 = m2_out;
   out.ba.reset(ctx, (size_t)m2_out);
   out.bw.reset(ctx, (size_t)m2_out);
@@ -368,7 +391,7 @@ void sparsify_graph(gp_ctx *ctx, const DevGraph &g, int64_t m_hat, int32_t level
   out.bv.reset(ctx, (size_t)n);
   out.vwgt = out.bv.get();
   if (n > 0 && m2_out > 0) {
-    a.oadj = out.adjncy; a.ow = out.adjwgt;
+    a.nxadj = out.xadj; a.oadj = out.adjncy; a.ow = out.adjwgt; a.room = (unsigned)m2_out;
     k_keep<true><<<kgrid, 256, 0, ctx->stream>>>(a);
     GP_LAUNCH_CHECK();
   }

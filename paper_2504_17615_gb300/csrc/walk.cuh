@@ -18,7 +18,7 @@ inline int grid_for(int64_t items, int per_block, int cap) {
 // With 32 rows per warp step one warp walked a hub's whole row (4e5 entries of the scale-24 R-MAT graph)
 // while the rest of the device waited; with even shares of the entries alone one warp walked all the empty
 // rows between two of them (8.4M nodes with 840 edges: modularity 1.3 ms, against .18 with 32 rows per warp step and
-// .14 now; sparsification .79, .13 and .16).
+// .14 now; sparsification .79, .13 and .14).
 //
 //   for (EntryWalk w(xadj, n, wid, nw); w.next(); )
 //     entries [w.e0, w.e1) lie in rows [w.u0, w.u0 + 32); lane i's row is [w.xs, w.xe) (past n: empty);
@@ -44,6 +44,7 @@ struct EntryWalk {
   unsigned u0;       // this window's first row
   int e0, e1;
   int xs, xe;        // this lane's row
+  int split;         // the lane whose row goes on in the next share (-1: none)
   bool no_empty;     // no row of the window is empty
   __device__ __forceinline__ EntryWalk(const int32_t *x, int nn, int wid, int nw) : xadj(x), n((unsigned)nn) {
     // the search's first 32 places, at doubling distances around where even degrees would put the share: read
@@ -68,7 +69,7 @@ struct EntryWalk {
       pos = cut(row, start, next, (unsigned)from);
       if (pos < lo) pos = lo;
     }
-    u0 = 0; e0 = e1 = xs = xe = 0; no_empty = false;
+    u0 = 0; e0 = e1 = xs = xe = 0; split = -1; no_empty = false;
   }
   __device__ __forceinline__ bool next() {
     while (row < n) {
@@ -86,6 +87,7 @@ struct EntryWalk {
         const int j = __ffs(past) - 1;
         const int b = __shfl_sync(0xFFFFFFFFu, xs, j), e = __shfl_sync(0xFFFFFFFFu, xe, j);
         stop = cut(u0 + j, b, e, until);
+        split = stop > b ? j : -1;
         row = n;
       }
       if (stop > hi) stop = hi;
