@@ -54,13 +54,19 @@ constexpr int kPSortSmem = 2048;    // overflow sets sorted in shared memory up 
 constexpr int kPBuckets = 4096;     // few-label overflow: priority buckets (top 12 bits)
 constexpr int kPScan = 8;           // few-label overflow: keys of the set in flight per thread
 constexpr int kPCross = 1024;       // few-label overflow: crossing-bucket entries kept in shared memory
-// overflow sets above kPSortOne entries with at most kPFewLabels labels are resolved one target per block
-// (every block reads the whole set, so more labels than a few per block would not pay); smaller sets are
-// sorted by one block in shared memory
+// overflow sets are resolved one target per block (every block reads the whole set) when no block has more than
+// one target, or when they hold more than kPSortOne entries and there are at most kPFewLabels labels, or more than
+// kPSortSmem entries and at most kPManyLabels labels a block; other sets are sorted by one block, in shared memory
+// up to kPSortSmem entries and in global memory beyond (refinement of a scale-18 R-MAT graph, k = 3000 and 9000, sets of up to
+// 13,000 entries: 47.7 and 30.3 ms sorted, 9.7 and 9.5 target by target; 216,000-node mesh, up to 3,000 entries:
+// 4.5 and 4.9, 2.2 and 2.6)
 constexpr int kPFewLabels = 1024;
+constexpr int kPManyLabels = 32;
 constexpr int kPSortOne = 1024;
-// with the label weights in shared memory, a sub-round of at most this many proposals is decided by every
-// block for itself (the same decisions from the same snapshot), which saves two grid barriers
+// with the label weights in shared memory, a sub-round of at most this many proposals is decided without grid
+// barriers: every block lists the proposals of overflowing targets, and a warp per proposal adds up the weights
+// that go before it and applies the move.  With the list sorted by every block instead (55 steps for 1024
+// entries) refinement of a scale-14 R-MAT graph, k = 64, took 1.83 ms against 1.43 (1.63 target by target)
 constexpr int kPLocal = 1024;
 // 2.5x cap: digits of the radix select (11 bits from the top), and the keys left at which the
 // remaining ones are listed and ranked directly
@@ -68,7 +74,7 @@ constexpr int kPCapBits = 11;
 constexpr int kPCapBins = 1 << kPCapBits;
 constexpr int kPCapPasses = 6;
 constexpr int kPCapList = 256;
-constexpr size_t kLocalBytes = (sizeof(uint64_t) + sizeof(uint32_t) + sizeof(int32_t) + sizeof(long long) + 1) * kPLocal;
+constexpr size_t kLocalBytes = (sizeof(uint64_t) + sizeof(uint32_t) + sizeof(int32_t) + 1) * kPLocal;
 // a class's list longer than this many nodes per warp is rated by a thread per node, a shorter one by lane
 // groups: a thread's whole row takes 1.5 to 4 us, a pass of lane groups (4, 2 or 1 nodes a warp) about 1 us
 constexpr int kPRows8 = 16, kPRows16 = 6, kPRows32 = 8;
@@ -465,7 +471,6 @@ __global__ void __launch_bounds__(kPThreads, GP_PLP_BLOCKS_PER_SM) k_lp_persiste
   int subs = 0, capped = 0;
   bool stop = false;
   unsigned long long ue = 0, uv = 0;
-  const bool few = a.nlabels <= kPFewLabels;
   const bool agg = !a.count_clusters && a.nlabels <= kPAggLabels;
   const bool few_w = !a.count_clusters && a.nlabels <= kPWeightSmem;  // label weights in shared memory
 
@@ -647,14 +652,13 @@ __global__ void __launch_bounds__(kPThreads, GP_PLP_BLOCKS_PER_SM) k_lp_persiste
       // -------------------------------------------------------- decide
       // when no target overflows every proposal is accepted, and there is nothing to decide
       const bool over_any = *(volatile int *)&c->over != 0;
-      // few proposals, and the label weights of the sub-round's start in shared memory: every block decides
-      // all of them from those and the incoming weights, into its own flags, and applies its share
+      // few proposals, and the label weights of the sub-round's start in shared memory: every block lists the
+      // proposers of overflowing targets from those and the incoming weights, and decides what its warps apply
       const bool local = over_any && few_w && nprop <= kPLocal;
-      uint64_t *lk = reinterpret_cast<uint64_t *>(area);               // [kPLocal] overflow keys
+      uint64_t *lk = reinterpret_cast<uint64_t *>(area);               // [kPLocal] overflow: target, priority
       uint32_t *lv = reinterpret_cast<uint32_t *>(lk + kPLocal);       // [kPLocal] nodes
-      int32_t *lx = reinterpret_cast<int32_t *>(lv + kPLocal);         // [kPLocal] proposal indices
-      long long *lp = reinterpret_cast<long long *>(lx + kPLocal);     // [kPLocal] running weights
-      uint8_t *lacc = reinterpret_cast<uint8_t *>(lp + kPLocal);       // [kPLocal] accepted
+      int32_t *lw = reinterpret_cast<int32_t *>(lv + kPLocal);         // [kPLocal] their weights
+      uint8_t *lfit = reinterpret_cast<uint8_t *>(lw + kPLocal);       // [kPLocal] per proposal: its target takes all
       int nov = 0;
       if (local) {
         __shared__ int s_no;
@@ -663,44 +667,17 @@ __global__ void __launch_bounds__(kPThreads, GP_PLP_BLOCKS_PER_SM) k_lp_persiste
         for (int i = threadIdx.x; i < nprop; i += blockDim.x) {
           const int4 p = a.prop[i];
           const bool fit = (int64_t)s_wl[p.y] + *(volatile int32_t *)&inc[p.y] <= a.bound;
-          lacc[i] = fit ? 1 : 0;
+          lfit[i] = fit ? 1 : 0;
           if (!fit) {
             const int j = atomicAdd(&s_no, 1);
             lk[j] = ((uint64_t)(uint32_t)p.y << 32) | h32(kprio, (uint32_t)p.x, 0);
             lv[j] = (uint32_t)p.x;
-            lx[j] = i;
+            lw[j] = p.w;
           }
         }
         __syncthreads();
         nov = s_no;
-        int P = 1;
-        while (P < nov) P <<= 1;
-        for (int i = nov + threadIdx.x; i < P; i += blockDim.x) { lk[i] = ~0ull; lv[i] = 0xFFFFFFFFu; lx[i] = -1; }
-        __syncthreads();
-        bitonic(lk, lv, lx, P);
-        long long carry = 0;
-        for (int c0 = 0; c0 < nov; c0 += blockDim.x) {
-          const int i = c0 + (int)threadIdx.x;
-          const long long x = i < nov ? (long long)a.vwgt[lv[i]] : 0;
-          long long tot;
-          const long long incl = block_incl_scan(x, s_ll, tot);
-          if (i < nov) lp[i] = carry + incl;
-          carry += tot;
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < nov; i += blockDim.x) {
-          const uint64_t seg = lk[i] & 0xFFFFFFFF00000000ull;
-          int l0 = 0, l1 = i;
-          while (l0 < l1) {
-            const int mid = (l0 + l1) >> 1;
-            if (lk[mid] < seg) l0 = mid + 1; else l1 = mid;
-          }
-          const long long w = lp[i] - (l0 > 0 ? lp[l0 - 1] : 0);
-          lacc[lx[i]] = (int64_t)s_wl[(int)(lk[i] >> 32)] + w <= a.bound ? 1 : 0;
-        }
-        __syncthreads();
       }
-      const uint8_t *acc = local ? lacc : a.acc;
       if (over_any && !local) {
       for (int b0 = blockIdx.x * blockDim.x; b0 < nprop; b0 += gthreads) {
         const int i = b0 + (int)threadIdx.x;
@@ -724,7 +701,8 @@ __global__ void __launch_bounds__(kPThreads, GP_PLP_BLOCKS_PER_SM) k_lp_persiste
       // ------------------------------------------------------ overflow
       if (over_any && !local) {
         nov = *(volatile int *)&c->nov;
-        if (few && nov > kPSortOne) {
+        if (a.nlabels <= (int64_t)gridDim.x || (nov > kPSortOne && a.nlabels <= kPFewLabels) ||
+            (nov > kPSortSmem && a.nlabels <= (int64_t)kPManyLabels * gridDim.x)) {
           // per target: weighted histogram over the top 12 priority bits finds the
           // bucket where the running weight passes the room; only that bucket's
           // entries are ranked exactly
@@ -999,10 +977,33 @@ __global__ void __launch_bounds__(kPThreads, GP_PLP_BLOCKS_PER_SM) k_lp_persiste
         __syncthreads();
       }
       long long moved = 0, delta = 0;
-      for (int i = gt; i < nprop; i += gthreads) {
+      for (int i = gw; local && i < nprop; i += nw) {  // a warp per proposal
+        const int4 p = a.prop[i];
+        if (!lfit[i]) {  // the longest prefix in (priority, node) order that fits
+          const uint64_t seg = (uint64_t)(uint32_t)p.y << 32, key = seg | h32(kprio, (uint32_t)p.x, 0);
+          int w = 0;
+          for (int j = lane; j < nov; j += 32) {
+            const uint64_t k = lk[j];
+            w += k >= seg && (k < key || (k == key && lv[j] <= (uint32_t)p.x)) ? lw[j] : 0;
+          }
+          w = (int)__reduce_add_sync(FULL, (unsigned)w);
+          if ((int64_t)s_wl[p.y] + w > a.bound) continue;
+        }
+        if (lane == 0) {
+          a.label[p.x] = p.y;
+          if (a.label8) a.label8[p.x] = (uint8_t)p.y;
+          atomicAdd(&s_dw[p.y], p.w);
+          atomicSub(&s_dw[p.z], p.w);
+          a.dirty[p.x] = 1;
+          moved++;
+        }
+        const int e0 = a.xadj[p.x], e1 = a.xadj[p.x + 1];
+        for (int e = e0 + lane; e < e1; e += 32) a.dirty[a.adjncy[e]] = 1;
+      }
+      for (int i = gt; !local && i < nprop; i += gthreads) {
         const int4 p = a.prop[i];
         if (!a.two_inc) inc[p.y] = 0;
-        if (over_any && !acc[i]) continue;
+        if (over_any && !a.acc[i]) continue;
         if (cutoff != ~0ull && pkey(kprio, p.x) >= cutoff) continue;
         a.label[p.x] = p.y;
         if (a.label8) a.label8[p.x] = (uint8_t)p.y;
@@ -1021,9 +1022,9 @@ __global__ void __launch_bounds__(kPThreads, GP_PLP_BLOCKS_PER_SM) k_lp_persiste
         for (int q = threadIdx.x; q < (int)a.nlabels; q += blockDim.x)
           if (s_dw[q]) atomicAdd(&a.weight[q], s_dw[q]);
       }
-      if (a.dirty) {  // every applied move marks its node and the node's neighbours, a warp per move
+      if (a.dirty && !local) {  // every applied move marks its node and the node's neighbours, a warp per move
         for (int i = gw; i < nprop; i += nw) {
-          if (over_any && !acc[i]) continue;
+          if (over_any && !a.acc[i]) continue;
           const int v = a.prop[i].x;
           if (cutoff != ~0ull && pkey(kprio, v) >= cutoff) continue;
           const int e0 = a.xadj[v], e1 = a.xadj[v + 1];
