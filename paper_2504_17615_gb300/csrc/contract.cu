@@ -457,9 +457,10 @@ void contract_graph(gp_ctx *ctx, const DevGraph &g, const int32_t *cmap, int32_t
   DBuf<int> chunk0, tchunk0;
   DBuf<int2> tab;
   int64_t slots = 0;
+  const int64_t table_bytes = ctx->limits.table_bytes(g.m2);
   for (sg.q4 = 8; sg.q4 > 4; sg.q4--) {  // two slots a key down to one and a quarter
     slots = (int64_t)hs.keys * sg.q4 / 4 + hs.huge;
-    if (slots <= g.m2 + ((int64_t)2 << 20)) break;
+    if (slots * (int64_t)sizeof(int2) <= table_bytes) break;
   }
   a.split_huge = hs.huge > 0 && sg.q4 > 4 ? 1 : 0;
   if (a.split_huge) {
@@ -470,7 +471,7 @@ void contract_graph(gp_ctx *ctx, const DevGraph &g, const int32_t *cmap, int32_t
     sg = SegArgs{segs.get(), chunk0.get(), tchunk0.get(), tab.get(), sg.q4};
   } else if (const int bits = table_bits(seg_keys(hs.longest, nc), 5); ((int64_t)1 << bits) > kBlockSmemSlots) {
     a.gstride = (int64_t)1 << bits;
-    lblocks = table_blocks(g.m2, a.gstride, lblocks);
+    lblocks = table_blocks(table_bytes, a.gstride, lblocks);
     gk.reset(ctx, (size_t)(a.gstride * lblocks));
     gv.reset(ctx, (size_t)(a.gstride * lblocks));
     a.gkeys = gk.get();

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstdio>
 #include <cstdlib>
@@ -99,7 +100,10 @@ namespace gp {
 // Sizes at which a context changes its way of working, never its results; gp_test_limits lowers them, so that
 // small graphs reach what otherwise only very large ones do.
 struct Limits {
-  int32_t hash_collect = 16384;  // exact sampler: edges fetched and ordered on the host
+  int32_t hash_collect = 16384;       // exact sampler: edges fetched and ordered on the host
+  int64_t table_slack = 16 << 20;     // hash tables in global memory: bytes beyond 8 per CSR entry
+
+  int64_t table_bytes(int64_t m2) const { return std::max<int64_t>(0, 8 * m2 + table_slack); }
 };
 
 }  // namespace gp

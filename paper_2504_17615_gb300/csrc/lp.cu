@@ -1685,7 +1685,7 @@ void make_tables(gp_ctx *ctx, const DevGraph &g, int64_t nlabels, RateTables &t)
   const int maxdeg = h.maxdeg;
   t.blocks = ctx->num_sms * 4;
   if (nlabels > 0) {
-    const int64_t cap = (8 * g.m2 + ((int64_t)16 << 20)) / (int64_t)sizeof(int2);
+    const int64_t cap = ctx->limits.table_bytes(g.m2) / (int64_t)sizeof(int2);
     t.dense = nlabels <= kHubDense && (int64_t)h.big * nlabels <= 2 * cap;
     const int64_t hubs = t.dense ? h.big : h.hubs;
     int64_t slots = 0;
@@ -1712,7 +1712,7 @@ void make_tables(gp_ctx *ctx, const DevGraph &g, int64_t nlabels, RateTables &t)
   const int bits = table_bits(maxdeg, 1);
   if (((int64_t)1 << bits) > kLargeSmemSlots) {
     t.stride = (int64_t)1 << bits;
-    t.blocks = table_blocks(g.m2, t.stride, t.blocks);
+    t.blocks = table_blocks(ctx->limits.table_bytes(g.m2), t.stride, t.blocks);
     t.gkeys.reset(ctx, (size_t)(t.stride * t.blocks));
     t.gvals.reset(ctx, (size_t)(t.stride * t.blocks));
     t.gkeys.fill_bytes(0xFF);

@@ -1173,7 +1173,7 @@ bool lp_run_small(gp_ctx *ctx, const DevGraph &g, int32_t *label, int32_t *weigh
   int hblocks = grid;  // blocks that rate the nodes of degree > kPLight
   if ((1 << bits) > kPHeavySlots) {
     gstride = (int64_t)1 << bits;
-    hblocks = table_blocks(g.m2, gstride, grid);
+    hblocks = table_blocks(ctx->limits.table_bytes(g.m2), gstride, grid);
     gtk.reset(ctx, (size_t)(gstride * hblocks));
     gtv.reset(ctx, (size_t)(gstride * hblocks));
     gtk.fill_bytes(0xFF);

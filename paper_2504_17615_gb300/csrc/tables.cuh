@@ -26,11 +26,10 @@ __host__ __device__ __forceinline__ int chunks_of(int count, int step) {
 }
 
 // Blocks that get a private global hash table of `slots` int pairs, at most
-// `want`: the tables together stay within 8 bytes per CSR entry plus 16 MiB,
-// so scratch memory grows with the graph, not with its largest degree.
-inline int table_blocks(int64_t m2, int64_t slots, int want) {
-  const int64_t cap = 8 * m2 + ((int64_t)16 << 20);
-  int64_t b = cap / (slots * 8);
+// `want`: the tables together stay within `bytes` (8 per CSR entry plus 16 MiB,
+// Limits), so scratch memory grows with the graph, not with its largest degree.
+inline int table_blocks(int64_t bytes, int64_t slots, int want) {
+  int64_t b = bytes / (slots * 8);
   if (b > want) b = want;
   return b < 1 ? 1 : (int)b;
 }

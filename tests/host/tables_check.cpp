@@ -33,10 +33,10 @@ int main() {
       if (c * step < k || (c - 1) * step >= k + (k == 0)) bad |= 64;
     }
   }
-  for (int64_t m2 : {(int64_t)0, (int64_t)1000000, M})
+  for (int64_t bytes : {(int64_t)0, (int64_t)24000000, 8 * M})
     for (int b : {13, 30, 31}) {
-      const int n = gp::table_blocks(m2, (int64_t)1 << b, 608);
-      if (n < 1 || n > 608 || (n > 1 && ((int64_t)n << b) * 8 > 8 * m2 + (16 << 20))) bad |= 128;
+      const int n = gp::table_blocks(bytes, (int64_t)1 << b, 608);
+      if (n < 1 || n > 608 || (n > 1 && ((int64_t)n << b) * 8 > bytes)) bad |= 128;
     }
   printf("bad=%d\n", bad);
   return bad != 0;

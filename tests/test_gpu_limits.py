@@ -9,6 +9,8 @@ import pytest
 
 import graphgen as gg
 import oracle as orc
+from tests.test_gpu_hubs import GRAPHS
+from tests.test_gpu_parity import HOST_PATH, canon
 
 pytestmark = pytest.mark.gpu
 
@@ -23,8 +25,8 @@ def ctx():
     c.close()
 
 
-def limits(ctx, hash_collect=16384):
-    ctx.lib.gp_test_limits(ctypes.c_void_p(ctx.ptr), ctypes.c_int32(hash_collect))
+def limits(ctx, hash_collect=16384, table_slack=16 << 20):
+    ctx.lib.gp_test_limits(ctypes.c_void_p(ctx.ptr), ctypes.c_int32(hash_collect), ctypes.c_int64(table_slack))
 
 
 # edges of one weight that share a hash prefix: with a limit of 16384 one digit is read, with 64 or 1 one or two,
@@ -44,3 +46,51 @@ def test_exact_sampler_digits(ctx, limit, name):
         assert got.m == m_hat and st.threshold == ost.threshold
         assert np.array_equal(got.xadj, np.asarray(exp.xadj)) and np.array_equal(got.adjncy, np.asarray(exp.adjncy))
         assert np.array_equal(got.adjwgt, np.asarray(exp.adjwgt))
+
+
+def _slack(m2, keys, tables, q4):
+    """Bytes that let `tables` tables of `keys` keys in all have q4 quarters of a slot a key, and not more; q4 = 0:
+    no such tables."""
+    return -8 * m2 if q4 == 0 else 8 * (keys * q4 // 4 + tables) - 8 * m2
+
+
+# hub tables of 3, 2.5, 2 and 1.5 slots a neighbour, and none: the hubs of more than 18432 neighbours then take a
+# block each (refinement with few labels counts them per label unless even that is too much)
+@pytest.mark.parametrize("q4", [12, 10, 8, 6, 0])
+def test_hub_tables(ctx, q4):
+    import torch
+    import paper_2504_17615_gb300 as gp
+    g = GRAPHS["weighted"]
+    deg = np.diff(np.asarray(g.xadj))
+    hubs = deg[deg > 18432]
+    assert len(hubs) >= 2
+    limits(ctx, table_slack=_slack(2 * g.m, int(hubs.sum()), len(hubs), q4))
+    dg = gp.DeviceGraph.from_host(g)
+    cmap, nc, st = ctx.gp_coarsen(dg, 400, 1, 5, gp.default_config(**HOST_PATH))
+    ocmap, onc, ost = orc.coarsen(g, 400, 1, 5)
+    assert nc == onc and np.array_equal(cmap.cpu().numpy(), ocmap)
+    for k in (2, 300, 1025):
+        blk = np.random.default_rng(k).integers(0, k, g.n).astype(np.int32)
+        lmax = int(np.bincount(blk, weights=g.vwgt, minlength=k).max()) + 2
+        for cfg in (HOST_PATH, {}):
+            t = torch.from_numpy(blk.copy()).cuda()
+            moves = ctx.gp_refine(dg, k, lmax, 1, 3, t, gp.default_config(**cfg))
+            oblk, omoves = orc.refine(g, k, lmax, 1, 3, blk)
+            assert moves == omoves and np.array_equal(t.cpu().numpy(), oblk)
+
+
+# segments above 2048 entries: tables of 2, 1.75, 1.5 and 1.25 slots a key, and a block a segment
+@pytest.mark.parametrize("q4", [8, 7, 6, 5, 0])
+@pytest.mark.parametrize("name,nc", [("weighted", 7), ("weighted", 5000), ("clique", 1500)])
+def test_segment_tables(ctx, name, nc, q4):
+    import torch
+    import paper_2504_17615_gb300 as gp
+    g = GRAPHS[name]
+    cmap = np.concatenate([np.arange(nc), np.random.default_rng(nc).integers(0, nc, g.n - nc)]).astype(np.int32)
+    seg = np.bincount(cmap, weights=np.diff(np.asarray(g.xadj)), minlength=nc).astype(np.int64)
+    long = np.minimum(seg[seg > 2048], nc)
+    assert len(long) > 0
+    limits(ctx, table_slack=_slack(2 * g.m, int(long.sum()), len(long), q4))
+    got = ctx.gp_contract(gp.DeviceGraph.from_host(g), torch.from_numpy(cmap).cuda(), nc).to_host()
+    for a, b in zip(canon(got), canon(orc.contract(g, cmap, nc))):
+        assert np.array_equal(a, b)
