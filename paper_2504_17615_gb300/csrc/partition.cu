@@ -377,7 +377,8 @@ struct Tail {
 bool tail_down(gp_ctx *ctx, const DevGraph &g, int level, int32_t k, int64_t U, int64_t Lmax, uint64_t seed,
                const gp_config &cfg, gp_level_stats *st, Tail &t) {
   ProfScope ps(ctx, PROF_LP_SMALL);
-  const int64_t bytes = 160 * (int64_t)g.n + 40 * g.m2 + 64 * (int64_t)k + ((int64_t)4 << 20);
+  const int64_t bytes =
+      std::max<int64_t>(4096, 160 * (int64_t)g.n + 40 * g.m2 + 64 * (int64_t)k + ctx->limits.tail_slack) & ~(int64_t)255;
   t.arena.reset(ctx, (size_t)bytes);
   t.lv.reset(ctx, GP_MAX_LEVELS + 1);
   t.out.reset(ctx, 1);

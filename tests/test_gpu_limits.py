@@ -25,8 +25,9 @@ def ctx():
     c.close()
 
 
-def limits(ctx, hash_collect=16384, table_slack=16 << 20):
-    ctx.lib.gp_test_limits(ctypes.c_void_p(ctx.ptr), ctypes.c_int32(hash_collect), ctypes.c_int64(table_slack))
+def limits(ctx, hash_collect=16384, table_slack=16 << 20, tail_slack=4 << 20):
+    ctx.lib.gp_test_limits(ctypes.c_void_p(ctx.ptr), ctypes.c_int32(hash_collect), ctypes.c_int64(table_slack),
+                           ctypes.c_int64(tail_slack))
 
 
 # edges of one weight that share a hash prefix: with a limit of 16384 one digit is read, with 64 or 1 one or two,
@@ -94,3 +95,39 @@ def test_segment_tables(ctx, name, nc, q4):
     got = ctx.gp_contract(gp.DeviceGraph.from_host(g), torch.from_numpy(cmap).cuda(), nc).to_host()
     for a, b in zip(canon(got), canon(orc.contract(g, cmap, nc))):
         assert np.array_equal(a, b)
+
+
+def _levels(ctx, g, k, **kw):
+    """Levels of a partition (checked against the oracle) and how many of them were contracted on their own, not
+    among the one-CTA levels."""
+    import paper_2504_17615_gb300 as gp
+    dg = gp.DeviceGraph.from_host(g)
+    ctx.profile_reset()
+    ctx.profile(True)
+    blocks, cut, st = ctx.gp_partition(dg, k, 0.03, 3, gp.default_config(**kw))
+    ctx.profile(False)
+    r = orc.partition(g, k, 0.03, 3, orc.Config.default(**{a: b for a, b in kw.items() if a != "small_lp_nodes"}))
+    assert cut == r.cut and np.array_equal(blocks.cpu().numpy(), r.blocks) and st.levels == r.stats.levels
+    return st.levels, ctx.profile_read()["contract"]["launches"]
+
+
+# 4608 nodes and 49152 entries are the limits; persistent launches switched off take the one-CTA levels with them.
+# 321 nodes have a cluster bound of 1: nothing merges, and the level is discarded where it was tried
+@pytest.mark.parametrize("n,m,kw,tail", [(321, 500, {}, True), (4608, 24576, {}, True), (4609, 20000, {}, False),
+                                         (4600, 24577, {}, False), (4600, 20000, {"small_lp_nodes": 1000}, False)])
+def test_one_cta_levels_run(ctx, n, m, kw, tail):
+    levels, alone = _levels(ctx, gg.er(n, m, 6), 2, max_levels=1, **kw)
+    assert levels == (0 if n == 321 else 1) and alone == (0 if tail else 1)
+
+
+def test_one_cta_levels_below_the_limits(ctx):
+    levels, alone = _levels(ctx, gg.er(30000, 90000, 6), 2)
+    assert 0 < alone < levels
+
+
+# the arena for the way down, and for the way down but not for the way up
+@pytest.mark.parametrize("slack", [-10 ** 9, -1500000, -1000000, -700000, -500000, -250000, 0])
+def test_one_cta_levels_without_room(ctx, slack):
+    limits(ctx, tail_slack=slack)
+    levels, alone = _levels(ctx, gg.with_edge_weights(gg.er(4000, 20000, 2), 3), 3)
+    assert levels > 0 and (alone > 0 if slack < -10 ** 8 else alone <= levels)
