@@ -78,10 +78,12 @@ void gp_set_wait_limit(gp_ctx *ctx, int64_t spins) {
 }
 
 // For tests, not part of the C-ABI (gp.h): the context's Limits.
-void gp_test_limits(gp_ctx *ctx, int32_t hash_collect, int64_t table_slack, int64_t tail_slack) {
+void gp_test_limits(gp_ctx *ctx, int32_t hash_collect, int64_t table_slack, int64_t tail_slack,
+                    int32_t few_nodes) {
   ctx->limits.hash_collect = hash_collect;
   ctx->limits.table_slack = table_slack;
   ctx->limits.tail_slack = tail_slack;
+  ctx->limits.few_nodes = few_nodes;
 }
 
 const char *gp_version(void) { return "gp-gb300 1.0 (sm_103a)"; }

@@ -102,6 +102,7 @@ namespace gp {
 struct Limits {
   int32_t hash_collect = 16384;       // exact sampler: edges fetched and ordered on the host
   int64_t table_slack = 16 << 20;     // hash tables in global memory: bytes beyond 8 per CSR entry
+  int32_t few_nodes = 72;             // LP sub-rounds: nodes an SM rated together per launch saved (0: a launch per class)
   int64_t tail_slack = 4 << 20;       // one-CTA levels: arena bytes beyond those per node, entry and block
 
   int64_t table_bytes(int64_t m2) const { return std::max<int64_t>(0, 8 * m2 + table_slack); }

@@ -35,6 +35,7 @@ struct RateArgs {
   const int4 *list;     // bucket list: (node, row offset, degree, node weight)
   const int32_t *offs;
   int key;
+  int nkeys;            // k_rate_warp, k_rate_block: buckets of the launch, from key on
   int64_t bound;
   uint64_t ktie;
   int2 *prop;           // RATE_LP: per list position (proposed label or -1, own label)
@@ -50,8 +51,17 @@ struct RateArgs {
   const int32_t *ccount;  // optional: the list holds ccount[key] records from offs[key] (compacted)
 };
 
-__device__ __forceinline__ int list_end(const RateArgs &a) {
-  return a.ccount ? a.offs[a.key] + a.ccount[a.key] : a.offs[a.key + 1];
+__device__ __forceinline__ int list_end(const RateArgs &a, int key) {
+  return a.ccount ? a.offs[key] + a.ccount[key] : a.offs[key + 1];
+}
+__device__ __forceinline__ int list_end(const RateArgs &a) { return list_end(a, a.key); }
+
+// The first of a bucket's records [begin, end) for worker `id` of nw, which go through the buckets of a launch as if
+// they were one list; done: records of the buckets before, modulo nw.
+__device__ __forceinline__ int bucket_first(int begin, int end, int id, int nw, int &done) {
+  const int at = id >= done ? id - done : id - done + nw;
+  done = (int)(((unsigned)done + (unsigned)(end - begin)) % (unsigned)nw);
+  return begin + at;
 }
 
 __device__ __forceinline__ void add_units(unsigned long long *units, unsigned long long e,
@@ -283,74 +293,76 @@ __global__ void __launch_bounds__(kThreads) k_rate_warp(RateArgs a, int slots) {
   for (int t = lane; t < slots; t += 32) { tk[t] = -1; tv[t] = 0; }
   __syncwarp();
   if (a.stop && *a.stop) return;
-  const int begin = a.offs[a.key], end = list_end(a);
   const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int nw = (int)((gridDim.x * blockDim.x) >> 5);
   unsigned long long ue = 0, uv = 0, uc = 0, up = 0;
-  for (int i = begin + wid; i < end; i += nw) {
-    const int4 rec = a.list[i];
-    const int v = rec.x, start = rec.y, deg = rec.z, cv = rec.w;
-    if (a.dirty && !a.dirty[v]) {  // clean: cannot move
-      if (MODE == RATE_LP && lane == 0) a.prop[i] = make_int2(-1, 0);
-      continue;
-    }
-    const int own = label_of(a, v);
-    const int tsize = tab_slots(deg, kTabQ4);
-    for (int j0 = lane; j0 < deg; j0 += 32 * kWarpUnroll) {
-      int L[kWarpUnroll], w[kWarpUnroll];
-#pragma unroll
-      for (int r = 0; r < kWarpUnroll; r++) {
-        const int j = j0 + r * 32;
-        L[r] = j < deg ? __ldcs(a.adjncy + start + j) : -1;
-        w[r] = j < deg && a.adjwgt ? __ldcs(a.adjwgt + start + j) : 1;
+  for (int b = 0, done = 0; b < a.nkeys; b++) {
+    const int begin = a.offs[a.key + b], end = list_end(a, a.key + b);
+    for (int i = bucket_first(begin, end, wid, nw, done); i < end; i += nw) {
+      const int4 rec = a.list[i];
+      const int v = rec.x, start = rec.y, deg = rec.z, cv = rec.w;
+      if (a.dirty && !a.dirty[v]) {  // clean: cannot move
+        if (MODE == RATE_LP && lane == 0) a.prop[i] = make_int2(-1, 0);
+        continue;
       }
+      const int own = label_of(a, v);
+      const int tsize = tab_slots(deg, kTabQ4);
+      for (int j0 = lane; j0 < deg; j0 += 32 * kWarpUnroll) {
+        int L[kWarpUnroll], w[kWarpUnroll];
 #pragma unroll
-      for (int r = 0; r < kWarpUnroll; r++) L[r] = L[r] >= 0 ? label_of(a, L[r]) : -1;
+        for (int r = 0; r < kWarpUnroll; r++) {
+          const int j = j0 + r * 32;
+          L[r] = j < deg ? __ldcs(a.adjncy + start + j) : -1;
+          w[r] = j < deg && a.adjwgt ? __ldcs(a.adjwgt + start + j) : 1;
+        }
 #pragma unroll
-      for (int r = 0; r < kWarpUnroll; r++) {
-        if (L[r] < 0) continue;
-        int s = (int)__umulhi((unsigned)L[r] * 2654435761u, (unsigned)tsize);
-        for (int probe = 0; probe < tsize; probe++) {  // bounded: more slots than neighbours
-          const int prev = atomicCAS(&tk[s], -1, L[r]);
-          if (prev == -1 || prev == L[r]) { atomicAdd(&tv[s], w[r]); break; }
-          s = s + 1 == tsize ? 0 : s + 1;
+        for (int r = 0; r < kWarpUnroll; r++) L[r] = L[r] >= 0 ? label_of(a, L[r]) : -1;
+#pragma unroll
+        for (int r = 0; r < kWarpUnroll; r++) {
+          if (L[r] < 0) continue;
+          int s = (int)__umulhi((unsigned)L[r] * 2654435761u, (unsigned)tsize);
+          for (int probe = 0; probe < tsize; probe++) {  // bounded: more slots than neighbours
+            const int prev = atomicCAS(&tk[s], -1, L[r]);
+            if (prev == -1 || prev == L[r]) { atomicAdd(&tv[s], w[r]); break; }
+            s = s + 1 == tsize ? 0 : s + 1;
+          }
         }
       }
-    }
-    __syncwarp();
-    int own_loc = 0, rloc = -1, nc = 0, rall = 0;
-    for (int t = lane; t < tsize; t += 32) {
-      const int L = tk[t];
-      if (L < 0) continue;
-      const int r = tv[t];
-      if (L == own) { own_loc = r; continue; }
-      nc++;
-      rall = r > rall ? r : rall;
-      if (r > rloc && (MODE != RATE_LP || (int64_t)a.weight[L] + cv <= a.bound)) rloc = r;  // only a better one matters
-    }
-    const int own_r = __reduce_max_sync(FULL, own_loc);
-    const int rmax = __reduce_max_sync(FULL, rloc);
-    if (a.dirty && __reduce_max_sync(FULL, rall) <= own_r && lane == 0) a.dirty[v] = 0;
-    ue += deg; uv += 1; uc += nc;
-    const bool want = !(rmax < 0 || (MODE == RATE_LP && rmax <= own_r));
-    uint64_t packed = ~0ull;
-    for (int t = lane; t < tsize; t += 32) {
-      const int L = tk[t];
-      if (L < 0) continue;
-      if (want && L != own && tv[t] == rmax && (MODE != RATE_LP || (int64_t)a.weight[L] + cv <= a.bound)) {
-        const uint64_t p = ((uint64_t)h32(a.ktie, (uint32_t)v, (uint32_t)L) << 32) | (uint32_t)L;
-        packed = p < packed ? p : packed;
+      __syncwarp();
+      int own_loc = 0, rloc = -1, nc = 0, rall = 0;
+      for (int t = lane; t < tsize; t += 32) {
+        const int L = tk[t];
+        if (L < 0) continue;
+        const int r = tv[t];
+        if (L == own) { own_loc = r; continue; }
+        nc++;
+        rall = r > rall ? r : rall;
+        if (r > rloc && (MODE != RATE_LP || (int64_t)a.weight[L] + cv <= a.bound)) rloc = r;  // only a better one matters
       }
-      tk[t] = -1;
-      tv[t] = 0;
+      const int own_r = __reduce_max_sync(FULL, own_loc);
+      const int rmax = __reduce_max_sync(FULL, rloc);
+      if (a.dirty && __reduce_max_sync(FULL, rall) <= own_r && lane == 0) a.dirty[v] = 0;
+      ue += deg; uv += 1; uc += nc;
+      const bool want = !(rmax < 0 || (MODE == RATE_LP && rmax <= own_r));
+      uint64_t packed = ~0ull;
+      for (int t = lane; t < tsize; t += 32) {
+        const int L = tk[t];
+        if (L < 0) continue;
+        if (want && L != own && tv[t] == rmax && (MODE != RATE_LP || (int64_t)a.weight[L] + cv <= a.bound)) {
+          const uint64_t p = ((uint64_t)h32(a.ktie, (uint32_t)v, (uint32_t)L) << 32) | (uint32_t)L;
+          packed = p < packed ? p : packed;
+        }
+        tk[t] = -1;
+        tv[t] = 0;
+      }
+      if (want) {
+        packed = warp_min(packed);
+        if (lane == 0) { emit<MODE>(a, i, v, (int)(uint32_t)packed, cv, own); up += 1; }
+      } else if (MODE == RATE_LP && lane == 0) {
+        a.prop[i] = make_int2(-1, 0);
+      }
+      __syncwarp();
     }
-    if (want) {
-      packed = warp_min(packed);
-      if (lane == 0) { emit<MODE>(a, i, v, (int)(uint32_t)packed, cv, own); up += 1; }
-    } else if (MODE == RATE_LP && lane == 0) {
-      a.prop[i] = make_int2(-1, 0);
-    }
-    __syncwarp();
   }
   add_units(a.units, ue * (lane == 0), uv * (lane == 0), uc, up, a.label8 != nullptr, a.adjwgt == nullptr);
 }
@@ -497,78 +509,80 @@ __global__ void __launch_bounds__(NT) k_rate_block(RateArgs a, int slots, int q4
   if (a.stop && *a.stop) return;
   int *tk = s_tab, *tv = s_tab + slots;
   for (int t = threadIdx.x; t < slots; t += NT) { tk[t] = -1; tv[t] = 0; }
-  const int begin = a.offs[a.key], end = list_end(a);
   unsigned long long ue = 0, uv = 0, uc = 0, up = 0;
-  for (int i = begin + (int)blockIdx.x; i < end; i += (int)gridDim.x) {
-    const int4 rec = a.list[i];
-    const int v = rec.x, start = rec.y, deg = rec.z, cv = rec.w;
-    if (a.dirty && !a.dirty[v]) {  // clean: cannot move (uniform in the block)
-      if (threadIdx.x == 0) a.prop[i] = make_int2(-1, 0);
-      continue;
-    }
-    const int own = label_of(a, v);
-    const int tsize = tab_slots(deg, q4);
-    if (threadIdx.x == 0) s_own = 0;
-    __syncthreads();  // the table is empty, and the flag of the clean nodes was read before it may change
-    for (int j0 = threadIdx.x; j0 < deg; j0 += NT * kBlockUnroll) {
-      int L[kBlockUnroll], w[kBlockUnroll];
-#pragma unroll
-      for (int r = 0; r < kBlockUnroll; r++) {
-        const int j = j0 + r * NT;
-        L[r] = j < deg ? __ldcs(a.adjncy + start + j) : -1;
-        w[r] = j < deg && a.adjwgt ? __ldcs(a.adjwgt + start + j) : 1;
+  for (int b = 0, done = 0; b < a.nkeys; b++) {
+    const int begin = a.offs[a.key + b], end = list_end(a, a.key + b);
+    for (int i = bucket_first(begin, end, (int)blockIdx.x, (int)gridDim.x, done); i < end; i += (int)gridDim.x) {
+      const int4 rec = a.list[i];
+      const int v = rec.x, start = rec.y, deg = rec.z, cv = rec.w;
+      if (a.dirty && !a.dirty[v]) {  // clean: cannot move (uniform in the block)
+        if (threadIdx.x == 0) a.prop[i] = make_int2(-1, 0);
+        continue;
       }
+      const int own = label_of(a, v);
+      const int tsize = tab_slots(deg, q4);
+      if (threadIdx.x == 0) s_own = 0;
+      __syncthreads();  // the table is empty, and the flag of the clean nodes was read before it may change
+      for (int j0 = threadIdx.x; j0 < deg; j0 += NT * kBlockUnroll) {
+        int L[kBlockUnroll], w[kBlockUnroll];
 #pragma unroll
-      for (int r = 0; r < kBlockUnroll; r++) L[r] = L[r] >= 0 ? label_of(a, L[r]) : -1;
+        for (int r = 0; r < kBlockUnroll; r++) {
+          const int j = j0 + r * NT;
+          L[r] = j < deg ? __ldcs(a.adjncy + start + j) : -1;
+          w[r] = j < deg && a.adjwgt ? __ldcs(a.adjwgt + start + j) : 1;
+        }
 #pragma unroll
-      for (int r = 0; r < kBlockUnroll; r++) {
-        if (L[r] < 0) continue;
-        int s = (int)__umulhi((unsigned)L[r] * 2654435761u, (unsigned)tsize);
-        for (int probe = 0; probe < tsize; probe++) {  // bounded: more slots than neighbours
-          const int prev = atomicCAS(&tk[s], -1, L[r]);
-          if (prev == -1 || prev == L[r]) { atomicAdd(&tv[s], w[r]); break; }
-          s = s + 1 == tsize ? 0 : s + 1;
+        for (int r = 0; r < kBlockUnroll; r++) L[r] = L[r] >= 0 ? label_of(a, L[r]) : -1;
+#pragma unroll
+        for (int r = 0; r < kBlockUnroll; r++) {
+          if (L[r] < 0) continue;
+          int s = (int)__umulhi((unsigned)L[r] * 2654435761u, (unsigned)tsize);
+          for (int probe = 0; probe < tsize; probe++) {  // bounded: more slots than neighbours
+            const int prev = atomicCAS(&tk[s], -1, L[r]);
+            if (prev == -1 || prev == L[r]) { atomicAdd(&tv[s], w[r]); break; }
+            s = s + 1 == tsize ? 0 : s + 1;
+          }
         }
       }
-    }
-    __syncthreads();
-    int rloc = -1, rall = 0, nc = 0;
-    for (int t = threadIdx.x; t < tsize; t += NT) {
-      const int L = tk[t];
-      if (L < 0) continue;
-      const int r = tv[t];
-      if (L == own) { s_own = r; continue; }
-      nc++;
-      rall = r > rall ? r : rall;
-      if (r > rloc && (int64_t)a.weight[L] + cv <= a.bound) rloc = r;  // only what beats the thread's best matters
-    }
-    const int rmax = block_max_n<NT>(rloc, s_ri);  // its barriers also publish s_own
-    const int own_r = s_own;
-    if (a.dirty) {
-      rall = block_max_n<NT>(rall, s_ri);
-      if (rall <= own_r && threadIdx.x == 0) a.dirty[v] = 0;
-    }
-    uc += nc;
-    const bool want = rmax >= 0 && rmax > own_r;
-    uint64_t packed = ~0ull;
-    for (int t = threadIdx.x; t < tsize; t += NT) {
-      const int L = tk[t];
-      if (L < 0) continue;
-      if (want && L != own && tv[t] == rmax && (int64_t)a.weight[L] + cv <= a.bound) {
-        const uint64_t p = ((uint64_t)h32(a.ktie, (uint32_t)v, (uint32_t)L) << 32) | (uint32_t)L;
-        packed = p < packed ? p : packed;
+      __syncthreads();
+      int rloc = -1, rall = 0, nc = 0;
+      for (int t = threadIdx.x; t < tsize; t += NT) {
+        const int L = tk[t];
+        if (L < 0) continue;
+        const int r = tv[t];
+        if (L == own) { s_own = r; continue; }
+        nc++;
+        rall = r > rall ? r : rall;
+        if (r > rloc && (int64_t)a.weight[L] + cv <= a.bound) rloc = r;  // only what beats the thread's best matters
       }
-      tk[t] = -1;
-      tv[t] = 0;
+      const int rmax = block_max_n<NT>(rloc, s_ri);  // its barriers also publish s_own
+      const int own_r = s_own;
+      if (a.dirty) {
+        rall = block_max_n<NT>(rall, s_ri);
+        if (rall <= own_r && threadIdx.x == 0) a.dirty[v] = 0;
+      }
+      uc += nc;
+      const bool want = rmax >= 0 && rmax > own_r;
+      uint64_t packed = ~0ull;
+      for (int t = threadIdx.x; t < tsize; t += NT) {
+        const int L = tk[t];
+        if (L < 0) continue;
+        if (want && L != own && tv[t] == rmax && (int64_t)a.weight[L] + cv <= a.bound) {
+          const uint64_t p = ((uint64_t)h32(a.ktie, (uint32_t)v, (uint32_t)L) << 32) | (uint32_t)L;
+          packed = p < packed ? p : packed;
+        }
+        tk[t] = -1;
+        tv[t] = 0;
+      }
+      if (want) packed = block_min_n<NT>(packed, s_ru);
+      if (threadIdx.x == 0) {
+        ue += deg;
+        uv += 1;
+        if (want) { emit<RATE_LP>(a, i, v, (int)(uint32_t)packed, cv, own); up += 1; }
+        else a.prop[i] = make_int2(-1, 0);
+      }
+      __syncthreads();
     }
-    if (want) packed = block_min_n<NT>(packed, s_ru);
-    if (threadIdx.x == 0) {
-      ue += deg;
-      uv += 1;
-      if (want) { emit<RATE_LP>(a, i, v, (int)(uint32_t)packed, cv, own); up += 1; }
-      else a.prop[i] = make_int2(-1, 0);
-    }
-    __syncthreads();
   }
   add_units(a.units, ue, uv, uc, up, a.label8 != nullptr, a.adjwgt == nullptr);
 }
@@ -1774,29 +1788,69 @@ void launch_block(gp_ctx *ctx, const RateArgs &a, int maxdeg, int q4, int grid) 
   GP_LAUNCH_CHECK();
 }
 
+template <int MODE>
+void launch_warps(gp_ctx *ctx, const RateArgs &a, int maxdeg, int count) {
+  const int slots = tab_slots(maxdeg, kTabQ4);
+  const size_t smem = 2 * sizeof(int) * (size_t)slots * kWarpsPerBlock;
+  if (smem > 48 * 1024)
+    GP_CUDA(cudaFuncSetAttribute(k_rate_warp<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k_rate_warp<MODE><<<rate_grid(ctx, count, kWarpsPerBlock, ctx->num_sms * 8), kThreads, smem, ctx->stream>>>(a, slots);
+  GP_LAUNCH_CHECK();
+}
+
+// A sub-round of few nodes is a chain of launches of some 5 us each, one per class that is not empty.  The classes
+// up to kWarpMaxDeg go through k_rate_warp together while they hold at most Limits::few_nodes nodes an SM for each launch
+// that this saves (24 warps an SM take about 1.5 us for a node each), and up to one node an SM of the block
+// classes through the largest of these.  A launch per class / together, on the per-phase path: refinement with k = 64 of
+// scale-10, -14 and -18 R-MAT graphs 4.5 / 3.0, 5.9 / 4.1 and 7.6 / 5.9 ms, of an ER graph of 65,536 nodes 4.4 / 3.2; clustering
+// of the scale-14 and -18 graphs 5.6 / 3.5 and 8.3 / 5.1 ms.  With one class (a mesh) nothing is saved and a warp per
+// node takes longer.
+
 // nlabels: number of labels
 template <int MODE>
 void launch_rate(gp_ctx *ctx, RateArgs a, int bucket_key_base, const RateTables &t, int64_t nlabels,
                  const int *hcnt) {
-  const int cap = ctx->num_sms * 8;
-  if (MODE == RATE_LP && a.label8) launch_groups<MODE, LK_NARROW>(ctx, a, bucket_key_base, hcnt);
-  else launch_groups<MODE, LK_WIDE>(ctx, a, bucket_key_base, hcnt);
-  for (int q = 0; q < 2; q++) {  // a warp per node; favourites of larger nodes: k_rate_large
-    const int b = kMediumBucket + q;
-    if ((hcnt && hcnt[b] == 0) || (q == 1 && MODE != RATE_LP)) continue;
-    a.key = bucket_key_base + b;
-    const int slots = tab_slots(q == 0 ? kMediumMaxDeg : kWarpMaxDeg, kTabQ4);
-    const size_t smem = 2 * sizeof(int) * (size_t)slots * kWarpsPerBlock;
-    if (smem > 48 * 1024)
-      GP_CUDA(cudaFuncSetAttribute(k_rate_warp<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_rate_warp<MODE><<<rate_grid(ctx, hcnt ? hcnt[b] : -1, kWarpsPerBlock, cap), kThreads, smem, ctx->stream>>>(a, slots);
-    GP_LAUNCH_CHECK();
+  a.nkeys = 1;
+  int warps = 0, warp_classes = 0, blocks = 0, block_classes = 0;
+  if (hcnt) {
+    for (int b = 0; b < kMediumBucket + 2; b++) {
+      warps += hcnt[b];
+      warp_classes += hcnt[b] > 0;
+    }
+    for (int b = kMediumBucket + 2; b < kMediumBucket + 5; b++) {
+      blocks += hcnt[b];
+      block_classes += hcnt[b] > 0;
+    }
+  }
+  const int few = ctx->limits.few_nodes * ctx->num_sms;
+  if (MODE == RATE_LP && warp_classes > 1 && warps <= (int64_t)few * (warp_classes - 1)) {
+    a.key = bucket_key_base;
+    a.nkeys = kMediumBucket + 2;
+    launch_warps<MODE>(ctx, a, kWarpMaxDeg, warps);
+    a.nkeys = 1;
+  } else {
+    if (MODE == RATE_LP && a.label8) launch_groups<MODE, LK_NARROW>(ctx, a, bucket_key_base, hcnt);
+    else launch_groups<MODE, LK_WIDE>(ctx, a, bucket_key_base, hcnt);
+    for (int q = 0; q < 2; q++) {  // a warp per node; favourites of larger nodes: k_rate_large
+      const int b = kMediumBucket + q;
+      if ((hcnt && hcnt[b] == 0) || (q == 1 && MODE != RATE_LP)) continue;
+      a.key = bucket_key_base + b;
+      launch_warps<MODE>(ctx, a, q == 0 ? kMediumMaxDeg : kWarpMaxDeg, hcnt ? hcnt[b] : -1);
+    }
+  }
+  const bool together =
+      MODE == RATE_LP && few > 0 && !(t.hubs && t.dense) && block_classes > 1 && blocks <= ctx->num_sms;
+  if (together) {
+    a.key = bucket_key_base + kMediumBucket + 2;
+    a.nkeys = 3;
+    launch_block<1024>(ctx, a, kHubDeg, kTabQ4Last, blocks);
+    a.nkeys = 1;
   }
   const int hgrid = ctx->num_sms * 6;
   for (int q = MODE == RATE_LP ? 0 : -1; q < 4; q++) {  // the three block classes, the hubs
     const int b = kMediumBucket + 2 + q;
     const int c = hcnt ? hcnt[b] : -1;
-    if (c == 0) continue;
+    if (c == 0 || (together && q < 3)) continue;
     a.key = bucket_key_base + b;
     if (MODE == RATE_LP && t.hubs && (q == 3 || (q > 0 && t.dense))) {
       HubArgs h{t.hub.get(), t.chunk0.get(), t.tchunk0.get(), t.tab.get(), t.hist.get(), (int)nlabels, t.q4};

@@ -25,9 +25,9 @@ def ctx():
     c.close()
 
 
-def limits(ctx, hash_collect=16384, table_slack=16 << 20, tail_slack=4 << 20):
+def limits(ctx, hash_collect=16384, table_slack=16 << 20, tail_slack=4 << 20, few_nodes=72):
     ctx.lib.gp_test_limits(ctypes.c_void_p(ctx.ptr), ctypes.c_int32(hash_collect), ctypes.c_int64(table_slack),
-                           ctypes.c_int64(tail_slack))
+                           ctypes.c_int64(tail_slack), ctypes.c_int32(few_nodes))
 
 
 # edges of one weight that share a hash prefix: with a limit of 16384 one digit is read, with 64 or 1 one or two,
