@@ -105,7 +105,11 @@ __device__ __forceinline__ void emit(const RateArgs &a, int i, int v, int best, 
 // array); with 8 or 16 lanes per node and tables in shared memory a node of 20 neighbours took 225-300
 // warp instructions, so that issue and latency bound it instead.  The pairs cost D (D - 1) / 2 x 3
 // instructions per 32 nodes, a tenth of that, and every label of the row is in flight at once.
-// The clustering and refinement of a level of 16.8M nodes and 268M entries went from 25.6 to 21.7 ms.
+// A level of 16.8M nodes and 336M entries (clustering, contraction, sparsification, clustering of the result) went from
+// 25.6 to 21.7 ms; where the label array passes L2 (2^26 nodes) clustering's rating stays at the rate of its misses
+// (44 ms).  Refinement of that graph, unit weights, 128 one-byte labels: 59.6 ms with lane groups, 54.7 with this,
+// 60.2 with byte counters per thread in shared memory instead of the pairs (a fifth of the instructions, but 39 % of
+// the warps active and 28 % of the issue slots used).
 //
 // The choice is lazy in the label weights: candidates are ranked by (rating, tie hash, label) without the
 // bound, and only the best one's weight is read; if it does not fit, the weights of all that are rated
@@ -172,105 +176,6 @@ __global__ void __launch_bounds__(ThreadShape<D>::NT, ThreadShape<D>::PER_SM) k_
     }
   }
   add_units(a.units, ue, uv, uc, up, a.label8 != nullptr, a.adjwgt == nullptr);
-}
-
-// ------------- degree <= 32, unit weights, one-byte labels: counters per thread
-//
-// Refinement of an input with unit weights (level 1, the largest level): a rating is a count of at most
-// 32, so every thread counts its row in byte counters of its own, four to a word, in shared memory (word
-// [label / 4][thread]: no two lanes of a warp meet in a bank).  The pairs of k_rate_thread took 3100
-// instructions per 32 nodes of degree 17-24 and 106 registers (16 warps an SM, 80e9 entries/s); this takes
-// about a fifth of the instructions and half the registers.  It reaches
-// 105e9 entries/s on 2^26 nodes of degree 16, bound by the L1 path of the gathers.
-
-template <int D>
-__global__ void __launch_bounds__(128, D <= 16 ? 8 : 6) k_rate_bytes(RateArgs a) {
-  constexpr int NT = 128;
-  extern __shared__ unsigned s_cnt[];  // (wlabels + 3) / 4 words a thread, then the label weights
-  if (a.stop && *a.stop) return;
-  const int words = (a.wlabels + 3) / 4;
-  int *s_w = reinterpret_cast<int *>(s_cnt + words * NT);
-  unsigned *cnt = s_cnt + threadIdx.x;
-  for (int t = 0; t < words; t++) cnt[t * NT] = 0;
-  for (int t = threadIdx.x; t < a.wlabels; t += NT) s_w[t] = a.weight[t];
-  __syncthreads();
-  const bool vec = ((uintptr_t)a.adjncy & 15) == 0;
-  const int begin = a.offs[a.key], end = list_end(a);
-  unsigned long long ue = 0, uv = 0, uc = 0, up = 0;
-  for (int i0 = begin + (int)(blockIdx.x * NT); i0 < end; i0 += (int)(gridDim.x * NT)) {
-    const int i = i0 + (int)threadIdx.x;
-    const int4 rec = i < end ? a.list[i] : make_int4(-1, 0, 0, 0);
-    const int v = rec.x, cv = rec.w;
-    const bool live = v >= 0 && !(a.dirty && !a.dirty[v]);
-    const int st = live ? rec.y : 0, deg = live ? rec.z : 0;
-    const int own = live ? (int)a.label8[v] : 0;
-    unsigned P[D / 4];  // the labels, four to a word
-    {
-      int u[D];
-      load_row<D>(a.adjncy, st, deg, a.m2, vec, u);
-#pragma unroll
-      for (int q = 0; q < D; q++) u[q] = q < deg ? (int)a.label8[u[q]] : 0;
-#pragma unroll
-      for (int q = 0; q < D / 4; q++)
-        P[q] = (unsigned)u[4 * q] | (unsigned)u[4 * q + 1] << 8 | (unsigned)u[4 * q + 2] << 16 | (unsigned)u[4 * q + 3] << 24;
-    }
-    auto label = [&](int q) -> int { return (int)((P[q / 4] >> (8 * (q & 3))) & 255u); };
-    const int dm = __reduce_max_sync(FULL, deg);
-#pragma unroll
-    for (int q = 0; q < D; q++) {
-      if (q >= dm) break;
-      const int L = label(q);
-      if (q < deg) cnt[(L >> 2) * NT] += 1u << ((L & 3) * 8);
-    }
-    const int own_r = (int)((cnt[(own >> 2) * NT] >> ((own & 3) * 8)) & 255u);
-    const int room = room_of(a.bound, cv);
-    int rall = 0, r = own_r, lb = -1, nc = 0;
-    bool tie = false;
-#pragma unroll
-    for (int q = 0; q < D; q++) {
-      if (q >= dm) break;
-      const int L = label(q);
-      if (q >= deg || L == own) continue;
-      const int c = (int)((cnt[(L >> 2) * NT] >> ((L & 3) * 8)) & 255u);
-      nc++;
-      rall = c > rall ? c : rall;
-      if (c > own_r && c >= r && s_w[L] <= room) {
-        if (c > r) { r = c; lb = L; tie = false; }
-        else if (L != lb) tie = true;
-      }
-    }
-    if (tie) {
-      unsigned hb = 0xFFFFFFFFu;
-      lb = 0x7FFFFFFF;
-#pragma unroll
-      for (int q = 0; q < D; q++) {
-        const int L = label(q);
-        if (q >= deg || L == own) continue;
-        const int c = (int)((cnt[(L >> 2) * NT] >> ((L & 3) * 8)) & 255u);
-        if (c != r || s_w[L] > room) continue;
-        const unsigned h = h32(a.ktie, (uint32_t)v, (uint32_t)L);
-        if (h < hb || (h == hb && L < lb)) { hb = h; lb = L; }
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < D; q++) {
-      if (q >= dm) break;
-      if (q < deg) cnt[(label(q) >> 2) * NT] = 0;
-    }
-    if (a.dirty && live && rall <= own_r) a.dirty[v] = 0;
-    uc += nc;
-    if (live) {
-      ue += deg;
-      uv += 1;
-    }
-    if (lb >= 0) {
-      emit<RATE_LP>(a, i, v, lb, cv, own);
-      up += 1;
-    } else if (v >= 0) {
-      a.prop[i] = make_int2(-1, 0);
-    }
-  }
-  add_units(a.units, ue, uv, uc, up, true, true);
 }
 
 // ------------------------- degree <= 128, <= 512: warp/node, shared table
@@ -1752,26 +1657,10 @@ void launch_threads(gp_ctx *ctx, RateArgs a, int key, int count) {
   GP_LAUNCH_CHECK();
 }
 
-template <int D>
-void launch_bytes(gp_ctx *ctx, RateArgs a, int key, int count) {
-  if (count == 0) return;
-  a.key = key;
-  const size_t smem = sizeof(int) * ((size_t)((a.wlabels + 3) / 4) * 128 + (size_t)a.wlabels);
-  k_rate_bytes<D><<<rate_grid(ctx, count, 128, ctx->num_sms * 16), 128, smem, ctx->stream>>>(a);
-  GP_LAUNCH_CHECK();
-}
-
 // hcnt: the bucket sizes of this sub-round when the host knows them (empty buckets are then not
 // launched), else nullptr
 template <int MODE, int LK>
 void launch_groups(gp_ctx *ctx, const RateArgs &a, int base, const int *hcnt) {
-  if (LK == LK_NARROW && a.adjwgt == nullptr && hcnt) {
-    launch_bytes<8>(ctx, a, base + 0, hcnt[0]);
-    launch_bytes<16>(ctx, a, base + 1, hcnt[1]);
-    launch_bytes<24>(ctx, a, base + 2, hcnt[2]);
-    launch_bytes<32>(ctx, a, base + 3, hcnt[3]);
-    return;
-  }
   launch_threads<MODE, 8, LK>(ctx, a, base + 0, hcnt ? hcnt[0] : -1);
   launch_threads<MODE, 16, LK>(ctx, a, base + 1, hcnt ? hcnt[1] : -1);
   launch_threads<MODE, 24, LK>(ctx, a, base + 2, hcnt ? hcnt[2] : -1);
@@ -1829,7 +1718,7 @@ void launch_rate(gp_ctx *ctx, RateArgs a, int bucket_key_base, const RateTables 
     launch_warps<MODE>(ctx, a, kWarpMaxDeg, warps);
     a.nkeys = 1;
   } else {
-    if (MODE == RATE_LP && a.label8) launch_groups<MODE, LK_NARROW>(ctx, a, bucket_key_base, hcnt);
+    if (MODE == RATE_LP && a.label8) launch_groups<MODE, MODE == RATE_LP ? LK_NARROW : LK_WIDE>(ctx, a, bucket_key_base, hcnt);
     else launch_groups<MODE, LK_WIDE>(ctx, a, bucket_key_base, hcnt);
     for (int q = 0; q < 2; q++) {  // a warp per node; favourites of larger nodes: k_rate_large
       const int b = kMediumBucket + q;
