@@ -355,6 +355,8 @@ typedef struct gp_batch_tuning {
   double class_path_gps[GP_TUNE_CLASSES];    /* per-graph path graphs/s on the class (0: not measured) */
   double tune_ms;                            /* wall time of the tuning */
 } gp_batch_tuning;
+/* gp_batch_get_tuning returns the settings in the context; while none has been set or measured these are the
+ * defaults before they are narrowed per batch.  Setting them as returned makes them the caller's: not narrowed. */
 void gp_batch_tuning_default(gp_batch_tuning *t);
 gp_status gp_batch_set_tuning(gp_ctx *ctx, const gp_batch_tuning *t);
 gp_status gp_batch_get_tuning(gp_ctx *ctx, gp_batch_tuning *t);
@@ -371,8 +373,8 @@ gp_status gp_batch_autotune(gp_ctx *ctx, const gp_batch_item *items, int32_t cou
  * admitted).  Requests in flight overlap on the GPU.  Each request is the
  * host-array partition of gp_partition_host, so its blocks and cut equal a
  * gp_partition_host call with the same arguments, alone or in any mix.
- * The estimate is 4x the request's CSR bytes plus 64 bytes per node plus
- * 64 MiB; a request whose estimate exceeds the budget is refused at submit
+ * The estimate is 4x the request's CSR bytes plus 8 bytes per CSR entry plus
+ * 128 bytes per node plus 80 MiB; a request whose estimate exceeds the budget is refused at submit
  * with GP_ERR_BUDGET.  A worker's pool is trimmed back to 1/workers of the
  * budget after each request.
  */

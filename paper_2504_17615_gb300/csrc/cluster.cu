@@ -59,11 +59,6 @@ __global__ void k_fav_apply(const uint64_t *keys, int count, const int32_t *merg
   }
 }
 
-__global__ void k_fav_clear(const uint64_t *keys, int count, int32_t *cmax) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x)
-    cmax[(int)(keys[i] >> 32)] = 0;
-}
-
 __global__ void k_iso_flags(const int32_t *xadj, const int32_t *vwgt, int n, int64_t U, int32_t *flag,
                             int *cmax) {
   int m = 0;

@@ -12,7 +12,8 @@
 //  merge  : each segment is summed by coarse neighbour in a hash table (a
 //           warp with a shared-memory table up to 128 entries, a block with
 //           a 4096-slot shared table up to 2048, many blocks with a table in
-//           global memory above) and written back in place, compacted;
+//           global memory above, or a block each where those tables together
+//           would pass the memory bound) and written back in place, compacted;
 // and the merged rows are finally packed into the coarse CSR.  Row order
 // inside a coarse row is unspecified.
 #include "gp_internal.cuh"

@@ -21,8 +21,7 @@
 // cut equal a gp_partition call with the same arguments.  Only the execution
 // differs: block-wide scans, an LSD radix sort in global memory, lane-group
 // rating (the per-graph path's rate_group) for nodes of degree <= 128 and a
-// CTA-wide table for larger ones, and a named barrier per group of four warps
-// that runs one bisection trial.
+// CTA-wide table for larger ones, and a warp per bisection trial.
 //
 // Memory: each CTA owns an arena of fixed size carved out of one allocation.
 // The hierarchy of the current graph grows from the bottom of the arena,

@@ -257,10 +257,6 @@ struct TraceTimer {
   }
 };
 
-// ---------------------------------------------------------------- launch
-
-constexpr int kWarp = 32;
-
 // ------------------------------------------------------------------ hash
 
 // Keyed counter hash of the method (SplitMix64 output finaliser of Steele,
@@ -340,15 +336,6 @@ __device__ __forceinline__ T warp_min(T v) {
     v = x < v ? x : v;
   }
   return v;
-}
-
-// Adds `val` into *addr, aggregating lanes that target the same address.
-__device__ __forceinline__ void warp_agg_add(int *base, int idx, int val, bool pred) {
-  unsigned act = __ballot_sync(0xFFFFFFFFu, pred);
-  if (!pred) return;
-  unsigned peers = __match_any_sync(act, idx);
-  int sum = __reduce_add_sync(peers, val);
-  if ((int)lane_id() == __ffs(peers) - 1) atomicAdd(base + idx, sum);
 }
 
 // Row of CSR entry e: the largest r < n with xadj[r] <= e.

@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(kThreads) k_rate_warp(RateArgs a, int slots) {
   add_units(a.units, ue * (lane == 0), uv * (lane == 0), uc, up, a.label8 != nullptr, a.adjwgt == nullptr);
 }
 
-// --------------------------------------------- degree > 128: block/node
+// ---- a block per node: favourites of degree > 128, and hubs when their tables would pass the memory bound
 
 __device__ __forceinline__ int block_max_i32(int v, int *s_red) {
   v = warp_max(v);
@@ -1537,13 +1537,6 @@ __global__ void __launch_bounds__(kThreads) k_close(ApplyArgs a, int64_t count_l
 __global__ void k_counters_init(Counters *cnt, long long nclusters) {
   cnt->stop = 0; cnt->nov = 0; cnt->nmov = 0; cnt->pad0 = 0; cnt->moved_sub = 0; cnt->moved_round = 0;
   cnt->moved_total = 0; cnt->nonempty = 0; cnt->nclusters = nclusters;
-}
-
-
-__global__ void k_fill_i32(int32_t *a, int64_t n, int32_t v) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    a[i] = v;
 }
 
 // Largest degree, number of nodes above kBlockDeg0, number of hubs and their neighbours.
