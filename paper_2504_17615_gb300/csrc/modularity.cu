@@ -27,7 +27,7 @@ __device__ __forceinline__ bool in_range(int L, int nl) { return L >= 0 && L < n
 constexpr int kModUnroll = 4;
 constexpr int kModShared = 2048;
 
-__global__ void __launch_bounds__(256) k_mod_rows(const int32_t *xadj, const int32_t *adjncy,
+__global__ void __launch_bounds__(256, 6) k_mod_rows(const int32_t *xadj, const int32_t *adjncy,
                                                   const int32_t *adjwgt, const int32_t *label, int n, int nl, int nsh,
                                                   unsigned long long *vol, ModOut *o) {
   __shared__ unsigned s_deg[8][32];

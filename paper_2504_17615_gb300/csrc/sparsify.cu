@@ -87,9 +87,8 @@ __device__ __forceinline__ bool keep_entry(const KeepArgs &a, int row, int v, in
 
 // WRITE = false: kept entries per row; WRITE = true: the kept entries, compacted.  Bound by the instructions of the
 // hash and of the walk (three quarters of the issue slots).  Against a warp per 32 rows, uniform mode: scale-21
-// R-MAT 5.8 -> .31 ms, meshes and random graphs of up to some million entries 3 to 20 % slower (216,000-node mesh
-// .064 -> .076 ms, 1M nodes and 21M entries .175 -> .195), 268M and 537M entries 3 %: every warp begins with a
-// search.
+// R-MAT 5.7 -> .31 ms; meshes and random graphs of up to some million entries 3 to 20 % slower, for every warp begins
+// with a search (216,000-node mesh .064 -> .077 ms, 1M nodes and 21M entries .176 -> .188); 134M and 537M entries the same.
 template <bool WRITE>
 __global__ void __launch_bounds__(256, 7) k_keep(KeepArgs a) {
   __shared__ int s_cnt[8][32];

@@ -46,6 +46,7 @@ struct EntryWalk {
   int xs, xe;        // this lane's row
   int split;         // the lane whose row goes on in the next share (-1: none)
   bool no_empty;     // no row of the window is empty
+  int ended;         // rows of the window that end at or before the entry that owner is asked for next
   __device__ __forceinline__ EntryWalk(const int32_t *x, int nn, int wid, int nw) : xadj(x), n((unsigned)nn) {
     // the search's first 32 places, at doubling distances around where even degrees would put the share: read
     // together with the first and the last offset
@@ -69,7 +70,7 @@ struct EntryWalk {
       pos = cut(row, start, next, (unsigned)from);
       if (pos < lo) pos = lo;
     }
-    u0 = 0; e0 = e1 = xs = xe = 0; split = -1; no_empty = false;
+    u0 = 0; e0 = e1 = xs = xe = 0; split = -1; no_empty = false; ended = 0;
   }
   __device__ __forceinline__ bool next() {
     while (row < n) {
@@ -95,6 +96,7 @@ struct EntryWalk {
       e0 = pos;
       e1 = pos = stop;
       no_empty = __all_sync(0xFFFFFFFFu, xs < xe);
+      ended = 0;
       return true;
     }
     return false;
@@ -129,15 +131,17 @@ struct EntryWalk {
     if (!upper) end = xadj[b];
     return a;
   }
-  // Lane index of the row that holds entry f + lane (f the same in the whole warp): the lanes whose row
-  // ends at or before it.  Without empty rows in the window every row end is another position, so the
-  // ends among the 32 entries form a bit mask, and a count of its lower bits replaces the search (one
-  // reduction instead of five dependent shuffles).
-  __device__ __forceinline__ int owner(int f) const {
+  // Lane index of the row that holds entry f + lane (f the same in the whole warp, 32 on from the call before in
+  // this window): the lanes whose row ends at or before it.  Without empty rows in the window every row end is
+  // another position, so the ends among the 32 entries form a bit mask, and a count of its lower bits replaces
+  // the search (one reduction instead of five dependent shuffles).
+  __device__ __forceinline__ int owner(int f) {
     if (no_empty) {
-      const int d = xe - f;
-      const unsigned ends = __reduce_or_sync(0xFFFFFFFFu, d > 0 && d < 32 ? 1u << d : 0u);
-      return __popc(__ballot_sync(0xFFFFFFFFu, d <= 0)) + __popc(ends & (lanemask_lt() | (1u << lane_id())));
+      const unsigned d = (unsigned)(xe - f - 1);
+      const unsigned ends = __reduce_or_sync(0xFFFFFFFFu, d < 32 ? 1u << d : 0u);
+      const int q = ended + __popc(ends & lanemask_lt());
+      ended += __popc(ends);
+      return q;
     }
     const int e = f + (int)lane_id();
     int q = 0;
